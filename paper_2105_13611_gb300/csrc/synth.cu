@@ -36,12 +36,6 @@ namespace {
 
 constexpr float kLn10 = 2.302585092994046f;
 constexpr float kFourPi = 12.566370614359172f;
-constexpr float kFarV = 41.f;            // far formula valid for |v| >= 40
-// The far evaluation v = G_k (kv B) + kv E1 rounds two terms, each at most the larger of
-// the tile's span and the centre's distance in x = d ln q; with the centre at least one
-// tile (2048 points) from every point of the tile, |x| is at least that span, so v keeps
-// about 2e-7 relative accuracy.
-constexpr int kFarDist = kTile;
 
 __device__ __forceinline__ int floordiv(int a, int b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
 
@@ -342,8 +336,8 @@ struct __align__(16) LineRec {
     int c;
     float f, kv, a;
     float srel;
-    int jlo, jhi, ilo;
-    int ihi, pad0, pad1, pad2;
+    int ilo, ihi, jlo;
+    int jhi, pad0, pad1, pad2;
 };
 
 struct PrepOut {
@@ -703,66 +697,33 @@ struct RowDesc {
     float* out;                 // [N]
 };
 
-// flag bits of the per-line records in shared memory
-constexpr int kFlKloBits = 5;
-constexpr int kFlMask = (1 << kFlKloBits) - 1;
-constexpr int kFlChk = 1 << 10;      // points near the cut: test s_rel H >= 1
-constexpr int kFlAlt = 1 << 11;      // far: "y" form; near: expm1 series for v
-constexpr int kFlFull = 1 << 12;     // the window covers every slot of the tile
-constexpr int kFlRat = 1 << 13;      // far: rational form sk / (|z|^2 - 3/2)
-constexpr int kFlScaled = 1 << 14;   // far, rational: the line may be evaluated in units of sk (far_rat_pairs_scaled)
-
-struct NearRec {
-    float cf, f, klnq, a, srel, kv;
-    int flags;
-    int jlo, jhi;    // outer cut window (grid indices)
-    int pad[3];
-};
-
-// far line, three forms (sk = s_rel a / sqrt(pi)).  v = G_k * (kv B) + kv E1 is the exact
-// expm1 split of the frequency offset around the tile start.
-//  * kFarRat, "rational": s_rel H = sk / (|z|^2 - 3/2), |z|^2 = v^2 + a^2.  Its relative
-//    error against H is below (2 + 2a^2)/|z|^4 (the asymptotic series of H to order |z|^-4),
-//    so it is used where that bound is <= 1e-6 over the whole tile: 3 FFMA + 1 reciprocal.
-//    p = {kv B, kv E1, a^2 - 3/2, sk}.
-//  * kFarExact: the one-level continued fraction without truncation, with
-//    v' = sqrt2 v and D = v'^2 + 2a^2 - 1 = 2|z|^2 - 1:
-//    s_rel H = (2 sk D + 4 sk) / (D^2 + 8 a^2): 5 FFMA + 1 reciprocal.
-//  * kFarY: where D^2 could overflow FP32 (|v| >= 1e9 somewhere in the tile),
-//    y = 1/D, s_rel H = sk y (2 + 4 y); there 8 a^2 y^2 is far below 1e-8.
-//    p = {sqrt2 kv B, sqrt2 kv E1, 2a^2 - 1, 8a^2}, q = {2 sk, 4 sk} for both.
-// The PTS points are evaluated without branches so that their dependency chains
-// interleave; MASKED lines (partial coverage or points near the cut) select with a mask.
-constexpr int kFarRat = 0, kFarExact = 1, kFarY = 2;
-
-template <int PTS, int FORM, bool MASKED>
-__device__ __forceinline__ void far_line(const float4 p, const float2 q, int klo, int khi, bool chk,
-                                         const float (&G)[PTS], float (&part)[PTS]) {
-#pragma unroll
-    for (int k = 0; k < PTS; ++k) {
-        const float vp = fmaf(G[k], p.x, p.y);
-        const float D = fmaf(vp, vp, p.z);
-        float t, y;
-        if (FORM == kFarRat) {
-            y = rcp_approx(D);
-            t = p.w;
-        } else if (FORM == kFarY) {
-            y = rcp_approx(D);
-            t = fmaf(q.y, y, q.x);
-        } else {
-            y = rcp_approx(fmaf(D, D, p.w));
-            t = fmaf(q.x, D, q.y);
-        }
-        if (MASKED) {
-            const float l = t * y;
-            bool ok = (k >= klo) & (k <= khi);
-            if (chk) ok = ok & (l >= 1.f);
-            part[k] += ok ? l : 0.f;
-        } else {
-            part[k] = fmaf(t, y, part[k]);
-        }
-    }
-}
+// ---------------------------------------------------------------------------
+// Wing sums by interpolation.
+//
+// Seen from a stretch of the grid that lies at least its own length away from the line's
+// centre, a profile is smooth: s_rel H has its nearest singularity (the centre) at three
+// half-lengths from the stretch's middle, so its Chebyshev interpolant converges like
+// 5.8^-n.  With kNodes = 12 nodes the interpolant of 1/v^2 is within 2.3e-8 of it anywhere on
+// the stretch (10 nodes: 6.7e-7, 8: 1.8e-5), below the 1e-6 of the profile formulas.  The sum
+// over such lines is therefore formed at the nodes only, and interpolated once per tile:
+// 12 evaluations per (line, stretch) instead of one per point.
+//
+// Two stretches are used, the CTA's tile (level 0) and a warp's part of it (level 1).  Lines
+// that neither level takes (centre too close, window edge inside, too small |z|) are
+// evaluated point by point.
+constexpr int kNodes = 12;
+// cos(i pi / 24): node k of a stretch is at (1 + x_k)/2 of its length, x_k = cos((2k + 1) pi / 24),
+// and T_m(x_k) = cos(m (2k + 1) pi / 24)
+__constant__ double c_cos24[48] = {
+    1.0, 0.99144486137381041, 0.96592582628906829, 0.92387953251128676, 0.86602540378443865, 0.79335334029123517,
+    0.70710678118654752, 0.60876142900872064, 0.5, 0.38268343236508977, 0.25881904510252076, 0.13052619222005159,
+    0.0, -0.13052619222005159, -0.25881904510252076, -0.38268343236508977, -0.5, -0.60876142900872064,
+    -0.70710678118654752, -0.79335334029123517, -0.86602540378443865, -0.92387953251128676, -0.96592582628906829,
+    -0.99144486137381041, -1.0, -0.99144486137381041, -0.96592582628906829, -0.92387953251128676,
+    -0.86602540378443865, -0.79335334029123517, -0.70710678118654752, -0.60876142900872064, -0.5,
+    -0.38268343236508977, -0.25881904510252076, -0.13052619222005159, 0.0, 0.13052619222005159, 0.25881904510252076,
+    0.38268343236508977, 0.5, 0.60876142900872064, 0.70710678118654752, 0.79335334029123517, 0.86602540378443865,
+    0.92387953251128676, 0.96592582628906829, 0.99144486137381041};
 
 // packed FP32: two lanes per instruction, rounded like fmaf
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
@@ -774,337 +735,496 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return d;
 }
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 
-// plain line in the rational form, two points per reciprocal, in packed FP32.  The
-// thread's points are taken as pairs (2j, 2j+1): v and D = v^2 + a^2 - 3/2 of both points
-// in one packed FFMA each, r = 1/(D_0 D_1) and, with sr = sk r,
-// sk/D_0 = sr D_1 and sk/D_1 = sr D_0 (about two ulps) in one packed FFMA into the pair's
-// partial sums, held as {part_{2j+1}, part_{2j}}.  Per pair: three packed FFMAs and two
-// FMULs on the FMA pipe (8 lane operations) and one reciprocal.  D_0 D_1 < 1e36 stays finite
-// because the form is used only where |v| < 1e9 on the whole tile.
-// u = {kv B, kv B, kv E1, kv E1}, w = {a^2 - 3/2, a^2 - 3/2, sk, sk} (duplicated so that
-// each operand pair comes straight from one 16-byte shared-memory load).
-template <int PTS>
-__device__ __forceinline__ void far_rat_pairs(const float4 u, const float4 w, const float (&G)[PTS],
-                                              float (&part)[PTS]) {
-    static_assert(PTS % 2 == 0, "points are taken in pairs");
-    const float2 B2 = make_float2(u.x, u.y), E2 = make_float2(u.z, u.w), C2 = make_float2(w.x, w.y);
-    const float sk = w.z;
+// The offset v of a line at the points of a stretch starting D points from its centre:
+// v = G (kv B) + kv E1 with E1 = expm1(-D ln q), B = 1 + E1 and G = expm1(-delta ln q) for the
+// point delta points into the stretch (the exact split of expm1).  Both terms are at most
+// the larger of the stretch's span and the centre's distance, so with the centre at least the
+// span away v keeps about 2e-7 relative accuracy.
+struct Wing {
+    float kvE, kvB;      // kv E1, kv B
+    float dist;          // distance [points] of the centre from the stretch, < 0 inside
+    float zmin2, zmax2;  // smallest and largest |z|^2 on the stretch
+};
+// span = its number of points - 1, gend = G at its end
+__device__ __forceinline__ Wing wing(int J, int c, float f, float kv, float A, float lnq, float span, float gend) {
+    Wing w;
+    const float D = (float)(J - c) - f;
+    const float E1 = expm1f(-D * lnq);
+    w.kvE = kv * E1;
+    w.kvB = kv + w.kvE;
+    const float v0 = fabsf(w.kvE), v1 = fabsf(fmaf(gend, w.kvB, w.kvE));
+    w.dist = fmaxf(D, -(D + span));
+    const float vm = fminf(v0, v1), vx = fmaxf(v0, v1);
+    w.zmin2 = fmaf(vm, vm, A);
+    w.zmax2 = fmaf(vx, vx, A);
+    return w;
+}
+// The rational far form s_rel H = sk / (|z|^2 - 3/2), sk = s_rel a / sqrt(pi): its relative error is
+// below (2 + 2 a^2)/|z|^4 (the asymptotic series of H to order |z|^-4), so it is used where
+// that is at most 1e-6 on the whole stretch; |z|^2 <= 1e18 keeps the product of two denominators
+// finite.
+__device__ __forceinline__ bool rational_ok(const Wing& w, float A) {
+    return w.zmin2 * w.zmin2 >= 1.0e6f * fmaf(2.f, A, 2.f) && w.zmax2 <= 1.0e18f;
+}
+// acc[k] += s_rel H at the nodes (G[k]: expm1(-delta_k ln q)), rational form, two nodes per
+// reciprocal in packed FP32: r = 1/(D_0 D_1), sk/D_0 = sk r D_1, sk/D_1 = sk r D_0, the pair's sums
+// held as {acc_{2j+1}, acc_{2j}}.  Per pair three packed FFMAs, two FMULs and one reciprocal.
+__device__ __forceinline__ void nodes_rational(const Wing& w, float A, float sk, const float* G, float2 (&acc)[kNodes / 2]) {
+    const float2 B2 = dup2(w.kvB), E2 = dup2(w.kvE), C2 = dup2(A - 1.5f);
 #pragma unroll
-    for (int j = 0; j < PTS / 2; ++j) {
+    for (int j = 0; j < kNodes / 2; ++j) {
         const float2 v = ffma2(make_float2(G[2 * j], G[2 * j + 1]), B2, E2);
         const float2 D = ffma2(v, v, C2);
-        const float P01 = D.x * D.y;
-        float2 acc = make_float2(part[2 * j + 1], part[2 * j]);
-        const float sr = sk * rcp_approx(P01);
-        acc = ffma2(make_float2(sr, sr), D, acc);
-        part[2 * j + 1] = acc.x;
-        part[2 * j] = acc.y;
+        const float sr = sk * rcp_approx(D.x * D.y);
+        acc[j] = ffma2(dup2(sr), D, acc[j]);
     }
 }
-
-// plain line in the rational form, in units of sk: with v' = v / sqrt(sk) and
-// D' = v'^2 + (a^2 - 3/2)/sk = D/sk, the contribution sk/D is 1/D', so the factor sk leaves
-// the inner loop: r = 1/(D'_0 D'_1), 1/D'_0 = r D'_1, 1/D'_1 = r D'_0.  Per pair: three
-// packed FFMAs and one FMUL (7 lane operations) and one reciprocal.  Used for lines with
-// sk <= 1e18 D_min and |v|_max <= 1e9 sqrt(sk) on the tile, so that every D' lies in
-// [1e-18, 1e18] and the products stay normal FP32 numbers.
-// u = {B', B', E', E'} = {kv B, kv B, kv E1, kv E1} / sqrt(sk), w = {c', c', -, -}.
-template <int PTS>
-__device__ __forceinline__ void far_rat_pairs_scaled(const float4 u, const float4 w, const float (&G)[PTS],
-                                                     float (&part)[PTS]) {
-    static_assert(PTS % 2 == 0, "points are taken in pairs");
-    const float2 B2 = make_float2(u.x, u.y), E2 = make_float2(u.z, u.w), C2 = make_float2(w.x, w.y);
+// the same by the series (LOW: a^2 <= 2)
+template <bool LOW>
+__device__ __forceinline__ void nodes_series(const Wing& w, float A, float sk, const float* G, float2 (&acc)[kNodes / 2]) {
+    const float2 B2 = dup2(w.kvB), E2 = dup2(w.kvE), A2 = dup2(A), S2 = dup2(sk), zero = dup2(0.f);
+    const float2 k2 = dup2(series_k2(A)), k3 = dup2(series_k3(A)), k4 = dup2(series_k4(A));
 #pragma unroll
-    for (int j = 0; j < PTS / 2; ++j) {
+    for (int j = 0; j < kNodes / 2; ++j) {
         const float2 v = ffma2(make_float2(G[2 * j], G[2 * j + 1]), B2, E2);
-        const float2 D = ffma2(v, v, C2);
-        const float r = rcp_approx(D.x * D.y);
-        const float2 acc = ffma2(make_float2(r, r), D, make_float2(part[2 * j + 1], part[2 * j]));
-        part[2 * j + 1] = acc.x;
-        part[2 * j] = acc.y;
-    }
-}
-
-// near line: exact offset d = (j - c) - f and the expm1 series for v; the tiers of H
-// branch per point.  Lines that do not cover the whole tile are culled per warp in
-// 32-point segments (a warp's lanes own 32 consecutive points of each slot).  The coverage
-// and cut-test flags are runtime arguments: one copy of this code instead of four template
-// copies measured 1.1 % faster on the 8-row table step (less instruction-cache pressure).
-template <int PTS, int THREADS>
-__device__ __forceinline__ void near_line(const NearRec& r, int seg0, bool series, bool full, bool chk,
-                                          const float (&jf)[PTS], float q1, float q2, float q3, float lnq,
-                                          float (&part)[PTS]) {
-#pragma unroll
-    for (int k = 0; k < PTS; ++k) {
-        if (!full) {
-            const int lo = seg0 + k * THREADS;
-            if (lo + 31 < r.jlo || lo > r.jhi) continue;
+        const float2 Z = ffma2(v, v, A2);
+        const float r = rcp_approx(Z.x * Z.y);
+        const float2 t = make_float2(r * Z.x, r * Z.y);   // {1/Z_{2j+1}, 1/Z_{2j}}
+        float2 h;
+        if (LOW) {
+            h = ffma2(t, ffma2(t, ffma2(t, k4, k3), k2), dup2(1.5f));
+        } else {
+            const float2 s = ffma2(A2, t, zero);
+            const float2 c1 = ffma2(s, dup2(-2.f), dup2(1.5f));
+            const float2 c2 = ffma2(s, ffma2(s, dup2(12.f), dup2(-15.f)), dup2(3.75f));
+            const float2 c3 = ffma2(s, ffma2(s, ffma2(s, dup2(-120.f), dup2(210.f)), dup2(-105.f)), dup2(13.125f));
+            h = ffma2(t, ffma2(t, c3, c2), c1);
         }
-        const float d = (jf[k] - r.cf) - r.f;
-        float v;
-        if (series) v = r.klnq * (d * fmaf(d, fmaf(d, fmaf(d, q3, q2), q1), 1.f));
-        else v = r.kv * expm1f(-d * lnq);
-        float l = r.srel * voigt_H_lean(v, r.a);
-        if (chk) l = (l >= 1.f) ? l : 0.f;
-        part[k] += l;
+        h = ffma2(t, h, dup2(1.f));
+        acc[j] = ffma2(ffma2(t, S2, zero), h, acc[j]);
     }
 }
 
-// One tile of one row.  Called by the grid kernel (one tile per CTA, or S CTAs per tile that
+// sum of one value over the warp, in every lane
+__device__ __forceinline__ float warp_sum_f(float v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+
+// total += y: Kahan-compensated, or a plain sum for the naive variant
+template <int PREC>
+__device__ __forceinline__ void fold(float& sum, float& comp, float v) {
+    if (PREC == MPSA_PREC_FP32_COMPENSATED) {
+        const float y = v - comp;
+        const float t = sum + y;
+        comp = (t - sum) - y;
+        sum = t;
+    } else {
+        sum += v;
+    }
+}
+
+// Add a warp's node sums (over its lanes) to the warp's totals F[k] = {sum, comp}; clears acc.
+template <int PREC>
+__device__ __forceinline__ void fold_nodes(float2 (&acc)[kNodes / 2], float2* F, int lane) {
+    float mine = 0.f;
+#pragma unroll
+    for (int j = 0; j < kNodes / 2; ++j) {
+        const float hi = warp_sum_f(acc[j].x), lo = warp_sum_f(acc[j].y);   // nodes 2j + 1 and 2j
+        if (lane == 2 * j) mine = lo;
+        if (lane == 2 * j + 1) mine = hi;
+        acc[j] = make_float2(0.f, 0.f);
+    }
+    if (lane < kNodes) {
+        float2 q = F[lane];
+        fold<PREC>(q.x, q.y, mine);
+        F[lane] = q;
+    }
+}
+
+// Clenshaw sum of the Chebyshev series c[0..kNodes) at x
+__device__ __forceinline__ float clenshaw(const float* c, float x) {
+    float b1 = 0.f, b2 = 0.f;
+    const float x2 = 2.f * x;
+#pragma unroll
+    for (int m = kNodes - 1; m >= 1; --m) {
+        const float b = fmaf(x2, b1, c[m] - b2);
+        b2 = b1;
+        b1 = b;
+    }
+    return fmaf(x, b1, c[0] - b2);
+}
+
+// A line that a warp evaluates point by point on its part of the tile: window edges inside the
+// part, centres on or next to it.  Window [lo, hi] relative to Js, kind one of
+//   kPtRat     rational form on the whole part, v from the expm1 split (u.z = kv E1, u.w = kv B)
+//   kPtWing    the series of H on the whole part, v from the expm1 split, a^2 <= 2
+//   kPtNear    centre within the part's length: v = kv (x - x^2/2 + x^3/6)-like series (|x| <= 0.01, the
+//              rest is below 5e-8 of it); the points jc0..jc1 (|z|^2 < 100, in u.z and u.w as
+//              integers) by voigt_small or, for a > 0.03, the Gauss-Hermite tiers; the others by
+//              the series of H
+//   kPtGen     any other case, decided point by point
+// with kPtChk where the part is not inside the inner window: a point then takes the line iff
+// s_rel H >= 1.
+struct __align__(16) PointRec {
+    float ci, f, klnq, A;          // ci = c - Js (exact)
+    float sk, srel, kvE, kvB;
+    int lo, hi, kind;
+    float a;
+};
+constexpr int kPtRat = 0, kPtWing = 1, kPtNear = 2, kPtGen = 3, kPtKind = 3, kPtAway = 4, kPtChk = 8;
+constexpr int kPtRecs = 32;    // records a warp holds
+
+// kPtNear's core, by voigt_small (TINY: a <= 3e-4)
+template <bool TINY>
+__device__ __forceinline__ void add_core(float* x, int j0, int j1, int lane, const float4 p, float srel, float a,
+                                         float floor1, float q1, float q2) {
+#pragma unroll 1
+    for (int j = j0 + lane; j <= j1; j += 32) {
+        const float d = ((float)j - p.x) - p.y;
+        const float v = p.z * (d * fmaf(d, fmaf(d, q2, q1), 1.f));
+        const float l = srel * voigt_small<TINY>(v * v, p.w, a);
+        if (l >= floor1) x[j] += l;
+    }
+}
+
+// One record added to the warp's points x[0..last].  The lanes take 32 consecutive points of the
+// window at a time, so a narrow window costs no idle segments and no two lanes share a point.
+// Every case has a loop of its own without branches: one loop deciding per point spent as
+// many integer and control instructions as FP32 ones.  Gp[j] = expm1(-j ln q).
+__device__ __forceinline__ void add_points(const PointRec& r, float* x, const float* Gp, int last, int lane, float q1,
+                                           float q2, float lnq) {
+    const int4 w = *reinterpret_cast<const int4*>(&r.lo);
+    const float4 u = *reinterpret_cast<const float4*>(&r.sk);
+    const float4 p = *reinterpret_cast<const float4*>(&r.ci);
+    const float floor1 = (w.z & kPtChk) ? 1.f : 0.f;
+    const int lo = max(w.x, 0), hi = min(w.y, last);
+    const int kind = w.z & kPtKind;
+    const float a = __int_as_float(w.w);
+    if (kind == kPtRat) {
+        const float C = p.w - 1.5f;
+#pragma unroll 1
+        for (int j = lo + lane; j <= hi; j += 32) {
+            const float v = fmaf(Gp[j], u.w, u.z);
+            const float l = u.x * rcp_approx(fmaf(v, v, C));
+            if (l >= floor1) x[j] += l;
+        }
+    } else if (kind == kPtNear) {
+        const int c0 = max(lo, __float_as_int(u.z)), c1 = min(hi, __float_as_int(u.w));
+        // the points outside the core, left then right, as one sequence; no core: all of them
+        const int nl = c0 <= c1 ? c0 - lo : hi - lo + 1, gap = c0 <= c1 ? c1 - c0 + 1 : 0, n = hi - lo + 1 - gap;
+        const float k2 = series_k2(p.w), k3 = series_k3(p.w), k4 = series_k4(p.w);
+#pragma unroll 1
+        for (int t = lane; t < n; t += 32) {
+            const int j = lo + t + (t >= nl ? gap : 0);
+            const float d = ((float)j - p.x) - p.y;
+            const float v = p.z * (d * fmaf(d, fmaf(d, q2, q1), 1.f));
+            const float y = rcp_approx(fmaf(v, v, p.w));
+            const float l = u.x * y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, k4, k3), k2), 1.5f), 1.f);
+            if (l >= floor1) x[j] += l;
+        }
+        if (a <= kTinyA) {
+            add_core<true>(x, c0, c1, lane, p, u.y, a, floor1, q1, q2);
+        } else if (a <= kSmallA) {
+            add_core<false>(x, c0, c1, lane, p, u.y, a, floor1, q1, q2);
+        } else {
+#pragma unroll 1
+            for (int j = c0 + lane; j <= c1; j += 32) {
+                const float d = ((float)j - p.x) - p.y;
+                const float v = p.z * (d * fmaf(d, fmaf(d, q2, q1), 1.f));
+                const float l = u.y * voigt_inner_tiers(v, a);
+                if (l >= floor1) x[j] += l;
+            }
+        }
+    } else if (kind == kPtWing) {
+        const float k2 = series_k2(p.w), k3 = series_k3(p.w), k4 = series_k4(p.w);
+#pragma unroll 1
+        for (int j = lo + lane; j <= hi; j += 32) {
+            const float v = fmaf(Gp[j], u.w, u.z);
+            const float y = rcp_approx(fmaf(v, v, p.w));
+            const float l = u.x * y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, k4, k3), k2), 1.5f), 1.f);
+            if (l >= floor1) x[j] += l;
+        }
+    } else {
+#pragma unroll 1
+        for (int j = lo + lane; j <= hi; j += 32) {
+            float v;
+            if (w.z & kPtAway) v = fmaf(Gp[j], u.w, u.z);
+            else v = p.z / lnq * expm1f(-(((float)j - p.x) - p.y) * lnq);
+            const float l = u.y * voigt_point(v, a);
+            if (l >= floor1) x[j] += l;
+        }
+    }
+}
+
+// One tile of one row.  Called by the grid kernel (one tile per CTA, or up to S CTAs per tile that
 // take every S-th chunk of the tile's candidate lines, sp = 0..S-1, when a call has too few
-// tiles to fill the GPU) and by the persistent kernel (a loop over a work list).
+// tiles to fill the GPU; *s_used says how many did) and by the persistent kernel (a loop over a work list).
+//
+// Candidate lines are taken THREADS at a time, one per thread: a thread adds its line to the
+// node sums of the tile (level 0) in its own registers, so that a line costs its set-up and 12
+// evaluations once, with no broadcast.  Lines that the tile cannot take are queued in shared
+// memory (in candidate order); when the queue holds more than kQueue lines every warp runs
+// over it, one line per lane, for its own part of the tile (level 1), and the lines that the
+// part cannot take are gathered (kPtRecs a warp) and evaluated at its points by the whole warp.
+//
+// FP32 partial sums run over at most 64 lines (level 0, points) or 2 THREADS / 32 lines (level 1)
+// and are folded into Kahan-compensated totals in shared memory.
+constexpr int kSplitChunks = 64;   // chunks of candidates that are worth a CTA of their own
+constexpr int kQueue = 1024;   // queued lines at which a tile turns to level 1
+
 template <int PREC, int PTS, int THREADS>
-__device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0, int S = 1) {
-    constexpr int TILE = PTS * THREADS;
-    __shared__ float4 sFarA[THREADS];
-    __shared__ float4 sFarB[THREADS];
-    __shared__ NearRec sNear[THREADS];
-    __shared__ int sCnt[6][THREADS / 32];
+__device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0, int S = 1, int S_free = 1,
+                                          int* s_used = nullptr) {
+    constexpr int TILE = PTS * THREADS, WARPS = THREADS / 32, QCAP = THREADS + kQueue;
+    __shared__ int sQ[QCAP];
+    __shared__ PointRec sP[WARPS][kPtRecs];
+    __shared__ float sX[WARPS][32 * PTS];   // sums of the gathered records at the warp's points
+    __shared__ float sGp[32 * PTS];         // expm1(-j ln q) at the points j of a warp's part
+    __shared__ float sG0[kNodes], sG1[WARPS][kNodes];
+    __shared__ float2 sF0[WARPS][kNodes], sF1[WARPS][kNodes];   // node totals {sum, comp}
+    __shared__ float sC0[kNodes], sC1[WARPS][kNodes];           // their Chebyshev coefficients
+    __shared__ int sCnt[2][WARPS];
+    __shared__ int sBeg[kNumClasses], sEnd[kNumClasses];        // each class's candidates
+    __shared__ float sSum[PTS][THREADS];
+    __shared__ float sComp[PREC == MPSA_PREC_FP32_COMPENSATED ? PTS : 1][THREADS];
 
     const int J0 = tile * TILE;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-    // Kahan totals live in shared memory ([point][thread], conflict-free): they change once
-    // per chunk, and keeping them out of registers lets more CTAs share an SM
-    __shared__ float sSum[PREC == MPSA_PREC_FP32_COMPENSATED ? PTS : 1][THREADS];
-    __shared__ float sComp[PREC == MPSA_PREC_FP32_COMPENSATED ? PTS : 1][THREADS];
-    float jf[PTS], G[PTS], part[PTS];
+    const float lnq = g.lnq;
+    // the tile's points on the grid, [J0, Te], and the warp's part of them, [Js, Je] (npt segments of
+    // 32): a short tile is shared out over all warps
+    const int Te = min(J0 + TILE, g.N) - 1;
+    const int sub = 32 * ((Te - J0 + 32 * WARPS) / (32 * WARPS)), npt = sub / 32;
+    const int Js = J0 + warp * sub, Je = min(Js + sub - 1, Te);
+    const bool active = Js <= Te;
+    const float span0 = (float)(Te - J0), span1 = active ? (float)(Je - Js) : 0.f;
+    const float gend0 = expm1f(-span0 * lnq), gend1 = expm1f(-span1 * lnq);
+    if (lane < kNodes) {
+        const float x = 0.5f + 0.5f * (float)c_cos24[2 * lane + 1];
+        sG1[warp][lane] = expm1f(-span1 * x * lnq);
+        if (warp == 0) sG0[lane] = expm1f(-span0 * x * lnq);
+        sF0[warp][lane] = sF1[warp][lane] = make_float2(0.f, 0.f);
+    }
+    if (tid < kNumClasses) {   // all classes at once: one memory latency instead of one per class
+        const int reach = 1 << tid;
+        const int tlo = max(floordiv(J0 - reach + 1, TILE), -1);
+        const int thi = min(floordiv(J0 + TILE - 1 + reach - 1, TILE), g.nT);
+        const int* cum = g.cum + (size_t)tid * (g.nT + 3);
+        sBeg[tid] = tlo <= thi ? cum[tlo + 1] : 0;
+        sEnd[tid] = tlo <= thi ? cum[thi + 2] : 0;
+    }
+    for (int t = tid; t < 32 * PTS; t += THREADS) sGp[t] = expm1f(-(float)t * lnq);
 #pragma unroll
     for (int k = 0; k < PTS; ++k) {
-        const int off = k * THREADS + tid;
-        jf[k] = (float)(J0 + off);
-        G[k] = expm1f(-(float)off * g.lnq);
-        if (PREC == MPSA_PREC_FP32_COMPENSATED) {
-            sSum[k][tid] = 0.f;
-            sComp[k][tid] = 0.f;
-        }
-        part[k] = 0.f;
+        sSum[k][tid] = 0.f;
+        (&sX[0][0])[k * THREADS + tid] = 0.f;
+        if (PREC == MPSA_PREC_FP32_COMPENSATED) sComp[k][tid] = 0.f;
+    }
+    __syncthreads();
+    if (S > 1) {   // as many of the tile's CTAs as its candidates are worth
+        int chunks = 0;
+        for (int b = 0; b < kNumClasses; ++b) chunks += (sEnd[b] - sBeg[b] + THREADS - 1) / THREADS;
+        S = max(1, max(min(S_free, chunks), min(S, chunks / kSplitChunks)));
+        if (sp == 0 && tid == 0) *s_used = S;
+        if (sp >= S) return;
     }
 
-    int chunk = 0;   // running chunk index over the classes: this CTA takes chunk % S == sp
-    for (int b = 0; b < kNumClasses; ++b) {
-        const int reach = 1 << b;
-        int tlo = floordiv(J0 - reach + 1, TILE), thi = floordiv(J0 + TILE - 1 + reach - 1, TILE);
-        tlo = max(tlo, -1);
-        thi = min(thi, g.nT);
-        if (tlo > thi) continue;
-        const int* cum = g.cum + (size_t)b * (g.nT + 3);
-        const int beg = cum[tlo + 1], end = cum[thi + 2];
-        for (int base = beg; base < end; base += THREADS) {
-            if (chunk++ % S != sp) continue;   // CTA-uniform
-            // ---- set-up: one candidate line per thread
-            const int pos = base + tid;
-            bool isFar = false, isNear = false;
-            float4 fa, fb;
-            NearRec nr;
+    // the warp's gathered point records at every segment of its part
+    auto points = [&](int n) {
+        __syncwarp();
+        for (int i = 0; i < n; ++i) {
+            add_points(sP[warp][i], sX[warp], sGp, Je - Js, lane, g.q1, g.q2, lnq);
+            __syncwarp();
+        }
+        for (int k = 0; k < npt; ++k) {
+            float dummy = 0.f;
+            fold<PREC>(sSum[k][tid], PREC == MPSA_PREC_FP32_COMPENSATED ? sComp[k][tid] : dummy, sX[warp][32 * k + lane]);
+            sX[warp][32 * k + lane] = 0.f;
+        }
+        __syncwarp();
+    };
+    // level 1 and the points, over the queued lines
+    auto flush = [&](int n) {
+        float2 acc[kNodes / 2];
+#pragma unroll
+        for (int j = 0; j < kNodes / 2; ++j) acc[j] = make_float2(0.f, 0.f);
+        int np = 0;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            bool direct = false, rat = false, ser = false;
+            Wing w{};
+            int4 r0, r1, r2;
+            float f = 0.f, kv = 0.f, a = 0.f, A = 0.f, sk = 0.f;
+            if (i < n) {
+                const int4* rp = reinterpret_cast<const int4*>(g.rec + sQ[i]);
+                r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2);
+                if (r2.x >= Js && r1.w <= Je) {
+                    f = __int_as_float(r0.y), kv = __int_as_float(r0.z), a = __int_as_float(r0.w);
+                    A = a * a;
+                    sk = __int_as_float(r1.x) * a * kInvSqrtPi;
+                    w = wing(Js, r0.x, f, kv, A, lnq, span1, gend1);
+                    const bool smooth = r1.y <= Js && r1.z >= Je && w.dist > span1;
+                    const bool ra = rational_ok(w, A);
+                    rat = smooth && ra;
+                    ser = smooth && !ra && w.zmin2 >= kSeriesZ2 && w.zmax2 <= 1.0e18f;
+                    direct = !rat && !ser;
+                }
+            }
+            if (rat) nodes_rational(w, A, sk, sG1[warp], acc);
+            if (__any_sync(0xffffffffu, ser)) {
+                if (__all_sync(0xffffffffu, !ser || A <= kSeriesA)) {
+                    if (ser) nodes_series<true>(w, A, sk, sG1[warp], acc);
+                } else {
+                    if (ser) nodes_series<false>(w, A, sk, sG1[warp], acc);
+                }
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, direct);
+            if (np + __popc(m) > kPtRecs) {
+                points(np);
+                np = 0;
+            }
+            if (direct) {
+                const bool away = w.dist > span1;
+                PointRec p;
+                p.ci = (float)(r0.x - Js);
+                p.f = f;
+                p.klnq = kv * lnq;
+                p.A = A;
+                p.sk = sk;
+                p.srel = __int_as_float(r1.x);
+                p.kvE = w.kvE;
+                p.kvB = w.kvB;
+                p.lo = r1.w - Js;
+                p.hi = r2.x - Js;
+                p.a = a;
+                const bool chk = !(r1.y <= Js && r1.z >= Je);
+                int kind = kPtGen;
+                if (away && rational_ok(w, A)) {
+                    kind = kPtRat;
+                } else if (A <= kSeriesA && away && w.zmin2 >= kSeriesZ2 && w.zmax2 <= 1.0e18f) {
+                    kind = kPtWing;
+                } else if (A <= kSeriesA && !away && (span1 + fmaxf(w.dist, 0.f) + 1.f) * lnq <= 0.01f &&
+                           w.zmax2 <= 1.0e18f) {
+                    kind = kPtNear;
+                    // |v| = 10 at about this many points from the centre
+                    const float h = fminf(sqrtf(kSeriesZ2 - A) / p.klnq, 1.0e6f), x0 = p.ci + f;
+                    p.kvE = __int_as_float((int)ceilf(x0 - h));
+                    p.kvB = __int_as_float((int)floorf(x0 + h));
+                }
+                p.kind = kind | (away ? kPtAway : 0) | (chk ? kPtChk : 0);
+                sP[warp][np + __popc(m & ((1u << lane) - 1u))] = p;
+            }
+            np += __popc(m);
+        }
+        if (np > 0) points(np);
+        fold_nodes<PREC>(acc, sF1[warp], lane);
+    };
+
+    float2 acc0[kNodes / 2];
+#pragma unroll
+    for (int j = 0; j < kNodes / 2; ++j) acc0[j] = make_float2(0.f, 0.f);
+    int chunk = 0;    // running chunk index over the classes: this CTA takes chunk % S == sp
+    int nq = 0;       // queued lines
+    int par = 0, run = 0;
+    int b = -1, base = 0, end = 0;   // class, next candidate, end of the class's candidates
+    for (bool more = true; more;) {
+        // ---- the next chunk of candidates (CTA-uniform)
+        int pos0 = -1;
+        while (pos0 < 0) {
+            if (base < end) {
+                if (chunk++ % S == sp) pos0 = base;
+                base += THREADS;
+            } else if (++b < kNumClasses) {
+                base = sBeg[b];
+                end = sEnd[b];
+            } else {
+                more = false;
+                break;
+            }
+        }
+        if (more) {
+            // ---- level 0: one candidate line per thread
+            const int pos = pos0 + tid;
+            bool queue = false;
+            int4 r0, r1, r2;
             if (pos < end) {
                 const int4* rp = reinterpret_cast<const int4*>(g.rec + pos);
-                const int4 r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2);
-                const int jlo = r1.y, jhi = r1.z;
-                if (jhi >= J0 && jlo <= J0 + TILE - 1) {
-                    const int c = r0.x;
-                    const float f = __int_as_float(r0.y), kv = __int_as_float(r0.z), a = __int_as_float(r0.w),
-                                srel = __int_as_float(r1.x);
-                    const int klo = max(0, (jlo - J0) / THREADS), khi = min(PTS - 1, (jhi - J0) / THREADS);
-                    const int P0 = J0 + klo * THREADS, P1 = J0 + khi * THREADS + THREADS - 1;
-                    const bool check = !(r1.w <= P0 && r2.x >= P1);
-                    // distance from the centre x0 = c + f to the nearest point of the tile
-                    // (far lines are evaluated at all points, masked to [klo, khi])
-                    const int T0 = J0, T1 = J0 + TILE - 1;
-                    float dist;
-                    bool red;
-                    if (c + 1 <= T0) { dist = (float)(T0 - c) - f; red = true; }
-                    else if (c >= T1) { dist = f + (float)(c - T1); red = false; }
-                    else { dist = 0.f; red = true; }
-                    float vmin = 0.f;
-                    if (dist >= (float)kFarDist)
-                        vmin = red ? -kv * expm1f(-dist * g.lnq) : kv * expm1f(dist * g.lnq);
-                    const int flags = klo | (khi << kFlKloBits) | (check ? kFlChk : 0) |
-                                      ((klo == 0 && khi == PTS - 1) ? kFlFull : 0);
-                    if (dist >= (float)kFarDist && vmin >= kFarV) {
-                        isFar = true;
-                        // a far line whose windows reach the grid's last point counts as covering
-                        // the tile there: the points past the grid's end (last tile only) are
-                        // evaluated but never stored, so narrow grids keep the unmasked forms
-                        const int Te = min(T1, g.N - 1);
-                        const int khf = jhi >= Te ? PTS - 1 : khi;
-                        const bool chf = !(r1.w <= P0 && r2.x >= min(J0 + khf * THREADS + THREADS - 1, Te));
-                        const int ff = klo | (khf << kFlKloBits) | (chf ? kFlChk : 0) |
-                                       ((klo == 0 && khf == PTS - 1) ? kFlFull : 0);
-                        const float D = (float)(J0 - c) - f;
-                        const float x = D * g.lnq;
-                        const float E1 = expm1f(-x), B = expf(-x);
-                        const float A = a * a;
-                        const float r2 = 1.41421356237309505f;
-                        // the largest |v| on the tile (both ends) decides between the two forms
-                        const float xe = ((float)(J0 + TILE - 1 - c) - f) * g.lnq;
-                        const float vmax = fmaxf(fabsf(kv * E1), fabsf(kv * expm1f(-xe)));
-                        const bool yform = vmax >= 1.0e9f;
-                        const float sk = srel * a * kInvSqrtPi;
-                        // rational form where (2 + 2a^2) / |z|^4 <= 1e-6 at the tile's nearest point
-                        const float zmin2 = fmaf(vmin, vmin, A);
-                        if (zmin2 * zmin2 >= 1.0e6f * fmaf(2.f, A, 2.f)) {
-                            fa = make_float4(kv * B, kv * E1, A - 1.5f, sk);
-                            // every D/sk of the tile within [1e-18, 1e18]: the form in units of sk
-                            const bool scaled = sk <= 1.0e18f * (zmin2 - 1.5f) && vmax <= 1.0e9f * sqrtf(sk);
-                            fb = make_float4(0.f, 0.f,
-                                             __int_as_float(ff | kFlRat | (yform ? kFlAlt : 0) |
-                                                            (scaled ? kFlScaled : 0)),
-                                             0.f);
-                        } else {
-                            fa = make_float4(r2 * kv * B, r2 * kv * E1, fmaf(2.f, A, -1.f), 8.f * A);
-                            fb = make_float4(2.f * sk, 4.f * sk, __int_as_float(ff | (yform ? kFlAlt : 0)), 0.f);
-                        }
+                r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2);
+                const int ilo = r1.y, ihi = r1.z, jlo = r1.w, jhi = r2.x;
+                if (jhi >= J0 && jlo <= Te) {
+                    const float a = __int_as_float(r0.w), A = a * a;
+                    const Wing w = wing(J0, r0.x, __int_as_float(r0.y), __int_as_float(r0.z), A, lnq, span0, gend0);
+                    if (ilo <= J0 && ihi >= Te && w.dist > span0 && rational_ok(w, A)) {
+                        float G[kNodes];
+#pragma unroll
+                        for (int k = 0; k < kNodes; ++k) G[k] = sG0[k];
+                        nodes_rational(w, A, __int_as_float(r1.x) * a * kInvSqrtPi, G, acc0);
                     } else {
-                        isNear = true;
-                        const float dmax = fmaxf(fabsf((float)(P0 - c) - f), fabsf((float)(P1 - c) - f));
-                        const bool series = dmax * g.lnq <= 0.05f;
-                        nr.cf = (float)c;
-                        nr.f = f;
-                        nr.klnq = kv * g.lnq;
-                        nr.a = a;
-                        nr.srel = srel;
-                        nr.kv = kv;
-                        nr.flags = flags | (series ? kFlAlt : 0);
-                        nr.jlo = jlo;
-                        nr.jhi = jhi;
-                        nr.pad[0] = nr.pad[1] = nr.pad[2] = 0;
+                        queue = true;
                     }
                 }
             }
-            // far lines are compacted into five lists: plain rational in units of sk, plain
-            // rational with two points per reciprocal (the few lines the scaled form cannot
-            // take), plain "exact" and plain "y" forms, and masked (partial coverage or cut
-            // test), so the hot loops dispatch nothing; near lines into a sixth
-            constexpr int kNearCat = 5;
-            int cat = -1;
-            if (isFar) {
-                const int fl = __float_as_int(fb.z);
-                const bool plain = (fl & kFlFull) && !(fl & kFlChk);
-                // rational lines with |v| >= 1e9 somewhere take the single-reciprocal masked path
-                // rational lines: in units of sk where allowed (list 0), else two points per
-                // reciprocal where |v| < 1e9 (list 1), else the single-reciprocal masked path
-                cat = !plain ? 4
-                             : ((fl & kFlRat) ? ((fl & kFlScaled) ? 0 : ((fl & kFlAlt) ? 4 : 1))
-                                              : ((fl & kFlAlt) ? 3 : 2));
-            } else if (isNear) {
-                cat = kNearCat;
-            }
-            unsigned bm = 0u;
-#pragma unroll
-            for (int q = 0; q <= kNearCat; ++q) {
-                const unsigned b = __ballot_sync(0xffffffffu, cat == q);
-                if (cat == q) bm = b;
-                if (lane == 0) sCnt[q][warp] = __popc(b);
-            }
+            // ---- queue the others, in candidate order
+            const unsigned bm = __ballot_sync(0xffffffffu, queue);
+            if (lane == 0) sCnt[par][warp] = __popc(bm);
             __syncthreads();
-            int off = 0, tot[kNearCat + 1] = {0, 0, 0, 0, 0, 0};
+            int off = nq, tot = 0;
 #pragma unroll
-            for (int w = 0; w < THREADS / 32; ++w) {
-#pragma unroll
-                for (int q = 0; q <= kNearCat; ++q) {
-                    const int cnt = sCnt[q][w];
-                    if (w < warp && q == cat) off += cnt;
-                    tot[q] += cnt;
-                }
+            for (int v = 0; v < WARPS; ++v) {
+                const int cnt = sCnt[par][v];
+                if (v < warp) off += cnt;
+                tot += cnt;
             }
-            const unsigned lt = (1u << lane) - 1u;
-            if (cat >= 0 && cat < kNearCat) {
-                int base2 = 0;
-#pragma unroll
-                for (int q = 0; q < kNearCat - 1; ++q)
-                    if (q < cat) base2 += tot[q];
-                const int p = base2 + off + __popc(bm & lt);
-                if (cat == 0) {
-                    const float rs = 1.f / sqrtf(fa.w), c1 = fa.z / fa.w;
-                    sFarA[p] = make_float4(fa.x * rs, fa.x * rs, fa.y * rs, fa.y * rs);
-                    sFarB[p] = make_float4(c1, c1, 0.f, 0.f);
-                } else if (cat <= 1) {
-                    sFarA[p] = make_float4(fa.x, fa.x, fa.y, fa.y);
-                    sFarB[p] = make_float4(fa.z, fa.z, fa.w, fa.w);
-                } else {
-                    sFarA[p] = fa;
-                    sFarB[p] = fb;
-                }
-            }
-            if (cat == kNearCat) sNear[off + __popc(bm & lt)] = nr;
-            const int nNear = tot[kNearCat];
+            par ^= 1;
+            if (queue) sQ[off + __popc(bm & ((1u << lane) - 1u))] = pos;
+            nq += tot;
+            ++run;
+        }
+        if (!more || run >= 64) {
+            fold_nodes<PREC>(acc0, sF0[warp], lane);
+            run = 0;
+        }
+        if (!more || nq > QCAP - THREADS) {
             __syncthreads();
-
-            // ---- evaluation: every thread, every compacted line, its PTS points
-            {
-                int r = 0;
-                // two lines per iteration: half the loop overhead, and two independent
-                // dependency chains per point for the scheduler
-                for (; r + 1 < tot[0]; r += 2) {
-                    const float4 ua = sFarA[r], wa = sFarB[r], ub = sFarA[r + 1], wb = sFarB[r + 1];
-                    far_rat_pairs_scaled<PTS>(ua, wa, G, part);
-                    far_rat_pairs_scaled<PTS>(ub, wb, G, part);
-                }
-                if (r < tot[0]) {
-                    far_rat_pairs_scaled<PTS>(sFarA[r], sFarB[r], G, part);
-                    ++r;
-                }
-                const int e1 = tot[0] + tot[1];
-                for (; r + 1 < e1; r += 2) {
-                    const float4 ua = sFarA[r], wa = sFarB[r], ub = sFarA[r + 1], wb = sFarB[r + 1];
-                    far_rat_pairs<PTS>(ua, wa, G, part);
-                    far_rat_pairs<PTS>(ub, wb, G, part);
-                }
-                if (r < e1) {
-                    far_rat_pairs<PTS>(sFarA[r], sFarB[r], G, part);
-                    ++r;
-                }
-                for (; r < e1 + tot[2]; ++r) {
-                    const float4 q4 = sFarB[r];
-                    far_line<PTS, kFarExact, false>(sFarA[r], make_float2(q4.x, q4.y), 0, PTS - 1, false, G, part);
-                }
-                for (; r < e1 + tot[2] + tot[3]; ++r) {
-                    const float4 q4 = sFarB[r];
-                    far_line<PTS, kFarY, false>(sFarA[r], make_float2(q4.x, q4.y), 0, PTS - 1, false, G, part);
-                }
-                for (; r < e1 + tot[2] + tot[3] + tot[4]; ++r) {
-                    const float4 p = sFarA[r];
-                    const float4 q4 = sFarB[r];
-                    const float2 q = make_float2(q4.x, q4.y);
-                    const int fl = __float_as_int(q4.z);
-                    const int klo = fl & kFlMask, khi = (fl >> kFlKloBits) & kFlMask;
-                    const bool chk = fl & kFlChk;
-                    if (fl & kFlRat) far_line<PTS, kFarRat, true>(p, q, klo, khi, chk, G, part);
-                    else if (fl & kFlAlt) far_line<PTS, kFarY, true>(p, q, klo, khi, chk, G, part);
-                    else far_line<PTS, kFarExact, true>(p, q, klo, khi, chk, G, part);
-                }
-            }
-            const int seg0 = J0 + warp * 32;
-            for (int r = 0; r < nNear; ++r) {
-                const NearRec nrr = sNear[r];
-                const bool series = nrr.flags & kFlAlt;
-                const bool full = nrr.flags & kFlFull, chk = nrr.flags & kFlChk;
-                near_line<PTS, THREADS>(nrr, seg0, series, full, chk, jf, g.q1, g.q2, g.q3, g.lnq, part);
-            }
-            if (PREC == MPSA_PREC_FP32_COMPENSATED) {
-                // fold the chunk's FP32 partial sums into the Kahan-compensated totals
-#pragma unroll
-                for (int k = 0; k < PTS; ++k) {
-                    const float s0 = sSum[k][tid], c0 = sComp[k][tid];
-                    const float y = part[k] - c0;
-                    const float t = s0 + y;
-                    sComp[k][tid] = (t - s0) - y;
-                    sSum[k][tid] = t;
-                    part[k] = 0.f;
-                }
-            }
+            if (active) flush(nq);
             __syncthreads();
+            nq = 0;
         }
     }
-    const float tp = expf(*g.ln_tp);
-#pragma unroll
-    for (int k = 0; k < PTS; ++k) {
-        const int j = J0 + k * THREADS + tid;
-        const float tot = (PREC == MPSA_PREC_FP32_COMPENSATED) ? (sSum[k][tid] - sComp[k][tid]) : part[k];
-        if (j < g.N) g.out[j] = tp * tot;
+    // ---- Chebyshev coefficients of the node totals, c_m = (2 - [m = 0])/n sum_k F_k T_m(x_k), in FP64
+    if (lane < kNodes) {
+        double s1 = 0.0, s0 = 0.0;
+        for (int k = 0; k < kNodes; ++k) {
+            const double tm = c_cos24[(lane * (2 * k + 1)) % 48];
+            s1 += tm * ((double)sF1[warp][k].x - (double)sF1[warp][k].y);
+            if (warp == 0) {
+                double F = 0.0;
+                for (int v = 0; v < WARPS; ++v) F += (double)sF0[v][k].x - (double)sF0[v][k].y;
+                s0 += tm * F;
+            }
+        }
+        const double sc = (lane == 0 ? 1.0 : 2.0) / kNodes;
+        sC1[warp][lane] = (float)(sc * s1);
+        if (warp == 0) sC0[lane] = (float)(sc * s0);
     }
+    __syncthreads();
+    const float tp = expf(*g.ln_tp);
+    if (active) {
+        const float r0 = span0 > 0.f ? 2.f / span0 : 0.f, r1 = span1 > 0.f ? 2.f / span1 : 0.f;
+#pragma unroll
+        for (int k = 0; k < PTS; ++k) {
+            const int j = Js + 32 * k + lane;
+            if (k >= npt || j > Je) continue;
+            const float near = PREC == MPSA_PREC_FP32_COMPENSATED ? sSum[k][tid] - sComp[k][tid] : sSum[k][tid];
+            const float far = clenshaw(sC0, fmaf((float)(j - J0), r0, -1.f)) + clenshaw(sC1[warp], fmaf((float)(j - Js), r1, -1.f));
+            g.out[j] = tp * (near + far);
+        }
+    }
+    __syncthreads();   // the shared memory is free for the persistent kernel's next tile
 }
 
 // Grid form: one CTA per (row, tile); the rows of one call share the prep arrays.
@@ -1126,8 +1246,10 @@ struct TileArgs {
     const int* ihi;
     const float* ln_tp;
     float* out;
-    int split;       // CTAs per tile (1: direct output)
+    int split;       // CTAs per tile at most (1: direct output)
+    int split_free;  // as many as the GPU holds at once
     float* part;     // split > 1: partial sums [n_sel][split][N], added by k_split_sum
+    int* used;       // split > 1: how many of a tile's CTAs wrote theirs, [n_sel][nT]
 };
 
 __device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s, int tile) {
@@ -1168,19 +1290,22 @@ __global__ void __launch_bounds__(kTileThreads, MPSA_TILES_MINB) k_tiles(TileArg
     if (SPLIT) {
         const int sp = blockIdx.x % g.split;
         r.out = g.part + ((size_t)blockIdx.y * g.split + sp) * g.N;
-        tile_body<PREC, kPtsPerThread, kTileThreads>(r, blockIdx.x / g.split, sp, g.split);
+        const int tile = blockIdx.x / g.split;
+        tile_body<PREC, kPtsPerThread, kTileThreads>(r, tile, sp, g.split, g.split_free, g.used + (size_t)blockIdx.y * g.nT + tile);
     } else {
         tile_body<PREC, kPtsPerThread, kTileThreads>(r, blockIdx.x);
     }
 }
 
 // kappa[s][j] = sum over the split CTAs' partial sums (FP64 sum, one rounding to FP32)
-__global__ void k_split_sum(int n_sel, int N, int split, const float* __restrict__ part, float* __restrict__ kappa) {
+__global__ void k_split_sum(int n_sel, int N, int split, const int* __restrict__ used, const float* __restrict__ part,
+                            float* __restrict__ kappa) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)n_sel * N) return;
     const int s = (int)(t / N), j = (int)(t % N);
+    const int n = used[(size_t)s * ((N + kTile - 1) / kTile) + j / kTile];
     double acc = 0.0;
-    for (int q = 0; q < split; ++q) acc += part[((size_t)s * split + q) * N + j];
+    for (int q = 0; q < n; ++q) acc += part[((size_t)s * split + q) * N + j];
     kappa[t] = (float)acc;
 }
 
@@ -1312,7 +1437,7 @@ __global__ void k_voigt_eval(int64_t n, const double* __restrict__ v, const doub
                              double* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    out[i] = fp64 ? voigt_H64(v[i], a[i]) : (double)voigt_H((float)v[i], (float)a[i]);
+    out[i] = fp64 ? voigt_H64(v[i], a[i]) : (double)voigt_point((float)v[i], (float)a[i]);
 }
 
 }  // namespace
@@ -1454,8 +1579,9 @@ TileArgs tile_args(const PrepBufs& b, float* kappa) {
     ta.ihi = b.po.ihi;
     ta.ln_tp = b.ln_tp;
     ta.out = kappa;
-    ta.split = 1;
+    ta.split = ta.split_free = 1;
     ta.part = nullptr;
+    ta.used = nullptr;
     return ta;
 }
 
@@ -1496,16 +1622,20 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         g.lnq64 = b.lnq;
         k_tiles64<<<dim3(b.nT, n_sel), 256, 0, st>>>(g);
     } else {
-        // a call with fewer tiles than two waves of the GPU (narrow windows) splits each tile's
-        // candidate lines over several CTAs, up to 64, and adds their partial sums afterwards
+        // a call with fewer tiles than the GPU holds CTAs (narrow windows) splits each tile's
+        // candidate lines over several CTAs, up to 64, and adds their partial sums afterwards: as
+        // many as run at once, one chunk each at least, and up to eight times that for
+        // the tiles with kSplitChunks each (deep rows have ten times the candidates of shallow ones)
         int dev = 0, sms = 0;
         MPSA_CUDA_TRY(cudaGetDevice(&dev));
         MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int64_t ctas = (int64_t)b.nT * n_sel, want = 2ll * sms * MPSA_TILES_MINB;
+        const int64_t ctas = (int64_t)b.nT * n_sel, slots = (int64_t)sms * MPSA_TILES_MINB;
+        const int64_t most = std::min<int64_t>(64, kNumClasses + b.L / kTileThreads);   // chunks a tile can have
         TileArgs tb = ta;
-        tb.split = ctas >= want ? 1 : (int)std::min<int64_t>(64, (want + ctas - 1) / ctas);
+        tb.split_free = (int)std::max<int64_t>(1, std::min(most, slots / ctas));
+        tb.split = ctas > slots ? 1 : (int)std::max<int64_t>(1, std::min(most, 8 * slots / ctas));
         tb.part = nullptr;
-        if (tb.split > 1 && (r = sc.alloc(&tb.part, (size_t)n_sel * tb.split * N))) return r;
+        if (tb.split > 1 && ((r = sc.alloc(&tb.part, (size_t)n_sel * tb.split * N)) || (r = sc.alloc(&tb.used, ctas)))) return r;
         const dim3 grid((unsigned)(b.nT * tb.split), n_sel);
         const bool naive = prec == MPSA_PREC_FP32_NAIVE;
         if (tb.split > 1) {
@@ -1517,7 +1647,7 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         }
         if (tb.split > 1) {
             const int64_t tot = (int64_t)n_sel * N;
-            k_split_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n_sel, N, tb.split, tb.part, kappa);
+            k_split_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n_sel, N, tb.split, tb.used, tb.part, kappa);
         }
     }
     prof_mark(ctx, MPSA_KERNEL_PROFILE, st);

@@ -302,3 +302,29 @@ def test_unsorted_list_is_sorted_by_the_library():
         pl, k, slack, W = oracle_dense(w, L, w.T[s], w.P[s])
         bad, _, _ = opacity_violations(kg2[s], k, pl.kappa_c, slack)
         assert len(bad) == 0
+
+
+@pytest.mark.parametrize("N,R", [(1, 5e5), (2, 5e5), (31, 5e5), (33, 5e5), (257, 5e5), (2047, 5e5), (2048, 5e5), (2049, 5e5),
+                                 (2081, 2e6), (4353, 2e6), (2300, 2e4), (2300, 1e3)])
+def test_interpolated_wings_on_grids_of_every_shape(N, R):
+    # tiles and warp parts of one point, of one segment and beside their full lengths, and grids so
+    # coarse that a part spans percents in wavelength: lines centred on the grid and up to 4
+    # tiles beside it, at pressures from a << 1e-6 to a >> 1, so that the wings reach the tiles from
+    # every distance; dense parity against the oracle
+    lam0 = 400.0
+    lnq = np.log1p(1 / R)
+    w = wl.config_tiny(n_lines=300, lam=(lam0, lam0 * np.exp((N - 0.5) * lnq)), R=R, seed=51)
+    w.T = np.array([4000.0, 9000.0, 6000.0, 2000.0])
+    w.P = np.array([1e4, 1e-2, 1e7, 1e8])
+    se, ss = wl.species_table(w.n_metals)
+    pad = np.exp(8192 * lnq) if R > 1e4 else np.exp(0.2)
+    L = wl.linelist(300, len(se), lam0 / pad, w.grid.lam1_nm * pad, 51)
+    ctx, _ = gpu_context(w, lines=L)
+    kg, kcg, evg = gpu_synth(ctx, w, np.arange(4))
+    assert kg.shape[1] == N
+    for s in range(4):
+        pl, k, slack, W = oracle_dense(w, L, w.T[s], w.P[s])
+        assert abs(kcg[s] / pl.kappa_c - 1) < 2e-5
+        bad, err, bound = opacity_violations(kg[s], k, pl.kappa_c, slack)
+        assert len(bad) == 0, (s, bad[:5], rel_report(kg[s], k, pl.kappa_c))
+        assert W <= evg[s] <= W + 8 * len(L) + 16

@@ -63,3 +63,21 @@ def test_fp64_tiers_against_oracle():
     rel = np.abs(g / o - 1)
     assert rel.max() <= FP64_RTOL, (rel.max(), v[np.argmax(rel)], a[np.argmax(rel)])
     ctx.close()
+
+
+def test_weakly_damped_and_series_forms_against_oracle():
+    # the profile's form for a <= 0.03 inside |z| = 10 (both of its branches, down to the damping of
+    # low-pressure lines) and the series outside it, hugging their boundaries.  Where e^{-V} makes up
+    # H, rounding V = v^2 costs V 2^-24, 2e-6 at V = 34 (a = 1e-16; beyond it the wing takes over)
+    from paper_2105_13611_gb300 import binding
+    ctx = binding.Context(0)
+    e = 1e-6
+    a = np.r_[np.geomspace(1e-16, 0.03, 60), 3e-4 * (1 - e), 3e-4 * (1 + e), 0.03 * (1 - e), 0.03 * (1 + e), 0.3, 3.0, 30.0]
+    v = np.r_[0.0, np.linspace(1e-3, 10.2, 2500), np.geomspace(10.0, 1e4, 200)]
+    V, A = (x.ravel() for x in np.meshgrid(v, a, indexing="ij"))
+    edge = [(np.sqrt(100.0 * f - x * x), x) for x in a if x < 9.9 for f in (1 - e, 1 + e)]
+    V, A = np.r_[V, [x for x, _ in edge]], np.r_[A, [y for _, y in edge]]
+    vf, af = V.astype(np.float32).astype(np.float64), A.astype(np.float32).astype(np.float64)
+    rel = np.abs(device_H(ctx, vf, af, binding.PREC_FP32_COMPENSATED) / H(vf, af) - 1)
+    assert rel.max() <= FP32_RTOL, (rel.max(), vf[np.argmax(rel)], af[np.argmax(rel)])
+    ctx.close()
