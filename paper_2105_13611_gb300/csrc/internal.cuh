@@ -27,9 +27,11 @@ int check_species(const mpsa_ctx* ctx, const char* who);
 int check_grid(const mpsa_lgrid* g, int* N);
 
 // ODF kernel launch on device-resident bounds [K+1], cumulative widths [n_steps+1]
-// and widths [n_steps]; mean_kind MPSA_MEAN_ARITH or MPSA_MEAN_GEOM (odf.cu).
+// and widths [n_steps]; mean_kind MPSA_MEAN_ARITH or MPSA_MEAN_GEOM; longest: the points of the
+// longest interval (odf_longest of the host bounds) (odf.cu).
 int odf_launch(const float* kappa, int n_rows, int64_t N, int K, const int64_t* d_bounds, int n_steps,
-               const double* d_cw, const double* d_w, double* d_out, int mean_kind, cudaStream_t st);
+               const double* d_cw, const double* d_w, double* d_out, int mean_kind, int64_t longest, cudaStream_t st);
+int64_t odf_longest(int K, const int64_t* bounds);
 
 // One-time kernel attribute set-up of the ODF kernel on the current device (call outside
 // stream capture) (odf.cu).

@@ -33,9 +33,11 @@
 // order statistics, exactly in 2^-30 fixed point, and
 //   G(u) = sum_{0 < x < theta} ln x + (u - #{x < theta}) ln theta   (u at or above the zeros);
 // a sub-bin that reaches into the zero values has geometric mean 0.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -337,10 +339,33 @@ __device__ __forceinline__ void resolve_warp(Target& t, const Hist& h, int wb, i
 #ifndef ODF_MINB
 #define ODF_MINB 2
 #endif
+// CLUSTER: a thread-block cluster per (row, interval) instead of one CTA, for calls whose few long
+// intervals would leave most of the GPU idle (odf_launch).  Every CTA of the cluster reads its
+// slice of the interval; the exact integer histograms and ln sums of the others are added to
+// CTA 0's through distributed shared memory, CTA 0 resolves the targets, and the others copy
+// them: the same integers as one CTA would form, so the same result bit for bit.  Ten intervals
+// of 1.4 M points, two rows, geometric means: 2.59 ms with 20 CTAs, 0.50 ms with 20 clusters of 16.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __restrict__ kappa, int64_t N, int K,
                                                      const int64_t* __restrict__ bounds, int n_steps,
                                                      const double* __restrict__ cw, const double* __restrict__ w,
                                                      double* __restrict__ out, int geom, int redo_only) {
+    namespace cg = cooperative_groups;
+    const int C = CLUSTER ? (int)cg::this_cluster().num_blocks() : 1;
+    const int rank = CLUSTER ? (int)cg::this_cluster().block_rank() : 0;
+    // add this CTA's n words at p to CTA 0's (all CTAs call it; a cluster barrier on either side)
+    auto merge = [&](unsigned* p, int n, bool first, bool last) {
+        if (!CLUSTER) return;
+        if (first) cg::this_cluster().sync();
+        if (rank != 0) {
+            unsigned* q = cg::this_cluster().map_shared_rank(p, 0);
+            for (int i = threadIdx.x; i < n; i += kOdfThreads) {
+                const unsigned v = p[i];
+                if (v) atomicAdd(q + i, v);
+            }
+        }
+        if (last) cg::this_cluster().sync();
+    };
     extern __shared__ __align__(16) unsigned sm[];
     const int nt = n_steps - 1;
     const int nslots = nt > kMinSlots ? nt : kMinSlots;
@@ -368,14 +393,28 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
     __shared__ unsigned gacc[5][kMaxTargets + 1];   // geometric pass: exact fixed-point sums per bucket
     __shared__ int n_thr;
 
-    const int k = blockIdx.x, row = blockIdx.y;
+    const int k = CLUSTER ? blockIdx.x / C : blockIdx.x, row = blockIdx.y;
     // after k_odf_gather: only the intervals it marked for this kernel (a uniform early exit)
     if (redo_only && *reinterpret_cast<const unsigned long long*>(out + ((size_t)row * K + k) * n_steps) != kOdfRedo)
         return;
     const int64_t b0 = bounds[k], b1 = bounds[k + 1];
     const long long n = b1 - b0;
-    const float* x = kappa + (size_t)row * N + b0;
+    // this CTA's slice [x, x + nx) of the interval's n values
+    const long long per = (((n + C - 1) / C) + 3) & ~3ll, s0 = min(n, rank * per), nx = min(per, n - s0);
+    const float* x = kappa + (size_t)row * N + b0 + s0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the targets as CTA 0 has them
+    auto share_targets = [&] {
+        if (!CLUSTER) return;
+        cg::this_cluster().sync();
+        if (rank != 0) {
+            constexpr int words = sizeof(Target) / sizeof(unsigned);
+            const unsigned* q = reinterpret_cast<const unsigned*>(cg::this_cluster().map_shared_rank(&tg[0], 0));
+            for (int i = tid; i < nt * words; i += kOdfThreads) reinterpret_cast<unsigned*>(&tg[0])[i] = q[i];
+            if (tid == 0) s_zero = *cg::this_cluster().map_shared_rank(&s_zero, 0);
+        }
+        __syncthreads();
+    };
 
     for (int i = tid; i < kL1Bins; i += kOdfThreads) h1.zero(i);
     if (tid < kL1Bins / 32) tbits[tid] = 0u;
@@ -386,7 +425,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
     {
         unsigned zeros = 0;
         RunAdd run;
-        for_each_value(x, n, [&](unsigned bits, bool valid) {
+        for_each_value(x, nx, [&](unsigned bits, bool valid) {
             if (!valid) return;
             bits &= 0x7fffffffu;
             zeros += bits == 0u ? 1u : 0u;
@@ -397,9 +436,11 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         if (lane == 0 && zeros) atomicAdd(&s_zero, zeros);
     }
     __syncthreads();
+    merge(sm, 3 * kL1Bins, true, false);
+    merge(&s_zero, 1, false, true);
 
     // ---- inclusive scan of the level-1 counts (8 bins per thread)
-    {
+    if (rank == 0) {
         int c[8], v = 0;
         for (int m = 0; m < 8; ++m) { c[m] = (int)h1.count(8 * tid + m); v += c[m]; }
         int incl = v;
@@ -421,7 +462,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         int run = wtot[warp] + incl - v;
         for (int m = 0; m < 8; ++m) { run += c[m]; cincl[8 * tid + m] = run; }
     }
-    if (tid < 256) {
+    if (rank == 0 && tid < 256) {
         unsigned long long acc = 0;
         for (int m = 0; m < kL1PerGroup; ++m) {
             const int b = tid * kL1PerGroup + m;
@@ -430,7 +471,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         gsum[tid] = acc;
     }
     __syncthreads();
-    if (warp == 0) {
+    if (rank == 0 && warp == 0) {
         // FP64 exclusive prefix over the 256 exponent groups (the only FP64 reduction)
         double loc[8];
         double tot = 0.0;
@@ -450,7 +491,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
             run += loc[m];
         }
         if (lane == 31) gpre[256] = run;
-    } else if (warp == 1 && lane < nt) {
+    } else if (rank == 0 && warp == 1 && lane < nt) {
         // each target's level-1 bin: the first bin whose inclusive count exceeds its rank
         Target t;
         // u = c_s n as one rounded FP64 product (no fused multiply-add), so that the rank is
@@ -485,6 +526,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         tg[lane] = t;
     }
     __syncthreads();
+    share_targets();
 
     // ---- levels 2..4.  The counts of the current target prefixes are known from the last
     // histogram; once they fit the candidate buffer, one pass (from L2) collects those
@@ -557,11 +599,11 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         };
         if (collect) {
             if (lvl == 0) {
-                collect_values(x, n, cand, &n_cand, [&](unsigned bits) {
+                collect_values(x, nx, cand, &n_cand, [&](unsigned bits) {
                     return bits != 0u && ((tbits[bits >> (kL1Shift + 5)] >> ((bits >> kL1Shift) & 31u)) & 1u);
                 });
             } else {
-                collect_values(x, n, cand, &n_cand, [&](unsigned bits) { return slot_of(bits) >= 0; });
+                collect_values(x, nx, cand, &n_cand, [&](unsigned bits) { return slot_of(bits) >= 0; });
             }
             __syncthreads();
             nc = min(n_cand, kCand);
@@ -578,7 +620,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
             }
         } else {
             RunAdd run;
-            for_each_value(x, n, [&](unsigned bits, bool valid) {
+            for_each_value(x, nx, [&](unsigned bits, bool valid) {
                 bits &= 0x7fffffffu;
                 const int q = valid ? slot_of(bits) : -1;
                 if (q < 0) return;
@@ -589,9 +631,12 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
             run.flush(h2);
         }
         __syncthreads();
-        if (tid < nd && dpre[tid] == 0u) h2.c[tid * kL2Bins] += s_zero;
+        merge(h2.c, nd * kL2Bins, true, false);
+        merge(h2.hi, nd * kL2Bins, false, false);
+        merge(h2.lo, nd * kL2Bins, false, true);
+        if (rank == 0 && tid < nd && dpre[tid] == 0u) h2.c[tid * kL2Bins] += s_zero;
         __syncthreads();
-        for (int t = warp; t < nt; t += kOdfWarps) {
+        for (int t = warp; t < nt && rank == 0; t += kOdfWarps) {
             if (tg[t].total) continue;
             Target tt = tg[t];
             const Hist hs{h2.c + tt.slot * kL2Bins, h2.hi + tt.slot * kL2Bins, h2.lo + tt.slot * kL2Bins};
@@ -600,6 +645,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         }
         nd_prev = nd;
         __syncthreads();
+        share_targets();
     }
 
     if (geom) {
@@ -634,7 +680,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
             atomicAdd(&gacc[3][rkey], (unsigned)((rsum >> 20) & 1023u));
             atomicAdd(&gacc[4][rkey], (unsigned)(rsum >> 30));
         };
-        for_each_value(x, n, [&](unsigned bits, bool valid) {
+        for_each_value(x, nx, [&](unsigned bits, bool valid) {
             bits &= 0x7fffffffu;
             if (!valid || bits == 0u) return;
             int b = 0;
@@ -650,6 +696,8 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         });
         flush();
         __syncthreads();
+        merge(&gacc[0][0], 5 * (kMaxTargets + 1), true, true);
+        if (rank != 0) return;
         if (tid <= m) {
             const unsigned long long tot = (unsigned long long)gacc[1][tid] + ((unsigned long long)gacc[2][tid] << 10) +
                                            ((unsigned long long)gacc[3][tid] << 20) +
@@ -682,6 +730,8 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         return;
     }
 
+    if (CLUSTER) cg::this_cluster().sync();   // the others have read CTA 0's targets: it may end
+    if (rank != 0) return;
     // ---- step means
     if (tid < n_steps) {
         const int s = tid;
@@ -1290,6 +1340,8 @@ int odf_check(const char* who, int n_rows, int64_t N, int K, const int64_t* boun
     return MPSA_OK;
 }
 
+static int g_odf_max_cluster[kMaxDevices];   // CTAs of k_odf<true> that a cluster can have
+
 int odf_setup() {
     int dev = 0;
     MPSA_CUDA_TRY(cudaGetDevice(&dev));
@@ -1298,12 +1350,27 @@ int odf_setup() {
     static std::once_flag once[kMaxDevices];
     static cudaError_t err[kMaxDevices];
     std::call_once(once[dev], [&] {
-        err[dev] = cudaFuncSetAttribute(k_odf, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        g_odf_max_cluster[dev] = 1;
+        err[dev] = cudaFuncSetAttribute(k_odf<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)odf_smem_bytes(kMaxSteps));
+        if (err[dev] == cudaSuccess)
+            err[dev] = cudaFuncSetAttribute(k_odf<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)odf_smem_bytes(kMaxSteps));
+        if (err[dev] == cudaSuccess)
+            err[dev] = cudaFuncSetAttribute(k_odf<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (err[dev] == cudaSuccess)
             err[dev] = cudaFuncSetAttribute(k_odf_gather<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
         if (err[dev] == cudaSuccess)
             err[dev] = cudaFuncSetAttribute(k_odf_gather<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSmem);
+        if (err[dev] == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(16);
+            cfg.blockDim = dim3(kOdfThreads);
+            cfg.dynamicSmemBytes = odf_smem_bytes(kMaxSteps);
+            int c = 1;
+            if (cudaOccupancyMaxPotentialClusterSize(&c, k_odf<true>, &cfg) == cudaSuccess) g_odf_max_cluster[dev] = c;
+            else cudaGetLastError();
+        }
     });
     if (err[dev] != cudaSuccess)
         return fail(MPSA_ECUDA, "build_odf: cudaFuncSetAttribute: %s", cudaGetErrorString(err[dev]));
@@ -1311,7 +1378,7 @@ int odf_setup() {
 }
 
 int odf_launch(const float* kappa, int n_rows, int64_t N, int K, const int64_t* d_bounds, int n_steps,
-               const double* d_cw, const double* d_w, double* d_out, int mean_kind, cudaStream_t st) {
+               const double* d_cw, const double* d_w, double* d_out, int mean_kind, int64_t longest, cudaStream_t st) {
     int r;
     if ((r = odf_setup())) return r;
     // at most 12 steps: count then gather, and the exact multi-select only for the intervals the
@@ -1325,10 +1392,45 @@ int odf_launch(const float* kappa, int n_rows, int64_t N, int K, const int64_t* 
             k_odf_gather<false><<<dim3(K, n_rows), kGThreads, kGSmem, st>>>(kappa, N, K, d_bounds, n_steps, d_cw, d_w, d_out);
         MPSA_CUDA_TRY(cudaGetLastError());
     }
-    k_odf<<<dim3(K, n_rows), kOdfThreads, odf_smem_bytes(n_steps), st>>>(kappa, N, K, d_bounds, n_steps, d_cw, d_w,
-                                                                         d_out, mean_kind == MPSA_MEAN_GEOM, gather);
+    // Long intervals (the gather leaves those above kGMaxN) in a call with fewer of them than the
+    // GPU holds CTAs of the multi-select (two per SM): a cluster of CTAs each, as large as fits, up
+    // to 16.  Below kGMaxN points a CTA is done in some 40 us, and the barriers of a cluster cost a
+    // good part of that.
+    int dev = 0, sms = 0;
+    MPSA_CUDA_TRY(cudaGetDevice(&dev));
+    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int C = 1;
+    while (longest > kGMaxN && 2 * C <= std::min(16, g_odf_max_cluster[dev]) &&
+           2ll * C * K * n_rows <= ODF_MINB * sms + sms / 8)
+        C *= 2;
+    const size_t smem = odf_smem_bytes(n_steps);
+    const int geom = mean_kind == MPSA_MEAN_GEOM;
+    if (C == 1) {
+        k_odf<false><<<dim3(K, n_rows), kOdfThreads, smem, st>>>(kappa, N, K, d_bounds, n_steps, d_cw, d_w, d_out, geom,
+                                                                 gather);
+    } else {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)K * C, n_rows);
+        cfg.blockDim = dim3(kOdfThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        MPSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_odf<true>, kappa, N, K, d_bounds, n_steps, d_cw, d_w, d_out, geom,
+                                         (int)gather));
+    }
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
+}
+
+int64_t odf_longest(int K, const int64_t* bounds) {
+    int64_t m = 0;
+    for (int k = 0; k < K; ++k) m = std::max(m, bounds[k + 1] - bounds[k]);
+    return m;
 }
 
 }  // namespace mpsa
@@ -1350,7 +1452,7 @@ extern "C" int build_odf(mpsa_ctx* ctx, const float* kappa, int32_t n_rows, int6
     MPSA_CUDA_TRY(cudaMemcpyAsync(d_cw, cw.data(), (n_steps + 1) * sizeof(double), cudaMemcpyHostToDevice, st));
     MPSA_CUDA_TRY(cudaMemcpyAsync(d_w, widths, n_steps * sizeof(double), cudaMemcpyHostToDevice, st));
     prof_mark(ctx, MPSA_KERNEL_ODF, st);
-    r = odf_launch(kappa, n_rows, N, K, d_b, n_steps, d_cw, d_w, odf_out, mean_kind, st);
+    r = odf_launch(kappa, n_rows, N, K, d_b, n_steps, d_cw, d_w, odf_out, mean_kind, odf_longest(K, bounds), st);
     prof_mark(ctx, MPSA_KERNEL_ODF, st);
     return r;
 }
@@ -1420,5 +1522,5 @@ extern "C" int build_odf_noalloc(int32_t device, const float* kappa, int32_t n_r
     MPSA_CUDA_TRY(cudaMemcpyAsync(d_b, bounds, (K + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     MPSA_CUDA_TRY(cudaMemcpyAsync(d_cw, cw, (n_steps + 1) * sizeof(double), cudaMemcpyHostToDevice, st));
     MPSA_CUDA_TRY(cudaMemcpyAsync(d_w, widths, n_steps * sizeof(double), cudaMemcpyHostToDevice, st));
-    return odf_launch(kappa, n_rows, N, K, d_b, n_steps, d_cw, d_w, odf_out, mean_kind, st);
+    return odf_launch(kappa, n_rows, N, K, d_b, n_steps, d_cw, d_w, odf_out, mean_kind, odf_longest(K, bounds), st);
 }

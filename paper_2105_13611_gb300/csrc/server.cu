@@ -199,7 +199,7 @@ int odf_chunk(mpsa_server* s, Req* r, Slot& sl) {
                          nullptr, nullptr, st)))
         return rc;
     if ((rc = odf_launch(r->kap, nrow, N, K, r->db, ns, r->dcw, r->dw, r->dout + (size_t)off * K * ns, r->mean_kind,
-                         st)))
+                         odf_longest(K, r->bounds.data()), st)))
         return rc;
     r->next_row = off + nrow;
     if (r->next_row == n_sel) {

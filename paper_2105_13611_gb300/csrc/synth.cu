@@ -1794,6 +1794,7 @@ struct mpsa_batch {
         int K = 0, n_steps = 0, mean_kind = MPSA_MEAN_ARITH;
         int64_t* d_bounds = nullptr;
         double *d_cw = nullptr, *d_w = nullptr, *odf = nullptr;
+        int64_t longest = 0;
     };
     std::vector<Group> groups;
     mpsa::RowDesc* d_rows = nullptr;
@@ -1895,6 +1896,7 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
             G.n_steps = q.n_steps;
             G.mean_kind = q.mean_kind;
             G.odf = q.odf_out;
+            G.longest = odf_longest(q.K, q.bounds);
             if ((r = balloc(b, &G.d_bounds, q.K + 1)) || (r = balloc(b, &G.d_cw, q.n_steps + 1)) ||
                 (r = balloc(b, &G.d_w, q.n_steps)))
                 return r;
@@ -2013,7 +2015,7 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
     if (rc == MPSA_OK) rc = persistent_launch(b->cfg, b->prec, b->d_rows, b->d_units, b->n_units, b->d_counter, cap);
     if (rc == MPSA_OK)
         for (auto& G : b->groups)
-            if (G.K > 0 && (rc = odf_launch(G.kappa, G.n_sel, G.N, G.K, G.d_bounds, G.n_steps, G.d_cw, G.d_w, G.odf, G.mean_kind, cap)))
+            if (G.K > 0 && (rc = odf_launch(G.kappa, G.n_sel, G.N, G.K, G.d_bounds, G.n_steps, G.d_cw, G.d_w, G.odf, G.mean_kind, G.longest, cap)))
                 break;
     e = cudaStreamEndCapture(cap, &b->graph);
     cudaStreamDestroy(cap);

@@ -180,3 +180,43 @@ def test_gather_and_multiselect_paths():
     # one step and two steps (no boundary, one boundary)
     check(x, b, [1.0])
     check(x, b, [0.5, 0.5])
+
+
+@pytest.mark.parametrize("geom", [False, True])
+@pytest.mark.parametrize("lens,n_steps,kind", [((65537,), 12, "lines"), ((65541, 70003), 12, "lines"), ((300007,), 1, "lines"),
+                                               ((131072, 3, 66000), 32, "lines"), ((2097151,), 12, "lines"),
+                                               ((200001,), 20, "equal"), ((90001,), 12, "zeros"), ((100003,), 5, "wide")])
+def test_clusters_give_the_bits_of_one_cta(lens, n_steps, kind, geom):
+    # a call with few long intervals shares each of them out over a cluster of CTAs; with many rows
+    # every interval has one CTA.  Both form the same exact integers: the results agree bit for
+    # bit (odd lengths and starts, one to 32 steps, equal values, zeros, every exponent)
+    import torch
+    from paper_2105_13611_gb300 import binding
+    rng = np.random.default_rng(sum(lens) + n_steps)
+    start = 5
+    b = start + np.r_[0, np.cumsum(lens)]
+    N = int(b[-1]) + 2
+    x = (10.0 ** rng.normal(-1, 2, N)).astype(np.float32)
+    if kind == "equal":
+        x[:] = 0.3
+    elif kind == "zeros":
+        x[: N // 3] = 0.0
+    elif kind == "wide":
+        x = (2.0 ** rng.uniform(-149, 127, N)).astype(np.float32)
+    w = wl.ODF_WIDTHS_12 if n_steps == 12 else np.full(n_steps, 1.0 / n_steps)
+    ctx = binding.Context(0)
+    kind_ = binding.MEAN_GEOM if geom else binding.MEAN_ARITH
+    one = torch.from_numpy(x)[None].cuda()
+    o1 = torch.empty((1, len(lens), n_steps), dtype=torch.float64, device="cuda")
+    ctx.build_odf(one, b, w, o1, kind_)
+    rows = 2 * torch.cuda.get_device_properties(0).multi_processor_count + 100
+    many = one.expand(rows, N).contiguous()
+    om = torch.empty((rows, len(lens), n_steps), dtype=torch.float64, device="cuda")
+    ctx.build_odf(many, b, w, om, kind_)
+    torch.cuda.synchronize()
+    assert torch.isfinite(o1).all() and torch.equal(om, o1.expand_as(om))
+    if not geom:
+        from oracle import odf as od
+        o = od.odf(x.astype(np.float64), b, w)
+        assert np.all(np.abs(o1[0].cpu().numpy() - o) <= 1e-5 * np.abs(o) + 1e-300)
+    ctx.close()
