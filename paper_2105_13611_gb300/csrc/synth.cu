@@ -7,19 +7,20 @@
 // opacity of the synthetic workload).
 //
 // Pipeline (all on the caller's stream):
-//   k_place        per line: centre index c and fraction f on the grid (FP64 log)
+//   k_distance     per line: how far off the grid its centre is
 //   k_consts       per (row, species): ln(sqrt(pi) e^2/(m_e c) N/U / rho), u, c/u from the FP64 table
 //   k_kappa0       per (row, line): ln S, a, ln kappa0 in FP32 log space
 //   k_med_*        per row: lower median of ln kappa0 by multi-CTA radix selection -> ln t_p, kappa_c
-//   k_prep         per (row, line): strength relative to t_p, cut windows (outer: no point
-//                  beyond can pass the cut; inner: every point inside passes), width class
+//   k_prep         per (row, line): peak against the cut, reach of the wing; the lines left, listed
+//   k_place        the listed lines' centre index c and fraction f on the grid (FP64 log)
+//   k_windows      per listed line: cut windows (outer: no point beyond can pass the cut; inner:
+//                  every point inside passes), width class
 //   k_scan_class, k_scan_fin, k_scatter   stable counting sort of the kept lines by width class
 //   k_ranges       per (row, class, tile boundary): first line whose centre lies at or
 //                  beyond the boundary (binary search in the centre-sorted class)
-//   k_tiles        the profile kernel: one CTA per (row, 2048-point tile); each thread owns
-//                  8 grid points in registers; every line whose window reaches the tile is
-//                  evaluated at the thread's points; FP32 partial sums per chunk of lines are
-//                  folded into Kahan-compensated totals; no atomics; coalesced stores.
+//   k_tiles        the profile kernel: one CTA per (row, 2048-point tile) (or several, on calls with
+//                  few tiles); wings summed at Chebyshev nodes, the rest point by point; FP32
+//                  partial sums folded into Kahan-compensated totals; no atomics; coalesced stores.
 #include <math.h>
 #include <stdio.h>
 
@@ -39,20 +40,76 @@ constexpr float kFourPi = 12.566370614359172f;
 
 __device__ __forceinline__ int floordiv(int a, int b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
 
+// A wavelength grid as the preparation kernels see it: lambda_j = lam0 e^{j lnq}, N points, the
+// index of its per-line arrays (distance, flags, placement).
+struct GridDesc {
+    double lam0_nm, lnq64;
+    float lnq, inv_first, inv_last;   // ln q and 1/lambda of the first and last point [1/nm]
+    int N, index;
+};
+// The grid of each row: one for all rows, or grids[row].
+struct RowGrids {
+    GridDesc one;
+    const GridDesc* many;
+    __device__ __forceinline__ GridDesc of(int s) const { return many ? many[s] : one; }
+};
+
 // ---------------------------------------------------------------------------
-// k_place: c = floor(x0), f = x0 - c with x0 = ln(lambda0/lambda_start)/ln(1+1/R)
-// (FP64: an FP32 logarithm would misplace lines by whole grid points).
-__global__ void k_place(int64_t L, const double* __restrict__ lam_nm, double lam0_nm, double lnq,
-                        int* __restrict__ c_out, float* __restrict__ f_out, float* __restrict__ lamcm_out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// k_distance: per (grid, line), a lower bound of the distance between a centre off the grid and
+// the grid's nearest point in relative frequency, |v| / kv there:
+//   1 - lambda/lambda_0 (centre shortward), lambda/lambda_{N-1} - 1 (longward),
+// negative for centres on the grid.  Four grid points and the FP32 rounding are taken off, so FP32 will do, and no
+// logarithm is needed: the exact position of a line (k_place) is formed only if it reaches the
+// grid.  Clears the line's flag.
+__global__ void k_distance(int64_t L, size_t ld, int n_grids, const double* __restrict__ lam_nm, GridDesc one,
+                           const GridDesc* __restrict__ many, float* __restrict__ dist, unsigned char* __restrict__ flag) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= L) return;
-    const double lam = lam_nm[i];
-    double x0 = log(lam / lam0_nm) / lnq;
-    x0 = fmin(fmax(x0, -268435456.0), 268435456.0);
-    const double c = floor(x0);
-    c_out[i] = (int)c;
-    f_out[i] = (float)(x0 - c);
-    lamcm_out[i] = (float)(lam * 1e-7);
+    const float lam = (float)lam_nm[i];
+    for (int g = blockIdx.y; g < n_grids; g += gridDim.y) {
+        const GridDesc q = many ? many[g] : one;
+        const float d = fmaxf(fmaf(-lam, q.inv_first, 1.f), fmaf(lam, q.inv_last, -1.f));
+        // lambda, 1/lambda_0 and the product round by 6e-8 each
+        dist[g * ld + i] = fmaf(d, 1.f - 4.2f * q.lnq - 1e-5f, -4.2f * q.lnq - 4e-7f);
+        flag[g * ld + i] = 0;
+    }
+}
+
+// k_place: c = floor(x0), f = x0 - c with x0 = ln(lambda0/lambda_start)/ln(1+1/R) (FP64: an FP32
+// logarithm would misplace lines by whole grid points) of the lines that some row of the
+// grid keeps.  A CTA gathers the kept ones of its 1024 lines and then takes their logarithms
+// with full warps: FP64 bounds this kernel, and of a 5e6-line list a window of a few nm keeps a
+// few per cent (all 5e6: 484 us, 104 us for the 3 per cent that 80 depths keep of a 7 nm window).
+__global__ void __launch_bounds__(kPrepThreads) k_place(int64_t L, size_t ld, const double* __restrict__ lam_nm, GridDesc one,
+                                                        const GridDesc* __restrict__ many,
+                                                        const unsigned char* __restrict__ flag, int* __restrict__ c_out,
+                                                        float* __restrict__ f_out) {
+    __shared__ short list[kPrepLines];
+    __shared__ int n_list;
+    const int g = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    const int64_t i0 = (int64_t)blockIdx.x * kPrepLines;
+    if (tid == 0) n_list = 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPrepLines / kPrepThreads; ++k) {
+        const int off = k * kPrepThreads + tid;
+        const bool on = i0 + off < L && flag[g * ld + i0 + off] != 0;
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(&n_list, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (on) list[base + __popc(m & ((1u << lane) - 1u))] = (short)off;
+    }
+    __syncthreads();
+    const GridDesc q = many ? many[g] : one;
+    for (int t = tid; t < n_list; t += kPrepThreads) {
+        const int64_t i = i0 + list[t];
+        double x0 = log(lam_nm[i] / q.lam0_nm) / q.lnq64;
+        x0 = fmin(fmax(x0, -268435456.0), 268435456.0);
+        const double c = floor(x0);
+        c_out[g * ld + i] = (int)c;
+        f_out[g * ld + i] = (float)(x0 - c);
+    }
 }
 
 // per-row scalars (FP32) and per-(row, species) scalars
@@ -104,15 +161,15 @@ __global__ void k_consts(int n_sel, const int* __restrict__ sel, int n_sp, const
 // constants are read and formed once, then each row's values follow.
 constexpr int kKappa0Rows = 8;
 
-__global__ void k_kappa0(int64_t L, int n_sel, const int* __restrict__ species, const float* __restrict__ loggf,
+__global__ void k_kappa0(int64_t L, size_t ld, int n_sel, const int* __restrict__ species, const float* __restrict__ loggf,
                          const float* __restrict__ E, const float* __restrict__ lgR, const float* __restrict__ lgS,
-                         const float* __restrict__ lgW, const float* __restrict__ lamcm, int n_sp,
+                         const float* __restrict__ lgW, const double* __restrict__ lam_nm, int n_sp,
                          const RowConst* __restrict__ rc, const SpConst* __restrict__ sc,
                          float* __restrict__ lnS_out, float* __restrict__ a_out, float* __restrict__ lnk0_out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= L) return;
     const int sp = species[i];
-    const float lam = lamcm[i], lglam = logf(lam), lg = loggf[i], Ei = E[i];
+    const float lam = (float)(lam_nm[i] * 1e-7), lglam = logf(lam), lg = loggf[i], Ei = E[i];
     const float gR = exp10f(lgR[i]), gS = exp10f(lgS[i]), gW = exp10f(lgW[i]);
     const int s1 = min(n_sel, (int)(blockIdx.y + 1) * kKappa0Rows);
     for (int s = blockIdx.y * kKappa0Rows; s < s1; ++s) {
@@ -123,7 +180,7 @@ __global__ void k_kappa0(int64_t L, int n_sel, const int* __restrict__ species, 
         const float lnDnu = logf(q.u) - lglam;
         const float stim = -expm1f(-r.hc_kT_cm / lam);
         const float lnS = q.lnC + lg * kLn10 - Ei * r.inv_kT_eV + logf(stim) - lnDnu;
-        const size_t o = (size_t)s * L + i;
+        const size_t o = s * ld + i;
         lnS_out[o] = lnS;
         a_out[o] = a;
         lnk0_out[o] = lnS + logf(voigt_H(0.f, a));
@@ -158,7 +215,7 @@ __global__ void k_med_init(int n_sel, int64_t L, MedState* __restrict__ st, unsi
     if (i < n_sel) st[i] = MedState{0u, (unsigned)((L - 1) / 2)};
 }
 
-__global__ void __launch_bounds__(1024) k_med_hist(int64_t L, const float* __restrict__ lnk0, int level,
+__global__ void __launch_bounds__(1024) k_med_hist(int64_t L, size_t ld, const float* __restrict__ lnk0, int level,
                                                    const MedState* __restrict__ st, unsigned* __restrict__ ghist) {
     __shared__ unsigned h[kMedBins];
     const int s = blockIdx.y;
@@ -167,7 +224,7 @@ __global__ void __launch_bounds__(1024) k_med_hist(int64_t L, const float* __res
     const unsigned prefix = st[s].prefix;
     for (int i = threadIdx.x; i < kMedBins; i += blockDim.x) h[i] = 0u;
     __syncthreads();
-    const float* x = lnk0 + (size_t)s * L;
+    const float* x = lnk0 + s * ld;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L; i += stride) {
         const unsigned k = fkey(__ldg(x + i));
@@ -306,11 +363,19 @@ __device__ void crossing(float a, float t, float vb, float* v_ge, float* v_lt) {
     *v_lt = expf(xhi);
 }
 
+// The inner speed lies just inside the outer crossing: where H falls at least like v^-1 there (wings
+// and the flanks of the core) it passes t_in at 2e-4 of v inside, which one evaluation confirms;
+// only lines whose peak is just above the cut take a search of their own.
 __device__ void cut_speeds(float a, float r, float* v_out, float* v_in) {
     const float t_out = r * (1.f - 1e-4f), t_in = r * (1.f + 1e-4f);
     float ge, lt;
     crossing(a, t_out, v_bound(a, t_out), &ge, &lt);
     *v_out = lt;
+    const float vi = ge * (1.f - 2e-4f);
+    if (ge > 0.f && voigt_H(vi, a) >= t_in) {
+        *v_in = vi;
+        return;
+    }
     if (voigt_H(0.f, a) < t_in) {
         *v_in = -1.f;
         return;
@@ -337,101 +402,112 @@ struct __align__(16) LineRec {
     float f, kv, a;
     float srel;
     int ilo, ihi, jlo;
-    int jhi, pad0, pad1, pad2;
+    int jhi, line, pad0, pad1;
 };
 
+// Lists of the lines that k_prep lets through, per row (compact: every array is indexed by the
+// position in the list).  The lines of a prep block are one run of the list, in line order.
 struct PrepOut {
-    int* c;
-    float* f;
-    float* srel;
-    float* a;
-    float* kv;
-    int* jlo;
-    int* jhi;
-    int* ilo;
-    int* ihi;
-    unsigned char* cls;
+    int* surv;            // [n_sel][L] line indices
+    int* nsurv;           // [n_sel] their number
+    int2* run;            // [n_sel][nb] each prep block's run: first position, length
+    float* srel;          // [n_sel][L]
+    int4* win;            // [n_sel][L] jlo, jhi, ilo, ihi
+    unsigned char* cls;   // [n_sel][L] width class, kDropped if the window misses the grid
     int* blkcnt;          // [n_sel][kNumClasses][nb]
     long long* wpart;     // [n_sel][nb]
-    int* surv;            // [n_sel][L] lines left for the crossing search, each prep block's together
-    int* nsurv;           // [n_sel] their number
 };
 
 // k_prep: one CTA of kPrepThreads threads per block of kPrepLines lines of one row.  Every line
-// is tested: its peak against the cut threshold, then the cheap bound below on its window's
-// reach.  The lines that remain are appended, as one run per block, to the row's list for
-// k_windows; the others are marked dropped.  The block's class counts and window-length sum,
-// which k_windows adds to, start at zero here.
-__global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, int N, float lnq, const int* __restrict__ species,
-                                                       const int* __restrict__ cpos, const float* __restrict__ fpos,
+// is tested: its peak against the cut threshold, then whether its wing can reach the grid.  With
+// H <= 4a/(sqrt(pi) v^2) + exp(-v^2/4) (the convolution split at |t| = v/2) and 1/r = s_rel =
+// e^rel, rel = ln S - ln t_p <= 88, a line stays below the cut beyond max(w, 2 sqrt(ln 2 + rel)),
+// w^2 = 8 a s_rel/sqrt(pi), the second of which is below 19: a line whose nearest grid point
+// lies at |v| = kv dist is dropped if that is above 22 and 3 per cent above w (k_windows drops
+// exactly what is left).  The squares are compared, so the test costs one exponential and no
+// logarithm, root or division: 3.4 -> 1.4 ms for 4e8 (row, line) pairs, which it reads at 16 B each.  The lines that
+// remain are appended, as one run per block in line order, to the row's list, and flagged for
+// k_place.  The block's class counts and window-length sum, which k_windows adds to, start at
+// zero here.
+__global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, RowGrids grids,
+                                                       const int* __restrict__ species,
+                                                       const float* __restrict__ dist, unsigned char* __restrict__ flag,
                                                        int n_sp, const SpConst* __restrict__ sc,
                                                        const float* __restrict__ lnS, const float* __restrict__ av,
                                                        const float* __restrict__ lnk0, const float* __restrict__ ln_tp,
                                                        int nb, PrepOut o) {
-    __shared__ short s_list[kPrepLines];
-    __shared__ int s_n, s_base;
-    const int s = blockIdx.y, lane = threadIdx.x & 31;
-    const int64_t i0 = (int64_t)blockIdx.x * kPrepLines;
-    if (threadIdx.x == 0) s_n = 0;
-    if (threadIdx.x < kNumClasses) o.blkcnt[((size_t)s * kNumClasses + threadIdx.x) * nb + blockIdx.x] = 0;
-    if (threadIdx.x == 0) o.wpart[(size_t)s * nb + blockIdx.x] = 0;
-    __syncthreads();
+    static_assert(kPrepLines == 4 * kPrepThreads, "four lines per thread");
+    constexpr int kWarps = kPrepThreads / 32;
+    __shared__ int s_cnt[kWarps], s_base;
+    const int s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t i0 = (int64_t)blockIdx.x * kPrepLines + 4 * tid;
+    if (tid < kNumClasses) o.blkcnt[((size_t)s * kNumClasses + tid) * nb + blockIdx.x] = 0;
+    if (tid == 0) o.wpart[(size_t)s * nb + blockIdx.x] = 0;
+    const size_t gL = grids.of(s).index * ld;
     const float ltp = ln_tp[s];
-    constexpr int kPer = kPrepLines / kPrepThreads;
-    // every load of the thread's lines first, so they are in flight together
-    float lk[kPer], ls[kPer], la[kPer], lf[kPer], lkv[kPer];
-    int lc[kPer];
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const int64_t i = i0 + k * kPrepThreads + threadIdx.x;
-        lk[k] = -INFINITY;
-        if (i < L) {
-            const size_t q = (size_t)s * L + i;
-            lk[k] = lnk0[q];
-            ls[k] = lnS[q];
-            la[k] = av[q];
-            lf[k] = fpos[i];
-            lc[k] = cpos[i];
-            lkv[k] = sc[(size_t)s * n_sp + species[i]].kv;
-        }
+    float lk[4], ls[4], la[4], di[4];
+    if (i0 < L) {   // rows are padded to a multiple of four lines
+        const float4 k4 = __ldcs(reinterpret_cast<const float4*>(lnk0 + s * ld + i0));
+        const float4 s4 = __ldg(reinterpret_cast<const float4*>(lnS + s * ld + i0));
+        const float4 a4 = __ldg(reinterpret_cast<const float4*>(av + s * ld + i0));
+        const float4 d4 = __ldg(reinterpret_cast<const float4*>(dist + gL + i0));
+        lk[0] = k4.x, lk[1] = k4.y, lk[2] = k4.z, lk[3] = k4.w;
+        ls[0] = s4.x, ls[1] = s4.y, ls[2] = s4.z, ls[3] = s4.w;
+        la[0] = a4.x, la[1] = a4.y, la[2] = a4.z, la[3] = a4.w;
+        di[0] = d4.x, di[1] = d4.y, di[2] = d4.z, di[3] = d4.w;
     }
+    float kv_min = INFINITY;   // of the row's species
+    for (int p = lane; p < n_sp; p += 32) kv_min = fminf(kv_min, sc[(size_t)s * n_sp + p].kv);
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const int off = k * kPrepThreads + threadIdx.x;
-        const int64_t i = i0 + off;
-        bool reach = false;
-        if (i < L) {
-            reach = lk[k] >= ltp;
-            const int c = lc[k];
-            if (reach && (c < -2 || c > N)) {
-                // A centre off the grid: H(v, a) <= 4a/(sqrt(pi) v^2) + exp(-v^2/4) (the convolution
-                // split at |t| = v/2), so the line stays below the cut beyond vb, with
-                // 1/r = s_rel = e^rel, rel = ln S - ln t_p >= 0 (the peak passed).  The line is
-                // kept if its bound window [c + f - d_blue(vb) - 2, c + f + d_red(vb) + 2] reaches
-                // the grid; the grid side's offset is compared in FP32 (FP64 issues slowly on this
-                // part) against an integer bound rounded towards keeping the line (k_windows drops
-                // the few extra ones exactly).  Centres on the grid are kept without a test.
-                const float rel = fminf(ls[k] - ltp, 88.f);
-                const float a = la[k], kv = lkv[k], f = lf[k];
-                const float vb =
-                    fmaxf(sqrtf(8.f * kInvSqrtPi * a * expf(rel)), 2.f * sqrtf(fmaxf(0.69314718f + rel, 0.f))) + 1.f;
-                if (c < -2) reach = fminf(f + d_red(vb, kv, lnq), 1.0e9f) >= __int2float_rd(-2 - c);
-                else reach = fmaxf(f - d_blue(vb, kv, lnq), -1.0e9f) <= __int2float_ru(N + 1 - c);
+    for (int d = 16; d > 0; d >>= 1) kv_min = fminf(kv_min, __shfl_xor_sync(0xffffffffu, kv_min, d));
+    unsigned reach = 0u;   // bit k: line i0 + k is kept
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (i0 + k < L && lk[k] >= ltp) {
+            const float w2 = 8.f * kInvSqrtPi * 1.06f * la[k] * __expf(fminf(ls[k] - ltp, 88.f));
+            float need = kv_min * di[k];
+            bool in = need <= 22.f || w2 >= need * need;
+            if (in && need > 0.f) {   // off the grid, and not too far for the slowest species: its own kv
+                need = sc[(size_t)s * n_sp + species[i0 + k]].kv * di[k];
+                in = need <= 22.f || w2 >= need * need;
             }
-            // only kept lines are read later (through their bucket), so dropped ones write the class alone
-            if (!reach) o.cls[(size_t)s * L + i] = kDropped;
+            if (in) reach |= 1u << k;
         }
-        const unsigned m = __ballot_sync(0xffffffffu, reach);
-        int base = 0;
-        if (lane == 0 && m) base = atomicAdd(&s_n, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (reach) s_list[base + __popc(m & ((1u << lane) - 1u))] = (short)off;
+    }
+    // the lines' places in the run: within the warp, then over the warps
+    const int cnt = __popc(reach);
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += y;
+    }
+    if (lane == 31) s_cnt[warp] = incl;
+    __syncthreads();
+    int before = 0, n = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const int c = s_cnt[w];
+        if (w < warp) before += c;
+        n += c;
+    }
+    if (n == 0) {
+        if (tid == 0) o.run[(size_t)s * nb + blockIdx.x] = make_int2(0, 0);
+        return;
+    }
+    if (tid == 0) {
+        const int base = atomicAdd(&o.nsurv[s], n);
+        s_base = base;
+        o.run[(size_t)s * nb + blockIdx.x] = make_int2(base, n);
     }
     __syncthreads();
-    const int n = s_n;
-    if (threadIdx.x == 0 && n > 0) s_base = atomicAdd(&o.nsurv[s], n);
-    __syncthreads();
-    for (int t = threadIdx.x; t < n; t += kPrepThreads) o.surv[(size_t)s * L + s_base + t] = (int)(i0 + s_list[t]);
+    int pos = s_base + before + incl - cnt;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if ((reach >> k) & 1u) {
+            o.surv[s * ld + pos++] = (int)(i0 + k);
+            flag[gL + i0 + k] = 1;
+        }
 }
 
 // k_windows: the outer and inner cut windows of every listed line (crossing searches on the
@@ -439,13 +515,17 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, int N, float l
 // dense whatever fraction of the lines the cheap bound kept.  The per-block class counts and
 // window-length sums are integer atomics, combined first across the lanes of a warp that
 // hold lines of the same prep block (a block's lines are one run of the list).
-__global__ void __launch_bounds__(kPrepThreads) k_windows(int64_t L, int N, float lnq, const int* __restrict__ species,
+__global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids grids, const int* __restrict__ species,
                                                           const int* __restrict__ cpos, const float* __restrict__ fpos,
                                                           int n_sp, const SpConst* __restrict__ sc,
                                                           const float* __restrict__ lnS, const float* __restrict__ av,
                                                           const float* __restrict__ ln_tp, int nb, PrepOut o) {
     const int s = blockIdx.y, lane = threadIdx.x & 31;
     const int n = o.nsurv[s];
+    const GridDesc gd = grids.of(s);
+    const int N = gd.N;
+    const float lnq = gd.lnq;
+    const size_t gL = gd.index * ld;
     const float ltp = ln_tp[s];
     const int stride = gridDim.x * kPrepThreads;
     // every lane of a warp runs the same number of passes (the warp-wide combining below)
@@ -455,13 +535,13 @@ __global__ void __launch_bounds__(kPrepThreads) k_windows(int64_t L, int N, floa
         int blk = -1 - lane, key2 = -1;   // lanes past the list: a segment of their own
         long long w = 0;
         if (t < n) {
-            const int64_t i = o.surv[(size_t)s * L + t];
-            const size_t q = (size_t)s * L + i;
+            const int64_t i = o.surv[s * ld + t];
+            const size_t q = s * ld + i;
             blk = (int)(i / kPrepLines);
             const float rel = fminf(lnS[q] - ltp, 88.f);
             const float r = expf(-rel);
-            const int c = cpos[i];
-            const float f = fpos[i], a = av[q], kv = sc[(size_t)s * n_sp + species[i]].kv;
+            const int c = cpos[gL + i];
+            const float f = fpos[gL + i], a = av[q], kv = sc[(size_t)s * n_sp + species[i]].kv;
             unsigned char cl = kDropped;
             const float srel = expf(rel);
             float vo, vi;
@@ -490,17 +570,10 @@ __global__ void __launch_bounds__(kPrepThreads) k_windows(int64_t L, int N, floa
                 cl = (unsigned char)(32 - __clz(hw));
                 key2 = blk * kNumClasses + cl;
                 w = (long long)(jhi - jlo + 1);
-                o.c[q] = c;
-                o.f[q] = f;
-                o.srel[q] = srel;
-                o.a[q] = a;
-                o.kv[q] = kv;
-                o.jlo[q] = jlo;
-                o.jhi[q] = jhi;
-                o.ilo[q] = ilo;
-                o.ihi[q] = ihi;
+                o.srel[s * ld + t] = srel;
+                o.win[s * ld + t] = make_int4(jlo, jhi, ilo, ihi);
             }
-            o.cls[q] = cl;
+            o.cls[s * ld + t] = cl;
         }
         // window-length sum of each prep block's run of lanes (runs are contiguous): segmented
         // inclusive scan, the run's last lane adds the total
@@ -584,79 +657,59 @@ __global__ void __launch_bounds__(1024) k_scan_fin(int nb, const int* __restrict
     }
 }
 
-// k_scatter: stable placement of kept lines into class buckets (centre order preserved), one
-// CTA per prep block of kPrepLines lines; warp w takes the block's w-th run of consecutive
-// lines.  A first pass counts each warp's lines per class, a scan over the warps gives the
-// offsets, and a second pass places the lines.  A block that kept no line (window-length sum
-// zero) returns at once.
-__global__ void __launch_bounds__(kPrepThreads) k_scatter(int64_t L, int N, const unsigned char* __restrict__ cls,
-                                                          const int* __restrict__ cpos, const int* __restrict__ blkoff,
-                                                          const int* __restrict__ classbase, int nb,
-                                                          int* __restrict__ bidx, int* __restrict__ bkey,
-                                                          const PrepOut o, LineRec* __restrict__ rec) {
-    constexpr int kWarps = kPrepThreads / 32, kGroups = kPrepLines / kPrepThreads;
-    __shared__ int wcnt[kWarps][kNumClasses];
-    const int s = blockIdx.y;
-    if (o.wpart[(size_t)s * nb + blockIdx.x] == 0) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int t = threadIdx.x; t < kWarps * kNumClasses; t += kPrepThreads) (&wcnt[0][0])[t] = 0;
-    __syncthreads();
-    const int64_t i0 = (int64_t)blockIdx.x * kPrepLines + (int64_t)warp * (32 * kGroups) + lane;
+// k_scatter: stable placement of the kept lines into class buckets (centre order preserved): a
+// warp per prep block's run of the row's list, 32 lines at a time; the lanes of one class rank
+// themselves, and the warp keeps how many of each class it has placed.  Blocks without kept lines
+// cost one load.
+__global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids grids, const int* __restrict__ species,
+                                                          const int* __restrict__ cpos, const float* __restrict__ fpos,
+                                                          int n_sp, const SpConst* __restrict__ sc,
+                                                          const float* __restrict__ av, const int* __restrict__ blkoff,
+                                                          const int* __restrict__ classbase, int nb, const PrepOut o,
+                                                          LineRec* __restrict__ rec) {
+    constexpr int kWarps = kPrepThreads / 32;
+    __shared__ int placed[kWarps][32];
+    const int s = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int blk = blockIdx.x * kWarps + warp;
+    if (blk >= nb) return;
+    const int2 run = o.run[(size_t)s * nb + blk];
+    if (run.y == 0) return;
+    const size_t sL = s * ld, gL = grids.of(s).index * ld;
+    if (lane < kNumClasses)
+        placed[warp][lane] = classbase[s * kNumClasses + lane] + blkoff[((size_t)s * kNumClasses + lane) * nb + blk];
+    __syncwarp();
     const unsigned lt = (1u << lane) - 1u;
-    int b[kGroups];
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g) {
-        const int64_t i = i0 + 32 * g;
-        b[g] = (i < L) ? (int)cls[(size_t)s * L + i] : (int)kDropped;
-        const unsigned same = __match_any_sync(0xffffffffu, b[g]);
-        if (b[g] < kNumClasses && __popc(same & lt) == 0) wcnt[warp][b[g]] += __popc(same);
-        __syncwarp();
-    }
-    __syncthreads();
-    if (threadIdx.x < kNumClasses) {
-        int run = 0;
-        for (int w = 0; w < kWarps; ++w) {
-            const int t = wcnt[w][threadIdx.x];
-            wcnt[w][threadIdx.x] = run;
-            run += t;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g) {
-        const int64_t i = i0 + 32 * g;
-        const int bg = b[g];
-        const unsigned same = __match_any_sync(0xffffffffu, bg);
+    for (int t0 = run.x; t0 < run.x + run.y; t0 += 32) {
+        const int t = t0 + lane;
+        const int b = t < run.x + run.y ? (int)o.cls[sL + t] : (int)kDropped;
+        const unsigned same = __match_any_sync(0xffffffffu, b);
         const int lrank = __popc(same & lt);
-        if (bg < kNumClasses) {
-            const int pos = classbase[s * kNumClasses + bg] + blkoff[((size_t)s * kNumClasses + bg) * nb + blockIdx.x] +
-                            wcnt[warp][bg] + lrank;
-            const int c = cpos[i];
-            bidx[(size_t)s * L + pos] = (int)i;
-            bkey[(size_t)s * L + pos] = c < -1 ? -1 : (c > N ? N : c);
-            const size_t q = (size_t)s * L + i;
+        if (b < kNumClasses) {
+            const int i = o.surv[sL + t];
+            const int4 w = o.win[sL + t];
             LineRec r;
-            r.c = o.c[q];
-            r.f = o.f[q];
-            r.kv = o.kv[q];
-            r.a = o.a[q];
-            r.srel = o.srel[q];
-            r.jlo = o.jlo[q];
-            r.jhi = o.jhi[q];
-            r.ilo = o.ilo[q];
-            r.ihi = o.ihi[q];
-            r.pad0 = r.pad1 = r.pad2 = 0;
-            rec[(size_t)s * L + pos] = r;
+            r.c = cpos[gL + i];
+            r.f = fpos[gL + i];
+            r.kv = sc[(size_t)s * n_sp + species[i]].kv;
+            r.a = av[sL + i];
+            r.srel = o.srel[sL + t];
+            r.jlo = w.x;
+            r.jhi = w.y;
+            r.ilo = w.z;
+            r.ihi = w.w;
+            r.line = i;
+            r.pad0 = r.pad1 = 0;
+            rec[sL + placed[warp][b] + lrank] = r;
         }
         __syncwarp();
-        if (bg < kNumClasses && lrank == 0) wcnt[warp][bg] += __popc(same);
+        if (b < kNumClasses && lrank == 0) placed[warp][b] += __popc(same);
         __syncwarp();
     }
 }
 
-// k_ranges: cum[s][b][ts] = position of the first line of class b whose centre key is
-// >= (ts - 1) * kTile, ts = 0 .. nT + 2 (tiles -1 .. nT, with off-grid centres clamped).
-__global__ void k_ranges(int n_sel, int64_t L, int nT, int tile, const int* __restrict__ bkey,
+// k_ranges: cum[s][b][ts] = position of the first line of class b whose centre key (its grid index,
+// off-grid centres clamped to -1 and N) is >= (ts - 1) * tile, ts = 0 .. nT + 2.
+__global__ void k_ranges(int n_sel, size_t ld, int N, int nT, int tile, const LineRec* __restrict__ rec,
                          const int* __restrict__ classbase, const int* __restrict__ classcnt, int* __restrict__ cum) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int W = nT + 3;
@@ -665,12 +718,12 @@ __global__ void k_ranges(int n_sel, int64_t L, int nT, int tile, const int* __re
     const int b = (int)((t / W) % kNumClasses);
     const int s = (int)(t / ((int64_t)W * kNumClasses));
     const int base = classbase[s * kNumClasses + b], n = classcnt[s * kNumClasses + b];
-    const int* k = bkey + (size_t)s * L + base;
+    const LineRec* k = rec + s * ld + base;
     const long long thr = (long long)(ts - 1) * tile;
     int lo = 0, hi = n;
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
-        if ((long long)k[mid] < thr) lo = mid + 1; else hi = mid;
+        if (min(max(k[mid].c, -1), N) < thr) lo = mid + 1; else hi = mid;
     }
     cum[t] = base + lo;
 }
@@ -683,17 +736,7 @@ struct RowDesc {
     float lnq, q1, q2, q3;      // expm1(-x)/(-x) ~ 1 + d (q1 + d (q2 + d q3)), x = d lnq
     const float* ln_tp;         // ln of the cut threshold t_p (outputs are t_p * sum of s_rel H)
     const int* cum;             // [kNumClasses][nT + 3]
-    const int* bidx;            // [L] bucketed line indices
-    const LineRec* rec;         // [L] their constants, in the same order
-    const int* c;
-    const float* f;
-    const float* srel;
-    const float* a;
-    const float* kv;
-    const int* jlo;
-    const int* jhi;
-    const int* ilo;
-    const int* ihi;
+    const LineRec* rec;         // [L] the bucketed lines
     float* out;                 // [N]
 };
 
@@ -1230,20 +1273,10 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
 // Grid form: one CTA per (row, tile); the rows of one call share the prep arrays.
 struct TileArgs {
     int N, nT;
-    int64_t L;
+    size_t ld;       // lines per row of the record array
     float lnq, q1, q2, q3;
     const int* cum;
-    const int* bidx;
     const LineRec* rec;
-    const int* c;
-    const float* f;
-    const float* srel;
-    const float* a;
-    const float* kv;
-    const int* jlo;
-    const int* jhi;
-    const int* ilo;
-    const int* ihi;
     const float* ln_tp;
     float* out;
     int split;       // CTAs per tile at most (1: direct output)
@@ -1253,7 +1286,7 @@ struct TileArgs {
 };
 
 __device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s, int tile) {
-    const size_t sL = (size_t)s * g.L;
+    const size_t sL = s * g.ld;
     RowDesc r;
     r.N = g.N;
     r.nT = g.nT;
@@ -1264,17 +1297,7 @@ __device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s, int tile) 
     r.q3 = g.q3;
     r.ln_tp = g.ln_tp + s;
     r.cum = g.cum + (size_t)s * kNumClasses * (g.nT + 3);
-    r.bidx = g.bidx + sL;
     r.rec = g.rec + sL;
-    r.c = g.c + sL;
-    r.f = g.f + sL;
-    r.srel = g.srel + sL;
-    r.a = g.a + sL;
-    r.kv = g.kv + sL;
-    r.jlo = g.jlo + sL;
-    r.jhi = g.jhi + sL;
-    r.ilo = g.ilo + sL;
-    r.ihi = g.ihi + sL;
     r.out = g.out + (size_t)s * g.N;
     return r;
 }
@@ -1387,8 +1410,8 @@ __global__ void __launch_bounds__(256) k_tiles64(Tile64Args g) {
             __syncthreads();
             const int pos = base + tid;
             if (pos < end) {
-                const int q = r.bidx[pos];
-                const int jlo = r.jlo[q], jhi = r.jhi[q];
+                const int q = r.rec[pos].line;
+                const int jlo = r.rec[pos].jlo, jhi = r.rec[pos].jhi;
                 if (jhi >= J0 && jlo <= J0 + TILE - 1) {
                     const int sp = g.species[q];
                     const int e = g.sp_el[sp], st = g.sp_stage[sp];
@@ -1456,15 +1479,15 @@ int synth_module_init(int device) {
 // Device buffers of the line preparation of n_sel rows (one grid, one tile size).
 struct PrepBufs {
     int64_t L = 0;
+    size_t ld = 0;   // lines per row of the per-(row, line) arrays: L rounded up to four
     int n_sel = 0, N = 0, nT = 0, nb = 0, tile = kTile;
     double lnq = 0.0;
-    int *c = nullptr, *bidx = nullptr, *bkey = nullptr, *blkcnt = nullptr, *classbase = nullptr, *classcnt = nullptr,
-        *cum = nullptr;
+    int *c = nullptr, *classbase = nullptr, *classcnt = nullptr, *cum = nullptr;
     LineRec* rec = nullptr;
-    float *f = nullptr, *lamcm = nullptr, *lnS = nullptr, *av = nullptr, *lnk0 = nullptr, *ln_tp = nullptr;
+    float *f = nullptr, *dist = nullptr, *lnS = nullptr, *av = nullptr, *lnk0 = nullptr, *ln_tp = nullptr;
+    unsigned char* flag = nullptr;
     RowConst* rc = nullptr;
     SpConst* spc = nullptr;
-    long long* wpart = nullptr;
     MedState* med = nullptr;
     unsigned* ghist = nullptr;
     PrepOut po{};
@@ -1480,26 +1503,27 @@ int prep_alloc(PrepBufs& b, const mpsa_ctx* ctx, int n_sel, int N, double R, int
     b.nT = (N + tile - 1) / tile;
     b.nb = (int)((b.L + kPrepLines - 1) / kPrepLines);
     b.lnq = log1p(1.0 / R);
-    const int64_t L = b.L;
-    const size_t SL = (size_t)n_sel * L;
+    b.ld = ((size_t)b.L + 3) & ~(size_t)3;
+    const size_t L = b.ld, SL = n_sel * L, Sb = (size_t)n_sel * b.nb;
     int r;
-    if ((r = al(&b.c, L)) || (r = al(&b.f, L)) || (r = al(&b.lamcm, L)) || (r = al(&b.rc, n_sel)) ||
+    if ((r = al(&b.c, L)) || (r = al(&b.f, L)) || (r = al(&b.dist, L)) || (r = al(&b.flag, L)) || (r = al(&b.rc, n_sel)) ||
         (r = al(&b.spc, (size_t)n_sel * ctx->n_sp)) || (r = al(&b.lnS, SL)) || (r = al(&b.av, SL)) ||
-        (r = al(&b.lnk0, SL)) || (r = al(&b.ln_tp, n_sel)) || (r = al(&b.po.c, SL)) || (r = al(&b.po.f, SL)) ||
-        (r = al(&b.po.srel, SL)) || (r = al(&b.po.a, SL)) || (r = al(&b.po.kv, SL)) || (r = al(&b.po.jlo, SL)) ||
-        (r = al(&b.po.jhi, SL)) || (r = al(&b.po.ilo, SL)) || (r = al(&b.po.ihi, SL)) || (r = al(&b.po.cls, SL)) ||
-        (r = al(&b.blkcnt, (size_t)n_sel * kNumClasses * b.nb)) || (r = al(&b.wpart, (size_t)n_sel * b.nb)) ||
+        (r = al(&b.lnk0, SL)) || (r = al(&b.ln_tp, n_sel)) || (r = al(&b.po.surv, SL)) || (r = al(&b.po.nsurv, n_sel)) ||
+        (r = al(&b.po.run, Sb)) || (r = al(&b.po.srel, SL)) || (r = al(&b.po.win, SL)) || (r = al(&b.po.cls, SL)) ||
+        (r = al(&b.po.blkcnt, Sb * kNumClasses)) || (r = al(&b.po.wpart, Sb)) ||
         (r = al(&b.classbase, (size_t)n_sel * kNumClasses)) || (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) ||
-        (r = al(&b.bidx, SL)) || (r = al(&b.bkey, SL)) || (r = al(&b.rec, SL)) ||
-        (r = al(&b.cum, (size_t)n_sel * kNumClasses * (b.nT + 3))) || (r = al(&b.med, n_sel)) ||
-        (r = al(&b.ghist, (size_t)n_sel * kMedBins)) || (r = al(&b.po.surv, SL)) || (r = al(&b.po.nsurv, n_sel)))
+        (r = al(&b.rec, SL)) || (r = al(&b.cum, (size_t)n_sel * kNumClasses * (b.nT + 3))) || (r = al(&b.med, n_sel)) ||
+        (r = al(&b.ghist, (size_t)n_sel * kMedBins)))
         return r;
-    b.po.blkcnt = b.blkcnt;
-    b.po.wpart = b.wpart;
     return MPSA_OK;
 }
 
 int ranges_launch(const PrepBufs& b, int tile, int* cum, cudaStream_t st);
+
+GridDesc grid_desc(double lam0_nm, double lnq, int N, int index) {
+    return GridDesc{lam0_nm, lnq, (float)lnq, (float)(1.0 / lam0_nm), (float)(1.0 / (lam0_nm * exp((double)(N - 1) * lnq))),
+                    N, index};
+}
 
 // Line preparation of the rows d_sel of `pop` on the grid (lam0, R, N): placement, line terms,
 // median continuum and cut threshold, cut windows, width-class buckets and tile ranges.
@@ -1510,26 +1534,30 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     const int64_t L = b.L;
     const int n_sel = b.n_sel, n_sp = ctx->n_sp;
     const int lb = (int)((L + 255) / 256);
-    k_place<<<lb, 256, 0, st>>>(L, ctx->d_lam, lam0_nm, b.lnq, b.c, b.f, b.lamcm);
+    RowGrids grids;
+    grids.one = grid_desc(lam0_nm, b.lnq, b.N, 0);
+    grids.many = nullptr;
+    k_distance<<<dim3(lb, 1), 256, 0, st>>>(L, b.ld, 1, ctx->d_lam, grids.one, nullptr, b.dist, b.flag);
     const int pop32 = (opts && opts->precision == MPSA_PREC_FP32_POP32) ? 1 : 0;
     k_consts<<<(n_sel * n_sp + 127) / 128, 128, 0, st>>>(n_sel, d_sel, n_sp, ctx->d_sp_el, ctx->d_sp_stage, ctx->n_el,
                                                            ctx->d_el, pop, ctx->vturb, pop32, b.rc, b.spc);
     k_kappa0<<<dim3(lb, (n_sel + kKappa0Rows - 1) / kKappa0Rows), 256, 0, st>>>(
-        L, n_sel, ctx->d_species, ctx->d_loggf, ctx->d_E, ctx->d_lgR, ctx->d_lgS, ctx->d_lgW, b.lamcm, n_sp, b.rc,
+        L, b.ld, n_sel, ctx->d_species, ctx->d_loggf, ctx->d_E, ctx->d_lgR, ctx->d_lgS, ctx->d_lgW, ctx->d_lam, n_sp, b.rc,
         b.spc, b.lnS, b.av, b.lnk0);
     {
         // median of ln kappa0 per row: three radix levels, each a multi-CTA histogram and a pick
         const int per_row = (int)std::max<int64_t>(1, std::min<int64_t>(128, (L + 8191) / 8192));
         k_med_init<<<(n_sel * kMedBins + 255) / 256, 256, 0, st>>>(n_sel, L, b.med, b.ghist);
         for (int level = 0; level < 3; ++level) {
-            k_med_hist<<<dim3(per_row, n_sel), 1024, 0, st>>>(L, b.lnk0, level, b.med, b.ghist);
+            k_med_hist<<<dim3(per_row, n_sel), 1024, 0, st>>>(L, b.ld, b.lnk0, level, b.med, b.ghist);
             k_med_pick<<<n_sel, 1024, 0, st>>>(level, b.med, b.ghist, (float)log(kcf), (float)log(cut), b.ln_tp,
                                                kc_out);
         }
     }
     MPSA_CUDA_TRY(cudaMemsetAsync(b.po.nsurv, 0, (size_t)n_sel * sizeof(int), st));
-    k_prep<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.N, (float)b.lnq, ctx->d_species, b.c, b.f, n_sp, b.spc,
-                                                       b.lnS, b.av, b.lnk0, b.ln_tp, b.nb, b.po);
+    k_prep<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS, b.av,
+                                                       b.lnk0, b.ln_tp, b.nb, b.po);
+    k_place<<<dim3(b.nb, 1), kPrepThreads, 0, st>>>(L, b.ld, ctx->d_lam, grids.one, nullptr, b.flag, b.c, b.f);
     {
         // the listed lines' count is known on the device only: about eight CTAs per SM in all,
         // each running over its row's list
@@ -1537,20 +1565,21 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
         MPSA_CUDA_TRY(cudaGetDevice(&dev));
         MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const int gx = std::max(1, std::min(b.nb, (8 * sms + n_sel - 1) / n_sel));
-        k_windows<<<dim3(gx, n_sel), kPrepThreads, 0, st>>>(L, b.N, (float)b.lnq, ctx->d_species, b.c, b.f, n_sp, b.spc,
-                                                            b.lnS, b.av, b.ln_tp, b.nb, b.po);
+        k_windows<<<dim3(gx, n_sel), kPrepThreads, 0, st>>>(b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.lnS, b.av,
+                                                            b.ln_tp, b.nb, b.po);
     }
-    k_scan_class<<<dim3(kNumClasses, n_sel), 1024, 0, st>>>(b.nb, b.blkcnt, b.classcnt);
-    k_scan_fin<<<n_sel, 1024, 0, st>>>(b.nb, b.classcnt, b.classbase, b.wpart, (long long*)evals);
-    k_scatter<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.N, b.po.cls, b.c, b.blkcnt, b.classbase, b.nb, b.bidx,
-                                                          b.bkey, b.po, b.rec);
+    k_scan_class<<<dim3(kNumClasses, n_sel), 1024, 0, st>>>(b.nb, b.po.blkcnt, b.classcnt);
+    k_scan_fin<<<n_sel, 1024, 0, st>>>(b.nb, b.classcnt, b.classbase, b.po.wpart, (long long*)evals);
+    constexpr int kWarps = kPrepThreads / 32;
+    k_scatter<<<dim3((b.nb + kWarps - 1) / kWarps, n_sel), kPrepThreads, 0, st>>>(
+        b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec);
     return ranges_launch(b, b.tile, b.cum, st);
 }
 
 int ranges_launch(const PrepBufs& b, int tile, int* cum, cudaStream_t st) {
     const int nT = (b.N + tile - 1) / tile;
     const int64_t nr = (int64_t)b.n_sel * kNumClasses * (nT + 3);
-    k_ranges<<<(unsigned)((nr + 255) / 256), 256, 0, st>>>(b.n_sel, b.L, nT, tile, b.bkey, b.classbase, b.classcnt,
+    k_ranges<<<(unsigned)((nr + 255) / 256), 256, 0, st>>>(b.n_sel, b.ld, b.N, nT, tile, b.rec, b.classbase, b.classcnt,
                                                           cum);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
@@ -1560,23 +1589,13 @@ TileArgs tile_args(const PrepBufs& b, float* kappa) {
     TileArgs ta;
     ta.N = b.N;
     ta.nT = b.nT;
-    ta.L = b.L;
+    ta.ld = b.ld;
     ta.lnq = (float)b.lnq;
     ta.q1 = (float)(-b.lnq / 2.0);
     ta.q2 = (float)(b.lnq * b.lnq / 6.0);
     ta.q3 = (float)(-b.lnq * b.lnq * b.lnq / 24.0);
     ta.cum = b.cum;
-    ta.bidx = b.bidx;
     ta.rec = b.rec;
-    ta.c = b.po.c;
-    ta.f = b.po.f;
-    ta.srel = b.po.srel;
-    ta.a = b.po.a;
-    ta.kv = b.po.kv;
-    ta.jlo = b.po.jlo;
-    ta.jhi = b.po.jhi;
-    ta.ilo = b.po.ilo;
-    ta.ihi = b.po.ihi;
     ta.ln_tp = b.ln_tp;
     ta.out = kappa;
     ta.split = ta.split_free = 1;
@@ -1836,7 +1855,7 @@ std::vector<RowDesc> row_descs(mpsa_batch* b, int tile, const std::vector<int*>&
             ta.nT = nT;
             ta.cum = cums[g];
             RowDesc r;
-            const size_t sL = (size_t)s * G.pb.L;
+            const size_t sL = s * G.pb.ld;
             r.N = G.N;
             r.nT = nT;
             r.tile = tile;
@@ -1846,17 +1865,7 @@ std::vector<RowDesc> row_descs(mpsa_batch* b, int tile, const std::vector<int*>&
             r.q3 = ta.q3;
             r.ln_tp = G.pb.ln_tp + s;
             r.cum = cums[g] + (size_t)s * kNumClasses * (nT + 3);
-            r.bidx = G.pb.bidx + sL;
             r.rec = G.pb.rec + sL;
-            r.c = G.pb.po.c + sL;
-            r.f = G.pb.po.f + sL;
-            r.srel = G.pb.po.srel + sL;
-            r.a = G.pb.po.a + sL;
-            r.kv = G.pb.po.kv + sL;
-            r.jlo = G.pb.po.jlo + sL;
-            r.jhi = G.pb.po.jhi + sL;
-            r.ilo = G.pb.po.ilo + sL;
-            r.ihi = G.pb.po.ihi + sL;
             r.out = G.kappa + (size_t)s * G.N;
             rows.push_back(r);
         }
