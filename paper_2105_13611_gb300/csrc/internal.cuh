@@ -6,7 +6,7 @@
 namespace mpsa {
 
 // Line preparation works on blocks of kPrepLines lines of one row, kPrepThreads threads each
-// (per-block class counts, window-length sums and stable bucket placement) (synth.cu).
+// (per-block class counts and stable bucket placement) (synth.cu).
 constexpr int kPrepThreads = 256;
 constexpr int kPrepLines = 1024;
 

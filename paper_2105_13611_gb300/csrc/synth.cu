@@ -80,18 +80,20 @@ __global__ void k_distance(int64_t L, size_t ld, int n_grids, const double* __re
 // grid keeps.  A CTA gathers the kept ones of its 1024 lines and then takes their logarithms
 // with full warps: FP64 bounds this kernel, and of a 5e6-line list a window of a few nm keeps a
 // few per cent (all 5e6: 484 us, 104 us for the 3 per cent that 80 depths keep of a 7 nm window).
+// LINES: 1024, or 256 for lists too short to give every SM a CTA of 1024.
+template <int LINES>
 __global__ void __launch_bounds__(kPrepThreads) k_place(int64_t L, size_t ld, const double* __restrict__ lam_nm, GridDesc one,
                                                         const GridDesc* __restrict__ many,
                                                         const unsigned char* __restrict__ flag, int* __restrict__ c_out,
                                                         float* __restrict__ f_out) {
-    __shared__ short list[kPrepLines];
+    __shared__ short list[LINES];
     __shared__ int n_list;
     const int g = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
-    const int64_t i0 = (int64_t)blockIdx.x * kPrepLines;
+    const int64_t i0 = (int64_t)blockIdx.x * LINES;
     if (tid == 0) n_list = 0;
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kPrepLines / kPrepThreads; ++k) {
+    for (int k = 0; k < LINES / kPrepThreads; ++k) {
         const int off = k * kPrepThreads + tid;
         const bool on = i0 + off < L && flag[g * ld + i0 + off] != 0;
         const unsigned m = __ballot_sync(0xffffffffu, on);
@@ -415,7 +417,6 @@ struct PrepOut {
     int4* win;            // [n_sel][L] jlo, jhi, ilo, ihi
     unsigned char* cls;   // [n_sel][L] width class, kDropped if the window misses the grid
     int* blkcnt;          // [n_sel][kNumClasses][nb]
-    long long* wpart;     // [n_sel][nb]
 };
 
 // k_prep: one CTA of kPrepThreads threads per block of kPrepLines lines of one row.  Every line
@@ -427,8 +428,7 @@ struct PrepOut {
 // exactly what is left).  The squares are compared, so the test costs one exponential and no
 // logarithm, root or division: 3.4 -> 1.4 ms for 4e8 (row, line) pairs, which it reads at 16 B each.  The lines that
 // remain are appended, as one run per block in line order, to the row's list, and flagged for
-// k_place.  The block's class counts and window-length sum, which k_windows adds to, start at
-// zero here.
+// k_place.  The block's class counts, which k_windows adds to, start at zero here.
 __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, RowGrids grids,
                                                        const int* __restrict__ species,
                                                        const float* __restrict__ dist, unsigned char* __restrict__ flag,
@@ -442,7 +442,6 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, Row
     const int s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t i0 = (int64_t)blockIdx.x * kPrepLines + 4 * tid;
     if (tid < kNumClasses) o.blkcnt[((size_t)s * kNumClasses + tid) * nb + blockIdx.x] = 0;
-    if (tid == 0) o.wpart[(size_t)s * nb + blockIdx.x] = 0;
     const size_t gL = grids.of(s).index * ld;
     const float ltp = ln_tp[s];
     float lk[4], ls[4], la[4], di[4];
@@ -511,29 +510,54 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, Row
 }
 
 // k_windows: the outer and inner cut windows of every listed line (crossing searches on the
-// FP32 H), its width class and window length.  Threads run over the row's list, so warps are
-// dense whatever fraction of the lines the cheap bound kept.  The per-block class counts and
-// window-length sums are integer atomics, combined first across the lanes of a warp that
-// hold lines of the same prep block (a block's lines are one run of the list).
+// FP32 H), its width class.  Threads run over the row's list, so warps are dense whatever
+// fraction of the lines the cheap bound kept.  A CTA first sorts its 256 lines by the tier of H
+// at their expected crossing (far wing, continued fraction, core): a warp whose lanes need
+// different tiers runs all of them at every evaluation.  The per-block class counts are integer
+// atomics, combined first across the lanes of a warp that hold lines of the same prep block.
 __global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids grids, const int* __restrict__ species,
                                                           const int* __restrict__ cpos, const float* __restrict__ fpos,
                                                           int n_sp, const SpConst* __restrict__ sc,
                                                           const float* __restrict__ lnS, const float* __restrict__ av,
                                                           const float* __restrict__ ln_tp, int nb, PrepOut o) {
-    const int s = blockIdx.y, lane = threadIdx.x & 31;
+    constexpr int kWarps = kPrepThreads / 32;
+    __shared__ unsigned char perm[kPrepThreads];
+    __shared__ int cnt[4][kWarps];
+    const int s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = o.nsurv[s];
     const GridDesc gd = grids.of(s);
     const int N = gd.N;
     const float lnq = gd.lnq;
     const size_t gL = gd.index * ld;
     const float ltp = ln_tp[s];
-    const int stride = gridDim.x * kPrepThreads;
-    // every lane of a warp runs the same number of passes (the warp-wide combining below)
-    const int t0 = blockIdx.x * kPrepThreads + (threadIdx.x & ~31);
-    for (int tw = t0; tw < n; tw += stride) {
-        const int t = tw + lane;
-        int blk = -1 - lane, key2 = -1;   // lanes past the list: a segment of their own
-        long long w = 0;
+    for (int base = blockIdx.x * kPrepThreads; base < n; base += gridDim.x * kPrepThreads) {
+        {   // ---- sort by tier
+            int cat = 3;
+            if (base + tid < n) {
+                const size_t q = s * ld + o.surv[s * ld + base + tid];
+                const float rel = fminf(lnS[q] - ltp, 88.f), a = av[q];
+                const float z2 = fmaxf(a * kInvSqrtPi * __expf(rel), rel) + a * a;
+                cat = z2 >= 1600.f ? 0 : (z2 >= 36.f ? 1 : 2);
+            }
+            unsigned mine = 0u;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const unsigned m = __ballot_sync(0xffffffffu, cat == q);
+                if (cat == q) mine = m;
+                if (lane == 0) cnt[q][warp] = __popc(m);
+            }
+            __syncthreads();
+            int off = __popc(mine & ((1u << lane) - 1u));
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w)
+                    if (q < cat || (q == cat && w < warp)) off += cnt[q][w];
+            perm[off] = (unsigned char)tid;
+            __syncthreads();
+        }
+        const int t = base + perm[tid];
+        int blk = 0, key2 = -1;
         if (t < n) {
             const int64_t i = o.surv[s * ld + t];
             const size_t q = s * ld + i;
@@ -569,26 +593,16 @@ __global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids
                 const int hw = max(jhi - key, key - jlo);
                 cl = (unsigned char)(32 - __clz(hw));
                 key2 = blk * kNumClasses + cl;
-                w = (long long)(jhi - jlo + 1);
                 o.srel[s * ld + t] = srel;
                 o.win[s * ld + t] = make_int4(jlo, jhi, ilo, ihi);
             }
             o.cls[s * ld + t] = cl;
         }
-        // window-length sum of each prep block's run of lanes (runs are contiguous): segmented
-        // inclusive scan, the run's last lane adds the total
-        for (int d = 1; d < 32; d <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, w, d);
-            const int yb = __shfl_up_sync(0xffffffffu, blk, d);
-            if (lane >= d && yb == blk) w += y;
-        }
-        const int nextb = __shfl_down_sync(0xffffffffu, blk, 1);
-        if (blk >= 0 && (lane == 31 || nextb != blk) && w > 0)
-            atomicAdd((unsigned long long*)&o.wpart[(size_t)s * nb + blk], (unsigned long long)w);
         // kept lines per (prep block, class)
         const unsigned same = __match_any_sync(0xffffffffu, key2);
         if (key2 >= 0 && lane == __ffs(same) - 1)
             atomicAdd(&o.blkcnt[((size_t)s * kNumClasses + key2 % kNumClasses) * nb + blk], __popc(same));
+        __syncthreads();   // perm and cnt are free for the next lines
     }
 }
 
@@ -631,57 +645,65 @@ __global__ void __launch_bounds__(1024) k_scan_class(int nb, int* __restrict__ b
     if (tid == 0) classcnt[s * kNumClasses + b] = carry;
 }
 
-// k_scan_fin: per row, the class base offsets and the total number of profile evaluations.
-__global__ void __launch_bounds__(1024) k_scan_fin(int nb, const int* __restrict__ classcnt,
-                                                   int* __restrict__ classbase, const long long* __restrict__ wpart,
-                                                   long long* __restrict__ evals) {
-    __shared__ long long wsum[32];
-    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) {
-        int acc = 0;
-        for (int b = 0; b < kNumClasses; ++b) {
-            classbase[s * kNumClasses + b] = acc;
-            acc += classcnt[s * kNumClasses + b];
-        }
+// k_scan_fin: per row, the class base offsets; the number of profile evaluations starts at zero.
+__global__ void k_scan_fin(int n_sel, const int* __restrict__ classcnt, int* __restrict__ classbase,
+                           unsigned long long* __restrict__ evals) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n_sel) return;
+    int acc = 0;
+    for (int b = 0; b < kNumClasses; ++b) {
+        classbase[s * kNumClasses + b] = acc;
+        acc += classcnt[s * kNumClasses + b];
     }
-    if (!evals) return;
-    long long acc = 0;
-    for (int k = tid; k < nb; k += blockDim.x) acc += wpart[(size_t)s * nb + k];
-    for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
-    if (lane == 0) wsum[warp] = acc;
-    __syncthreads();
-    if (tid == 0) {
-        long long t = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
-        evals[s] = t;
-    }
+    if (evals) evals[s] = 0;
 }
 
-// k_scatter: stable placement of the kept lines into class buckets (centre order preserved): a
-// warp per prep block's run of the row's list, 32 lines at a time; the lanes of one class rank
-// themselves, and the warp keeps how many of each class it has placed.  Blocks without kept lines
-// cost one load.
+// k_scatter: stable placement of the kept lines into class buckets (centre order preserved): W
+// warps per prep block's run of the row's list (one, or eight where the call has too few blocks to
+// fill the GPU with one each), each taking a part of the run, 32 lines at a time; the lanes of
+// one class rank themselves, and a warp keeps how many of each class are placed.  Blocks
+// without kept lines cost one load.  The window lengths are added to the row's evaluations.
+template <int W>
 __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids grids, const int* __restrict__ species,
                                                           const int* __restrict__ cpos, const float* __restrict__ fpos,
                                                           int n_sp, const SpConst* __restrict__ sc,
                                                           const float* __restrict__ av, const int* __restrict__ blkoff,
                                                           const int* __restrict__ classbase, int nb, const PrepOut o,
-                                                          LineRec* __restrict__ rec) {
+                                                          LineRec* __restrict__ rec,
+                                                          unsigned long long* __restrict__ evals) {
     constexpr int kWarps = kPrepThreads / 32;
+    static_assert(W == 1 || W == kWarps, "a run is one warp's or one CTA's");
     __shared__ int placed[kWarps][32];
     const int s = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int blk = blockIdx.x * kWarps + warp;
-    if (blk >= nb) return;
-    const int2 run = o.run[(size_t)s * nb + blk];
-    if (run.y == 0) return;
+    const int blk = blockIdx.x * (kWarps / W) + warp / W, part = warp % W;
+    const int2 run = blk < nb ? o.run[(size_t)s * nb + blk] : make_int2(0, 0);
+    if (run.y == 0) return;   // all of the run's warps
     const size_t sL = s * ld, gL = grids.of(s).index * ld;
-    if (lane < kNumClasses)
-        placed[warp][lane] = classbase[s * kNumClasses + lane] + blkoff[((size_t)s * kNumClasses + lane) * nb + blk];
-    __syncwarp();
+    const int len = W == 1 ? run.y : 32 * ((run.y + 32 * W - 1) / (32 * W));   // lines of one warp
+    const int t1 = min(run.x + run.y, run.x + (part + 1) * len), tb = run.x + part * len;
     const unsigned lt = (1u << lane) - 1u;
-    for (int t0 = run.x; t0 < run.x + run.y; t0 += 32) {
+    int first = lane < kNumClasses
+                    ? classbase[s * kNumClasses + lane] + blkoff[((size_t)s * kNumClasses + lane) * nb + blk]
+                    : 0;
+    if (W > 1) {   // the lines of each class in the parts before this one
+        placed[warp][lane] = 0;
+        __syncwarp();
+        for (int t0 = tb; t0 < t1; t0 += 32) {
+            const int b = t0 + lane < t1 ? (int)o.cls[sL + t0 + lane] : (int)kDropped;
+            const unsigned same = __match_any_sync(0xffffffffu, b);
+            if (b < kNumClasses && (same & lt) == 0u) placed[warp][b] += __popc(same);
+            __syncwarp();
+        }
+        __syncthreads();
+        for (int v = 0; v < part; ++v) first += placed[v][lane];
+        __syncthreads();
+    }
+    placed[warp][lane] = first;
+    __syncwarp();
+    unsigned long long len_sum = 0;
+    for (int t0 = tb; t0 < t1; t0 += 32) {
         const int t = t0 + lane;
-        const int b = t < run.x + run.y ? (int)o.cls[sL + t] : (int)kDropped;
+        const int b = t < t1 ? (int)o.cls[sL + t] : (int)kDropped;
         const unsigned same = __match_any_sync(0xffffffffu, b);
         const int lrank = __popc(same & lt);
         if (b < kNumClasses) {
@@ -699,11 +721,17 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
             r.ihi = w.w;
             r.line = i;
             r.pad0 = r.pad1 = 0;
+            len_sum += (unsigned long long)(w.y - w.x + 1);
             rec[sL + placed[warp][b] + lrank] = r;
         }
         __syncwarp();
         if (b < kNumClasses && lrank == 0) placed[warp][b] += __popc(same);
         __syncwarp();
+    }
+    if (evals) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) len_sum += __shfl_down_sync(0xffffffffu, len_sum, d);
+        if (lane == 0 && len_sum) atomicAdd(evals + s, len_sum);
     }
 }
 
@@ -1510,7 +1538,7 @@ int prep_alloc(PrepBufs& b, const mpsa_ctx* ctx, int n_sel, int N, double R, int
         (r = al(&b.spc, (size_t)n_sel * ctx->n_sp)) || (r = al(&b.lnS, SL)) || (r = al(&b.av, SL)) ||
         (r = al(&b.lnk0, SL)) || (r = al(&b.ln_tp, n_sel)) || (r = al(&b.po.surv, SL)) || (r = al(&b.po.nsurv, n_sel)) ||
         (r = al(&b.po.run, Sb)) || (r = al(&b.po.srel, SL)) || (r = al(&b.po.win, SL)) || (r = al(&b.po.cls, SL)) ||
-        (r = al(&b.po.blkcnt, Sb * kNumClasses)) || (r = al(&b.po.wpart, Sb)) ||
+        (r = al(&b.po.blkcnt, Sb * kNumClasses)) ||
         (r = al(&b.classbase, (size_t)n_sel * kNumClasses)) || (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) ||
         (r = al(&b.rec, SL)) || (r = al(&b.cum, (size_t)n_sel * kNumClasses * (b.nT + 3))) || (r = al(&b.med, n_sel)) ||
         (r = al(&b.ghist, (size_t)n_sel * kMedBins)))
@@ -1557,22 +1585,32 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     MPSA_CUDA_TRY(cudaMemsetAsync(b.po.nsurv, 0, (size_t)n_sel * sizeof(int), st));
     k_prep<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS, b.av,
                                                        b.lnk0, b.ln_tp, b.nb, b.po);
-    k_place<<<dim3(b.nb, 1), kPrepThreads, 0, st>>>(L, b.ld, ctx->d_lam, grids.one, nullptr, b.flag, b.c, b.f);
+    int dev = 0, sms = 0;
+    MPSA_CUDA_TRY(cudaGetDevice(&dev));
+    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (b.nb >= 2 * sms)
+        k_place<kPrepLines><<<dim3(b.nb, 1), kPrepThreads, 0, st>>>(L, b.ld, ctx->d_lam, grids.one, nullptr, b.flag, b.c, b.f);
+    else
+        k_place<kPrepThreads><<<dim3((unsigned)((L + kPrepThreads - 1) / kPrepThreads), 1), kPrepThreads, 0, st>>>(
+            L, b.ld, ctx->d_lam, grids.one, nullptr, b.flag, b.c, b.f);
     {
         // the listed lines' count is known on the device only: about eight CTAs per SM in all,
         // each running over its row's list
-        int dev = 0, sms = 0;
-        MPSA_CUDA_TRY(cudaGetDevice(&dev));
-        MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const int gx = std::max(1, std::min(b.nb, (8 * sms + n_sel - 1) / n_sel));
         k_windows<<<dim3(gx, n_sel), kPrepThreads, 0, st>>>(b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.lnS, b.av,
                                                             b.ln_tp, b.nb, b.po);
     }
     k_scan_class<<<dim3(kNumClasses, n_sel), 1024, 0, st>>>(b.nb, b.po.blkcnt, b.classcnt);
-    k_scan_fin<<<n_sel, 1024, 0, st>>>(b.nb, b.classcnt, b.classbase, b.po.wpart, (long long*)evals);
+    k_scan_fin<<<(n_sel + 31) / 32, 32, 0, st>>>(n_sel, b.classcnt, b.classbase, (unsigned long long*)evals);
     constexpr int kWarps = kPrepThreads / 32;
-    k_scatter<<<dim3((b.nb + kWarps - 1) / kWarps, n_sel), kPrepThreads, 0, st>>>(
-        b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec);
+    if ((int64_t)b.nb * n_sel * kWarps <= 64ll * sms)
+        k_scatter<kWarps><<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(
+            b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
+            (unsigned long long*)evals);
+    else
+        k_scatter<1><<<dim3((b.nb + kWarps - 1) / kWarps, n_sel), kPrepThreads, 0, st>>>(
+            b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
+            (unsigned long long*)evals);
     return ranges_launch(b, b.tile, b.cum, st);
 }
 
