@@ -10,7 +10,7 @@
 //   k_distance     per line: how far off the grid its centre is
 //   k_consts       per (row, species): ln(sqrt(pi) e^2/(m_e c) N/U / rho), u, c/u from the FP64 table
 //   k_kappa0       per (row, line): ln S, a, ln kappa0 in FP32 log space
-//   k_med_*        per row: lower median of ln kappa0 by multi-CTA radix selection -> ln t_p, kappa_c
+//   k_med_*        per row: lower median of ln kappa0 -> ln t_p, kappa_c
 //   k_prep         per (row, line): peak against the cut, reach of the wing; the lines left, listed
 //   k_place        the listed lines' centre index c and fraction f on the grid (FP64 log)
 //   k_windows      per listed line: cut windows (outer: no point beyond can pass the cut; inner:
@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(kPrepThreads) k_place(int64_t L, size_t ld, co
 struct RowConst {
     float ne, nHI, inv_kT_eV, hc_kT_cm;
 };
-struct SpConst {
-    float lnC, u, kv;
+struct __align__(16) SpConst {
+    float lnC, u, kv, lnu;   // lnu = logf(u)
 };
 
 __global__ void k_consts(int n_sel, const int* __restrict__ sel, int n_sp, const int* __restrict__ sp_el,
@@ -143,6 +143,7 @@ __global__ void k_consts(int n_sel, const int* __restrict__ sel, int n_sp, const
         o.lnC = NU > 0 ? (float)(log(pre) + log(NU) - log(row[kPopRho])) : -INFINITY;
     o.u = (float)u;
     o.kv = (float)(kC / u);
+    o.lnu = logf(o.u);
     sc[t] = o;
     if (sp == 0) {
         RowConst r;
@@ -161,40 +162,38 @@ __global__ void k_consts(int n_sel, const int* __restrict__ sel, int n_sp, const
 //   ln kappa0 = ln S + ln H(0, a).
 // One thread per line and up to kKappa0Rows rows: the line's data and its three damping
 // constants are read and formed once, then each row's values follow.
-constexpr int kKappa0Rows = 8;
+//
+// H(0, a) is bound by its arithmetic: at v = 0 the two poles of a pair of voigt_core give the same
+// term, so voigt_core0 forms it once (60 operations instead of 130), with every rounding that the general
+// form takes there (median, cut and windows follow from these bits).  4e8 (row, line) pairs: 3.60 ms
+// before, 2.58 ms now; their 12 bytes each would take 0.7 ms.
+constexpr int kKappa0Rows = 16;
 
-__global__ void k_kappa0(int64_t L, size_t ld, int n_sel, const int* __restrict__ species, const float* __restrict__ loggf,
-                         const float* __restrict__ E, const float* __restrict__ lgR, const float* __restrict__ lgS,
-                         const float* __restrict__ lgW, const double* __restrict__ lam_nm, int n_sp,
-                         const RowConst* __restrict__ rc, const SpConst* __restrict__ sc,
-                         float* __restrict__ lnS_out, float* __restrict__ a_out, float* __restrict__ lnk0_out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L) return;
-    const int sp = species[i];
-    const float lam = (float)(lam_nm[i] * 1e-7), lglam = logf(lam), lg = loggf[i], Ei = E[i];
-    const float gR = exp10f(lgR[i]), gS = exp10f(lgS[i]), gW = exp10f(lgW[i]);
-    const int s1 = min(n_sel, (int)(blockIdx.y + 1) * kKappa0Rows);
-    for (int s = blockIdx.y * kKappa0Rows; s < s1; ++s) {
-        const RowConst r = rc[s];
-        const SpConst q = sc[(size_t)s * n_sp + sp];
-        const float gamma = gR + gS * r.ne + gW * r.nHI;
-        const float a = gamma * lam / (kFourPi * q.u);
-        const float lnDnu = logf(q.u) - lglam;
-        const float stim = -expm1f(-r.hc_kT_cm / lam);
-        const float lnS = q.lnC + lg * kLn10 - Ei * r.inv_kT_eV + logf(stim) - lnDnu;
-        const size_t o = s * ld + i;
-        lnS_out[o] = lnS;
-        a_out[o] = a;
-        lnk0_out[o] = lnS + logf(voigt_H(0.f, a));
+__device__ __forceinline__ float voigt_core0(float a) {
+    const float d = kGHDelta, Y1 = __fadd_rn(a, d);
+    float sum = 0.f;
+    if (a < 2.f) {
+        const float Yd = __fadd_rn(Y1, d);
+#pragma unroll
+        for (int k = 0; k < kGHPairs; ++k) {
+            const float sk = c_voigt.s[k], s2 = __fmul_rn(sk, sk);
+            const float p = __fmul_rn(__fadd_rn(s2, d * d), __fmaf_rn(Y1, Y1, s2));
+            const float t = __fmaf_rn(c_voigt.U[k], __fmaf_rn(-Y1, d, s2), __fmul_rn(__fmul_rn(c_voigt.S[k], -sk), Yd));
+            sum = __fmaf_rn(__fmaf_rn(t, p, __fmul_rn(t, p)), rcp_approx(__fmul_rn(p, p)), sum);
+        }
+        return __fmaf_rn(a, sum, 1.f);
     }
+    const float Y12 = __fmul_rn(Y1, Y1);
+#pragma unroll
+    for (int k = 0; k < kGHPairs; ++k) {
+        const float sk = c_voigt.s[k];
+        const float q = __fmaf_rn(sk, sk, Y12), g = __fmaf_rn(c_voigt.S[k], sk, __fmul_rn(c_voigt.U[k], Y1));
+        sum = __fmaf_rn(__fmaf_rn(q, g, __fmul_rn(q, g)), rcp_approx(__fmul_rn(q, q)), sum);
+    }
+    return sum;
 }
 
-// ---------------------------------------------------------------------------
-// Lower median (rank (L-1)/2) of ln kappa0 per row: MSB radix selection on order-preserving
-// keys of the FP32 bit patterns in three levels of 11, 11 and 10 bits.  At every level a grid
-// of CTAs per row histograms its share of the row (the values whose key matches the prefix
-// resolved so far) in shared memory and adds the non-empty bins to the row's global
-// histogram; one CTA per row then finds the bin holding the rank (k_med_pick).
+// order-preserving keys of the FP32 bit patterns
 __device__ __forceinline__ unsigned fkey(float x) {
     unsigned b = __float_as_uint(x);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
@@ -203,86 +202,194 @@ __device__ __forceinline__ float unkey(unsigned k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
+// Where the median of a row is looked for (see the median below).
 struct MedState {
-    unsigned prefix;   // key bits resolved so far
-    unsigned rank;     // rank of the median among the keys with that prefix
+    unsigned lo, hi;   // keys that bracket it
+    unsigned below;    // lines below lo
+    unsigned n;        // lines in the bracket, listed
 };
-constexpr int kMedBins = 2048;
-__host__ __device__ constexpr int med_shift(int level) { return level == 0 ? 21 : (level == 1 ? 10 : 0); }
-__host__ __device__ constexpr int med_bits(int level) { return level == 2 ? 10 : 11; }
 
-__global__ void k_med_init(int n_sel, int64_t L, MedState* __restrict__ st, unsigned* __restrict__ ghist) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_sel * kMedBins) ghist[i] = 0u;
-    if (i < n_sel) st[i] = MedState{0u, (unsigned)((L - 1) / 2)};
+// SAMPLE: every kMedStride-th line only, ln kappa0 alone, into lnk0_out [n_sel][ld].
+constexpr int kMedStride = 128;
+template <bool SAMPLE>
+__global__ void k_kappa0(int64_t L, size_t ld, int n_sel, const int* __restrict__ species, const float* __restrict__ loggf,
+                         const float* __restrict__ E, const float* __restrict__ lgR, const float* __restrict__ lgS,
+                         const float* __restrict__ lgW, const double* __restrict__ lam_nm, int n_sp,
+                         const RowConst* __restrict__ rc, const SpConst* __restrict__ sc,
+                         float* __restrict__ lnS_out, float* __restrict__ a_out, float* __restrict__ lnk0_out) {
+    const int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = SAMPLE ? at * kMedStride : at;
+    if (i >= L) return;
+    const int sp = species[i];
+    const float lam = (float)(lam_nm[i] * 1e-7), lglam = logf(lam), lg = loggf[i], Ei = E[i];
+    const float gR = exp10f(lgR[i]), gS = exp10f(lgS[i]), gW = exp10f(lgW[i]);
+    const int s1 = min(n_sel, (int)(blockIdx.y + 1) * kKappa0Rows);
+#pragma unroll 1
+    for (int s = blockIdx.y * kKappa0Rows; s < s1; ++s) {
+        const RowConst r = rc[s];
+        const SpConst q = sc[(size_t)s * n_sp + sp];
+        const float gamma = gR + gS * r.ne + gW * r.nHI;
+        const float a = gamma * lam / (kFourPi * q.u);
+        const float lnDnu = q.lnu - lglam;
+        const float stim = -expm1f(-r.hc_kT_cm / lam);
+        const float lnS = q.lnC + lg * kLn10 - Ei * r.inv_kT_eV + logf(stim) - lnDnu;
+        const size_t o = s * ld + at;
+        if (!SAMPLE) {
+            lnS_out[o] = lnS;
+            a_out[o] = a;
+        }
+        lnk0_out[o] = lnS + logf(a * a >= 36.f ? voigt_H(0.f, a) : voigt_core0(a));
+    }
 }
 
-__global__ void __launch_bounds__(1024) k_med_hist(int64_t L, size_t ld, const float* __restrict__ lnk0, int level,
-                                                   const MedState* __restrict__ st, unsigned* __restrict__ ghist) {
-    __shared__ unsigned h[kMedBins];
-    const int s = blockIdx.y;
-    const int shift = med_shift(level), nbits = med_bits(level);
-    const unsigned pmask = level == 0 ? 0u : (0xffffffffu << (shift + nbits));
-    const unsigned prefix = st[s].prefix;
-    for (int i = threadIdx.x; i < kMedBins; i += blockDim.x) h[i] = 0u;
-    __syncthreads();
-    const float* x = lnk0 + s * ld;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L; i += stride) {
-        const unsigned k = fkey(__ldg(x + i));
-        if ((k & pmask) == prefix) atomicAdd(&h[(k >> shift) & ((1u << nbits) - 1u)], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < (1 << nbits); i += blockDim.x)
-        if (h[i]) atomicAdd(&ghist[(size_t)s * kMedBins + i], h[i]);
-}
+// ---------------------------------------------------------------------------
+// Lower median (rank (L-1)/2) of ln kappa0 per row, exact, on the order-preserving keys.
+//
+// Lists of up to kMedSmall lines: one CTA per row selects it in three radix levels of 11, 11 and 10
+// bits (k_med_select).  Longer ones are read once instead of three times: every 128th line is formed
+// ahead, two order statistics of that sample bracket the median (k_med_bracket: five standard
+// deviations of its rank on either side), one pass over the row counts the lines below the bracket
+// and lists the 3 per cent inside (k_med_collect), and the median is selected among those
+// (k_med_select again; from the whole row should the bracket have missed it).  5e6 lines x 80
+// rows: 1.10 ms for three passes, 0.62 ms now.  (Counting and listing in k_kappa0 itself took one
+// global atomic per warp and row: 2.6 -> 11.5 ms.)
+constexpr int kMedBins = 2048, kMedThreads = 1024;
+constexpr int64_t kMedSmall = 65536;
 
-__global__ void __launch_bounds__(1024) k_med_pick(int level, MedState* __restrict__ st,
-                                                   unsigned* __restrict__ ghist, float ln_kc_factor, float ln_cut,
-                                                   float* __restrict__ ln_tp, float* __restrict__ kc_out) {
-    __shared__ int wsum[32];
-    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned* h = ghist + (size_t)s * kMedBins;
-    const int nb = 1 << med_bits(level);
-    // two bins per thread; block-wide inclusive scan of their counts
-    const unsigned c0 = 2 * tid < nb ? h[2 * tid] : 0u, c1 = 2 * tid + 1 < nb ? h[2 * tid + 1] : 0u;
-    const int v = (int)(c0 + c1);
-    int incl = v;
-    for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += y;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int t = lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0;
-        int ti = t;
+// The key of rank `rank` among the keys key(x[0..n)), x 16-byte aligned: all threads of the CTA
+// call it.
+template <class F>
+__device__ __forceinline__ unsigned block_select(const float* __restrict__ x, int64_t n, unsigned rank, unsigned* h,
+                                                 F&& key) {
+    __shared__ unsigned wsum[32];
+    __shared__ unsigned s_bin, s_rank;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned prefix = 0u;
+    for (int level = 0; level < 3; ++level) {
+        const int shift = level == 0 ? 21 : (level == 1 ? 10 : 0), nb = level == 2 ? 1024 : 2048;
+        const unsigned pmask = level == 0 ? 0u : (0xffffffffu << (level == 1 ? 21 : 10));
+        for (int i = tid; i < kMedBins; i += kMedThreads) h[i] = 0u;
+        __syncthreads();
+        auto add = [&](float v) {
+            const unsigned k = key(v);
+            if ((k & pmask) == prefix) atomicAdd(&h[(k >> shift) & (nb - 1)], 1u);
+        };
+        const int64_t n4 = n >> 2;
+#pragma unroll 4
+        for (int64_t i = tid; i < n4; i += kMedThreads) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(x) + i);
+            add(q.x), add(q.y), add(q.z), add(q.w);
+        }
+        if (tid < (int)(n & 3)) add(__ldg(x + 4 * n4 + tid));
+        __syncthreads();
+        // two bins per thread; block-wide inclusive scan of their counts
+        const unsigned c0 = h[2 * tid], c1 = h[2 * tid + 1], v = c0 + c1;
+        unsigned incl = v;
+#pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, ti, d);
-            if (lane >= d) ti += y;
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += y;
         }
-        wsum[lane] = ti - t;
-    }
-    __syncthreads();
-    const unsigned before = (unsigned)(wsum[warp] + incl - v);
-    const MedState cur = st[s];
-    if (cur.rank >= before && cur.rank < before + (unsigned)v) {
-        const bool lo = cur.rank < before + c0;
-        const unsigned bin = 2u * tid + (lo ? 0u : 1u);
-        MedState nx;
-        nx.rank = cur.rank - (lo ? before : before + c0);
-        nx.prefix = cur.prefix | (bin << med_shift(level));
-        st[s] = nx;
-        if (level == 2) {
-            const float med = unkey(nx.prefix);
-            ln_tp[s] = med + ln_kc_factor + ln_cut;
-            if (kc_out) kc_out[s] = expf(med + ln_kc_factor);
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        unsigned before = incl - v;
+        for (int w = 0; w < warp; ++w) before += wsum[w];
+        if (rank >= before && rank < before + v) {   // one thread
+            const bool low = rank < before + c0;
+            s_bin = 2u * tid + (low ? 0u : 1u);
+            s_rank = rank - (low ? before : before + c0);
         }
+        __syncthreads();
+        prefix |= s_bin << shift;
+        rank = s_rank;
+        __syncthreads();
     }
+    return prefix;
+}
+
+// sample [n_sel][ld] of n values: keys around the middle, wide enough for the median of the whole
+__global__ void __launch_bounds__(kMedThreads) k_med_bracket(int64_t n, size_t ld, const float* __restrict__ sample,
+                                                             MedState* __restrict__ st) {
+    __shared__ unsigned h[kMedBins];
+    const int s = blockIdx.x;
+    const float* x = sample + s * ld;
+    const int64_t mid = (n - 1) / 2, w = (int64_t)(2.5 * sqrt((double)n)) + 2;
+    const unsigned lo = block_select(x, n, (unsigned)(mid - w < 0 ? 0 : mid - w), h, [](float v) { return fkey(v); });
+    const unsigned hi = block_select(x, n, (unsigned)(mid + w >= n ? n - 1 : mid + w), h, [](float v) { return fkey(v); });
+    if (threadIdx.x == 0) st[s] = MedState{lo, hi, 0u, 0u};
+}
+
+// Count the row's lines below its bracket, list those inside (list [n_sel][list_ld], any order).
+constexpr int kMedStage = 8192;
+__global__ void __launch_bounds__(kMedThreads) k_med_collect(int64_t L, size_t ld, const float* __restrict__ lnk0,
+                                                             MedState* __restrict__ st, float* __restrict__ list,
+                                                             size_t list_ld) {
+    __shared__ float stage[kMedStage];
+    __shared__ unsigned s_n, s_base, s_below;
+    const int s = blockIdx.y, tid = threadIdx.x;
+    const unsigned lo = st[s].lo, hi = st[s].hi;
+    const float* x = lnk0 + s * ld;   // 16-byte aligned rows
+    if (tid == 0) s_n = s_below = 0u;
     __syncthreads();
-    // clear the histogram for the next level
-    if (2 * tid < kMedBins) h[2 * tid] = 0u;
-    if (2 * tid + 1 < kMedBins) h[2 * tid + 1] = 0u;
+    unsigned below = 0u;
+    auto flush = [&] {
+        __syncthreads();
+        const unsigned n = s_n;
+        if (tid == 0 && n) s_base = atomicAdd(&st[s].n, n);
+        __syncthreads();
+        for (unsigned i = tid; i < n; i += kMedThreads) list[s * list_ld + s_base + i] = stage[i];
+        __syncthreads();
+        if (tid == 0) s_n = 0u;
+        __syncthreads();
+    };
+    const int64_t step = (int64_t)gridDim.x * 4 * kMedThreads;
+    for (int64_t i0 = (int64_t)blockIdx.x * 4 * kMedThreads; i0 < L; i0 += step) {
+        const int64_t i = i0 + 4 * tid;
+        if (i < L) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(x + i));
+            const float v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const unsigned k = fkey(v[c]);
+                if (i + c < L) {
+                    below += k < lo;
+                    if (k >= lo && k <= hi) stage[atomicAdd(&s_n, 1u)] = v[c];
+                }
+            }
+        }
+        __syncthreads();
+        if (s_n > kMedStage - 4 * kMedThreads) flush();
+    }
+    below = __reduce_add_sync(0xffffffffu, below);
+    if ((tid & 31) == 0 && below) atomicAdd(&s_below, below);
+    flush();
+    if (tid == 0 && s_below) atomicAdd(&st[s].below, s_below);
+}
+
+// st: null, or the bracket whose lines are listed
+__global__ void __launch_bounds__(kMedThreads) k_med_select(int64_t L, size_t ld, const float* __restrict__ lnk0,
+                                                            const MedState* __restrict__ st,
+                                                            const float* __restrict__ list, size_t list_ld,
+                                                            float ln_kc_factor, float ln_cut, float* __restrict__ ln_tp,
+                                                            float* __restrict__ kc_out) {
+    __shared__ unsigned h[kMedBins];
+    const int s = blockIdx.x;
+    const float* x = lnk0 + s * ld;
+    int64_t n = L;
+    unsigned rank = (unsigned)((L - 1) / 2), lo = 0u;
+    int sh = 0;
+    if (st && rank >= st[s].below && rank - st[s].below < st[s].n) {
+        x = list + s * list_ld;
+        n = st[s].n;
+        rank -= st[s].below;
+        // listed keys differ in their low bits only: spread them over the bins
+        lo = st[s].lo;
+        sh = __clz((int)((st[s].hi - lo) | 1u));
+    }
+    const float med = unkey(lo + (block_select(x, n, rank, h, [&](float v) { return (fkey(v) - lo) << sh; }) >> sh));
+    if (threadIdx.x == 0) {
+        ln_tp[s] = med + ln_kc_factor + ln_cut;
+        if (kc_out) kc_out[s] = expf(med + ln_kc_factor);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1517,7 +1624,6 @@ struct PrepBufs {
     RowConst* rc = nullptr;
     SpConst* spc = nullptr;
     MedState* med = nullptr;
-    unsigned* ghist = nullptr;
     PrepOut po{};
 };
 
@@ -1540,8 +1646,7 @@ int prep_alloc(PrepBufs& b, const mpsa_ctx* ctx, int n_sel, int N, double R, int
         (r = al(&b.po.run, Sb)) || (r = al(&b.po.srel, SL)) || (r = al(&b.po.win, SL)) || (r = al(&b.po.cls, SL)) ||
         (r = al(&b.po.blkcnt, Sb * kNumClasses)) ||
         (r = al(&b.classbase, (size_t)n_sel * kNumClasses)) || (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) ||
-        (r = al(&b.rec, SL)) || (r = al(&b.cum, (size_t)n_sel * kNumClasses * (b.nT + 3))) || (r = al(&b.med, n_sel)) ||
-        (r = al(&b.ghist, (size_t)n_sel * kMedBins)))
+        (r = al(&b.rec, SL)) || (r = al(&b.cum, (size_t)n_sel * kNumClasses * (b.nT + 3))) || (r = al(&b.med, n_sel)))
         return r;
     return MPSA_OK;
 }
@@ -1569,18 +1674,31 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     const int pop32 = (opts && opts->precision == MPSA_PREC_FP32_POP32) ? 1 : 0;
     k_consts<<<(n_sel * n_sp + 127) / 128, 128, 0, st>>>(n_sel, d_sel, n_sp, ctx->d_sp_el, ctx->d_sp_stage, ctx->n_el,
                                                            ctx->d_el, pop, ctx->vturb, pop32, b.rc, b.spc);
-    k_kappa0<<<dim3(lb, (n_sel + kKappa0Rows - 1) / kKappa0Rows), 256, 0, st>>>(
-        L, b.ld, n_sel, ctx->d_species, ctx->d_loggf, ctx->d_E, ctx->d_lgR, ctx->d_lgS, ctx->d_lgW, ctx->d_lam, n_sp, b.rc,
-        b.spc, b.lnS, b.av, b.lnk0);
     {
-        // median of ln kappa0 per row: three radix levels, each a multi-CTA histogram and a pick
-        const int per_row = (int)std::max<int64_t>(1, std::min<int64_t>(128, (L + 8191) / 8192));
-        k_med_init<<<(n_sel * kMedBins + 255) / 256, 256, 0, st>>>(n_sel, L, b.med, b.ghist);
-        for (int level = 0; level < 3; ++level) {
-            k_med_hist<<<dim3(per_row, n_sel), 1024, 0, st>>>(L, b.ld, b.lnk0, level, b.med, b.ghist);
-            k_med_pick<<<n_sel, 1024, 0, st>>>(level, b.med, b.ghist, (float)log(kcf), (float)log(cut), b.ln_tp,
-                                               kc_out);
+        // ln S, a, ln kappa0 and the median; the record array, not in use yet, holds the listed lines
+        // and the sample
+        const int rows = (n_sel + kKappa0Rows - 1) / kKappa0Rows;
+        const int64_t ns = (L + kMedStride - 1) / kMedStride;
+        const size_t ns_ld = ((size_t)ns + 3) & ~(size_t)3;
+        float* const list = reinterpret_cast<float*>(b.rec);
+        float* const sample = list + (size_t)n_sel * b.ld;
+        const bool small = L <= kMedSmall;
+        auto kappa0 = [&](auto kernel, int64_t lines, size_t ld, float* k0) {
+            kernel<<<dim3((unsigned)((lines + 255) / 256), rows), 256, 0, st>>>(
+                L, ld, n_sel, ctx->d_species, ctx->d_loggf, ctx->d_E, ctx->d_lgR, ctx->d_lgS, ctx->d_lgW, ctx->d_lam, n_sp,
+                b.rc, b.spc, b.lnS, b.av, k0);
+        };
+        if (!small) {
+            kappa0(k_kappa0<true>, ns, ns_ld, sample);
+            k_med_bracket<<<n_sel, kMedThreads, 0, st>>>(ns, ns_ld, sample, b.med);
         }
+        kappa0(k_kappa0<false>, L, b.ld, b.lnk0);
+        if (!small) {
+            const int per_row = (int)std::max<int64_t>(1, std::min<int64_t>(128, L / (8 * 4 * kMedThreads)));
+            k_med_collect<<<dim3(per_row, n_sel), kMedThreads, 0, st>>>(L, b.ld, b.lnk0, b.med, list, b.ld);
+        }
+        k_med_select<<<n_sel, kMedThreads, 0, st>>>(L, b.ld, b.lnk0, small ? nullptr : b.med, list, b.ld,
+                                                    (float)log(kcf), (float)log(cut), b.ln_tp, kc_out);
     }
     MPSA_CUDA_TRY(cudaMemsetAsync(b.po.nsurv, 0, (size_t)n_sel * sizeof(int), st));
     k_prep<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS, b.av,

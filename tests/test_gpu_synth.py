@@ -328,3 +328,42 @@ def test_interpolated_wings_on_grids_of_every_shape(N, R):
         bad, err, bound = opacity_violations(kg[s], k, pl.kappa_c, slack)
         assert len(bad) == 0, (s, bad[:5], rel_report(kg[s], k, pl.kappa_c))
         assert W <= evg[s] <= W + 8 * len(L) + 16
+
+
+@pytest.mark.parametrize("n_lines,kind", [(1, "random"), (2, "random"), (6, "equal"), (65536, "random"), (65537, "random"),
+                                          (70003, "equal"), (262147, "random"), (262146, "two values"),
+                                          (131101, "sample off"), (131101, "no atoms")])
+def test_median_continuum_of_lists_of_every_length(n_lines, kind):
+    # the lower median of ln kappa0 behind kappa_c: one CTA up to 65,536 lines, a bracket from every
+    # 128th line beyond; ties, a sample that misses the median (every 128th line far stronger than
+    # the rest: the whole row is searched), and species without atoms (ln kappa0 = -inf for half of
+    # the lines or more).  kappa_c is FP32 line terms of one line: 1e-5
+    import torch
+    from paper_2105_13611_gb300 import binding
+    w = wl.config_tiny(n_lines=40, lam=(300.0, 300.1), seed=81)
+    se, ss = wl.species_table(w.n_metals)
+    L = wl.linelist(n_lines, len(se), 200.0, 500.0, 82)
+    ab = None
+    if kind in ("equal", "two values"):
+        L.lam_nm[:], L.log_gf[:], L.E_eV[:], L.species[:] = 300.05, -1.0, 2.0, 3
+        L.log_gR[:] = L.log_gS[:] = L.log_gW[:] = -8.0
+        if kind == "two values":
+            L.log_gf[n_lines // 2:] = 0.5
+    elif kind == "sample off":
+        L.log_gf[::128] = 9.0
+    elif kind == "no atoms":
+        ab = np.ones((1, wl.elements(w.n_metals).n))
+        ab[0, 2:5] = 0.0            # three of the five metals
+    ctx, _ = gpu_context(w, lines=L, abund=ab)
+    kap = torch.empty((4, binding.grid_size(w.grid.lam0_nm, w.grid.lam1_nm, w.grid.R)), device="cuda")
+    kc = torch.empty(4, device="cuda")
+    ctx.synth_opacity(w.grid, np.arange(4), kap, kc)
+    torch.cuda.synchronize()
+    for s in range(4):
+        with np.errstate(divide="ignore"):
+            pl = sy.prepare(L, se, ss, wl.elements(w.n_metals), w.T[s], w.P[s], w.grid, w.cut, w.kc_factor,
+                            abund_scale=None if ab is None else ab[0])
+        if pl.kappa_c == 0.0:
+            assert float(kc[s]) == 0.0
+        else:
+            assert abs(float(kc[s]) / pl.kappa_c - 1) < 1e-5, s
