@@ -53,6 +53,18 @@ struct RowGrids {
     const GridDesc* many;
     __device__ __forceinline__ GridDesc of(int s) const { return many ? many[s] : one; }
 };
+// Where the rows' continuum and evaluation counts go (either may be null): one array for all
+// rows, or a pointer per row.
+struct RowOut {
+    float* kc;
+    unsigned long long* ev;
+    float* const* kc_many;
+    unsigned long long* const* ev_many;
+    __device__ __forceinline__ float* kc_of(int s) const { return kc_many ? kc_many[s] : (kc ? kc + s : nullptr); }
+    __device__ __forceinline__ unsigned long long* ev_of(int s) const {
+        return ev_many ? ev_many[s] : (ev ? ev + s : nullptr);
+    }
+};
 
 // ---------------------------------------------------------------------------
 // k_distance: per (grid, line), a lower bound of the distance between a centre off the grid and
@@ -370,7 +382,7 @@ __global__ void __launch_bounds__(kMedThreads) k_med_select(int64_t L, size_t ld
                                                             const MedState* __restrict__ st,
                                                             const float* __restrict__ list, size_t list_ld,
                                                             float ln_kc_factor, float ln_cut, float* __restrict__ ln_tp,
-                                                            float* __restrict__ kc_out) {
+                                                            RowOut out) {
     __shared__ unsigned h[kMedBins];
     const int s = blockIdx.x;
     const float* x = lnk0 + s * ld;
@@ -388,7 +400,8 @@ __global__ void __launch_bounds__(kMedThreads) k_med_select(int64_t L, size_t ld
     const float med = unkey(lo + (block_select(x, n, rank, h, [&](float v) { return (fkey(v) - lo) << sh; }) >> sh));
     if (threadIdx.x == 0) {
         ln_tp[s] = med + ln_kc_factor + ln_cut;
-        if (kc_out) kc_out[s] = expf(med + ln_kc_factor);
+        float* const kc = out.kc_of(s);
+        if (kc) *kc = expf(med + ln_kc_factor);
     }
 }
 
@@ -754,7 +767,7 @@ __global__ void __launch_bounds__(1024) k_scan_class(int nb, int* __restrict__ b
 
 // k_scan_fin: per row, the class base offsets; the number of profile evaluations starts at zero.
 __global__ void k_scan_fin(int n_sel, const int* __restrict__ classcnt, int* __restrict__ classbase,
-                           unsigned long long* __restrict__ evals) {
+                           RowOut out) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n_sel) return;
     int acc = 0;
@@ -762,7 +775,8 @@ __global__ void k_scan_fin(int n_sel, const int* __restrict__ classcnt, int* __r
         classbase[s * kNumClasses + b] = acc;
         acc += classcnt[s * kNumClasses + b];
     }
-    if (evals) evals[s] = 0;
+    unsigned long long* const ev = out.ev_of(s);
+    if (ev) *ev = 0;
 }
 
 // k_scatter: stable placement of the kept lines into class buckets (centre order preserved): W
@@ -776,8 +790,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
                                                           int n_sp, const SpConst* __restrict__ sc,
                                                           const float* __restrict__ av, const int* __restrict__ blkoff,
                                                           const int* __restrict__ classbase, int nb, const PrepOut o,
-                                                          LineRec* __restrict__ rec,
-                                                          unsigned long long* __restrict__ evals) {
+                                                          LineRec* __restrict__ rec, RowOut out) {
     constexpr int kWarps = kPrepThreads / 32;
     static_assert(W == 1 || W == kWarps, "a run is one warp's or one CTA's");
     __shared__ int placed[kWarps][32];
@@ -835,32 +848,12 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
         if (b < kNumClasses && lrank == 0) placed[warp][b] += __popc(same);
         __syncwarp();
     }
-    if (evals) {
+    unsigned long long* const ev = out.ev_of(s);
+    if (ev) {
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) len_sum += __shfl_down_sync(0xffffffffu, len_sum, d);
-        if (lane == 0 && len_sum) atomicAdd(evals + s, len_sum);
+        if (lane == 0 && len_sum) atomicAdd(ev, len_sum);
     }
-}
-
-// k_ranges: cum[s][b][ts] = position of the first line of class b whose centre key (its grid index,
-// off-grid centres clamped to -1 and N) is >= (ts - 1) * tile, ts = 0 .. nT + 2.
-__global__ void k_ranges(int n_sel, size_t ld, int N, int nT, int tile, const LineRec* __restrict__ rec,
-                         const int* __restrict__ classbase, const int* __restrict__ classcnt, int* __restrict__ cum) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int W = nT + 3;
-    if (t >= (int64_t)n_sel * kNumClasses * W) return;
-    const int ts = (int)(t % W);
-    const int b = (int)((t / W) % kNumClasses);
-    const int s = (int)(t / ((int64_t)W * kNumClasses));
-    const int base = classbase[s * kNumClasses + b], n = classcnt[s * kNumClasses + b];
-    const LineRec* k = rec + s * ld + base;
-    const long long thr = (long long)(ts - 1) * tile;
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (min(max(k[mid].c, -1), N) < thr) lo = mid + 1; else hi = mid;
-    }
-    cum[t] = base + lo;
 }
 
 // ---------------------------------------------------------------------------
@@ -868,12 +861,39 @@ __global__ void k_ranges(int n_sel, size_t ld, int N, int nT, int tile, const Li
 // thread t owns the points J0 + k THREADS + t, k = 0..PTS-1.
 struct RowDesc {
     int N, nT, tile;
-    float lnq, q1, q2, q3;      // expm1(-x)/(-x) ~ 1 + d (q1 + d (q2 + d q3)), x = d lnq
+    float lnq, q1, q2;          // expm1(-x)/(-x) ~ 1 + d (q1 + d q2), x = d lnq
     const float* ln_tp;         // ln of the cut threshold t_p (outputs are t_p * sum of s_rel H)
-    const int* cum;             // [kNumClasses][nT + 3]
+    int* cum;                   // [kNumClasses][nT + 3]
     const LineRec* rec;         // [L] the bucketed lines
     float* out;                 // [N]
 };
+
+// k_ranges: cum[b][ts] of a row = position of its first line of class b whose centre key (its grid
+// index, off-grid centres clamped to -1 and N) is >= (ts - 1) * tile, ts = 0 .. nT + 2.  rows: a
+// descriptor per row, or null: `one` for all, with their arrays following one another.
+__global__ void k_ranges(int n_sel, size_t ld, RowDesc one, const RowDesc* __restrict__ rows,
+                         const int* __restrict__ classbase, const int* __restrict__ classcnt) {
+    const int s = blockIdx.y;
+    RowDesc g = one;
+    if (rows) {
+        g = rows[s];
+    } else {
+        g.cum += (size_t)s * kNumClasses * (g.nT + 3);
+        g.rec += s * ld;
+    }
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, W = g.nT + 3;
+    if (t >= kNumClasses * W) return;
+    const int b = t / W, ts = t - b * W;
+    const int base = classbase[s * kNumClasses + b], n = classcnt[s * kNumClasses + b];
+    const LineRec* k = g.rec + base;
+    const long long thr = (long long)(ts - 1) * g.tile;
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (min(max(k[mid].c, -1), g.N) < thr) lo = mid + 1; else hi = mid;
+    }
+    g.cum[t] = base + lo;
+}
 
 // ---------------------------------------------------------------------------
 // Wing sums by interpolation.
@@ -1405,35 +1425,22 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
     __syncthreads();   // the shared memory is free for the persistent kernel's next tile
 }
 
-// Grid form: one CTA per (row, tile); the rows of one call share the prep arrays.
+// Grid form: one CTA per (row, tile); the rows of one call follow one another in the prep arrays.
 struct TileArgs {
-    int N, nT;
+    RowDesc row;     // row 0
     size_t ld;       // lines per row of the record array
-    float lnq, q1, q2, q3;
-    const int* cum;
-    const LineRec* rec;
-    const float* ln_tp;
-    float* out;
     int split;       // CTAs per tile at most (1: direct output)
     int split_free;  // as many as the GPU holds at once
     float* part;     // split > 1: partial sums [n_sel][split][N], added by k_split_sum
     int* used;       // split > 1: how many of a tile's CTAs wrote theirs, [n_sel][nT]
 };
 
-__device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s, int tile) {
-    const size_t sL = s * g.ld;
-    RowDesc r;
-    r.N = g.N;
-    r.nT = g.nT;
-    r.tile = tile;
-    r.lnq = g.lnq;
-    r.q1 = g.q1;
-    r.q2 = g.q2;
-    r.q3 = g.q3;
-    r.ln_tp = g.ln_tp + s;
-    r.cum = g.cum + (size_t)s * kNumClasses * (g.nT + 3);
-    r.rec = g.rec + sL;
-    r.out = g.out + (size_t)s * g.N;
+__device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s) {
+    RowDesc r = g.row;
+    r.ln_tp += s;
+    r.cum += (size_t)s * kNumClasses * (r.nT + 3);
+    r.rec += s * g.ld;
+    r.out += (size_t)s * r.N;
     return r;
 }
 
@@ -1444,12 +1451,12 @@ __device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s, int tile) 
 // instantiation, so that the one-CTA-per-tile form compiles as it would without it)
 template <int PREC, bool SPLIT>
 __global__ void __launch_bounds__(kTileThreads, MPSA_TILES_MINB) k_tiles(TileArgs g) {
-    RowDesc r = row_desc(g, blockIdx.y, kTile);
+    RowDesc r = row_desc(g, blockIdx.y);
     if (SPLIT) {
         const int sp = blockIdx.x % g.split;
-        r.out = g.part + ((size_t)blockIdx.y * g.split + sp) * g.N;
+        r.out = g.part + ((size_t)blockIdx.y * g.split + sp) * r.N;
         const int tile = blockIdx.x / g.split;
-        tile_body<PREC, kPtsPerThread, kTileThreads>(r, tile, sp, g.split, g.split_free, g.used + (size_t)blockIdx.y * g.nT + tile);
+        tile_body<PREC, kPtsPerThread, kTileThreads>(r, tile, sp, g.split, g.split_free, g.used + (size_t)blockIdx.y * r.nT + tile);
     } else {
         tile_body<PREC, kPtsPerThread, kTileThreads>(r, blockIdx.x);
     }
@@ -1522,7 +1529,7 @@ __global__ void __launch_bounds__(256) k_tiles64(Tile64Args g) {
     __shared__ int sLo[THREADS], sHi[THREADS];
     __shared__ int sN;
     const int s = blockIdx.y, tile = blockIdx.x, tid = threadIdx.x;
-    const RowDesc r = row_desc(g.t, s, kTile64);
+    const RowDesc r = row_desc(g.t, s);
     const int J0 = tile * TILE;
     const double* row = g.pop + (size_t)g.sel[s] * g.pop_stride_;
     const double T = row[kPopT], ne = row[kPopNe], nHI = row[kPopNHI], rho = row[kPopRho];
@@ -1614,10 +1621,10 @@ int synth_module_init(int device) {
 // Device buffers of the line preparation of n_sel rows (one grid, one tile size).
 struct PrepBufs {
     int64_t L = 0;
+    int n_grids = 1;
     size_t ld = 0;   // lines per row of the per-(row, line) arrays: L rounded up to four
-    int n_sel = 0, N = 0, nT = 0, nb = 0, tile = kTile;
-    double lnq = 0.0;
-    int *c = nullptr, *classbase = nullptr, *classcnt = nullptr, *cum = nullptr;
+    int n_sel = 0, nb = 0;
+    int *c = nullptr, *classbase = nullptr, *classcnt = nullptr;
     LineRec* rec = nullptr;
     float *f = nullptr, *dist = nullptr, *lnS = nullptr, *av = nullptr, *lnk0 = nullptr, *ln_tp = nullptr;
     unsigned char* flag = nullptr;
@@ -1627,50 +1634,45 @@ struct PrepBufs {
     PrepOut po{};
 };
 
-// Allocate every prep buffer through `al` (stream-ordered scratch or persistent memory).
+// Allocate every prep buffer of n_sel rows on n_grids grids through `al` (stream-ordered scratch or
+// persistent memory).
 template <class Alloc>
-int prep_alloc(PrepBufs& b, const mpsa_ctx* ctx, int n_sel, int N, double R, int tile, Alloc&& al) {
+int prep_alloc(PrepBufs& b, const mpsa_ctx* ctx, int n_sel, int n_grids, Alloc&& al) {
     b.L = ctx->L;
     b.n_sel = n_sel;
-    b.N = N;
-    b.tile = tile;
-    b.nT = (N + tile - 1) / tile;
+    b.n_grids = n_grids;
     b.nb = (int)((b.L + kPrepLines - 1) / kPrepLines);
-    b.lnq = log1p(1.0 / R);
     b.ld = ((size_t)b.L + 3) & ~(size_t)3;
-    const size_t L = b.ld, SL = n_sel * L, Sb = (size_t)n_sel * b.nb;
+    const size_t GL = n_grids * b.ld, SL = n_sel * b.ld, Sb = (size_t)n_sel * b.nb;
     int r;
-    if ((r = al(&b.c, L)) || (r = al(&b.f, L)) || (r = al(&b.dist, L)) || (r = al(&b.flag, L)) || (r = al(&b.rc, n_sel)) ||
+    if ((r = al(&b.c, GL)) || (r = al(&b.f, GL)) || (r = al(&b.dist, GL)) || (r = al(&b.flag, GL)) || (r = al(&b.rc, n_sel)) ||
         (r = al(&b.spc, (size_t)n_sel * ctx->n_sp)) || (r = al(&b.lnS, SL)) || (r = al(&b.av, SL)) ||
         (r = al(&b.lnk0, SL)) || (r = al(&b.ln_tp, n_sel)) || (r = al(&b.po.surv, SL)) || (r = al(&b.po.nsurv, n_sel)) ||
         (r = al(&b.po.run, Sb)) || (r = al(&b.po.srel, SL)) || (r = al(&b.po.win, SL)) || (r = al(&b.po.cls, SL)) ||
-        (r = al(&b.po.blkcnt, Sb * kNumClasses)) ||
-        (r = al(&b.classbase, (size_t)n_sel * kNumClasses)) || (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) ||
-        (r = al(&b.rec, SL)) || (r = al(&b.cum, (size_t)n_sel * kNumClasses * (b.nT + 3))) || (r = al(&b.med, n_sel)))
+        (r = al(&b.po.blkcnt, Sb * kNumClasses)) || (r = al(&b.classbase, (size_t)n_sel * kNumClasses)) ||
+        (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) || (r = al(&b.rec, SL)) || (r = al(&b.med, n_sel)))
         return r;
     return MPSA_OK;
 }
-
-int ranges_launch(const PrepBufs& b, int tile, int* cum, cudaStream_t st);
 
 GridDesc grid_desc(double lam0_nm, double lnq, int N, int index) {
     return GridDesc{lam0_nm, lnq, (float)lnq, (float)(1.0 / lam0_nm), (float)(1.0 / (lam0_nm * exp((double)(N - 1) * lnq))),
                     N, index};
 }
 
-// Line preparation of the rows d_sel of `pop` on the grid (lam0, R, N): placement, line terms,
-// median continuum and cut threshold, cut windows, width-class buckets and tile ranges.
-int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const int* d_sel, double lam0_nm,
-                float* kc_out, int64_t* evals, const mpsa_synth_opts* opts, cudaStream_t st) {
+// Line preparation of the rows d_sel of `pop`: line terms, median continuum and cut threshold, the
+// lines that reach the grid, their placement, cut windows and width-class buckets.  One grid for
+// all rows (grid), or, with b.n_grids > 1, grid g's descriptor at d_grids[g] and row s's at d_row_grids[s].
+int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const int* d_sel, const GridDesc& grid,
+                const GridDesc* d_grids, const GridDesc* d_row_grids, const RowOut& out, const mpsa_synth_opts* opts,
+                cudaStream_t st) {
     const double cut = (opts && opts->cut > 0) ? opts->cut : 1e-3;
     const double kcf = (opts && opts->kc_factor > 0) ? opts->kc_factor : 1e-2;
     const int64_t L = b.L;
     const int n_sel = b.n_sel, n_sp = ctx->n_sp;
     const int lb = (int)((L + 255) / 256);
-    RowGrids grids;
-    grids.one = grid_desc(lam0_nm, b.lnq, b.N, 0);
-    grids.many = nullptr;
-    k_distance<<<dim3(lb, 1), 256, 0, st>>>(L, b.ld, 1, ctx->d_lam, grids.one, nullptr, b.dist, b.flag);
+    const RowGrids grids{grid, d_row_grids};
+    k_distance<<<dim3(lb, 1), 256, 0, st>>>(L, b.ld, b.n_grids, ctx->d_lam, grid, d_grids, b.dist, b.flag);
     const int pop32 = (opts && opts->precision == MPSA_PREC_FP32_POP32) ? 1 : 0;
     k_consts<<<(n_sel * n_sp + 127) / 128, 128, 0, st>>>(n_sel, d_sel, n_sp, ctx->d_sp_el, ctx->d_sp_stage, ctx->n_el,
                                                            ctx->d_el, pop, ctx->vturb, pop32, b.rc, b.spc);
@@ -1698,7 +1700,7 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
             k_med_collect<<<dim3(per_row, n_sel), kMedThreads, 0, st>>>(L, b.ld, b.lnk0, b.med, list, b.ld);
         }
         k_med_select<<<n_sel, kMedThreads, 0, st>>>(L, b.ld, b.lnk0, small ? nullptr : b.med, list, b.ld,
-                                                    (float)log(kcf), (float)log(cut), b.ln_tp, kc_out);
+                                                    (float)log(kcf), (float)log(cut), b.ln_tp, out);
     }
     MPSA_CUDA_TRY(cudaMemsetAsync(b.po.nsurv, 0, (size_t)n_sel * sizeof(int), st));
     k_prep<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS, b.av,
@@ -1706,11 +1708,12 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     int dev = 0, sms = 0;
     MPSA_CUDA_TRY(cudaGetDevice(&dev));
     MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (b.nb >= 2 * sms)
-        k_place<kPrepLines><<<dim3(b.nb, 1), kPrepThreads, 0, st>>>(L, b.ld, ctx->d_lam, grids.one, nullptr, b.flag, b.c, b.f);
+    if ((int64_t)b.nb * b.n_grids >= 2 * sms)
+        k_place<kPrepLines><<<dim3(b.nb, b.n_grids), kPrepThreads, 0, st>>>(L, b.ld, ctx->d_lam, grid, d_grids, b.flag, b.c,
+                                                                            b.f);
     else
-        k_place<kPrepThreads><<<dim3((unsigned)((L + kPrepThreads - 1) / kPrepThreads), 1), kPrepThreads, 0, st>>>(
-            L, b.ld, ctx->d_lam, grids.one, nullptr, b.flag, b.c, b.f);
+        k_place<kPrepThreads><<<dim3((unsigned)((L + kPrepThreads - 1) / kPrepThreads), b.n_grids), kPrepThreads, 0, st>>>(
+            L, b.ld, ctx->d_lam, grid, d_grids, b.flag, b.c, b.f);
     {
         // the listed lines' count is known on the device only: about eight CTAs per SM in all,
         // each running over its row's list
@@ -1719,45 +1722,42 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
                                                             b.ln_tp, b.nb, b.po);
     }
     k_scan_class<<<dim3(kNumClasses, n_sel), 1024, 0, st>>>(b.nb, b.po.blkcnt, b.classcnt);
-    k_scan_fin<<<(n_sel + 31) / 32, 32, 0, st>>>(n_sel, b.classcnt, b.classbase, (unsigned long long*)evals);
+    k_scan_fin<<<(n_sel + 31) / 32, 32, 0, st>>>(n_sel, b.classcnt, b.classbase, out);
     constexpr int kWarps = kPrepThreads / 32;
     if ((int64_t)b.nb * n_sel * kWarps <= 64ll * sms)
         k_scatter<kWarps><<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(
             b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
-            (unsigned long long*)evals);
+            out);
     else
         k_scatter<1><<<dim3((b.nb + kWarps - 1) / kWarps, n_sel), kPrepThreads, 0, st>>>(
             b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
-            (unsigned long long*)evals);
-    return ranges_launch(b, b.tile, b.cum, st);
-}
-
-int ranges_launch(const PrepBufs& b, int tile, int* cum, cudaStream_t st) {
-    const int nT = (b.N + tile - 1) / tile;
-    const int64_t nr = (int64_t)b.n_sel * kNumClasses * (nT + 3);
-    k_ranges<<<(unsigned)((nr + 255) / 256), 256, 0, st>>>(b.n_sel, b.ld, b.N, nT, tile, b.rec, b.classbase, b.classcnt,
-                                                          cum);
+            out);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
 }
 
-TileArgs tile_args(const PrepBufs& b, float* kappa) {
-    TileArgs ta;
-    ta.N = b.N;
-    ta.nT = b.nT;
-    ta.ld = b.ld;
-    ta.lnq = (float)b.lnq;
-    ta.q1 = (float)(-b.lnq / 2.0);
-    ta.q2 = (float)(b.lnq * b.lnq / 6.0);
-    ta.q3 = (float)(-b.lnq * b.lnq * b.lnq / 24.0);
-    ta.cum = b.cum;
-    ta.rec = b.rec;
-    ta.ln_tp = b.ln_tp;
-    ta.out = kappa;
-    ta.split = ta.split_free = 1;
-    ta.part = nullptr;
-    ta.used = nullptr;
-    return ta;
+// Tile ranges of all rows for the descriptors (see k_ranges); most: the largest number of tiles.
+int ranges_launch(const PrepBufs& b, const RowDesc& one, const RowDesc* d_rows, int most, cudaStream_t st) {
+    const int n = kNumClasses * (most + 3);
+    k_ranges<<<dim3((n + 255) / 256, b.n_sel), 256, 0, st>>>(b.n_sel, b.ld, one, d_rows, b.classbase, b.classcnt);
+    MPSA_CUDA_TRY(cudaGetLastError());
+    return MPSA_OK;
+}
+
+// A row on a grid for tiles of `tile` points: its tile ranges, output, cut threshold and records.
+RowDesc row_of(const GridDesc& q, int tile, int* cum, const float* ln_tp, const LineRec* rec, float* out) {
+    RowDesc r;
+    r.N = q.N;
+    r.nT = (q.N + tile - 1) / tile;
+    r.tile = tile;
+    r.lnq = q.lnq;
+    r.q1 = (float)(-q.lnq64 / 2.0);
+    r.q2 = (float)(q.lnq64 * q.lnq64 / 6.0);
+    r.ln_tp = ln_tp;
+    r.cum = cum;
+    r.rec = rec;
+    r.out = out;
+    return r;
 }
 
 int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, double lam0_nm, double R, int N,
@@ -1768,11 +1768,20 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         return fail(MPSA_EINVAL, "synth: precision %d", prec);
     Scratch sc(st, ctx->pool);
     PrepBufs b;
-    int r;
-    const int tile = prec == MPSA_PREC_FP64 ? kTile64 : kTile;
-    if ((r = prep_alloc(b, ctx, n_sel, N, R, tile, [&](auto** p, size_t n) { return sc.alloc(p, n); }))) return r;
-    if ((r = prep_launch(b, ctx, pop, d_sel, lam0_nm, kc_out, evals, opts, st))) return r;
-    const TileArgs ta = tile_args(b, kappa);
+    int r, *cum;
+    const int tile = prec == MPSA_PREC_FP64 ? kTile64 : kTile, nT = (N + tile - 1) / tile;
+    if ((r = prep_alloc(b, ctx, n_sel, 1, [&](auto** p, size_t n) { return sc.alloc(p, n); }))) return r;
+    if ((r = sc.alloc(&cum, (size_t)n_sel * kNumClasses * (nT + 3)))) return r;
+    const GridDesc grid = grid_desc(lam0_nm, log1p(1.0 / R), N, 0);
+    const RowOut out{kc_out, (unsigned long long*)evals, nullptr, nullptr};
+    if ((r = prep_launch(b, ctx, pop, d_sel, grid, nullptr, nullptr, out, opts, st))) return r;
+    TileArgs ta;
+    ta.row = row_of(grid, tile, cum, b.ln_tp, b.rec, kappa);
+    ta.ld = b.ld;
+    ta.split = ta.split_free = 1;
+    ta.part = nullptr;
+    ta.used = nullptr;
+    if ((r = ranges_launch(b, ta.row, nullptr, nT, st))) return r;
     prof_mark(ctx, MPSA_KERNEL_PROFILE, st);
     if (prec == MPSA_PREC_FP64) {
         Tile64Args g;
@@ -1794,8 +1803,8 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         g.lgW = ctx->d_lgW;
         g.species = ctx->d_species;
         g.lam0_nm = lam0_nm;
-        g.lnq64 = b.lnq;
-        k_tiles64<<<dim3(b.nT, n_sel), 256, 0, st>>>(g);
+        g.lnq64 = grid.lnq64;
+        k_tiles64<<<dim3(nT, n_sel), 256, 0, st>>>(g);
     } else {
         // a call with fewer tiles than the GPU holds CTAs (narrow windows) splits each tile's
         // candidate lines over several CTAs, up to 64, and adds their partial sums afterwards: as
@@ -1804,21 +1813,21 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         int dev = 0, sms = 0;
         MPSA_CUDA_TRY(cudaGetDevice(&dev));
         MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int64_t ctas = (int64_t)b.nT * n_sel, slots = (int64_t)sms * MPSA_TILES_MINB;
+        const int64_t ctas = (int64_t)nT * n_sel, slots = (int64_t)sms * MPSA_TILES_MINB;
         const int64_t most = std::min<int64_t>(64, kNumClasses + b.L / kTileThreads);   // chunks a tile can have
         TileArgs tb = ta;
         tb.split_free = (int)std::max<int64_t>(1, std::min(most, slots / ctas));
         tb.split = ctas > slots ? 1 : (int)std::max<int64_t>(1, std::min(most, 8 * slots / ctas));
         tb.part = nullptr;
         if (tb.split > 1 && ((r = sc.alloc(&tb.part, (size_t)n_sel * tb.split * N)) || (r = sc.alloc(&tb.used, ctas)))) return r;
-        const dim3 grid((unsigned)(b.nT * tb.split), n_sel);
+        const dim3 blocks((unsigned)(nT * tb.split), n_sel);
         const bool naive = prec == MPSA_PREC_FP32_NAIVE;
         if (tb.split > 1) {
-            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, true><<<grid, kTileThreads, 0, st>>>(tb);
-            else k_tiles<MPSA_PREC_FP32_COMPENSATED, true><<<grid, kTileThreads, 0, st>>>(tb);
+            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, true><<<blocks, kTileThreads, 0, st>>>(tb);
+            else k_tiles<MPSA_PREC_FP32_COMPENSATED, true><<<blocks, kTileThreads, 0, st>>>(tb);
         } else {
-            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, false><<<grid, kTileThreads, 0, st>>>(tb);
-            else k_tiles<MPSA_PREC_FP32_COMPENSATED, false><<<grid, kTileThreads, 0, st>>>(tb);
+            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, false><<<blocks, kTileThreads, 0, st>>>(tb);
+            else k_tiles<MPSA_PREC_FP32_COMPENSATED, false><<<blocks, kTileThreads, 0, st>>>(tb);
         }
         if (tb.split > 1) {
             const int64_t tot = (int64_t)n_sel * N;
@@ -1961,17 +1970,26 @@ struct mpsa_batch {
     struct Group {
         mpsa_lgrid grid{};
         int N = 0, n_sel = 0;
-        int* d_sel = nullptr;
+        int part = 0, row0 = 0;   // its rows' place in a part
+        mpsa::GridDesc q{};
+        const int32_t* sel = nullptr;   // host, during creation only
         float *kappa = nullptr, *kc = nullptr;
         int64_t* evals = nullptr;
-        mpsa::PrepBufs pb;
-        int* cum = nullptr;   // tile ranges for the chosen tile size
         int K = 0, n_steps = 0, mean_kind = MPSA_MEAN_ARITH;
         int64_t* d_bounds = nullptr;
         double *d_cw = nullptr, *d_w = nullptr, *odf = nullptr;
         int64_t longest = 0;
     };
     std::vector<Group> groups;
+    // consecutive groups whose rows are prepared together (one launch per kernel, not one per group)
+    struct Part {
+        int n_rows = 0, n_grids = 0, row0 = 0;   // row0: its first row among all
+        mpsa::PrepBufs pb;
+        int* d_sel = nullptr;
+        mpsa::GridDesc *d_grids = nullptr, *d_row_grids = nullptr;
+        mpsa::RowOut out{};
+    };
+    std::vector<Part> parts;
     mpsa::RowDesc* d_rows = nullptr;
     int n_rows = 0;
     int2* d_units = nullptr;
@@ -2000,34 +2018,46 @@ int balloc(mpsa_batch* b, T** p, size_t n) {
     return MPSA_OK;
 }
 
-// Row descriptors for every row of every group with the tile ranges `cums[g]` of tile size `tile`.
-std::vector<RowDesc> row_descs(mpsa_batch* b, int tile, const std::vector<int*>& cums) {
-    std::vector<RowDesc> rows;
-    for (size_t g = 0; g < b->groups.size(); ++g) {
-        auto& G = b->groups[g];
-        const int nT = (G.N + tile - 1) / tile;
+// Row descriptors of every row of every group for tiles of `tile` points, with a new array of tile
+// ranges, on the device; the tile ranges themselves by batch_ranges.
+int batch_rows(mpsa_batch* b, int tile, std::vector<RowDesc>* rows) {
+    size_t n = 0;
+    for (auto& G : b->groups) n += (size_t)G.n_sel * kNumClasses * ((G.N + tile - 1) / tile + 3);
+    int r, *cum;
+    if ((r = balloc(b, &cum, n))) return r;
+    rows->clear();
+    for (auto& G : b->groups) {
+        const PrepBufs& pb = b->parts[G.part].pb;
         for (int s = 0; s < G.n_sel; ++s) {
-            TileArgs ta = tile_args(G.pb, G.kappa);
-            ta.nT = nT;
-            ta.cum = cums[g];
-            RowDesc r;
-            const size_t sL = s * G.pb.ld;
-            r.N = G.N;
-            r.nT = nT;
-            r.tile = tile;
-            r.lnq = ta.lnq;
-            r.q1 = ta.q1;
-            r.q2 = ta.q2;
-            r.q3 = ta.q3;
-            r.ln_tp = G.pb.ln_tp + s;
-            r.cum = cums[g] + (size_t)s * kNumClasses * (nT + 3);
-            r.rec = G.pb.rec + sL;
-            r.out = G.kappa + (size_t)s * G.N;
-            rows.push_back(r);
+            rows->push_back(row_of(G.q, tile, cum, pb.ln_tp + G.row0 + s, pb.rec + (G.row0 + s) * pb.ld,
+                                   G.kappa + (size_t)s * G.N));
+            cum += (size_t)kNumClasses * (rows->back().nT + 3);
         }
     }
-    return rows;
+    MPSA_CUDA_TRY(cudaMemcpy(b->d_rows, rows->data(), rows->size() * sizeof(RowDesc), cudaMemcpyHostToDevice));
+    return MPSA_OK;
 }
+
+int batch_ranges(const mpsa_batch* b, int tile, cudaStream_t st) {
+    for (auto& P : b->parts) {
+        int most = 0, r;
+        for (auto& G : b->groups)
+            if (&b->parts[G.part] == &P) most = std::max(most, (G.N + tile - 1) / tile);
+        if ((r = ranges_launch(P.pb, RowDesc{}, b->d_rows + P.row0, most, st))) return r;
+    }
+    return MPSA_OK;
+}
+
+int batch_prep(const mpsa_batch* b, cudaStream_t st) {
+    for (auto& P : b->parts) {
+        const int r = prep_launch(P.pb, b->ctx, b->ctx->d_pop, P.d_sel, GridDesc{}, P.d_grids, P.d_row_grids, P.out, &b->opts,
+                                  st);
+        if (r) return r;
+    }
+    return MPSA_OK;
+}
+
+constexpr int kPartRows = 32768;   // rows of one preparation (the y dimension of its launches)
 
 int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int autotune, cudaStream_t st) {
     mpsa_ctx* c = b->ctx;
@@ -2047,10 +2077,17 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
         G.kappa = q.kappa_out;
         G.kc = q.kappa_c_out;
         G.evals = q.evals_out;
-        if ((r = balloc(b, &G.d_sel, q.n_sel))) return r;
-        MPSA_CUDA_TRY(cudaMemcpy(G.d_sel, q.sel, q.n_sel * sizeof(int), cudaMemcpyHostToDevice));
-        if ((r = prep_alloc(G.pb, c, q.n_sel, G.N, q.grid.R, kTile, [&](auto** p, size_t n) { return balloc(b, p, n); })))
-            return r;
+        G.sel = q.sel;
+        if (b->parts.empty() || b->parts.back().n_rows + q.n_sel > kPartRows) {
+            b->parts.emplace_back();
+            b->parts.back().row0 = b->n_rows;
+        }
+        mpsa_batch::Part& P = b->parts.back();
+        G.part = (int)b->parts.size() - 1;
+        G.row0 = P.n_rows;
+        G.q = grid_desc(q.grid.lambda0_nm, log1p(1.0 / q.grid.R), G.N, P.n_grids);
+        P.n_rows += q.n_sel;
+        ++P.n_grids;
         if (q.K > 0) {
             if (!q.bounds || !q.widths || !q.odf_out) return fail(MPSA_EINVAL, "mpsa_batch_create: group %d ODF args", g);
             std::vector<double> cw(q.n_steps >= 1 && q.n_steps <= 32 ? q.n_steps + 1 : 1);
@@ -2072,8 +2109,39 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
         b->groups.push_back(G);
         b->n_rows += q.n_sel;
     }
-    for (auto& G : b->groups)
-        if ((r = prep_launch(G.pb, c, c->d_pop, G.d_sel, G.grid.lambda0_nm, G.kc, G.evals, &b->opts, st))) return r;
+    // ---- parts: buffers, rows, grids and output pointers
+    for (size_t p = 0; p < b->parts.size(); ++p) {
+        mpsa_batch::Part& P = b->parts[p];
+        if ((r = prep_alloc(P.pb, c, P.n_rows, P.n_grids, [&](auto** q, size_t n) { return balloc(b, q, n); }))) return r;
+        std::vector<int> sel;
+        std::vector<GridDesc> grids, row_grids;
+        std::vector<float*> kc;
+        std::vector<unsigned long long*> ev;
+        for (auto& G : b->groups) {
+            if (G.part != (int)p) continue;
+            grids.push_back(G.q);
+            for (int s = 0; s < G.n_sel; ++s) {
+                sel.push_back(G.sel[s]);
+                row_grids.push_back(G.q);
+                kc.push_back(G.kc ? G.kc + s : nullptr);
+                ev.push_back(G.evals ? (unsigned long long*)G.evals + s : nullptr);
+            }
+            G.sel = nullptr;
+        }
+        float** d_kc;
+        unsigned long long** d_ev;
+        if ((r = balloc(b, &P.d_sel, sel.size())) || (r = balloc(b, &P.d_grids, grids.size())) ||
+            (r = balloc(b, &P.d_row_grids, sel.size())) || (r = balloc(b, &d_kc, sel.size())) ||
+            (r = balloc(b, &d_ev, sel.size())))
+            return r;
+        MPSA_CUDA_TRY(cudaMemcpy(P.d_sel, sel.data(), sel.size() * sizeof(int), cudaMemcpyHostToDevice));
+        MPSA_CUDA_TRY(cudaMemcpy(P.d_grids, grids.data(), grids.size() * sizeof(GridDesc), cudaMemcpyHostToDevice));
+        MPSA_CUDA_TRY(cudaMemcpy(P.d_row_grids, row_grids.data(), sel.size() * sizeof(GridDesc), cudaMemcpyHostToDevice));
+        MPSA_CUDA_TRY(cudaMemcpy(d_kc, kc.data(), sel.size() * sizeof(float*), cudaMemcpyHostToDevice));
+        MPSA_CUDA_TRY(cudaMemcpy(d_ev, ev.data(), sel.size() * sizeof(unsigned long long*), cudaMemcpyHostToDevice));
+        P.out = RowOut{nullptr, nullptr, d_kc, d_ev};
+    }
+    if ((r = batch_prep(b, st))) return r;
     MPSA_CUDA_TRY(cudaStreamSynchronize(st));
     if ((r = balloc(b, &b->d_rows, b->n_rows)) || (r = balloc(b, &b->d_counter, 1))) return r;
 
@@ -2086,15 +2154,8 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
         double best = 1e300;
         for (int k = 0; k < kNumCfgs; ++k) {
             const int tile = kCfgs[k].pts * kCfgs[k].threads;
-            std::vector<int*> cums;
-            for (auto& G : b->groups) {
-                const int nT = (G.N + tile - 1) / tile;
-                int* cum;
-                if ((r = balloc(b, &cum, (size_t)G.n_sel * kNumClasses * (nT + 3)))) return r;
-                if ((r = ranges_launch(G.pb, tile, cum, st))) return r;
-                cums.push_back(cum);
-            }
-            std::vector<RowDesc> rows = row_descs(b, tile, cums);
+            std::vector<RowDesc> rows;
+            if ((r = batch_rows(b, tile, &rows)) || (r = batch_ranges(b, tile, st))) return r;
             // sample: at least 2048 (row, tile) units (all of them if there are fewer) spread
             // evenly over all units of the batch, so that rows weigh by their tile counts as in
             // the real launch and every CTA of the persistent launch runs several units (the
@@ -2107,7 +2168,6 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
             for (size_t u = step / 2; u < all.size(); u += step) units.push_back(all[u]);
             int2* du;
             if ((r = balloc(b, &du, units.size()))) return r;
-            MPSA_CUDA_TRY(cudaMemcpy(b->d_rows, rows.data(), rows.size() * sizeof(RowDesc), cudaMemcpyHostToDevice));
             MPSA_CUDA_TRY(cudaMemcpy(du, units.data(), units.size() * sizeof(int2), cudaMemcpyHostToDevice));
             float ms_best = 1e30f;
             for (int rep = 0; rep < 2; ++rep) {
@@ -2133,15 +2193,9 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
 
     // ---- final tile ranges, row descriptors and the cost-ordered work list
     const int tile = kCfgs[b->cfg].pts * kCfgs[b->cfg].threads;
-    std::vector<int*> cums;
-    for (auto& G : b->groups) {
-        const int nT = (G.N + tile - 1) / tile;
-        if ((r = balloc(b, &G.cum, (size_t)G.n_sel * kNumClasses * (nT + 3)))) return r;
-        if ((r = ranges_launch(G.pb, tile, G.cum, st))) return r;
-        cums.push_back(G.cum);
-    }
-    std::vector<RowDesc> rows = row_descs(b, tile, cums);
-    MPSA_CUDA_TRY(cudaMemcpy(b->d_rows, rows.data(), rows.size() * sizeof(RowDesc), cudaMemcpyHostToDevice));
+    std::vector<RowDesc> rows;
+    MPSA_CUDA_TRY(cudaStreamSynchronize(st));   // the descriptors of the last trial are overwritten
+    if ((r = batch_rows(b, tile, &rows)) || (r = batch_ranges(b, tile, st))) return r;
     std::vector<int2> units;
     for (int i = 0; i < (int)rows.size(); ++i)
         for (int t = 0; t < rows[i].nT; ++t) units.push_back(make_int2(i, t));
@@ -2173,10 +2227,7 @@ int batch_build(mpsa_batch* b, const mpsa_batch_group* gin, int n_groups, int au
         return fail(MPSA_ECUDA, "mpsa_batch_create: begin capture: %s", cudaGetErrorString(e));
     }
     int rc = MPSA_OK;
-    for (auto& G : b->groups) {
-        if ((rc = prep_launch(G.pb, c, c->d_pop, G.d_sel, G.grid.lambda0_nm, G.kc, G.evals, &b->opts, cap))) break;
-        if ((rc = ranges_launch(G.pb, tile, G.cum, cap))) break;
-    }
+    if ((rc = batch_prep(b, cap)) == MPSA_OK) rc = batch_ranges(b, tile, cap);
     if (rc == MPSA_OK) rc = persistent_launch(b->cfg, b->prec, b->d_rows, b->d_units, b->n_units, b->d_counter, cap);
     if (rc == MPSA_OK)
         for (auto& G : b->groups)
