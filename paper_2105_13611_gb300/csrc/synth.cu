@@ -923,18 +923,6 @@ __constant__ double c_cos24[48] = {
     0.38268343236508977, 0.5, 0.60876142900872064, 0.70710678118654752, 0.79335334029123517, 0.86602540378443865,
     0.92387953251128676, 0.96592582628906829, 0.99144486137381041};
 
-// packed FP32: two lanes per instruction, rounded like fmaf
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
-        "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
-
 // The offset v of a line at the points of a stretch starting D points from its centre:
 // v = G (kv B) + kv E1 with E1 = expm1(-D ln q), B = 1 + E1 and G = expm1(-delta ln q) for the
 // point delta points into the stretch (the exact split of expm1).  Both terms are at most
@@ -1061,9 +1049,10 @@ __device__ __forceinline__ float clenshaw(const float* c, float x) {
 //   kPtRat     rational form on the whole part, v from the expm1 split (u.z = kv E1, u.w = kv B)
 //   kPtWing    the series of H on the whole part, v from the expm1 split, a^2 <= 2
 //   kPtNear    centre within the part's length: v = kv (x - x^2/2 + x^3/6)-like series (|x| <= 0.01, the
-//              rest is below 5e-8 of it); the points jc0..jc1 (|z|^2 < 100, in u.z and u.w as
-//              integers) by voigt_small or, for a > 0.03, the Gauss-Hermite tiers; the others by
-//              the series of H
+//              rest is below 5e-8 of it); the pairs of points jc0..jc1 (|z|^2 < 64, in u.z and u.w
+//              as integers) by voigt_small2 or, for a > 0.03, the Gauss-Hermite tiers; the others
+//              by the series of H (grids of at most 2 in v per point, so that no point of
+//              those pairs is beyond |v| = 10)
 //   kPtGen     any other case, decided point by point
 // with kPtChk where the part is not inside the inner window: a point then takes the line iff
 // s_rel H >= 1.
@@ -1076,24 +1065,46 @@ struct __align__(16) PointRec {
 constexpr int kPtRat = 0, kPtWing = 1, kPtNear = 2, kPtGen = 3, kPtKind = 3, kPtAway = 4, kPtChk = 8;
 constexpr int kPtRecs = 32;    // records a warp holds
 
-// kPtNear's core, by voigt_small (TINY: a <= 3e-4)
-template <bool TINY>
-__device__ __forceinline__ void add_core(float* x, int j0, int j1, int lane, const float4 p, float srel, float a,
-                                         float floor1, float q1, float q2) {
-#pragma unroll 1
-    for (int j = j0 + lane; j <= j1; j += 32) {
-        const float d = ((float)j - p.x) - p.y;
-        const float v = p.z * (d * fmaf(d, fmaf(d, q2, q1), 1.f));
-        const float l = srel * voigt_small<TINY>(v * v, p.w, a);
-        if (l >= floor1) x[j] += l;
-    }
+// two neighbouring points: x[2p], x[2p + 1] += l where l passes the cut
+__device__ __forceinline__ void add_pair(float2* x, int p, float2 l, float floor1) {
+    l.x = l.x >= floor1 ? l.x : 0.f;
+    l.y = l.y >= floor1 ? l.y : 0.f;
+    x[p] = fadd2(x[p], l);
+}
+// offsets d = j - c - f of the points j = 2p, 2p + 1
+__device__ __forceinline__ float2 pair_offsets(int p, const float4 q) {
+    const float j = (float)(2 * p);
+    return fadd2(fadd2(make_float2(j, j + 1.f), dup2(-q.x)), dup2(-q.y));
+}
+__device__ __forceinline__ float2 pair_v(float2 d, const float4 q, float q1, float q2) {
+    return fmul2(dup2(q.z), fmul2(d, ffma2(d, ffma2(d, dup2(q2), dup2(q1)), dup2(1.f))));
+}
+// sk times the series of H at two points (a^2 <= 2), one reciprocal for both
+__device__ __forceinline__ float2 pair_series(float2 v, float A, float sk, float k2, float k3, float k4) {
+    const float2 Z = ffma2(v, v, dup2(A));
+    const float r = rcp_approx(Z.x * Z.y);
+    const float2 y = make_float2(r * Z.y, r * Z.x);
+    const float2 h = ffma2(y, ffma2(y, ffma2(y, ffma2(y, dup2(k4), dup2(k3)), dup2(k2)), dup2(1.5f)), dup2(1.f));
+    return fmul2(fmul2(dup2(sk), y), h);
 }
 
-// One record added to the warp's points x[0..last].  The lanes take 32 consecutive points of the
-// window at a time, so a narrow window costs no idle segments and no two lanes share a point.
-// Every case has a loop of its own without branches: one loop deciding per point spent as
-// many integer and control instructions as FP32 ones.  Gp[j] = expm1(-j ln q).
-__device__ __forceinline__ void add_points(const PointRec& r, float* x, const float* Gp, int last, int lane, float q1,
+// kPtNear's core, the pairs p0..p1, by voigt_small2 (TINY: a <= 3e-4)
+template <bool TINY>
+__device__ __forceinline__ void add_core(float2* x, int p0, int p1, int lane, const float4 p, float srel, float a,
+                                         float floor1, float q1, float q2) {
+#pragma unroll 1
+    for (int i = p0 + lane; i <= p1; i += 32)
+        add_pair(x, i, fmul2(dup2(srel), voigt_small2<TINY>(pair_v(pair_offsets(i, p), p, q1, q2), p.w, a)), floor1);
+}
+
+// One record added to the warp's points x[0..last].  A lane takes two neighbouring points at a
+// time, in packed FP32, and the lanes 64 consecutive points of the window, so a narrow window
+// costs no idle segments and no two lanes share a point.  (Points of a pair outside the window
+// fail the test of the cut by its margin; points past the part's end are never stored.)  Every
+// case has a loop of its own without branches: one loop deciding per point spent as many integer
+// and control instructions as FP32 ones.  The kernel is bound by instruction issue; points one at
+// a time took 16.5 ms for two table rows, pairs PAIRNOW ms.  Gp[j] = expm1(-j ln q).
+__device__ __forceinline__ void add_points(const PointRec& r, float* xs, const float* Gs, int last, int lane, float q1,
                                            float q2, float lnq) {
     const int4 w = *reinterpret_cast<const int4*>(&r.lo);
     const float4 u = *reinterpret_cast<const float4*>(&r.sk);
@@ -1102,27 +1113,27 @@ __device__ __forceinline__ void add_points(const PointRec& r, float* x, const fl
     const int lo = max(w.x, 0), hi = min(w.y, last);
     const int kind = w.z & kPtKind;
     const float a = __int_as_float(w.w);
+    float2* const x = reinterpret_cast<float2*>(xs);
+    const float2* const Gp = reinterpret_cast<const float2*>(Gs);
+    const int p0 = lo >> 1, p1 = hi >> 1;
     if (kind == kPtRat) {
-        const float C = p.w - 1.5f;
+        const float2 E = dup2(u.z), B = dup2(u.w), C = dup2(p.w - 1.5f);
 #pragma unroll 1
-        for (int j = lo + lane; j <= hi; j += 32) {
-            const float v = fmaf(Gp[j], u.w, u.z);
-            const float l = u.x * rcp_approx(fmaf(v, v, C));
-            if (l >= floor1) x[j] += l;
+        for (int i = p0 + lane; i <= p1; i += 32) {
+            const float2 v = ffma2(Gp[i], B, E);
+            const float2 D = ffma2(v, v, C);
+            const float sr = u.x * rcp_approx(D.x * D.y);
+            add_pair(x, i, make_float2(sr * D.y, sr * D.x), floor1);
         }
     } else if (kind == kPtNear) {
-        const int c0 = max(lo, __float_as_int(u.z)), c1 = min(hi, __float_as_int(u.w));
-        // the points outside the core, left then right, as one sequence; no core: all of them
-        const int nl = c0 <= c1 ? c0 - lo : hi - lo + 1, gap = c0 <= c1 ? c1 - c0 + 1 : 0, n = hi - lo + 1 - gap;
+        const int c0 = max(p0, __float_as_int(u.z) >> 1), c1 = min(p1, __float_as_int(u.w) >> 1);
+        // the pairs outside the core, left then right, as one sequence; no core: all of them
+        const int nl = c0 <= c1 ? c0 - p0 : p1 - p0 + 1, gap = c0 <= c1 ? c1 - c0 + 1 : 0, n = p1 - p0 + 1 - gap;
         const float k2 = series_k2(p.w), k3 = series_k3(p.w), k4 = series_k4(p.w);
 #pragma unroll 1
         for (int t = lane; t < n; t += 32) {
-            const int j = lo + t + (t >= nl ? gap : 0);
-            const float d = ((float)j - p.x) - p.y;
-            const float v = p.z * (d * fmaf(d, fmaf(d, q2, q1), 1.f));
-            const float y = rcp_approx(fmaf(v, v, p.w));
-            const float l = u.x * y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, k4, k3), k2), 1.5f), 1.f);
-            if (l >= floor1) x[j] += l;
+            const int i = p0 + t + (t >= nl ? gap : 0);
+            add_pair(x, i, pair_series(pair_v(pair_offsets(i, p), p, q1, q2), p.w, u.x, k2, k3, k4), floor1);
         }
         if (a <= kTinyA) {
             add_core<true>(x, c0, c1, lane, p, u.y, a, floor1, q1, q2);
@@ -1130,30 +1141,25 @@ __device__ __forceinline__ void add_points(const PointRec& r, float* x, const fl
             add_core<false>(x, c0, c1, lane, p, u.y, a, floor1, q1, q2);
         } else {
 #pragma unroll 1
-            for (int j = c0 + lane; j <= c1; j += 32) {
-                const float d = ((float)j - p.x) - p.y;
-                const float v = p.z * (d * fmaf(d, fmaf(d, q2, q1), 1.f));
-                const float l = u.y * voigt_inner_tiers(v, a);
-                if (l >= floor1) x[j] += l;
+            for (int i = c0 + lane; i <= c1; i += 32) {
+                const float2 v = pair_v(pair_offsets(i, p), p, q1, q2);
+                add_pair(x, i, make_float2(u.y * voigt_inner_tiers(v.x, a), u.y * voigt_inner_tiers(v.y, a)), floor1);
             }
         }
     } else if (kind == kPtWing) {
         const float k2 = series_k2(p.w), k3 = series_k3(p.w), k4 = series_k4(p.w);
+        const float2 E = dup2(u.z), B = dup2(u.w);
 #pragma unroll 1
-        for (int j = lo + lane; j <= hi; j += 32) {
-            const float v = fmaf(Gp[j], u.w, u.z);
-            const float y = rcp_approx(fmaf(v, v, p.w));
-            const float l = u.x * y * fmaf(y, fmaf(y, fmaf(y, fmaf(y, k4, k3), k2), 1.5f), 1.f);
-            if (l >= floor1) x[j] += l;
-        }
+        for (int i = p0 + lane; i <= p1; i += 32)
+            add_pair(x, i, pair_series(ffma2(Gp[i], B, E), p.w, u.x, k2, k3, k4), floor1);
     } else {
 #pragma unroll 1
         for (int j = lo + lane; j <= hi; j += 32) {
             float v;
-            if (w.z & kPtAway) v = fmaf(Gp[j], u.w, u.z);
+            if (w.z & kPtAway) v = fmaf(Gs[j], u.w, u.z);
             else v = p.z / lnq * expm1f(-(((float)j - p.x) - p.y) * lnq);
             const float l = u.y * voigt_point(v, a);
-            if (l >= floor1) x[j] += l;
+            if (l >= floor1) xs[j] += l;
         }
     }
 }
@@ -1180,8 +1186,8 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
     constexpr int TILE = PTS * THREADS, WARPS = THREADS / 32, QCAP = THREADS + kQueue;
     __shared__ int sQ[QCAP];
     __shared__ PointRec sP[WARPS][kPtRecs];
-    __shared__ float sX[WARPS][32 * PTS];   // sums of the gathered records at the warp's points
-    __shared__ float sGp[32 * PTS];         // expm1(-j ln q) at the points j of a warp's part
+    __shared__ __align__(8) float sX[WARPS][32 * PTS];   // sums of the gathered records at the warp's points
+    __shared__ __align__(8) float sGp[32 * PTS];         // expm1(-j ln q) at the points j of a warp's part
     __shared__ float sG0[kNodes], sG1[WARPS][kNodes];
     __shared__ float2 sF0[WARPS][kNodes], sF1[WARPS][kNodes];   // node totals {sum, comp}
     __shared__ float sC0[kNodes], sC1[WARPS][kNodes];           // their Chebyshev coefficients
@@ -1268,7 +1274,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
                     const bool smooth = r1.y <= Js && r1.z >= Je && w.dist > span1;
                     const bool ra = rational_ok(w, A);
                     rat = smooth && ra;
-                    ser = smooth && !ra && w.zmin2 >= kSeriesZ2 && w.zmax2 <= 1.0e18f;
+                    ser = smooth && !ra && w.zmin2 >= (A <= kSeriesA ? kSeriesZ2Low : kSeriesZ2) && w.zmax2 <= 1.0e18f;
                     direct = !rat && !ser;
                 }
             }
@@ -1303,13 +1309,13 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
                 int kind = kPtGen;
                 if (away && rational_ok(w, A)) {
                     kind = kPtRat;
-                } else if (A <= kSeriesA && away && w.zmin2 >= kSeriesZ2 && w.zmax2 <= 1.0e18f) {
+                } else if (A <= kSeriesA && away && w.zmin2 >= kSeriesZ2Low && w.zmax2 <= 1.0e18f) {
                     kind = kPtWing;
                 } else if (A <= kSeriesA && !away && (span1 + fmaxf(w.dist, 0.f) + 1.f) * lnq <= 0.01f &&
-                           w.zmax2 <= 1.0e18f) {
+                           w.zmax2 <= 1.0e18f && p.klnq <= 2.f) {
                     kind = kPtNear;
-                    // |v| = 10 at about this many points from the centre
-                    const float h = fminf(sqrtf(kSeriesZ2 - A) / p.klnq, 1.0e6f), x0 = p.ci + f;
+                    // |z| = 8 at this many points from the centre (v is linear to 0.5 per cent there)
+                    const float h = fminf(sqrtf(kSeriesZ2Low - A) / p.klnq * 1.005f, 1.0e6f), x0 = p.ci + f;
                     p.kvE = __int_as_float((int)ceilf(x0 - h));
                     p.kvB = __int_as_float((int)floorf(x0 + h));
                 }

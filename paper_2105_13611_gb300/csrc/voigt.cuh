@@ -140,13 +140,44 @@ __device__ __forceinline__ float voigt_core(float v, float a) {
     return sum;
 }
 
+// packed FP32: two lanes per instruction, rounded like fmaf, * and +
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+        "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+
 // Asymptotic series of H to order |z|^-6, for |z|^2 >= 100: with t = 1/|z|^2 and s = a^2 t,
 //   H = (a t / sqrt(pi)) (1 + t (3/2 - 2 s) + t^2 (15/4 - 15 s + 12 s^2)
 //                           + t^3 (105/8 - 105 s + 210 s^2 - 120 s^3)),
 // relative error 6.2e-7 at |z|^2 = 100 over all a.  For a^2 <= 2 the powers of t are collected,
-// 1 + t (3/2 + t (k2 + t (k3 + t k4))), whose dropped terms stay below 1e-7.  The functions return
-// the factor in brackets.
-constexpr float kSeriesZ2 = 100.f;
+// 1 + t (3/2 + t (k2 + t (k3 + t k4))), which reaches one order further at small a: 3.3e-7 at
+// |z|^2 = 64, the dropped a^2 terms included below 8e-7.  The functions return the factor in
+// brackets.
+constexpr float kSeriesZ2 = 100.f, kSeriesZ2Low = 64.f;
 constexpr float kSeriesA = 2.f;
 __device__ __forceinline__ float series_k2(float A) { return fmaf(-2.f, A, 3.75f); }
 __device__ __forceinline__ float series_k3(float A) { return fmaf(-15.f, A, 13.125f); }
@@ -167,42 +198,59 @@ __device__ __forceinline__ float voigt_series(float t, float A) {
 // rational function of V of degree 8/9, fitted by iteratively weighted least squares to D1 in 40
 // digits on 0 <= V <= 100, with the errors measured against the H of a = 0.03 (7.2e-8); q3 and q5
 // share its denominator (their terms' errors 1.1e-7 and 3e-8).  In FP32 the error is that of
-// rounding V in e^{-V} (1e-6 at V = 16) and 6e-7 elsewhere.  Below a = 3e-4 the a^2 terms are under
-// 1e-7.  The 12-point sum of voigt_core takes about 150 FP32 operations, this 33 (a <= 3e-4) or 50.
+// the quotient and e^{-V}, 6e-7.  Below a = 3e-4 the a^2 terms are under 1e-7.  The 12-point sum of
+// voigt_core takes about 150 FP32 operations a point, this 33 (a <= 3e-4) or 50, half of them
+// instructions.
 constexpr float kSmallA = 0.03f, kTinyA = 3e-4f;
+__device__ __forceinline__ float ex2_approx(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// Two points at once in packed FP32.  e^{-v^2} = 2^{-V log2 e}, V = v^2, with the rounding errors of V and of
+// its product with log2 e (both grow with V) put back as a factor, so that it keeps the 2^-22 of
+// ex2.approx at every V.  One reciprocal serves both points.
 template <bool TINY>
-__device__ __forceinline__ float voigt_small(float V, float A, float a) {
-    float num = fmaf(V, 2.305875414e-07f, -1.762603615e-06f);
-    num = fmaf(V, num, 3.279474764e-05f);
-    num = fmaf(V, num, 5.095594350e-05f);
-    num = fmaf(V, num, 9.224279876e-04f);
-    num = fmaf(V, num, 2.128481715e-02f);
-    num = fmaf(V, num, -1.116970724e-01f);
-    num = fmaf(V, num, 1.400493778e+00f);
-    num = fmaf(V, num, -1.128381491e+00f);
-    float den = fmaf(V, 4.087151467e-07f, -3.740103610e-06f);
-    den = fmaf(V, den, 6.256900470e-05f);
-    den = fmaf(V, den, -1.926362426e-05f);
-    den = fmaf(V, den, 2.406517031e-03f);
-    den = fmaf(V, den, 1.126780977e-02f);
-    den = fmaf(V, den, 7.061498180e-02f);
-    den = fmaf(V, den, 2.827565242e-01f);
-    den = fmaf(V, den, 7.589423457e-01f);
-    den = fmaf(V, den, 1.f);
-    float e = expf(-V);
+__device__ __forceinline__ float2 voigt_small2(float2 v, float A, float a) {
+    const float2 V = fmul2(v, v);
+    float2 num = ffma2(V, dup2(2.305875414e-07f), dup2(-1.762603615e-06f));
+    float2 den = ffma2(V, dup2(4.087151467e-07f), dup2(-3.740103610e-06f));
+    num = ffma2(V, num, dup2(3.279474764e-05f));
+    den = ffma2(V, den, dup2(6.256900470e-05f));
+    num = ffma2(V, num, dup2(5.095594350e-05f));
+    den = ffma2(V, den, dup2(-1.926362426e-05f));
+    num = ffma2(V, num, dup2(9.224279876e-04f));
+    den = ffma2(V, den, dup2(2.406517031e-03f));
+    num = ffma2(V, num, dup2(2.128481715e-02f));
+    den = ffma2(V, den, dup2(1.126780977e-02f));
+    num = ffma2(V, num, dup2(-1.116970724e-01f));
+    den = ffma2(V, den, dup2(7.061498180e-02f));
+    num = ffma2(V, num, dup2(1.400493778e+00f));
+    den = ffma2(V, den, dup2(2.827565242e-01f));
+    num = ffma2(V, num, dup2(-1.128381491e+00f));
+    den = ffma2(V, den, dup2(7.589423457e-01f));
+    den = ffma2(V, den, dup2(1.f));
+    const float2 hi = fmul2(V, dup2(1.44269504f));
+    const float2 lo = ffma2(V, dup2(-1.44269504f), hi);              // hi - V log2e (its rounding)
+    const float cx = fmaf(lo.x, 0.69314718f, fmaf(-v.x, v.x, V.x));   // ... and that of V
+    const float cy = fmaf(lo.y, 0.69314718f, fmaf(-v.y, v.y, V.y));
+    const float ex = ex2_approx(-hi.x), ey = ex2_approx(-hi.y);
+    float2 e = make_float2(fmaf(ex, cx, ex), fmaf(ey, cy, ey));
     if (!TINY) {
-        float p3 = fmaf(V, -2.027746242e-07f, -3.567472225e-06f);
-        p3 = fmaf(V, p3, 2.367759875e-04f);
-        p3 = fmaf(V, p3, -7.864333038e-03f);
-        p3 = fmaf(V, p3, 1.155756054e-01f);
-        p3 = fmaf(V, p3, -9.202488923e-01f);
-        p3 = fmaf(V, p3, 2.417829106e+00f);
-        p3 = fmaf(V, p3, -7.482371018e-01f);
-        num = fmaf(A, fmaf(A, -0.3440872f, p3), num);
-        const float c2 = fmaf(V, fmaf(V, 2.f / 3.f, -2.f), 0.5f);
-        e *= fmaf(A, fmaf(A, c2, fmaf(-2.f, V, 1.f)), 1.f);
+        const float2 A2 = dup2(A);
+        float2 p3 = ffma2(V, dup2(-2.027746242e-07f), dup2(-3.567472225e-06f));
+        p3 = ffma2(V, p3, dup2(2.367759875e-04f));
+        p3 = ffma2(V, p3, dup2(-7.864333038e-03f));
+        p3 = ffma2(V, p3, dup2(1.155756054e-01f));
+        p3 = ffma2(V, p3, dup2(-9.202488923e-01f));
+        p3 = ffma2(V, p3, dup2(2.417829106e+00f));
+        p3 = ffma2(V, p3, dup2(-7.482371018e-01f));
+        num = ffma2(A2, ffma2(A2, dup2(-0.3440872f), p3), num);
+        const float2 c2 = ffma2(V, ffma2(V, dup2(2.f / 3.f), dup2(-2.f)), dup2(0.5f));
+        e = fmul2(e, ffma2(A2, ffma2(A2, c2, ffma2(V, dup2(-2.f), dup2(1.f))), dup2(1.f)));
     }
-    return fmaf(a * rcp_approx(den), num, e);
+    const float r = a * rcp_approx(den.x * den.y);
+    return ffma2(make_float2(r * den.y, r * den.x), num, e);
 }
 
 // H(v, a) for any v (sign ignored) and a > 0.
@@ -234,8 +282,8 @@ __device__ __forceinline__ float voigt_point(float v, float a) {
         const float t = rcp_approx(Z);
         return a * kInvSqrtPi * t * voigt_series(t, A);
     }
-    if (a <= kTinyA) return voigt_small<true>(V, A, a);
-    if (a <= kSmallA) return voigt_small<false>(V, A, a);
+    if (a <= kTinyA) return voigt_small2<true>(make_float2(v, v), A, a).x;
+    if (a <= kSmallA) return voigt_small2<false>(make_float2(v, v), A, a).x;
     return voigt_H_lean(v, a);
 }
 
