@@ -517,15 +517,26 @@ __device__ __forceinline__ float d_blue(float vv, float kv, float lnq) { return 
 constexpr unsigned char kDropped = 255;
 
 // The tile kernel's constants of one kept (row, line), stored in bucket order so that a
-// tile's candidates are one contiguous run of records (three 16-byte loads per line)
-// instead of gathers from nine line-indexed arrays.
+// tile's candidates are one contiguous run of records (two 16-byte loads per line) instead of
+// gathers from nine line-indexed arrays.  The inner cut window [ilo, ihi] is kept as its
+// distances from the ends of the outer one, 16 bits each (the windows differ by about 2e-4 of
+// their width); a line without an inner window, or with one further in than that, has none.
 struct __align__(16) LineRec {
     int c;
     float f, kv, a;
     float srel;
-    int ilo, ihi, jlo;
-    int jhi, line, pad0, pad1;
+    int jlo, jhi;
+    unsigned in;
 };
+constexpr unsigned kNoInner = 0xffffffffu;
+__device__ __forceinline__ unsigned pack_inner(int jlo, int jhi, int ilo, int ihi) {
+    const int l = ilo - jlo, h = jhi - ihi;
+    return ilo <= ihi && l < 65535 && h < 65535 ? (unsigned)l | ((unsigned)h << 16) : kNoInner;
+}
+// every point of [j0, j1] is inside the inner window
+__device__ __forceinline__ bool inner_covers(int jlo, int jhi, unsigned in, int j0, int j1) {
+    return in != kNoInner && jlo + (int)(in & 0xffffu) <= j0 && jhi - (int)(in >> 16) >= j1;
+}
 
 // Lists of the lines that k_prep lets through, per row (compact: every array is indexed by the
 // position in the list).  The lines of a prep block are one run of the list, in line order.
@@ -790,7 +801,8 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
                                                           int n_sp, const SpConst* __restrict__ sc,
                                                           const float* __restrict__ av, const int* __restrict__ blkoff,
                                                           const int* __restrict__ classbase, int nb, const PrepOut o,
-                                                          LineRec* __restrict__ rec, RowOut out) {
+                                                          LineRec* __restrict__ rec, int* __restrict__ line,
+                                                          RowOut out) {
     constexpr int kWarps = kPrepThreads / 32;
     static_assert(W == 1 || W == kWarps, "a run is one warp's or one CTA's");
     __shared__ int placed[kWarps][32];
@@ -837,12 +849,10 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
             r.srel = o.srel[sL + t];
             r.jlo = w.x;
             r.jhi = w.y;
-            r.ilo = w.z;
-            r.ihi = w.w;
-            r.line = i;
-            r.pad0 = r.pad1 = 0;
+            r.in = pack_inner(w.x, w.y, w.z, w.w);
             len_sum += (unsigned long long)(w.y - w.x + 1);
             rec[sL + placed[warp][b] + lrank] = r;
+            line[sL + placed[warp][b] + lrank] = i;
         }
         __syncwarp();
         if (b < kNumClasses && lrank == 0) placed[warp][b] += __popc(same);
@@ -865,6 +875,7 @@ struct RowDesc {
     const float* ln_tp;         // ln of the cut threshold t_p (outputs are t_p * sum of s_rel H)
     int* cum;                   // [kNumClasses][nT + 3]
     const LineRec* rec;         // [L] the bucketed lines
+    const int* line;            // [L] their indices in the list
     float* out;                 // [N]
 };
 
@@ -933,11 +944,18 @@ struct Wing {
     float dist;          // distance [points] of the centre from the stretch, < 0 inside
     float zmin2, zmax2;  // smallest and largest |z|^2 on the stretch
 };
+// expm1(x): its series to x^6 for |x| <= 1/8 (below 8e-10 of it; stretches within a ninth of the wavelength of
+// the centre, which almost all are), a quarter of expm1f's instructions
+__device__ __forceinline__ float expm1_near(float x) {
+    if (fabsf(x) <= 0.125f)
+        return x * fmaf(x, fmaf(x, fmaf(x, fmaf(x, fmaf(x, 1.f / 720.f, 1.f / 120.f), 1.f / 24.f), 1.f / 6.f), 0.5f), 1.f);
+    return expm1f(x);
+}
 // span = its number of points - 1, gend = G at its end
 __device__ __forceinline__ Wing wing(int J, int c, float f, float kv, float A, float lnq, float span, float gend) {
     Wing w;
     const float D = (float)(J - c) - f;
-    const float E1 = expm1f(-D * lnq);
+    const float E1 = expm1_near(-D * lnq);
     w.kvE = kv * E1;
     w.kvB = kv + w.kvE;
     const float v0 = fabsf(w.kvE), v1 = fabsf(fmaf(gend, w.kvB, w.kvE));
@@ -1103,7 +1121,7 @@ __device__ __forceinline__ void add_core(float2* x, int p0, int p1, int lane, co
 // fail the test of the cut by its margin; points past the part's end are never stored.)  Every
 // case has a loop of its own without branches: one loop deciding per point spent as many integer
 // and control instructions as FP32 ones.  The kernel is bound by instruction issue; points one at
-// a time took 16.5 ms for two table rows, pairs PAIRNOW ms.  Gp[j] = expm1(-j ln q).
+// a time took 16.5 ms for two table rows, pairs 14.3 ms.  Gp[j] = expm1(-j ln q).
 __device__ __forceinline__ void add_points(const PointRec& r, float* xs, const float* Gs, int last, int lane, float q1,
                                            float q2, float lnq) {
     const int4 w = *reinterpret_cast<const int4*>(&r.lo);
@@ -1175,10 +1193,10 @@ __device__ __forceinline__ void add_points(const PointRec& r, float* xs, const f
 // over it, one line per lane, for its own part of the tile (level 1), and the lines that the
 // part cannot take are gathered (kPtRecs a warp) and evaluated at its points by the whole warp.
 //
-// FP32 partial sums run over at most 64 lines (level 0, points) or 2 THREADS / 32 lines (level 1)
+// FP32 partial sums run over at most 64 lines (level 0, points) or 72 lines (level 1)
 // and are folded into Kahan-compensated totals in shared memory.
 constexpr int kSplitChunks = 64;   // chunks of candidates that are worth a CTA of their own
-constexpr int kQueue = 1024;   // queued lines at which a tile turns to level 1
+constexpr int kQueue = 2048;   // queued lines at which a tile turns to level 1
 
 template <int PREC, int PTS, int THREADS>
 __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0, int S = 1, int S_free = 1,
@@ -1261,17 +1279,19 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
             const int i = i0 + lane;
             bool direct = false, rat = false, ser = false;
             Wing w{};
-            int4 r0, r1, r2;
+            int4 r0, r1;
             float f = 0.f, kv = 0.f, a = 0.f, A = 0.f, sk = 0.f;
+            bool inside = false;
             if (i < n) {
                 const int4* rp = reinterpret_cast<const int4*>(g.rec + sQ[i]);
-                r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2);
-                if (r2.x >= Js && r1.w <= Je) {
+                r0 = __ldg(rp), r1 = __ldg(rp + 1);
+                if (r1.z >= Js && r1.y <= Je) {
                     f = __int_as_float(r0.y), kv = __int_as_float(r0.z), a = __int_as_float(r0.w);
                     A = a * a;
                     sk = __int_as_float(r1.x) * a * kInvSqrtPi;
                     w = wing(Js, r0.x, f, kv, A, lnq, span1, gend1);
-                    const bool smooth = r1.y <= Js && r1.z >= Je && w.dist > span1;
+                    inside = inner_covers(r1.y, r1.z, (unsigned)r1.w, Js, Je);
+                    const bool smooth = inside && w.dist > span1;
                     const bool ra = rational_ok(w, A);
                     rat = smooth && ra;
                     ser = smooth && !ra && w.zmin2 >= (A <= kSeriesA ? kSeriesZ2Low : kSeriesZ2) && w.zmax2 <= 1.0e18f;
@@ -1302,10 +1322,9 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
                 p.srel = __int_as_float(r1.x);
                 p.kvE = w.kvE;
                 p.kvB = w.kvB;
-                p.lo = r1.w - Js;
-                p.hi = r2.x - Js;
+                p.lo = r1.y - Js;
+                p.hi = r1.z - Js;
                 p.a = a;
-                const bool chk = !(r1.y <= Js && r1.z >= Je);
                 int kind = kPtGen;
                 if (away && rational_ok(w, A)) {
                     kind = kPtRat;
@@ -1319,7 +1338,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
                     p.kvE = __int_as_float((int)ceilf(x0 - h));
                     p.kvB = __int_as_float((int)floorf(x0 + h));
                 }
-                p.kind = kind | (away ? kPtAway : 0) | (chk ? kPtChk : 0);
+                p.kind = kind | (away ? kPtAway : 0) | (inside ? 0 : kPtChk);
                 sP[warp][np + __popc(m & ((1u << lane) - 1u))] = p;
             }
             np += __popc(m);
@@ -1354,35 +1373,25 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
             // ---- level 0: one candidate line per thread
             const int pos = pos0 + tid;
             bool queue = false;
-            int4 r0, r1, r2;
             if (pos < end) {
                 const int4* rp = reinterpret_cast<const int4*>(g.rec + pos);
-                r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2);
-                const int ilo = r1.y, ihi = r1.z, jlo = r1.w, jhi = r2.x;
-                if (jhi >= J0 && jlo <= Te) {
+                const int4 r0 = __ldg(rp), r1 = __ldg(rp + 1);
+                if (r1.z >= J0 && r1.y <= Te) {
                     const float a = __int_as_float(r0.w), A = a * a;
                     const Wing w = wing(J0, r0.x, __int_as_float(r0.y), __int_as_float(r0.z), A, lnq, span0, gend0);
-                    if (ilo <= J0 && ihi >= Te && w.dist > span0 && rational_ok(w, A)) {
-                        float G[kNodes];
-#pragma unroll
-                        for (int k = 0; k < kNodes; ++k) G[k] = sG0[k];
-                        nodes_rational(w, A, __int_as_float(r1.x) * a * kInvSqrtPi, G, acc0);
-                    } else {
+                    if (inner_covers(r1.y, r1.z, (unsigned)r1.w, J0, Te) && w.dist > span0 && rational_ok(w, A))
+                        nodes_rational(w, A, __int_as_float(r1.x) * a * kInvSqrtPi, sG0, acc0);
+                    else
                         queue = true;
-                    }
                 }
             }
             // ---- queue the others, in candidate order
             const unsigned bm = __ballot_sync(0xffffffffu, queue);
             if (lane == 0) sCnt[par][warp] = __popc(bm);
             __syncthreads();
-            int off = nq, tot = 0;
-#pragma unroll
-            for (int v = 0; v < WARPS; ++v) {
-                const int cnt = sCnt[par][v];
-                if (v < warp) off += cnt;
-                tot += cnt;
-            }
+            const unsigned cnt = lane < WARPS ? (unsigned)sCnt[par][lane] : 0u;
+            const int tot = (int)__reduce_add_sync(0xffffffffu, cnt);
+            const int off = nq + (int)__reduce_add_sync(0xffffffffu, lane < warp ? cnt : 0u);
             par ^= 1;
             if (queue) sQ[off + __popc(bm & ((1u << lane) - 1u))] = pos;
             nq += tot;
@@ -1446,6 +1455,7 @@ __device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s) {
     r.ln_tp += s;
     r.cum += (size_t)s * kNumClasses * (r.nT + 3);
     r.rec += s * g.ld;
+    r.line += s * g.ld;
     r.out += (size_t)s * r.N;
     return r;
 }
@@ -1558,7 +1568,7 @@ __global__ void __launch_bounds__(256) k_tiles64(Tile64Args g) {
             __syncthreads();
             const int pos = base + tid;
             if (pos < end) {
-                const int q = r.rec[pos].line;
+                const int q = r.line[pos];
                 const int jlo = r.rec[pos].jlo, jhi = r.rec[pos].jhi;
                 if (jhi >= J0 && jlo <= J0 + TILE - 1) {
                     const int sp = g.species[q];
@@ -1630,7 +1640,7 @@ struct PrepBufs {
     int n_grids = 1;
     size_t ld = 0;   // lines per row of the per-(row, line) arrays: L rounded up to four
     int n_sel = 0, nb = 0;
-    int *c = nullptr, *classbase = nullptr, *classcnt = nullptr;
+    int *c = nullptr, *classbase = nullptr, *classcnt = nullptr, *line = nullptr;
     LineRec* rec = nullptr;
     float *f = nullptr, *dist = nullptr, *lnS = nullptr, *av = nullptr, *lnk0 = nullptr, *ln_tp = nullptr;
     unsigned char* flag = nullptr;
@@ -1656,7 +1666,8 @@ int prep_alloc(PrepBufs& b, const mpsa_ctx* ctx, int n_sel, int n_grids, Alloc&&
         (r = al(&b.lnk0, SL)) || (r = al(&b.ln_tp, n_sel)) || (r = al(&b.po.surv, SL)) || (r = al(&b.po.nsurv, n_sel)) ||
         (r = al(&b.po.run, Sb)) || (r = al(&b.po.srel, SL)) || (r = al(&b.po.win, SL)) || (r = al(&b.po.cls, SL)) ||
         (r = al(&b.po.blkcnt, Sb * kNumClasses)) || (r = al(&b.classbase, (size_t)n_sel * kNumClasses)) ||
-        (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) || (r = al(&b.rec, SL)) || (r = al(&b.med, n_sel)))
+        (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) || (r = al(&b.rec, SL)) || (r = al(&b.line, SL)) ||
+        (r = al(&b.med, n_sel)))
         return r;
     return MPSA_OK;
 }
@@ -1733,11 +1744,11 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     if ((int64_t)b.nb * n_sel * kWarps <= 64ll * sms)
         k_scatter<kWarps><<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(
             b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
-            out);
+            b.line, out);
     else
         k_scatter<1><<<dim3((b.nb + kWarps - 1) / kWarps, n_sel), kPrepThreads, 0, st>>>(
             b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
-            out);
+            b.line, out);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
 }
@@ -1751,7 +1762,7 @@ int ranges_launch(const PrepBufs& b, const RowDesc& one, const RowDesc* d_rows, 
 }
 
 // A row on a grid for tiles of `tile` points: its tile ranges, output, cut threshold and records.
-RowDesc row_of(const GridDesc& q, int tile, int* cum, const float* ln_tp, const LineRec* rec, float* out) {
+RowDesc row_of(const GridDesc& q, int tile, int* cum, const float* ln_tp, const LineRec* rec, const int* line, float* out) {
     RowDesc r;
     r.N = q.N;
     r.nT = (q.N + tile - 1) / tile;
@@ -1762,6 +1773,7 @@ RowDesc row_of(const GridDesc& q, int tile, int* cum, const float* ln_tp, const 
     r.ln_tp = ln_tp;
     r.cum = cum;
     r.rec = rec;
+    r.line = line;
     r.out = out;
     return r;
 }
@@ -1782,7 +1794,7 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
     const RowOut out{kc_out, (unsigned long long*)evals, nullptr, nullptr};
     if ((r = prep_launch(b, ctx, pop, d_sel, grid, nullptr, nullptr, out, opts, st))) return r;
     TileArgs ta;
-    ta.row = row_of(grid, tile, cum, b.ln_tp, b.rec, kappa);
+    ta.row = row_of(grid, tile, cum, b.ln_tp, b.rec, b.line, kappa);
     ta.ld = b.ld;
     ta.split = ta.split_free = 1;
     ta.part = nullptr;
@@ -2036,7 +2048,7 @@ int batch_rows(mpsa_batch* b, int tile, std::vector<RowDesc>* rows) {
         const PrepBufs& pb = b->parts[G.part].pb;
         for (int s = 0; s < G.n_sel; ++s) {
             rows->push_back(row_of(G.q, tile, cum, pb.ln_tp + G.row0 + s, pb.rec + (G.row0 + s) * pb.ld,
-                                   G.kappa + (size_t)s * G.N));
+                                   pb.line + (G.row0 + s) * pb.ld, G.kappa + (size_t)s * G.N));
             cum += (size_t)kNumClasses * (rows->back().nT + 3);
         }
     }
