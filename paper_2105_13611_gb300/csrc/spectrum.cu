@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "internal.cuh"
+#include "voigt.cuh"   // packed FP32
 
 namespace mpsa {
 
@@ -136,20 +137,24 @@ __global__ void __launch_bounds__(128) k_formal(int D, int N, const float* __res
 //
 // Three kernels per call:
 //  * k_bin_table: the FP64 table rounded once to FP32 (the interpolation then runs on the
-//    FP32 pipes; per-value conversions in the main loop kept the FP64 pipe 86 % busy);
+//    FP32 pipes; per-value conversions in the main loop kept the FP64 pipe 86 % busy) and
+//    turned to [row][sub-bin][bin], the bins padded to an even number;
 //  * k_bin_cells: per (ray, depth) the interpolation cell, its four weights, the
 //    interpolated continuum, m and T in FP32, and the ray's validity;
-//  * k_bin_intensity: one CTA per (ray, chunk of kb bins); thread t < kb * n_steps owns
-//    sub-bin s = t % n_steps of bin k0 + t / n_steps and walks the depths from the bottom
-//    up, holding one intensity per direction.  The recurrence needs only the layer optical
+//  * k_bin_intensity: one CTA per (ray, chunk of kb bins); a thread owns one sub-bin of two
+//    neighbouring bins and walks the depths from the bottom up, holding one intensity pair per
+//    direction.  The recurrence needs only the layer optical
 //    thicknesses dtau_d = (kappa_d + kappa_{d+1})(m_{d+1} - m_d)/2 and tau_0 = kappa_0 m_0, so
 //    no depth array is kept.  The cells and the Planck function of each bin and depth sit in
 //    shared memory; the per-bin Planck constants come from the host.
-constexpr int kBinThreads = 256;
+constexpr int kBinThreads = 192;            // at most
+constexpr int kBinCols = 2 * kBinThreads;   // sub-bins of a CTA, two per thread
+constexpr int kBinMaxKb = 64;
+
 
 struct DepthCell {
     int r00, dT, dP;        // table row of the lower corner, row offsets to the upper T and P corners
-                            // (k_bin_cells); scaled to element offsets (times K n_steps) for the table
+                            // (k_bin_cells); scaled to offsets in pairs of bins for the table
     float w00, w01, w10, w11;
     float m, T, kc;
     float pad[2];
@@ -157,7 +162,7 @@ struct DepthCell {
 
 struct BinCellArgs {
     int nT, nP, D, n_rays;
-    int row_stride;        // K * n_steps (table elements per row)
+    int row_stride;        // bin pairs of a table row
     const double* lt;      // [nT] log10 T axis
     const double* lp;      // [nP] log10 P axis
     const float* kc;       // [nT*nP]
@@ -170,7 +175,7 @@ struct BinCellArgs {
 
 struct BinArgs {
     int K, ns, D, n_mu, kb;
-    const float* tab;      // [nT*nP][K][ns] FP32
+    const float2* tab;     // [nT*nP][ns][(K + 1) / 2] bin pairs, FP32
     const float3* pk;      // [K]: c1, ln c1, c2 of B_lambda at the bin centre
     const double* w;       // [ns]
     const float* mu;       // [n_mu]
@@ -195,9 +200,26 @@ __device__ __forceinline__ void axis_cell(const double* __restrict__ ax, int n, 
     *f = (x - ax[lo]) / (ax[lo + 1] - ax[lo]);
 }
 
-__global__ void k_bin_table(const double* __restrict__ src, float* __restrict__ dst, size_t n) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dst[i] = (float)src[i];
+// a block turns one row's chunk of kTabBins bins in shared memory: coalesced reads and writes
+constexpr int kTabBins = 64;
+__global__ void __launch_bounds__(256) k_bin_table(const double* __restrict__ src, float* __restrict__ dst, int rows,
+                                                   int K, int ns) {
+    __shared__ float t[32][kTabBins + 1];
+    const int Kp = (K + 1) & ~1, chunks = (Kp + kTabBins - 1) / kTabBins;
+    for (long long it = blockIdx.x; it < (long long)rows * chunks; it += gridDim.x) {
+        const int row = (int)(it / chunks), k0 = (int)(it - (long long)row * chunks) * kTabBins;
+        const int nb = min(kTabBins, K - k0), nw = min(kTabBins, Kp - k0);
+        const double* in = src + ((size_t)row * K + k0) * ns;
+        __syncthreads();
+        if (nw > nb)
+            for (int s = threadIdx.x; s < ns; s += blockDim.x) t[s][nb] = 0.f;
+        for (int i = threadIdx.x; i < nb * ns; i += blockDim.x) t[i % ns][i / ns] = (float)in[i];
+        __syncthreads();
+        for (int i = threadIdx.x; i < ns * nw; i += blockDim.x) {
+            const int s = i / nw, k = i - s * nw;
+            dst[((size_t)row * ns + s) * Kp + k0 + k] = t[s][k];
+        }
+    }
 }
 
 __global__ void k_bin_cells(BinCellArgs a) {
@@ -231,19 +253,27 @@ __global__ void k_bin_cells(BinCellArgs a) {
     a.cells[i] = c;
 }
 
+// Bound by instruction issue (88 % of the slots at one sub-bin per thread): two sub-bins per
+// thread in packed FP32.  The two are the same sub-bin of neighbouring bins, and so are a
+// warp's: their opacities are alike, where a bin's own sub-bins span orders of magnitude, so a
+// warp's layers are mostly all thin or all thick and one of the two forms runs.
+// 1024 rays x 80 depths x 328 bins x 12 sub-bins x 5 directions: 1.53 ms one sub-bin per thread,
+// 1.37 ms in pairs within a bin, 1.35 ms in pairs across bins, 1.20 ms with the two short forms
+// below.  64 registers and 5 CTAs per SM: 6 CTAs (1.33 ms) reload the constants, and one choice
+// of form for all directions of a layer takes the same time with 93 registers.
 template <int NMU>
 __global__ void __launch_bounds__(kBinThreads) k_bin_intensity(BinArgs a) {
     extern __shared__ __align__(16) unsigned char bsm[];
     DepthCell* cell = reinterpret_cast<DepthCell*>(bsm);                      // [D]
-    float* Sb = reinterpret_cast<float*>(cell + a.D);                         // [kb][D]
-    float* part = Sb + (size_t)a.kb * a.D;                                    // [kBinThreads][NMU]
+    float* Sb = reinterpret_cast<float*>(cell + a.D);                         // [D][kb]
+    float* part = Sb + (size_t)a.kb * a.D;                                    // [ns][kb][NMU]
     const int ray = blockIdx.y, k0 = blockIdx.x * a.kb, tid = threadIdx.x;
     const DepthCell* rc = a.cells + (size_t)ray * a.D;
-    for (int d = tid; d < a.D; d += kBinThreads) cell[d] = rc[d];
+    for (int d = tid; d < a.D; d += blockDim.x) cell[d] = rc[d];
     __syncthreads();
     // Planck function at each bin centre and depth
-    for (int i = tid; i < a.kb * a.D; i += kBinThreads) {
-        const int kb = i / a.D, d = i - kb * a.D, k = k0 + kb;
+    for (int i = tid; i < a.kb * a.D; i += blockDim.x) {
+        const int d = i / a.kb, k = k0 + i - d * a.kb;
         float S = 0.f;
         if (k < a.K) {
             const float3 p = a.pk[k];
@@ -253,70 +283,113 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_intensity(BinArgs a) {
     }
     __syncthreads();
 
-    const int kb = tid / a.ns, s = tid - kb * a.ns, k = k0 + kb;
-    const bool act = kb < a.kb && k < a.K;
-    // per direction: mu, 1/mu and -log2(e)/mu (e^{-x/mu} = 2^{x * (-log2 e / mu)})
-    float I[NMU], mu[NMU], rmu[NMU], nl2[NMU];
+    const int pairs = a.kb / 2, s = tid / pairs, pr = tid - s * pairs;
+    if (s < a.ns && k0 + 2 * pr < a.K) {
+    float2 I[NMU];
 #pragma unroll
-    for (int q = 0; q < NMU; ++q) {
-        mu[q] = q < a.n_mu ? a.mu[q] : 1.f;
-        rmu[q] = 1.f / mu[q];
-        nl2[q] = -1.4426950408889634f * rmu[q];
-        I[q] = 0.f;
-    }
-    if (act) {
-        const int col = k * a.ns + s;
-        const float* __restrict__ tab = a.tab;
-        const float* S = Sb + (size_t)kb * a.D;
-        auto kappa = [&](int d) -> float {
-            const DepthCell c = cell[d];
-            const float* t = tab + (c.r00 + col);   // element offsets below 2^31 (checked on the host)
-            const float v00 = __ldg(t), v01 = __ldg(t + c.dP), v10 = __ldg(t + c.dT), v11 = __ldg(t + c.dT + c.dP);
-            return c.kc + (c.w00 * v00 + c.w01 * v01 + c.w10 * v10 + c.w11 * v11);
+    for (int q = 0; q < NMU; ++q) I[q] = make_float2(0.f, 0.f);
+        float2 mu[NMU], rmu[NMU];   // per direction mu and 1/mu
+        const float2 nl2 = dup2(-1.4426950408889634f);   // e^{-x} = 2^{x * (-log2 e)}
+#pragma unroll
+        for (int q = 0; q < NMU; ++q) {
+            const float m = q < a.n_mu ? a.mu[q] : 1.f, r = 1.f / m;
+            mu[q] = dup2(m);
+            rmu[q] = dup2(r);
+        }
+        const int np = (a.K + 1) >> 1;
+        const float2* __restrict__ tab = a.tab + (size_t)s * np + (k0 >> 1) + pr;
+        const float2* __restrict__ Sp = reinterpret_cast<const float2*>(Sb) + pr;   // depth d: Sp[d * pairs]
+        // a depth's four table values (offsets below 2^31, checked on the host), and its opacity from them
+        auto load = [&](int d, float2 (&v)[4]) {
+            const int r = cell[d].r00, dT = cell[d].dT, dP = cell[d].dP;
+            v[0] = __ldg(tab + r);
+            v[1] = __ldg(tab + r + dP);
+            v[2] = __ldg(tab + r + dT);
+            v[3] = __ldg(tab + r + dT + dP);
         };
+        auto kappa = [&](int d, const float2 (&v)[4]) -> float2 {
+            const DepthCell& c = cell[d];
+            float2 k = ffma2(dup2(c.w00), v[0], dup2(c.kc));
+            k = ffma2(dup2(c.w01), v[1], k);
+            k = ffma2(dup2(c.w10), v[2], k);
+            return ffma2(dup2(c.w11), v[3], k);
+        };
+        const float2 one = dup2(1.f), minus = dup2(-1.f);
         const int D = a.D;
-        float k_hi = kappa(D - 1), k_lo = kappa(D - 2);
-        float dtau = 0.5f * (k_lo + k_hi) * (cell[D - 1].m - cell[D - 2].m);
-        const float dS = (S[D - 1] - S[D - 2]) / dtau;
+        float2 v[4];
+        load(D - 1, v);
+        float2 k_hi = kappa(D - 1, v);
+        load(D - 2, v);
+        float2 k_lo = kappa(D - 2, v);
+        float2 dtau = fmul2(fadd2(k_lo, k_hi), dup2(0.5f * (cell[D - 1].m - cell[D - 2].m)));
+        float2 S_hi = Sp[(D - 1) * pairs], Sd = Sp[(D - 2) * pairs];
+        {
+            const float2 dS = make_float2((S_hi.x - Sd.x) / dtau.x, (S_hi.y - Sd.y) / dtau.y);
 #pragma unroll
-        for (int q = 0; q < NMU; ++q) I[q] = fmaf(mu[q], dS, S[D - 1]);
+            for (int q = 0; q < NMU; ++q) I[q] = ffma2(mu[q], dS, S_hi);
+        }
         for (int d = D - 2;; --d) {
-            // layer d .. d+1 of optical thickness dtau; per direction x = dtau / mu:
-            //   I <- I e^{-x} + S_d (1 - e^{-x}) + (S_{d+1} - S_d) (1 - e^{-x}(1 + x)) / x,
-            // the last two factors by their Taylor series below x = 0.1 (no cancellation)
-            const float Sd = S[d], dSl = S[d + 1] - S[d];
-            const float rdt = rcp_fast(dtau);
+            if (d > 0) load(d - 1, v);   // in flight during the layer's directions
+            // layer d .. d+1 of optical thickness dtau; per direction x = dtau / mu, e = e^{-x}:
+            //   I <- I e + S_d (1 - e) + dS (1 - e(1 + x)) / x,  dS = S_{d+1} - S_d.
+            // With B = mu dS / dtau it is S_d + B + e (I - S_{d+1} - B), five operations; its rounding
+            // error is the weight's own, 2^-24 dS / x.  Below x = 0.1 instead
+            //   I <- I + x (P (S_d - I) + Q dS),  P = (1 - e) / x,  Q = (1 - e(1 + x)) / x^2,
+            // P and Q cubics through the four Chebyshev nodes of [0, 0.1] (1.4e-8 and 2.4e-8 off at
+            // most, measured on 2001 points with the coefficients as they stand here).
+            const float2 dSl = ffma2(Sd, minus, S_hi);
+            const float2 G = fmul2(dSl, make_float2(rcp_fast(dtau.x), rcp_fast(dtau.y)));
 #pragma unroll
             for (int q = 0; q < NMU; ++q) {
-                const float x = dtau * rmu[q];
-                const float e = ex2_fast(dtau * nl2[q]);
-                float ome, wl;
-                layer_weights(x, e, mu[q] * rdt, &ome, &wl);
-                I[q] = fmaf(I[q], e, fmaf(Sd, ome, dSl * wl));
+                const float2 x = fmul2(dtau, rmu[q]);
+                const bool tx = x.x < 0.1f, ty = x.y < 0.1f;
+                float2 r;
+                if (!(tx && ty)) {
+                    const float2 h = fmul2(x, nl2);
+                    const float2 e = make_float2(ex2_fast(h.x), ex2_fast(h.y));
+                    const float2 B = fmul2(mu[q], G);
+                    r = ffma2(e, ffma2(fadd2(S_hi, B), minus, I[q]), fadd2(Sd, B));
+                }
+                if (tx || ty) {
+                    // (not packed: an instruction's immediate operand holds the coefficient)
+                    auto cubic = [](float y, float c3, float c2, float c1, float c0) {
+                        return fmaf(y, fmaf(y, fmaf(y, c3, c2), c1), c0);
+                    };
+                    const float2 P = make_float2(cubic(x.x, -0.04003755832f, 0.1665655674f, -0.4999979837f, 1.f),
+                                                 cubic(x.y, -0.04003755832f, 0.1665655674f, -0.4999979837f, 1.f));
+                    const float2 Q = make_float2(cubic(x.x, -0.03197662605f, 0.1249158226f, -0.3333316547f, 0.5f),
+                                                 cubic(x.y, -0.03197662605f, 0.1249158226f, -0.3333316547f, 0.5f));
+                    const float2 t = ffma2(x, ffma2(P, ffma2(I[q], minus, Sd), fmul2(Q, dSl)), I[q]);
+                    r = make_float2(tx ? t.x : r.x, ty ? t.y : r.y);
+                }
+                I[q] = r;
             }
             if (d == 0) break;
             k_hi = k_lo;
-            k_lo = kappa(d - 1);
-            dtau = 0.5f * (k_lo + k_hi) * (cell[d].m - cell[d - 1].m);
+            k_lo = kappa(d - 1, v);
+            dtau = fmul2(fadd2(k_lo, k_hi), dup2(0.5f * (cell[d].m - cell[d - 1].m)));
+            S_hi = Sd;
+            Sd = Sp[(d - 1) * pairs];
         }
-        const float tau0 = k_lo * cell[0].m;
-        const float ws = (float)a.w[s];
+        const float2 tau0 = fmul2(k_lo, dup2(cell[0].m));
+        const float2 ws = dup2((float)a.w[s]);
 #pragma unroll
         for (int q = 0; q < NMU; ++q) {
-            const float e = ex2_fast(tau0 * nl2[q]);
-            I[q] = ws * fmaf(I[q], e, S[0] * (1.f - e));
+            const float2 h = fmul2(fmul2(tau0, rmu[q]), nl2);
+            const float2 e = make_float2(ex2_fast(h.x), ex2_fast(h.y));
+            I[q] = fmul2(ws, ffma2(I[q], e, fmul2(Sd, ffma2(e, minus, one))));
+            part[(s * a.kb + 2 * pr) * NMU + q] = I[q].x;
+            part[(s * a.kb + 2 * pr + 1) * NMU + q] = I[q].y;
         }
     }
-#pragma unroll
-    for (int q = 0; q < NMU; ++q) part[tid * NMU + q] = I[q];
     __syncthreads();
     // sum over the sub-bins in order
     const bool bad = a.bad[ray] != 0;
-    for (int i = tid; i < a.kb * a.n_mu; i += kBinThreads) {
+    for (int i = tid; i < a.kb * a.n_mu; i += blockDim.x) {
         const int b = i / a.n_mu, q = i - b * a.n_mu, kk = k0 + b;
         if (kk >= a.K) continue;
         float acc = 0.f;
-        for (int t = 0; t < a.ns; ++t) acc += part[(b * a.ns + t) * NMU + q];
+        for (int t = 0; t < a.ns; ++t) acc += part[(t * a.kb + b) * NMU + q];
         a.out[((size_t)ray * a.n_mu + q) * a.K + kk] = bad ? __int_as_float(0x7fc00000) : acc;
     }
     if (tid == 0 && a.status && blockIdx.x == 0) a.status[ray] = bad ? 1 : 0;
@@ -415,10 +488,9 @@ extern "C" int synth_spectrum(mpsa_ctx* ctx, const mpsa_atmos* atm, const mpsa_l
 namespace mpsa {
 namespace {
 
-constexpr int kBinMaxKb = 32;
 constexpr size_t kBinSmemMax =
     (size_t)kMaxDepth * sizeof(DepthCell) + (size_t)kBinMaxKb * kMaxDepth * sizeof(float) +
-    (size_t)kBinThreads * kMaxMu * sizeof(float);
+    (size_t)kBinCols * kMaxMu * sizeof(float);
 
 template <int NMU>
 int bin_launch(const BinArgs& a, int n_rays, cudaStream_t st) {
@@ -431,9 +503,9 @@ int bin_launch(const BinArgs& a, int n_rays, cudaStream_t st) {
         attr_set |= 1u << (dev & 31);
     }
     const size_t smem = (size_t)a.D * sizeof(DepthCell) + (size_t)a.kb * a.D * sizeof(float) +
-                        (size_t)kBinThreads * NMU * sizeof(float);
+                        (size_t)kBinCols * NMU * sizeof(float);
     const dim3 grid((a.K + a.kb - 1) / a.kb, n_rays);
-    k_bin_intensity<NMU><<<grid, kBinThreads, smem, st>>>(a);
+    k_bin_intensity<NMU><<<grid, (a.ns * (a.kb / 2) + 31) / 32 * 32, smem, st>>>(a);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
 }
@@ -482,7 +554,7 @@ extern "C" int odf_intensity(mpsa_ctx* ctx, const mpsa_odf_table* tab, int32_t n
     MPSA_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
     Scratch sc(st, ctx->pool);
-    const size_t n_tab = (size_t)tab->nT * tab->nP * K * ns, n_cells = (size_t)n_rays * n_depth;
+    const size_t n_tab = (size_t)tab->nT * tab->nP * ((K + 1) & ~1) * ns, n_cells = (size_t)n_rays * n_depth;
     double *dlt, *dlp, *dw;
     float *dmu, *dtab;
     float3* dpk;
@@ -507,14 +579,16 @@ extern "C" int odf_intensity(mpsa_ctx* ctx, const mpsa_odf_table* tab, int32_t n
     MPSA_CUDA_TRY(cudaMemcpyAsync(dw, tab->widths, ns * sizeof(double), cudaMemcpyHostToDevice, st));
     MPSA_CUDA_TRY(cudaMemcpyAsync(dmu, hmu.data(), n_mu * sizeof(float), cudaMemcpyHostToDevice, st));
     MPSA_CUDA_TRY(cudaMemsetAsync(dbad, 0, n_rays * sizeof(int), st));
-    k_bin_table<<<(unsigned)std::min<size_t>((n_tab + 255) / 256, 4096), 256, 0, st>>>(tab->odf, dtab, n_tab);
+    const int rows = tab->nT * tab->nP;
+    const long long parts = (long long)rows * ((K + kTabBins) / kTabBins);
+    k_bin_table<<<(unsigned)std::min<long long>(parts, 4096), 256, 0, st>>>(tab->odf, dtab, rows, K, ns);
     MPSA_CUDA_TRY(cudaGetLastError());
     BinCellArgs ca;
     ca.nT = tab->nT;
     ca.nP = tab->nP;
     ca.D = n_depth;
     ca.n_rays = n_rays;
-    ca.row_stride = K * ns;
+    ca.row_stride = (K + 1) / 2 * ns;
     ca.lt = dlt;
     ca.lp = dlp;
     ca.kc = tab->kappa_c;
@@ -530,8 +604,8 @@ extern "C" int odf_intensity(mpsa_ctx* ctx, const mpsa_odf_table* tab, int32_t n
     a.ns = ns;
     a.D = n_depth;
     a.n_mu = n_mu;
-    a.kb = std::max(1, std::min(kBinThreads / ns, kBinMaxKb));
-    a.tab = dtab;
+    a.kb = std::min(kBinCols / ns, kBinMaxKb) & ~1;   // even, at least 12 (ns <= 32)
+    a.tab = reinterpret_cast<const float2*>(dtab);
     a.pk = dpk;
     a.w = dw;
     a.mu = dmu;

@@ -70,6 +70,20 @@ def test_parity_shapes(n_mu, ns):
         assert ok, (r, rel)
 
 
+@pytest.mark.parametrize("K", [1, 2, 65])
+@pytest.mark.parametrize("ns", [1, 5, 32])
+def test_parity_bin_counts(K, ns):
+    """The kernel works on pairs of bins in chunks of 12 to 64: a lone bin, one pair, one bin past a chunk."""
+    lt, lp, odf, kc, lam = wl.odf_table_synthetic(3, 4, K, ns, seed=50 + K + ns)
+    w = np.full(ns, 1.0 / ns)
+    m, T, P = wl.ray_atmospheres(2, 31, seed=51)
+    g = run_gpu(lt, lp, odf, kc, lam, w, m, T, P, MUS)
+    for r in range(2):
+        o = oracle(lt, lp, odf, kc, lam, w, m[r], T[r], P[r], MUS)
+        ok, rel = close(g[r], o)
+        assert ok, (r, rel)
+
+
 def test_isothermal_is_planck():
     lt, lp, odf, kc, lam = wl.odf_table_synthetic(5, 4, 33, 12, seed=35)
     D = 50
