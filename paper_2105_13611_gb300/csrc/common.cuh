@@ -4,8 +4,10 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/mpsa.h"
@@ -76,6 +78,43 @@ struct Scratch {
     }
     ~Scratch() {
         for (void* p : ptrs) cudaFreeAsync(p, stream);
+    }
+};
+
+// The arrays of one call in one scratch block: add() each, then take() allocates the block and sets
+// the pointers.  An allocation and its release cost the host about a microsecond each, and a call took
+// 26 to 36 of them: one row of 40 lines 137 us, 122 us with one block and two launches less; eight
+// spectrum requests on eight streams 15.1 ms, 12.9 ms.
+struct ScratchBlock {
+    std::vector<std::pair<void*, size_t>> at;   // address of the pointer, offset in the block
+    size_t bytes = 0;
+    template <class T>
+    int add(T** p, size_t n) {
+        at.emplace_back(p, bytes);
+        bytes += (n * sizeof(T) + 16 + 255) & ~(size_t)255;
+        return MPSA_OK;
+    }
+    int take(Scratch& sc) {
+        char* base;
+        const int r = sc.alloc(&base, bytes);
+        if (r) return r;
+        for (auto& a : at) {
+            void* const q = base + a.second;
+            memcpy(a.first, &q, sizeof q);
+        }
+        return MPSA_OK;
+    }
+};
+
+// Small host arrays that go to the device in one copy: add() returns the offset in bytes.
+struct HostPack {
+    std::vector<char> data;
+    template <class T>
+    size_t add(const T* p, size_t n) {
+        const size_t off = (data.size() + 15) & ~(size_t)15;
+        data.resize(off + n * sizeof(T));
+        memcpy(data.data() + off, p, n * sizeof(T));
+        return off;
     }
 };
 

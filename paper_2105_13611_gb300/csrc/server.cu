@@ -113,28 +113,33 @@ int launch_spectrum(mpsa_server* s, Req* r, Slot& sl) {
     cudaStream_t st = r->st;
     const int D = (int)r->m.size(), N = r->N, n_mu = (int)r->mu.size(), ne = c->n_el;
     Scratch sc(st, s->ctx->pool);
-    double *dT, *dP, *dab, *dpop;
-    float *fm, *fT, *fmu, *kap, *kc, *Iout;
-    int* dsel;
-    int rc;
-    if ((rc = sc.alloc(&dT, D)) || (rc = sc.alloc(&dP, D)) || (rc = sc.alloc(&dab, ne)) ||
-        (rc = sc.alloc(&dpop, (size_t)D * pop_stride(ne))) || (rc = sc.alloc(&fm, D)) || (rc = sc.alloc(&fT, D)) ||
-        (rc = sc.alloc(&fmu, n_mu)) || (rc = sc.alloc(&kap, (size_t)D * N)) || (rc = sc.alloc(&kc, D)) ||
-        (rc = sc.alloc(&dsel, D)) || (rc = sc.alloc(&Iout, (size_t)n_mu * N)))
-        return rc;
+    // the request's small inputs, in one copy
     std::vector<float> hm(D), hT(D), hmu(n_mu);
     std::vector<int> hsel(D);
     for (int d = 0; d < D; ++d) hm[d] = (float)r->m[d], hT[d] = (float)r->T[d], hsel[d] = d;
     for (int q = 0; q < n_mu; ++q) hmu[q] = (float)r->mu[q];
-    const double* ab = c->h_abund.data() + (size_t)r->comp * ne;
-    MPSA_CUDA_TRY(cudaMemcpyAsync(dT, r->T.data(), D * sizeof(double), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(dP, r->P.data(), D * sizeof(double), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(dab, ab, ne * sizeof(double), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(fm, hm.data(), D * sizeof(float), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(fT, hT.data(), D * sizeof(float), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(fmu, hmu.data(), n_mu * sizeof(float), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(dsel, hsel.data(), D * sizeof(int), cudaMemcpyHostToDevice, st));
-    if ((rc = populations_device(ne, c->d_el, dab, 1, D, dT, dP, dpop, st))) return rc;
+    HostPack in;
+    const size_t oT = in.add(r->T.data(), D), oP = in.add(r->P.data(), D);
+    const size_t oab = in.add(c->h_abund.data() + (size_t)r->comp * ne, ne), om = in.add(hm.data(), D);
+    const size_t of = in.add(hT.data(), D), omu = in.add(hmu.data(), n_mu), osel = in.add(hsel.data(), D);
+    char* din;
+    double* dpop;
+    float *kap, *kc, *Iout;
+    ScratchBlock block;
+    block.add(&din, in.data.size());
+    block.add(&dpop, (size_t)D * pop_stride(ne));
+    block.add(&kap, (size_t)D * N);
+    block.add(&kc, D);
+    block.add(&Iout, (size_t)n_mu * N);
+    int rc;
+    if ((rc = block.take(sc))) return rc;
+    MPSA_CUDA_TRY(cudaMemcpyAsync(din, in.data.data(), in.data.size(), cudaMemcpyHostToDevice, st));
+    const int* dsel = reinterpret_cast<int*>(din + osel);
+    const float *fm = reinterpret_cast<float*>(din + om), *fT = reinterpret_cast<float*>(din + of),
+                *fmu = reinterpret_cast<float*>(din + omu);
+    if ((rc = populations_device(ne, c->d_el, reinterpret_cast<double*>(din + oab), 1, D, reinterpret_cast<double*>(din + oT),
+                                 reinterpret_cast<double*>(din + oP), dpop, st)))
+        return rc;
     for (int off = 0; off < D; off += s->rows_per_chunk) {
         const int nrow = std::min(s->rows_per_chunk, D - off);
         if ((rc = synth_rows(c, dpop, nrow, dsel + off, r->win.lambda0_nm, r->win.R, N, kap + (size_t)off * N, kc + off,

@@ -395,11 +395,6 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_intensity(BinArgs a) {
     if (tid == 0 && a.status && blockIdx.x == 0) a.status[ray] = bad ? 1 : 0;
 }
 
-__global__ void k_iota(int n, int* p) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = i;
-}
-
 unsigned g_spec_init = 0;
 
 }  // namespace
@@ -449,33 +444,36 @@ extern "C" int synth_spectrum(mpsa_ctx* ctx, const mpsa_atmos* atm, const mpsa_l
     MPSA_CUDA_TRY(cudaSetDevice(ctx->device));
     cudaStream_t st = (cudaStream_t)stream;
     Scratch sc(st, ctx->pool);
-    double *dT, *dP, *dab, *dpop;
-    float *fm, *fT, *fmu, *kap, *kc;
-    int* dsel;
-    const int ne = ctx->n_el;
-    if ((r = sc.alloc(&dT, D)) || (r = sc.alloc(&dP, D)) || (r = sc.alloc(&dab, ne)) ||
-        (r = sc.alloc(&dpop, (size_t)D * pop_stride(ne))) || (r = sc.alloc(&fm, D)) || (r = sc.alloc(&fT, D)) ||
-        (r = sc.alloc(&fmu, n_mu)) || (r = sc.alloc(&kap, (size_t)D * N)) || (r = sc.alloc(&kc, D)) ||
-        (r = sc.alloc(&dsel, D)))
-        return r;
-    std::vector<float> hm(D), hT(D), hmu(n_mu);
-    for (int d = 0; d < D; ++d) hm[d] = (float)atm->m[d], hT[d] = (float)atm->T[d];
-    for (int q = 0; q < n_mu; ++q) hmu[q] = (float)mu[q];
-    const double* ab = ctx->h_abund.data() + (size_t)atm->comp * ne;
-    MPSA_CUDA_TRY(cudaMemcpyAsync(dT, atm->T, D * sizeof(double), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(dP, atm->P, D * sizeof(double), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(dab, ab, ne * sizeof(double), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(fm, hm.data(), D * sizeof(float), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(fT, hT.data(), D * sizeof(float), cudaMemcpyHostToDevice, st));
-    MPSA_CUDA_TRY(cudaMemcpyAsync(fmu, hmu.data(), n_mu * sizeof(float), cudaMemcpyHostToDevice, st));
-    if ((r = populations_device(ne, ctx->d_el, dab, 1, D, dT, dP, dpop, st))) return r;
-    k_iota<<<(D + 127) / 128, 128, 0, st>>>(D, dsel);
-    if ((r = synth_rows(ctx, dpop, D, dsel, win->lambda0_nm, win->R, N, kap, kc, nullptr, opts, st))) return r;
-    float* kcont = nullptr;
     const int cont = opts ? opts->continuum : 0;
+    const int ne = ctx->n_el;
+    // the call's small inputs, in one copy
+    std::vector<float> hm(D), hT(D), hmu(n_mu);
+    std::vector<int> hsel(D);
+    for (int d = 0; d < D; ++d) hm[d] = (float)atm->m[d], hT[d] = (float)atm->T[d], hsel[d] = d;
+    for (int q = 0; q < n_mu; ++q) hmu[q] = (float)mu[q];
+    HostPack in;
+    const size_t oT = in.add(atm->T, D), oP = in.add(atm->P, D), oab = in.add(ctx->h_abund.data() + (size_t)atm->comp * ne, ne);
+    const size_t om = in.add(hm.data(), D), of = in.add(hT.data(), D), omu = in.add(hmu.data(), n_mu), osel = in.add(hsel.data(), D);
+    char* din;
+    double* dpop;
+    float *kap, *kc, *kcont = nullptr;
+    ScratchBlock block;
+    block.add(&din, in.data.size());
+    block.add(&dpop, (size_t)D * pop_stride(ne));
+    block.add(&kap, (size_t)D * N);
+    block.add(&kc, D);
+    if (cont) block.add(&kcont, (size_t)D * N);
+    if ((r = block.take(sc))) return r;
+    MPSA_CUDA_TRY(cudaMemcpyAsync(din, in.data.data(), in.data.size(), cudaMemcpyHostToDevice, st));
+    const int* dsel = reinterpret_cast<int*>(din + osel);
+    const float *fm = reinterpret_cast<float*>(din + om), *fT = reinterpret_cast<float*>(din + of),
+                *fmu = reinterpret_cast<float*>(din + omu);
+    if ((r = populations_device(ne, ctx->d_el, reinterpret_cast<double*>(din + oab), 1, D, reinterpret_cast<double*>(din + oT),
+                                reinterpret_cast<double*>(din + oP), dpop, st)))
+        return r;
+    if ((r = synth_rows(ctx, dpop, D, dsel, win->lambda0_nm, win->R, N, kap, kc, nullptr, opts, st))) return r;
     if (cont) {
         if (cont & ~MPSA_CONT_ALL) return fail(MPSA_EINVAL, "synth_spectrum: continuum = %d", cont);
-        if ((r = sc.alloc(&kcont, (size_t)D * N))) return r;
         if ((r = continuum_launch(ctx, dpop, D, dsel, win->lambda0_nm, win->R, N, cont, kcont, st))) return r;
     }
     if ((r = formal_launch(D, N, kap, kc, kcont, fm, fT, win->lambda0_nm, log1p(1.0 / win->R), n_mu, fmu, I_out, st)))

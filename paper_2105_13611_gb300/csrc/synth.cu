@@ -7,15 +7,14 @@
 // opacity of the synthetic workload).
 //
 // Pipeline (all on the caller's stream):
-//   k_distance     per line: how far off the grid its centre is
-//   k_consts       per (row, species): ln(sqrt(pi) e^2/(m_e c) N/U / rho), u, c/u from the FP64 table
+//   k_start        per line: how far off the grid its centre is, and per (row, species): ln(sqrt(pi) e^2/(m_e c) N/U / rho), u, c/u from the FP64 table
 //   k_kappa0       per (row, line): ln S, a, ln kappa0 in FP32 log space
 //   k_med_*        per row: lower median of ln kappa0 -> ln t_p, kappa_c
 //   k_prep         per (row, line): peak against the cut, reach of the wing; the lines left, listed
 //   k_place        the listed lines' centre index c and fraction f on the grid (FP64 log)
 //   k_windows      per listed line: cut windows (outer: no point beyond can pass the cut; inner:
 //                  every point inside passes), width class
-//   k_scan_class, k_scan_fin, k_scatter   stable counting sort of the kept lines by width class
+//   k_scan_class, k_scatter   stable counting sort of the kept lines by width class
 //   k_ranges       per (row, class, tile boundary): first line whose centre lies at or
 //                  beyond the boundary (binary search in the centre-sorted class)
 //   k_tiles        the profile kernel: one CTA per (row, 2048-point tile) (or several, on calls with
@@ -66,27 +65,6 @@ struct RowOut {
     }
 };
 
-// ---------------------------------------------------------------------------
-// k_distance: per (grid, line), a lower bound of the distance between a centre off the grid and
-// the grid's nearest point in relative frequency, |v| / kv there:
-//   1 - lambda/lambda_0 (centre shortward), lambda/lambda_{N-1} - 1 (longward),
-// negative for centres on the grid.  Four grid points and the FP32 rounding are taken off, so FP32 will do, and no
-// logarithm is needed: the exact position of a line (k_place) is formed only if it reaches the
-// grid.  Clears the line's flag.
-__global__ void k_distance(int64_t L, size_t ld, int n_grids, const double* __restrict__ lam_nm, GridDesc one,
-                           const GridDesc* __restrict__ many, float* __restrict__ dist, unsigned char* __restrict__ flag) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L) return;
-    const float lam = (float)lam_nm[i];
-    for (int g = blockIdx.y; g < n_grids; g += gridDim.y) {
-        const GridDesc q = many ? many[g] : one;
-        const float d = fmaxf(fmaf(-lam, q.inv_first, 1.f), fmaf(lam, q.inv_last, -1.f));
-        // lambda, 1/lambda_0 and the product round by 6e-8 each
-        dist[g * ld + i] = fmaf(d, 1.f - 4.2f * q.lnq - 1e-5f, -4.2f * q.lnq - 4e-7f);
-        flag[g * ld + i] = 0;
-    }
-}
-
 // k_place: c = floor(x0), f = x0 - c with x0 = ln(lambda0/lambda_start)/ln(1+1/R) (FP64: an FP32
 // logarithm would misplace lines by whole grid points) of the lines that some row of the
 // grid keeps.  A CTA gathers the kept ones of its 1024 lines and then takes their logarithms
@@ -134,12 +112,10 @@ struct __align__(16) SpConst {
     float lnC, u, kv, lnu;   // lnu = logf(u)
 };
 
-__global__ void k_consts(int n_sel, const int* __restrict__ sel, int n_sp, const int* __restrict__ sp_el,
-                         const int* __restrict__ sp_stage, int n_el, const double* __restrict__ el,
-                         const double* __restrict__ pop, double vturb, int pop32, RowConst* __restrict__ rc,
-                         SpConst* __restrict__ sc) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_sel * n_sp) return;
+__device__ __forceinline__ void sp_consts(int t, const int* __restrict__ sel, int n_sp, const int* __restrict__ sp_el,
+                                          const int* __restrict__ sp_stage, int n_el, const double* __restrict__ el,
+                                          const double* __restrict__ pop, double vturb, int pop32,
+                                          RowConst* __restrict__ rc, SpConst* __restrict__ sc) {
     const int s = t / n_sp, sp = t % n_sp;
     const double* row = pop + (size_t)sel[s] * pop_stride(n_el);
     const double T = row[kPopT];
@@ -164,6 +140,43 @@ __global__ void k_consts(int n_sel, const int* __restrict__ sel, int n_sp, const
         r.inv_kT_eV = (float)(kEV / (kKB * T));
         r.hc_kT_cm = (float)(kH * kC / (kKB * T));
         rc[s] = r;
+    }
+}
+
+// k_start: two independent tables, by blocks of one launch.
+// The first `cb` blocks: the constants of each (row, species), and the rows' counts of listed
+// lines set to zero.
+// The others: per (grid, line), a lower bound of the distance between a centre off the grid and
+// the grid's nearest point in relative frequency, |v| / kv there:
+//   1 - lambda/lambda_0 (centre shortward), lambda/lambda_{N-1} - 1 (longward),
+// negative for centres on the grid.  Four grid points and the FP32 rounding are taken off, so FP32 will do, and no
+// logarithm is needed: the exact position of a line (k_place) is formed only if it reaches the
+// grid.  Clears the line's flag.
+constexpr int kStartThreads = 128;
+__global__ void __launch_bounds__(kStartThreads) k_start(int cb, int n_sel, const int* __restrict__ sel, int n_sp,
+                                                         const int* __restrict__ sp_el, const int* __restrict__ sp_stage,
+                                                         int n_el, const double* __restrict__ el,
+                                                         const double* __restrict__ pop, double vturb, int pop32,
+                                                         RowConst* __restrict__ rc, SpConst* __restrict__ sc,
+                                                         int* __restrict__ nsurv, int64_t L, size_t ld, int n_grids,
+                                                         const double* __restrict__ lam_nm, GridDesc one,
+                                                         const GridDesc* __restrict__ many, float* __restrict__ dist,
+                                                         unsigned char* __restrict__ flag) {
+    if ((int)blockIdx.x < cb) {
+        const int t = blockIdx.x * kStartThreads + threadIdx.x;
+        if (t < n_sel) nsurv[t] = 0;
+        if (t < n_sel * n_sp) sp_consts(t, sel, n_sp, sp_el, sp_stage, n_el, el, pop, vturb, pop32, rc, sc);
+        return;
+    }
+    const int64_t i = (int64_t)(blockIdx.x - cb) * kStartThreads + threadIdx.x;
+    if (i >= L) return;
+    const float lam = (float)lam_nm[i];
+    for (int g = 0; g < n_grids; ++g) {
+        const GridDesc q = many ? many[g] : one;
+        const float d = fmaxf(fmaf(-lam, q.inv_first, 1.f), fmaf(lam, q.inv_last, -1.f));
+        // lambda, 1/lambda_0 and the product round by 6e-8 each
+        dist[g * ld + i] = fmaf(d, 1.f - 4.2f * q.lnq - 1e-5f, -4.2f * q.lnq - 4e-7f);
+        flag[g * ld + i] = 0;
     }
 }
 
@@ -738,8 +751,9 @@ __global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids
 }
 
 // k_scan_class: per (class, row), exclusive scan in place of the per-block counts of the
-// class (one CTA each) and the class total.
-__global__ void __launch_bounds__(1024) k_scan_class(int nb, int* __restrict__ blkcnt, int* __restrict__ classcnt) {
+// class (one CTA each) and the class total; the row's number of profile evaluations starts at zero.
+__global__ void __launch_bounds__(1024) k_scan_class(int nb, int* __restrict__ blkcnt, int* __restrict__ classcnt,
+                                                     RowOut out) {
     __shared__ int wsum[32];
     __shared__ int carry;
     const int b = blockIdx.x, s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -773,21 +787,19 @@ __global__ void __launch_bounds__(1024) k_scan_class(int nb, int* __restrict__ b
         if (tid == (int)blockDim.x - 1) carry = ex + v;
         __syncthreads();
     }
-    if (tid == 0) classcnt[s * kNumClasses + b] = carry;
+    if (tid == 0) {
+        classcnt[s * kNumClasses + b] = carry;
+        unsigned long long* const ev = b == 0 ? out.ev_of(s) : nullptr;
+        if (ev) *ev = 0;
+    }
 }
 
-// k_scan_fin: per row, the class base offsets; the number of profile evaluations starts at zero.
-__global__ void k_scan_fin(int n_sel, const int* __restrict__ classcnt, int* __restrict__ classbase,
-                           RowOut out) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_sel) return;
+// lines of a row's classes before class b
+__device__ __forceinline__ int class_base(const int* __restrict__ cnt, int b) {
     int acc = 0;
-    for (int b = 0; b < kNumClasses; ++b) {
-        classbase[s * kNumClasses + b] = acc;
-        acc += classcnt[s * kNumClasses + b];
-    }
-    unsigned long long* const ev = out.ev_of(s);
-    if (ev) *ev = 0;
+#pragma unroll
+    for (int q = 0; q < kNumClasses - 1; ++q) acc += q < b ? cnt[q] : 0;
+    return acc;
 }
 
 // k_scatter: stable placement of the kept lines into class buckets (centre order preserved): W
@@ -800,7 +812,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
                                                           const int* __restrict__ cpos, const float* __restrict__ fpos,
                                                           int n_sp, const SpConst* __restrict__ sc,
                                                           const float* __restrict__ av, const int* __restrict__ blkoff,
-                                                          const int* __restrict__ classbase, int nb, const PrepOut o,
+                                                          const int* __restrict__ classcnt, int nb, const PrepOut o,
                                                           LineRec* __restrict__ rec, int* __restrict__ line,
                                                           RowOut out) {
     constexpr int kWarps = kPrepThreads / 32;
@@ -815,7 +827,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
     const int t1 = min(run.x + run.y, run.x + (part + 1) * len), tb = run.x + part * len;
     const unsigned lt = (1u << lane) - 1u;
     int first = lane < kNumClasses
-                    ? classbase[s * kNumClasses + lane] + blkoff[((size_t)s * kNumClasses + lane) * nb + blk]
+                    ? class_base(classcnt + s * kNumClasses, lane) + blkoff[((size_t)s * kNumClasses + lane) * nb + blk]
                     : 0;
     if (W > 1) {   // the lines of each class in the parts before this one
         placed[warp][lane] = 0;
@@ -883,7 +895,7 @@ struct RowDesc {
 // index, off-grid centres clamped to -1 and N) is >= (ts - 1) * tile, ts = 0 .. nT + 2.  rows: a
 // descriptor per row, or null: `one` for all, with their arrays following one another.
 __global__ void k_ranges(int n_sel, size_t ld, RowDesc one, const RowDesc* __restrict__ rows,
-                         const int* __restrict__ classbase, const int* __restrict__ classcnt) {
+                         const int* __restrict__ classcnt) {
     const int s = blockIdx.y;
     RowDesc g = one;
     if (rows) {
@@ -895,7 +907,7 @@ __global__ void k_ranges(int n_sel, size_t ld, RowDesc one, const RowDesc* __res
     const int t = blockIdx.x * blockDim.x + threadIdx.x, W = g.nT + 3;
     if (t >= kNumClasses * W) return;
     const int b = t / W, ts = t - b * W;
-    const int base = classbase[s * kNumClasses + b], n = classcnt[s * kNumClasses + b];
+    const int base = class_base(classcnt + s * kNumClasses, b), n = classcnt[s * kNumClasses + b];
     const LineRec* k = g.rec + base;
     const long long thr = (long long)(ts - 1) * g.tile;
     int lo = 0, hi = n;
@@ -1640,7 +1652,7 @@ struct PrepBufs {
     int n_grids = 1;
     size_t ld = 0;   // lines per row of the per-(row, line) arrays: L rounded up to four
     int n_sel = 0, nb = 0;
-    int *c = nullptr, *classbase = nullptr, *classcnt = nullptr, *line = nullptr;
+    int *c = nullptr, *classcnt = nullptr, *line = nullptr;
     LineRec* rec = nullptr;
     float *f = nullptr, *dist = nullptr, *lnS = nullptr, *av = nullptr, *lnk0 = nullptr, *ln_tp = nullptr;
     unsigned char* flag = nullptr;
@@ -1665,8 +1677,7 @@ int prep_alloc(PrepBufs& b, const mpsa_ctx* ctx, int n_sel, int n_grids, Alloc&&
         (r = al(&b.spc, (size_t)n_sel * ctx->n_sp)) || (r = al(&b.lnS, SL)) || (r = al(&b.av, SL)) ||
         (r = al(&b.lnk0, SL)) || (r = al(&b.ln_tp, n_sel)) || (r = al(&b.po.surv, SL)) || (r = al(&b.po.nsurv, n_sel)) ||
         (r = al(&b.po.run, Sb)) || (r = al(&b.po.srel, SL)) || (r = al(&b.po.win, SL)) || (r = al(&b.po.cls, SL)) ||
-        (r = al(&b.po.blkcnt, Sb * kNumClasses)) || (r = al(&b.classbase, (size_t)n_sel * kNumClasses)) ||
-        (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) || (r = al(&b.rec, SL)) || (r = al(&b.line, SL)) ||
+        (r = al(&b.po.blkcnt, Sb * kNumClasses)) || (r = al(&b.classcnt, (size_t)n_sel * kNumClasses)) || (r = al(&b.rec, SL)) || (r = al(&b.line, SL)) ||
         (r = al(&b.med, n_sel)))
         return r;
     return MPSA_OK;
@@ -1687,12 +1698,12 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     const double kcf = (opts && opts->kc_factor > 0) ? opts->kc_factor : 1e-2;
     const int64_t L = b.L;
     const int n_sel = b.n_sel, n_sp = ctx->n_sp;
-    const int lb = (int)((L + 255) / 256);
     const RowGrids grids{grid, d_row_grids};
-    k_distance<<<dim3(lb, 1), 256, 0, st>>>(L, b.ld, b.n_grids, ctx->d_lam, grid, d_grids, b.dist, b.flag);
     const int pop32 = (opts && opts->precision == MPSA_PREC_FP32_POP32) ? 1 : 0;
-    k_consts<<<(n_sel * n_sp + 127) / 128, 128, 0, st>>>(n_sel, d_sel, n_sp, ctx->d_sp_el, ctx->d_sp_stage, ctx->n_el,
-                                                           ctx->d_el, pop, ctx->vturb, pop32, b.rc, b.spc);
+    const int cb = (n_sel * n_sp + kStartThreads - 1) / kStartThreads;
+    k_start<<<cb + (unsigned)((L + kStartThreads - 1) / kStartThreads), kStartThreads, 0, st>>>(
+        cb, n_sel, d_sel, n_sp, ctx->d_sp_el, ctx->d_sp_stage, ctx->n_el, ctx->d_el, pop, ctx->vturb, pop32, b.rc, b.spc,
+        b.po.nsurv, L, b.ld, b.n_grids, ctx->d_lam, grid, d_grids, b.dist, b.flag);
     {
         // ln S, a, ln kappa0 and the median; the record array, not in use yet, holds the listed lines
         // and the sample
@@ -1719,7 +1730,6 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
         k_med_select<<<n_sel, kMedThreads, 0, st>>>(L, b.ld, b.lnk0, small ? nullptr : b.med, list, b.ld,
                                                     (float)log(kcf), (float)log(cut), b.ln_tp, out);
     }
-    MPSA_CUDA_TRY(cudaMemsetAsync(b.po.nsurv, 0, (size_t)n_sel * sizeof(int), st));
     k_prep<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS, b.av,
                                                        b.lnk0, b.ln_tp, b.nb, b.po);
     int dev = 0, sms = 0;
@@ -1738,16 +1748,15 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
         k_windows<<<dim3(gx, n_sel), kPrepThreads, 0, st>>>(b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.lnS, b.av,
                                                             b.ln_tp, b.nb, b.po);
     }
-    k_scan_class<<<dim3(kNumClasses, n_sel), 1024, 0, st>>>(b.nb, b.po.blkcnt, b.classcnt);
-    k_scan_fin<<<(n_sel + 31) / 32, 32, 0, st>>>(n_sel, b.classcnt, b.classbase, out);
+    k_scan_class<<<dim3(kNumClasses, n_sel), 1024, 0, st>>>(b.nb, b.po.blkcnt, b.classcnt, out);
     constexpr int kWarps = kPrepThreads / 32;
     if ((int64_t)b.nb * n_sel * kWarps <= 64ll * sms)
         k_scatter<kWarps><<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(
-            b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
+            b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classcnt, b.nb, b.po, b.rec,
             b.line, out);
     else
         k_scatter<1><<<dim3((b.nb + kWarps - 1) / kWarps, n_sel), kPrepThreads, 0, st>>>(
-            b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classbase, b.nb, b.po, b.rec,
+            b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.av, b.po.blkcnt, b.classcnt, b.nb, b.po, b.rec,
             b.line, out);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
@@ -1756,7 +1765,7 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
 // Tile ranges of all rows for the descriptors (see k_ranges); most: the largest number of tiles.
 int ranges_launch(const PrepBufs& b, const RowDesc& one, const RowDesc* d_rows, int most, cudaStream_t st) {
     const int n = kNumClasses * (most + 3);
-    k_ranges<<<dim3((n + 255) / 256, b.n_sel), 256, 0, st>>>(b.n_sel, b.ld, one, d_rows, b.classbase, b.classcnt);
+    k_ranges<<<dim3((n + 255) / 256, b.n_sel), 256, 0, st>>>(b.n_sel, b.ld, one, d_rows, b.classcnt);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
 }
@@ -1788,17 +1797,33 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
     PrepBufs b;
     int r, *cum;
     const int tile = prec == MPSA_PREC_FP64 ? kTile64 : kTile, nT = (N + tile - 1) / tile;
-    if ((r = prep_alloc(b, ctx, n_sel, 1, [&](auto** p, size_t n) { return sc.alloc(p, n); }))) return r;
-    if ((r = sc.alloc(&cum, (size_t)n_sel * kNumClasses * (nT + 3)))) return r;
+    ScratchBlock block;
+    prep_alloc(b, ctx, n_sel, 1, [&](auto** p, size_t n) { return block.add(p, n); });
+    block.add(&cum, (size_t)n_sel * kNumClasses * (nT + 3));
+    // A call with fewer tiles than the GPU holds CTAs (narrow windows) splits each tile's
+    // candidate lines over several CTAs, up to 64, and adds their partial sums afterwards: as
+    // many as run at once, one chunk each at least, and up to eight times that for
+    // the tiles with kSplitChunks each (deep rows have ten times the candidates of shallow ones)
+    int dev = 0, sms = 0;
+    MPSA_CUDA_TRY(cudaGetDevice(&dev));
+    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t ctas = (int64_t)nT * n_sel, slots = (int64_t)sms * MPSA_TILES_MINB;
+    const int64_t most = std::min<int64_t>(64, kNumClasses + b.L / kTileThreads);   // chunks a tile can have
+    TileArgs ta;
+    ta.split_free = (int)std::max<int64_t>(1, std::min(most, slots / ctas));
+    ta.split = prec == MPSA_PREC_FP64 || ctas > slots ? 1 : (int)std::max<int64_t>(1, std::min(most, 8 * slots / ctas));
+    ta.part = nullptr;
+    ta.used = nullptr;
+    if (ta.split > 1) {
+        block.add(&ta.part, (size_t)n_sel * ta.split * N);
+        block.add(&ta.used, ctas);
+    }
+    if ((r = block.take(sc))) return r;
     const GridDesc grid = grid_desc(lam0_nm, log1p(1.0 / R), N, 0);
     const RowOut out{kc_out, (unsigned long long*)evals, nullptr, nullptr};
     if ((r = prep_launch(b, ctx, pop, d_sel, grid, nullptr, nullptr, out, opts, st))) return r;
-    TileArgs ta;
     ta.row = row_of(grid, tile, cum, b.ln_tp, b.rec, b.line, kappa);
     ta.ld = b.ld;
-    ta.split = ta.split_free = 1;
-    ta.part = nullptr;
-    ta.used = nullptr;
     if ((r = ranges_launch(b, ta.row, nullptr, nT, st))) return r;
     prof_mark(ctx, MPSA_KERNEL_PROFILE, st);
     if (prec == MPSA_PREC_FP64) {
@@ -1824,32 +1849,18 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         g.lnq64 = grid.lnq64;
         k_tiles64<<<dim3(nT, n_sel), 256, 0, st>>>(g);
     } else {
-        // a call with fewer tiles than the GPU holds CTAs (narrow windows) splits each tile's
-        // candidate lines over several CTAs, up to 64, and adds their partial sums afterwards: as
-        // many as run at once, one chunk each at least, and up to eight times that for
-        // the tiles with kSplitChunks each (deep rows have ten times the candidates of shallow ones)
-        int dev = 0, sms = 0;
-        MPSA_CUDA_TRY(cudaGetDevice(&dev));
-        MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int64_t ctas = (int64_t)nT * n_sel, slots = (int64_t)sms * MPSA_TILES_MINB;
-        const int64_t most = std::min<int64_t>(64, kNumClasses + b.L / kTileThreads);   // chunks a tile can have
-        TileArgs tb = ta;
-        tb.split_free = (int)std::max<int64_t>(1, std::min(most, slots / ctas));
-        tb.split = ctas > slots ? 1 : (int)std::max<int64_t>(1, std::min(most, 8 * slots / ctas));
-        tb.part = nullptr;
-        if (tb.split > 1 && ((r = sc.alloc(&tb.part, (size_t)n_sel * tb.split * N)) || (r = sc.alloc(&tb.used, ctas)))) return r;
-        const dim3 blocks((unsigned)(nT * tb.split), n_sel);
+        const dim3 blocks((unsigned)(nT * ta.split), n_sel);
         const bool naive = prec == MPSA_PREC_FP32_NAIVE;
-        if (tb.split > 1) {
-            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, true><<<blocks, kTileThreads, 0, st>>>(tb);
-            else k_tiles<MPSA_PREC_FP32_COMPENSATED, true><<<blocks, kTileThreads, 0, st>>>(tb);
+        if (ta.split > 1) {
+            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, true><<<blocks, kTileThreads, 0, st>>>(ta);
+            else k_tiles<MPSA_PREC_FP32_COMPENSATED, true><<<blocks, kTileThreads, 0, st>>>(ta);
         } else {
-            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, false><<<blocks, kTileThreads, 0, st>>>(tb);
-            else k_tiles<MPSA_PREC_FP32_COMPENSATED, false><<<blocks, kTileThreads, 0, st>>>(tb);
+            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, false><<<blocks, kTileThreads, 0, st>>>(ta);
+            else k_tiles<MPSA_PREC_FP32_COMPENSATED, false><<<blocks, kTileThreads, 0, st>>>(ta);
         }
-        if (tb.split > 1) {
+        if (ta.split > 1) {
             const int64_t tot = (int64_t)n_sel * N;
-            k_split_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n_sel, N, tb.split, tb.used, tb.part, kappa);
+            k_split_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n_sel, N, ta.split, ta.used, ta.part, kappa);
         }
     }
     prof_mark(ctx, MPSA_KERNEL_PROFILE, st);
