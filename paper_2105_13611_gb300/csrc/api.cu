@@ -372,6 +372,7 @@ int load_linelist(mpsa_ctx* c, int32_t n_species, const int32_t* sp_el, const in
     c->h_sp_el.assign(sp_el, sp_el + n_species);
     c->h_sp_stage.assign(sp_stage, sp_stage + n_species);
     c->L = L;
+    c->log_span = log(src.lambda_nm[L - 1] / src.lambda_nm[0]);
     return MPSA_OK;
 }
 

@@ -137,6 +137,7 @@ struct mpsa_ctx {
     std::vector<int32_t> h_sp_el, h_sp_stage;
     // line list (device, ascending lambda)
     int64_t L = 0;
+    double log_span = 0;             // ln(last wavelength / first)
     double* d_lam = nullptr;
     float* d_loggf = nullptr;
     float* d_E = nullptr;

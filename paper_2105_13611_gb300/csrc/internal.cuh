@@ -15,9 +15,10 @@ int populations_device(int n_el, const double* d_el, const double* d_abund, int 
                        const double* d_T, const double* d_P, double* d_pop, cudaStream_t s);
 
 // Line-by-line opacity for rows d_sel of a population table onto the grid
-// (lam0_nm, R, N): kappa [n_sel][N], optional kappa_c [n_sel] and evaluation counts (synth.cu).
+// (lam0_nm, R, N): kappa [n_sel][N], optional kappa_c [n_sel] and evaluation counts; peers: calls that
+// share the GPU with this one on other streams (synth.cu).
 int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, double lam0_nm, double R, int N,
-               float* kappa, float* kc_out, int64_t* evals, const mpsa_synth_opts* opts, cudaStream_t st);
+               float* kappa, float* kc_out, int64_t* evals, const mpsa_synth_opts* opts, cudaStream_t st, int peers = 1);
 
 // Every species of the line list refers to an element of the table and to a stage that
 // element has (synth.cu).

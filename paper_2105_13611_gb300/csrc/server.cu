@@ -140,10 +140,12 @@ int launch_spectrum(mpsa_server* s, Req* r, Slot& sl) {
     if ((rc = populations_device(ne, c->d_el, reinterpret_cast<double*>(din + oab), 1, D, reinterpret_cast<double*>(din + oT),
                                  reinterpret_cast<double*>(din + oP), dpop, st)))
         return rc;
+    // every slot may hold a request: the chunks leave the others their part of the GPU (by the number of slots, not
+    // of requests in flight, on which the result would then depend)
     for (int off = 0; off < D; off += s->rows_per_chunk) {
         const int nrow = std::min(s->rows_per_chunk, D - off);
         if ((rc = synth_rows(c, dpop, nrow, dsel + off, r->win.lambda0_nm, r->win.R, N, kap + (size_t)off * N, kc + off,
-                             nullptr, nullptr, st)))
+                             nullptr, nullptr, st, (int)s->slots.size())))
             return rc;
     }
     if ((rc = formal_launch(D, N, kap, kc, nullptr, fm, fT, r->win.lambda0_nm, log1p(1.0 / r->win.R), n_mu, fmu, Iout,

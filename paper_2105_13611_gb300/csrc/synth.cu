@@ -935,16 +935,21 @@ __global__ void k_ranges(int n_sel, size_t ld, RowDesc one, const RowDesc* __res
 constexpr int kNodes = 12;
 // cos(i pi / 24): node k of a stretch is at (1 + x_k)/2 of its length, x_k = cos((2k + 1) pi / 24),
 // and T_m(x_k) = cos(m (2k + 1) pi / 24)
-__constant__ double c_cos24[48] = {
-    1.0, 0.99144486137381041, 0.96592582628906829, 0.92387953251128676, 0.86602540378443865, 0.79335334029123517,
-    0.70710678118654752, 0.60876142900872064, 0.5, 0.38268343236508977, 0.25881904510252076, 0.13052619222005159,
-    0.0, -0.13052619222005159, -0.25881904510252076, -0.38268343236508977, -0.5, -0.60876142900872064,
-    -0.70710678118654752, -0.79335334029123517, -0.86602540378443865, -0.92387953251128676, -0.96592582628906829,
-    -0.99144486137381041, -1.0, -0.99144486137381041, -0.96592582628906829, -0.92387953251128676,
-    -0.86602540378443865, -0.79335334029123517, -0.70710678118654752, -0.60876142900872064, -0.5,
-    -0.38268343236508977, -0.25881904510252076, -0.13052619222005159, 0.0, 0.13052619222005159, 0.25881904510252076,
-    0.38268343236508977, 0.5, 0.60876142900872064, 0.70710678118654752, 0.79335334029123517, 0.86602540378443865,
-    0.92387953251128676, 0.96592582628906829, 0.99144486137381041};
+__constant__ float c_cos24[48] = {
+    1.f, 0.991444886f, 0.965925813f, 0.923879504f, 0.866025388f, 0.793353319f, 0.707106769f, 0.60876143f,
+    0.5f, 0.382683426f, 0.258819044f, 0.130526185f, 0.f, -0.130526185f, -0.258819044f, -0.382683426f,
+    -0.5f, -0.60876143f, -0.707106769f, -0.793353319f, -0.866025388f, -0.923879504f, -0.965925813f, -0.991444886f,
+    -1.f, -0.991444886f, -0.965925813f, -0.923879504f, -0.866025388f, -0.793353319f, -0.707106769f, -0.60876143f,
+    -0.5f, -0.382683426f, -0.258819044f, -0.130526185f, 0.f, 0.130526185f, 0.258819044f, 0.382683426f,
+    0.5f, 0.60876143f, 0.707106769f, 0.793353319f, 0.866025388f, 0.923879504f, 0.965925813f, 0.991444886f};
+// and what FP32 rounds off
+__constant__ float c_cos24_lo[48] = {
+    0.f, -2.43569325e-08f, 1.35678162e-08f, 2.83074897e-08f, 1.55436251e-08f, 2.11231441e-08f, 1.21016175e-08f, -7.77961473e-10f,
+    0.f, 6.22335072e-09f, 1.46619872e-09f, 7.18434601e-09f, 0.f, -7.18434601e-09f, -1.46619872e-09f, -6.22335072e-09f,
+    0.f, 7.77961473e-10f, -1.21016175e-08f, -2.11231441e-08f, -1.55436251e-08f, -2.83074897e-08f, -1.35678162e-08f, 2.43569325e-08f,
+    0.f, 2.43569325e-08f, -1.35678162e-08f, -2.83074897e-08f, -1.55436251e-08f, -2.11231441e-08f, -1.21016175e-08f, 7.77961473e-10f,
+    0.f, -6.22335072e-09f, -1.46619872e-09f, -7.18434601e-09f, 0.f, 7.18434601e-09f, 1.46619872e-09f, 6.22335072e-09f,
+    0.f, -7.77961473e-10f, 1.21016175e-08f, 2.11231441e-08f, 1.55436251e-08f, 2.83074897e-08f, 1.35678162e-08f, -2.43569325e-08f};
 
 // The offset v of a line at the points of a stretch starting D points from its centre:
 // v = G (kv B) + kv E1 with E1 = expm1(-D ln q), B = 1 + E1 and G = expm1(-delta ln q) for the
@@ -1059,6 +1064,29 @@ __device__ __forceinline__ void fold_nodes(float2 (&acc)[kNodes / 2], float2* F,
         fold<PREC>(q.x, q.y, mine);
         F[lane] = q;
     }
+}
+
+// {hi, lo} += v (lo takes the rounding error of hi + v; Knuth's two-sum)
+__device__ __forceinline__ void acc_pair(float& hi, float& lo, float v) {
+    const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
+    hi = t;
+}
+
+// Chebyshev coefficients c_m = (2 - [m = 0])/n sum_k F_k T_m(x_k) of the node totals F_k = fx - fy,
+// node k in lane k of the warp; lane m < n gets c_m.  In FP32 pairs (products and sums with their
+// errors): FP64 has 1/64 of the FP32 rate here, and with it the two transforms cost a tile some 5 us.
+__device__ __forceinline__ float cheb_coefs(float fx, float fy, int lane) {
+    float hi = 0.f, lo = 0.f;
+#pragma unroll
+    for (int k = 0; k < kNodes; ++k) {
+        const float x = __shfl_sync(0xffffffffu, fx, k), y = __shfl_sync(0xffffffffu, fy, k);
+        const int i = (lane * (2 * k + 1)) % 48;
+        const float t = c_cos24[i], tl = c_cos24_lo[i], pr = __fmul_rn(t, x);
+        acc_pair(hi, lo, pr);
+        lo += fmaf(t, x, -pr) + fmaf(tl, x, -t * y);
+    }
+    return (hi + lo) * ((lane == 0 ? 1.f : 2.f) / kNodes);
 }
 
 // Clenshaw sum of the Chebyshev series c[0..kNodes) at x
@@ -1211,8 +1239,8 @@ constexpr int kSplitChunks = 64;   // chunks of candidates that are worth a CTA 
 constexpr int kQueue = 2048;   // queued lines at which a tile turns to level 1
 
 template <int PREC, int PTS, int THREADS>
-__device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0, int S = 1, int S_free = 1,
-                                          int* s_used = nullptr) {
+__device__ __forceinline__ void tile_body(const RowDesc& g, int J0, int size, int sp = 0, int S = 1,
+                                          int S_free = 1, int* s_used = nullptr) {
     constexpr int TILE = PTS * THREADS, WARPS = THREADS / 32, QCAP = THREADS + kQueue;
     __shared__ int sQ[QCAP];
     __shared__ PointRec sP[WARPS][kPtRecs];
@@ -1226,19 +1254,18 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
     __shared__ float sSum[PTS][THREADS];
     __shared__ float sComp[PREC == MPSA_PREC_FP32_COMPENSATED ? PTS : 1][THREADS];
 
-    const int J0 = tile * TILE;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float lnq = g.lnq;
     // the tile's points on the grid, [J0, Te], and the warp's part of them, [Js, Je] (npt segments of
     // 32): a short tile is shared out over all warps
-    const int Te = min(J0 + TILE, g.N) - 1;
+    const int Te = min(J0 + size, g.N) - 1;
     const int sub = 32 * ((Te - J0 + 32 * WARPS) / (32 * WARPS)), npt = sub / 32;
     const int Js = J0 + warp * sub, Je = min(Js + sub - 1, Te);
     const bool active = Js <= Te;
     const float span0 = (float)(Te - J0), span1 = active ? (float)(Je - Js) : 0.f;
     const float gend0 = expm1f(-span0 * lnq), gend1 = expm1f(-span1 * lnq);
     if (lane < kNodes) {
-        const float x = 0.5f + 0.5f * (float)c_cos24[2 * lane + 1];
+        const float x = 0.5f + 0.5f * c_cos24[2 * lane + 1];
         sG1[warp][lane] = expm1f(-span1 * x * lnq);
         if (warp == 0) sG0[lane] = expm1f(-span0 * x * lnq);
         sF0[warp][lane] = sF1[warp][lane] = make_float2(0.f, 0.f);
@@ -1246,7 +1273,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
     if (tid < kNumClasses) {   // all classes at once: one memory latency instead of one per class
         const int reach = 1 << tid;
         const int tlo = max(floordiv(J0 - reach + 1, TILE), -1);
-        const int thi = min(floordiv(J0 + TILE - 1 + reach - 1, TILE), g.nT);
+        const int thi = min(floordiv(Te + reach - 1, TILE), g.nT);
         const int* cum = g.cum + (size_t)tid * (g.nT + 3);
         sBeg[tid] = tlo <= thi ? cum[tlo + 1] : 0;
         sEnd[tid] = tlo <= thi ? cum[thi + 2] : 0;
@@ -1420,21 +1447,21 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
             nq = 0;
         }
     }
-    // ---- Chebyshev coefficients of the node totals, c_m = (2 - [m = 0])/n sum_k F_k T_m(x_k), in FP64
-    if (lane < kNodes) {
-        double s1 = 0.0, s0 = 0.0;
-        for (int k = 0; k < kNodes; ++k) {
-            const double tm = c_cos24[(lane * (2 * k + 1)) % 48];
-            s1 += tm * ((double)sF1[warp][k].x - (double)sF1[warp][k].y);
-            if (warp == 0) {
-                double F = 0.0;
-                for (int v = 0; v < WARPS; ++v) F += (double)sF0[v][k].x - (double)sF0[v][k].y;
-                s0 += tm * F;
+    // ---- Chebyshev coefficients of the node totals, level 0's summed over the warps first
+    {
+        const bool node = lane < kNodes;
+        const float2 f1 = node ? sF1[warp][lane] : make_float2(0.f, 0.f);
+        const float c1 = cheb_coefs(f1.x, f1.y, lane);
+        if (node) sC1[warp][lane] = c1;
+        if (warp == 0) {
+            float hi = 0.f, lo = 0.f;
+            for (int v = 0; v < WARPS && node; ++v) {
+                acc_pair(hi, lo, sF0[v][lane].x);
+                lo -= sF0[v][lane].y;
             }
+            const float c0 = cheb_coefs(hi, -lo, lane);
+            if (node) sC0[lane] = c0;
         }
-        const double sc = (lane == 0 ? 1.0 : 2.0) / kNodes;
-        sC1[warp][lane] = (float)(sc * s1);
-        if (warp == 0) sC0[lane] = (float)(sc * s0);
     }
     __syncthreads();
     const float tp = expf(*g.ln_tp);
@@ -1456,6 +1483,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int tile, int sp = 0
 struct TileArgs {
     RowDesc row;     // row 0
     size_t ld;       // lines per row of the record array
+    int size;        // points of a CTA: a tile, or an even part of one (a multiple of 256)
     int split;       // CTAs per tile at most (1: direct output)
     int split_free;  // as many as the GPU holds at once
     float* part;     // split > 1: partial sums [n_sel][split][N], added by k_split_sum
@@ -1472,31 +1500,33 @@ __device__ __forceinline__ RowDesc row_desc(const TileArgs& g, int s) {
     return r;
 }
 
-#ifndef MPSA_TILES_MINB
-#define MPSA_TILES_MINB 4
-#endif
+// CTAs of an SM: 64 registers, or 80 with the wide tile's shared memory (3 CTAs fit)
+constexpr int kTilesPerSM = 4, kWidePerSM = 3;
+constexpr int kWidePts = 16, kWideTile = kWidePts * kTileThreads;   // 4096 points
 // SPLIT: g.split CTAs per tile, each writing its partial sums to g.part (a separate
-// instantiation, so that the one-CTA-per-tile form compiles as it would without it)
-template <int PREC, bool SPLIT>
-__global__ void __launch_bounds__(kTileThreads, MPSA_TILES_MINB) k_tiles(TileArgs g) {
+// instantiation, so that the one-CTA-per-tile form compiles as it would without it).
+// PTS: 8, or 16 for the wide tile (tile_size has the rule).
+template <int PREC, bool SPLIT, int PTS>
+__global__ void __launch_bounds__(kTileThreads, PTS == kWidePts ? kWidePerSM : kTilesPerSM) k_tiles(TileArgs g) {
     RowDesc r = row_desc(g, blockIdx.y);
     if (SPLIT) {
         const int sp = blockIdx.x % g.split;
         r.out = g.part + ((size_t)blockIdx.y * g.split + sp) * r.N;
-        const int tile = blockIdx.x / g.split;
-        tile_body<PREC, kPtsPerThread, kTileThreads>(r, tile, sp, g.split, g.split_free, g.used + (size_t)blockIdx.y * r.nT + tile);
+        const int part = blockIdx.x / g.split, parts = gridDim.x / g.split;
+        tile_body<PREC, PTS, kTileThreads>(r, part * g.size, g.size, sp, g.split, g.split_free,
+                                           g.used + (size_t)blockIdx.y * parts + part);
     } else {
-        tile_body<PREC, kPtsPerThread, kTileThreads>(r, blockIdx.x);
+        tile_body<PREC, PTS, kTileThreads>(r, blockIdx.x * g.size, g.size);
     }
 }
 
 // kappa[s][j] = sum over the split CTAs' partial sums (FP64 sum, one rounding to FP32)
-__global__ void k_split_sum(int n_sel, int N, int split, const int* __restrict__ used, const float* __restrict__ part,
+__global__ void k_split_sum(int n_sel, int N, int size, int split, const int* __restrict__ used, const float* __restrict__ part,
                             float* __restrict__ kappa) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)n_sel * N) return;
     const int s = (int)(t / N), j = (int)(t % N);
-    const int n = used[(size_t)s * ((N + kTile - 1) / kTile) + j / kTile];
+    const int n = used[(size_t)s * ((N + size - 1) / size) + j / size];
     double acc = 0.0;
     for (int q = 0; q < n; ++q) acc += part[((size_t)s * split + q) * N + j];
     kappa[t] = (float)acc;
@@ -1517,7 +1547,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tiles_persistent(const RowDes
         if (u >= n_units) break;
         const int2 rt = units[u];
         const RowDesc r = rows[rt.x];
-        tile_body<PREC, PTS, THREADS>(r, rt.y);
+        tile_body<PREC, PTS, THREADS>(r, rt.y * (PTS * THREADS), PTS * THREADS);
     }
 }
 
@@ -1787,8 +1817,44 @@ RowDesc row_of(const GridDesc& q, int tile, int* cum, const float* ln_tp, const 
     return r;
 }
 
+// Points per tile.  Level 0 works through a tile's candidate lines once, so a tile of twice the points halves
+// it, and the tile's fixed cost; but the parts of its warps are twice as long as well, and a line
+// near a part costs an evaluation at each of its points.  Windows are wider in grid points on finer
+// grids, and few lines leave the fixed cost: 4096 points from R = 1e6 on, or below one line in 20
+// points of the list's range, if these tiles fill the GPU.  2048 -> 4096 points, whole calls: two rows
+// of 5e6 lines, 300 - 1500 nm, at R = 2e6 4829 -> 4178 us, 1e6 3767 -> 3562, 5e5 3316 -> 3304 and 2e5
+// 2726 -> 3665 us; eight rows at R = 5e5 with 1.5e6 lines 5220 -> 6003 us, 5e5 lines 2120 -> 2156, 1e5
+// lines 712 -> 651 us.
+int tile_size(const mpsa_ctx* ctx, int n_sel, int N, double R, int sms) {
+    const bool fine = R >= 1e6, sparse = (double)ctx->L * 20.0 < ctx->log_span * R;
+    const int64_t wide = (int64_t)((N + kWideTile - 1) / kWideTile) * n_sel;
+    return (fine || sparse) && wide >= (int64_t)kWidePerSM * sms ? kWideTile : kTile;
+}
+
+// A call with fewer tiles than the GPU holds CTAs (narrow windows) shares each tile out:
+//  * of lists up to 1e5 lines, by points, down to 256 a CTA, while half the GPU stays free: near lines are
+//    evaluated point by point, and a shorter part has fewer of them.  Every CTA runs over the
+//    tile's candidates, so not with long lists.  40 depths, 20,000 lines, 1000 points: 478 -> 380 us;
+//  * of lists above 2048 lines, by candidate lines, over up to 64 CTAs, with partial sums added afterwards: as
+//    many as run at once, one chunk each at least, and up to eight times that for
+//    the tiles with kSplitChunks each (deep rows have ten times the candidates of shallow ones).
+//    Shorter lists save the second kernel: one row of 1350 lines 93 -> 84 us, of 40 lines 107 -> 103 us.
+// peers: calls that run beside this one take their part of the GPU.  Eight spectrum requests at once on eight
+// streams: 12.8 ms when each counts on the whole GPU, 11.5 ms on an eighth; seven on 25,000 lines 5.6, 3.7 ms.
+void tile_split(TileArgs& ta, int tile, int n_sel, int N, int64_t L, int sms, int peers) {
+    const int64_t slots = (int64_t)sms * kTilesPerSM / peers;
+    auto ctas = [&](int size) { return (int64_t)((N + size - 1) / size) * n_sel; };
+    ta.size = tile;
+    while (tile == kTile && L <= 100000 && ta.size > 256 && 2 * ctas(ta.size / 2) <= slots) ta.size /= 2;
+    const int64_t n = ctas(ta.size), most = std::min<int64_t>(64, kNumClasses + L / kTileThreads);   // chunks a tile can have
+    ta.split_free = (int)std::max<int64_t>(1, std::min(most, slots / n));
+    ta.split = tile != kTile || L <= 2048 || n > slots ? 1 : (int)std::max<int64_t>(1, std::min(most, 8 * slots / n));
+    ta.part = nullptr;
+    ta.used = nullptr;
+}
+
 int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, double lam0_nm, double R, int N,
-               float* kappa, float* kc_out, int64_t* evals, const mpsa_synth_opts* opts, cudaStream_t st) {
+               float* kappa, float* kc_out, int64_t* evals, const mpsa_synth_opts* opts, cudaStream_t st, int peers) {
     const int prec = opts ? opts->precision : 0;
     if (prec != MPSA_PREC_FP32_COMPENSATED && prec != MPSA_PREC_FP32_NAIVE && prec != MPSA_PREC_FP64 &&
         prec != MPSA_PREC_FP32_POP32)
@@ -1796,27 +1862,19 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
     Scratch sc(st, ctx->pool);
     PrepBufs b;
     int r, *cum;
-    const int tile = prec == MPSA_PREC_FP64 ? kTile64 : kTile, nT = (N + tile - 1) / tile;
-    ScratchBlock block;
-    prep_alloc(b, ctx, n_sel, 1, [&](auto** p, size_t n) { return block.add(p, n); });
-    block.add(&cum, (size_t)n_sel * kNumClasses * (nT + 3));
-    // A call with fewer tiles than the GPU holds CTAs (narrow windows) splits each tile's
-    // candidate lines over several CTAs, up to 64, and adds their partial sums afterwards: as
-    // many as run at once, one chunk each at least, and up to eight times that for
-    // the tiles with kSplitChunks each (deep rows have ten times the candidates of shallow ones)
     int dev = 0, sms = 0;
     MPSA_CUDA_TRY(cudaGetDevice(&dev));
     MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t ctas = (int64_t)nT * n_sel, slots = (int64_t)sms * MPSA_TILES_MINB;
-    const int64_t most = std::min<int64_t>(64, kNumClasses + b.L / kTileThreads);   // chunks a tile can have
+    const int tile = prec == MPSA_PREC_FP64 ? kTile64 : tile_size(ctx, n_sel, N, R, sms), nT = (N + tile - 1) / tile;
+    ScratchBlock block;
+    prep_alloc(b, ctx, n_sel, 1, [&](auto** p, size_t n) { return block.add(p, n); });
+    block.add(&cum, (size_t)n_sel * kNumClasses * (nT + 3));
     TileArgs ta;
-    ta.split_free = (int)std::max<int64_t>(1, std::min(most, slots / ctas));
-    ta.split = prec == MPSA_PREC_FP64 || ctas > slots ? 1 : (int)std::max<int64_t>(1, std::min(most, 8 * slots / ctas));
-    ta.part = nullptr;
-    ta.used = nullptr;
+    tile_split(ta, tile, n_sel, N, b.L, sms, peers);
+    const int nC = (N + ta.size - 1) / ta.size;   // CTAs of a row, before the split by candidates
     if (ta.split > 1) {
         block.add(&ta.part, (size_t)n_sel * ta.split * N);
-        block.add(&ta.used, ctas);
+        block.add(&ta.used, (size_t)n_sel * nC);
     }
     if ((r = block.take(sc))) return r;
     const GridDesc grid = grid_desc(lam0_nm, log1p(1.0 / R), N, 0);
@@ -1849,18 +1907,22 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         g.lnq64 = grid.lnq64;
         k_tiles64<<<dim3(nT, n_sel), 256, 0, st>>>(g);
     } else {
-        const dim3 blocks((unsigned)(nT * ta.split), n_sel);
+        const dim3 blocks((unsigned)(nC * ta.split), n_sel);
+        auto go = [&](auto kernel) { kernel<<<blocks, kTileThreads, 0, st>>>(ta); };
         const bool naive = prec == MPSA_PREC_FP32_NAIVE;
-        if (ta.split > 1) {
-            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, true><<<blocks, kTileThreads, 0, st>>>(ta);
-            else k_tiles<MPSA_PREC_FP32_COMPENSATED, true><<<blocks, kTileThreads, 0, st>>>(ta);
+        if (tile == kWideTile) {
+            if (naive) go(k_tiles<MPSA_PREC_FP32_NAIVE, false, kWidePts>);
+            else go(k_tiles<MPSA_PREC_FP32_COMPENSATED, false, kWidePts>);
+        } else if (ta.split > 1) {
+            if (naive) go(k_tiles<MPSA_PREC_FP32_NAIVE, true, kPtsPerThread>);
+            else go(k_tiles<MPSA_PREC_FP32_COMPENSATED, true, kPtsPerThread>);
         } else {
-            if (naive) k_tiles<MPSA_PREC_FP32_NAIVE, false><<<blocks, kTileThreads, 0, st>>>(ta);
-            else k_tiles<MPSA_PREC_FP32_COMPENSATED, false><<<blocks, kTileThreads, 0, st>>>(ta);
+            if (naive) go(k_tiles<MPSA_PREC_FP32_NAIVE, false, kPtsPerThread>);
+            else go(k_tiles<MPSA_PREC_FP32_COMPENSATED, false, kPtsPerThread>);
         }
         if (ta.split > 1) {
             const int64_t tot = (int64_t)n_sel * N;
-            k_split_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n_sel, N, ta.split, ta.used, ta.part, kappa);
+            k_split_sum<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(n_sel, N, ta.size, ta.split, ta.used, ta.part, kappa);
         }
     }
     prof_mark(ctx, MPSA_KERNEL_PROFILE, st);

@@ -330,6 +330,31 @@ def test_interpolated_wings_on_grids_of_every_shape(N, R):
         assert W <= evg[s] <= W + 8 * len(L) + 16
 
 
+@pytest.mark.parametrize("n_lines,N,R,rows", [(2048, 257, 5e5, 2), (2049, 257, 5e5, 2), (2049, 4097, 5e5, 1),
+                                              (100000, 300, 5e5, 1), (100001, 300, 5e5, 1), (100, 480000, 2e6, 4),
+                                              (100, 466945, 1e6, 4), (100, 466944, 5e5, 4)])
+def test_shares_of_a_tile_and_wide_tiles(n_lines, N, R, rows):
+    # narrow windows share a tile out by points (lists to 1e5 lines) and by candidate lines (from 2049
+    # lines), long ones of fine grids or sparse lists take tiles of 4096 points (114 of them a row
+    # at 466,944 points); dense parity against the oracle
+    lam0 = 400.0
+    lnq = np.log1p(1 / R)
+    w = wl.config_tiny(n_lines=40, lam=(lam0, lam0 * np.exp((N - 0.5) * lnq)), R=R, seed=61)
+    w.T, w.P = np.array([4000.0, 9000.0, 6000.0, 2500.0]), np.array([1e4, 1e2, 1e6, 1e5])
+    se, ss = wl.species_table(w.n_metals)
+    pad = np.exp(1000 * lnq)
+    L = wl.linelist(n_lines, len(se), lam0 / pad, w.grid.lam1_nm * pad, 62)
+    ctx, _ = gpu_context(w, lines=L)
+    kg, kcg, evg = gpu_synth(ctx, w, np.arange(rows))
+    assert kg.shape == (rows, N)
+    for s in range(rows):
+        pl, k, slack, W = oracle_dense(w, L, w.T[s], w.P[s])
+        assert abs(kcg[s] / pl.kappa_c - 1) < 2e-5
+        bad, err, bound = opacity_violations(kg[s], k, pl.kappa_c, slack)
+        assert len(bad) == 0, (s, bad[:5], rel_report(kg[s], k, pl.kappa_c))
+        assert W <= evg[s] <= W + 8 * len(L) + 16
+
+
 @pytest.mark.parametrize("n_lines,kind", [(1, "random"), (2, "random"), (6, "equal"), (65536, "random"), (65537, "random"),
                                           (70003, "equal"), (262147, "random"), (262146, "two values"),
                                           (131101, "sample off"), (131101, "no atoms")])
