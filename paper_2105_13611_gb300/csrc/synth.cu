@@ -234,35 +234,106 @@ struct MedState {
     unsigned n;        // lines in the bracket, listed
 };
 
+// The line list, and one line's parameters with what does not depend on the row.
+struct LineList {
+    const int* species;
+    const float *loggf, *E, *lgR, *lgS, *lgW;
+    const double* lam_nm;
+};
+struct LineConst {
+    float lam, lglam, lg, E, gR, gS, gW;
+};
+__device__ __forceinline__ LineConst line_const(const LineList& l, int64_t i) {
+    const float lam = (float)(l.lam_nm[i] * 1e-7);
+    return LineConst{lam, logf(lam), l.loggf[i], l.E[i], exp10f(l.lgR[i]), exp10f(l.lgS[i]), exp10f(l.lgW[i])};
+}
+// ln kappa0, ln S and a of a line in a row.  Every kernel that forms them takes the same roundings
+// (the fused operations are spelled out), so a line has one value wherever it is formed.
+__device__ __forceinline__ float line_terms(const LineConst& l, const RowConst& r, const SpConst& q, float* lnS, float* a) {
+    const float gamma = __fmaf_rn(l.gW, r.nHI, __fmaf_rn(l.gS, r.ne, l.gR));
+    *a = __fmul_rn(gamma, l.lam) / __fmul_rn(kFourPi, q.u);
+    const float stim = -expm1f(-r.hc_kT_cm / l.lam);
+    const float t = __fmaf_rn(-l.E, r.inv_kT_eV, __fmaf_rn(l.lg, kLn10, q.lnC));
+    *lnS = __fsub_rn(__fadd_rn(t, logf(stim)), __fsub_rn(q.lnu, l.lglam));
+    return __fadd_rn(*lnS, logf(*a * *a >= 36.f ? voigt_H(0.f, *a) : voigt_core0(*a)));
+}
+
 // SAMPLE: every kMedStride-th line only, ln kappa0 alone, into lnk0_out [n_sel][ld].
 constexpr int kMedStride = 128;
 template <bool SAMPLE>
-__global__ void k_kappa0(int64_t L, size_t ld, int n_sel, const int* __restrict__ species, const float* __restrict__ loggf,
-                         const float* __restrict__ E, const float* __restrict__ lgR, const float* __restrict__ lgS,
-                         const float* __restrict__ lgW, const double* __restrict__ lam_nm, int n_sp,
-                         const RowConst* __restrict__ rc, const SpConst* __restrict__ sc,
-                         float* __restrict__ lnS_out, float* __restrict__ a_out, float* __restrict__ lnk0_out) {
+__global__ void k_kappa0(int64_t L, size_t ld, int n_sel, LineList lines, int n_sp, const RowConst* __restrict__ rc,
+                         const SpConst* __restrict__ sc, float* __restrict__ lnS_out, float* __restrict__ a_out,
+                         float* __restrict__ lnk0_out) {
     const int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = SAMPLE ? at * kMedStride : at;
     if (i >= L) return;
-    const int sp = species[i];
-    const float lam = (float)(lam_nm[i] * 1e-7), lglam = logf(lam), lg = loggf[i], Ei = E[i];
-    const float gR = exp10f(lgR[i]), gS = exp10f(lgS[i]), gW = exp10f(lgW[i]);
+    const int sp = lines.species[i];
+    const LineConst l = line_const(lines, i);
     const int s1 = min(n_sel, (int)(blockIdx.y + 1) * kKappa0Rows);
 #pragma unroll 1
     for (int s = blockIdx.y * kKappa0Rows; s < s1; ++s) {
-        const RowConst r = rc[s];
-        const SpConst q = sc[(size_t)s * n_sp + sp];
-        const float gamma = gR + gS * r.ne + gW * r.nHI;
-        const float a = gamma * lam / (kFourPi * q.u);
-        const float lnDnu = q.lnu - lglam;
-        const float stim = -expm1f(-r.hc_kT_cm / lam);
-        const float lnS = q.lnC + lg * kLn10 - Ei * r.inv_kT_eV + logf(stim) - lnDnu;
         const size_t o = s * ld + at;
+        float lnS, a;
+        lnk0_out[o] = line_terms(l, rc[s], sc[(size_t)s * n_sp + sp], &lnS, &a);
         if (!SAMPLE) {
             lnS_out[o] = lnS;
             a_out[o] = a;
         }
-        lnk0_out[o] = lnS + logf(a * a >= 36.f ? voigt_H(0.f, a) : voigt_core0(a));
+    }
+}
+
+// k_bounds: upper bounds of ln kappa0 and of ln(a S) of every (row, line), for long lists.
+// Of such a list a window keeps some per cent, and the median needs the few per cent around it, so
+// only those take the full terms (k_med_collect, k_windows); the rest is sorted out by bounds
+// that cost a tenth: ln(1 - e^-x) through ex2/lg2 (x itself below 0.02, at most 1 per cent
+// more), and H(0, a) = e^{a^2} erfc(a) <= 2/(sqrt(pi) (a + sqrt(a^2 + 4/pi))) (Abramowitz & Stegun
+// 7.1.13), at most 0.057 in the logarithm above it for any a.  kBoundUp lies above the roundings of
+// both forms; ln kappa0 is above its bound less kBoundGap.  Both grow with the magnitude, for
+// lists whose terms leave the usual range.
+// 4e8 pairs: 2.58 ms for the full terms, 0.74 ms for the bounds, 8 bytes each.
+constexpr float kBoundUp = 0.02f, kBoundGap = 0.12f, kBoundRel = 1e-6f;
+__device__ __forceinline__ float lg2_fast(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float ex2_fast(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float sqrt_fast(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// up by the margin; an infinity stays what it is
+__device__ __forceinline__ float bound_up(float x) { return x + fmaf(kBoundRel, fminf(fabsf(x), 1e30f), kBoundUp); }
+// a value that ln kappa0 is not below, from its upper bound
+__device__ __forceinline__ float bound_low(float up) { return up - fmaf(3.f * kBoundRel, fminf(fabsf(up), 1e30f), kBoundGap); }
+
+__global__ void __launch_bounds__(256) k_bounds(int64_t L, size_t ld, int n_sel, LineList lines, int n_sp,
+                                                const RowConst* __restrict__ rc, const SpConst* __restrict__ sc,
+                                                float* __restrict__ lnaS_up, float* __restrict__ lnk0_up) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L) return;
+    constexpr float kLn2 = 0.6931471805599453f, kLog2E = 1.4426950408889634f;
+    const int sp = lines.species[i];
+    const LineConst l = line_const(lines, i);
+    const float lgk = fmaf(l.lg, kLn10, l.lglam), inv = kLog2E / l.lam;
+    const float da = l.lam * (float)(1.0 / (4.0 * kPI * kC));   // a = gamma lambda kv / (4 pi c), kv = c / u
+    const int s1 = min(n_sel, (int)(blockIdx.y + 1) * kKappa0Rows);
+#pragma unroll 2
+    for (int s = blockIdx.y * kKappa0Rows; s < s1; ++s) {
+        const RowConst r = rc[s];
+        const SpConst q = sc[(size_t)s * n_sp + sp];
+        const float a = fmaf(l.gW, r.nHI, fmaf(l.gS, r.ne, l.gR)) * (da * q.kv);
+        const float x2 = r.hc_kT_cm * inv;   // x log2(e)
+        const float w = x2 < 0.02f * kLog2E ? x2 * kLn2 : 1.f - ex2_fast(-x2);
+        const float lnS = fmaf(kLn2, lg2_fast(w), fmaf(-l.E, r.inv_kT_eV, (q.lnC - q.lnu) + lgk));
+        const float k0 = fmaf(-kLn2, lg2_fast(a + sqrt_fast(fmaf(a, a, 1.2732395f))), lnS + 0.1207822f);   // ln(2/sqrt(pi))
+        const size_t o = s * ld + i;
+        lnaS_up[o] = bound_up(fmaf(kLn2, lg2_fast(a), lnS));
+        lnk0_up[o] = bound_up(k0);
     }
 }
 
@@ -344,50 +415,87 @@ __global__ void __launch_bounds__(kMedThreads) k_med_bracket(int64_t n, size_t l
 }
 
 // Count the row's lines below its bracket, list those inside (list [n_sel][list_ld], any order).
-constexpr int kMedStage = 8192;
-__global__ void __launch_bounds__(kMedThreads) k_med_collect(int64_t L, size_t ld, const float* __restrict__ lnk0,
-                                                             MedState* __restrict__ st, float* __restrict__ list,
-                                                             size_t list_ld) {
-    __shared__ float stage[kMedStage];
-    __shared__ unsigned s_n, s_base, s_below;
-    const int s = blockIdx.y, tid = threadIdx.x;
-    const unsigned lo = st[s].lo, hi = st[s].hi;
-    const float* x = lnk0 + s * ld;   // 16-byte aligned rows
-    if (tid == 0) s_n = s_below = 0u;
-    __syncthreads();
+// The row holds upper bounds: the lines that these leave open go to the warp's queue, and take
+// their full terms 32 at a time.  (A queue per CTA of 1024 threads, 1.51 ms for 5e6 lines x 80 rows, waited at
+// its barriers; 0.68 ms now.)
+constexpr int kCollectThreads = 256;
+__global__ void __launch_bounds__(kCollectThreads) k_med_collect(int64_t L, size_t ld, const float* __restrict__ lnk0_up,
+                                                                 LineList lines, int n_sp, const RowConst* __restrict__ rc,
+                                                                 const SpConst* __restrict__ sc, MedState* __restrict__ st,
+                                                                 float* __restrict__ list, size_t list_ld) {
+    constexpr int kWarps = kCollectThreads / 32;
+    __shared__ int queue[kWarps][32 + 128];
+    const int s = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lo = st[s].lo, hi = st[s].hi, lt = (1u << lane) - 1u;
+    const float flo = unkey(lo), fhi = unkey(hi);
+    const float* x = lnk0_up + s * ld;   // rows 16-byte aligned and padded to four lines
+    const RowConst r = rc[s];
+    int* const q = queue[warp];
+    int nq = 0;
     unsigned below = 0u;
-    auto flush = [&] {
-        __syncthreads();
-        const unsigned n = s_n;
-        if (tid == 0 && n) s_base = atomicAdd(&st[s].n, n);
-        __syncthreads();
-        for (unsigned i = tid; i < n; i += kMedThreads) list[s * list_ld + s_base + i] = stage[i];
-        __syncthreads();
-        if (tid == 0) s_n = 0u;
-        __syncthreads();
-    };
-    const int64_t step = (int64_t)gridDim.x * 4 * kMedThreads;
-    for (int64_t i0 = (int64_t)blockIdx.x * 4 * kMedThreads; i0 < L; i0 += step) {
-        const int64_t i = i0 + 4 * tid;
-        if (i < L) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(x + i));
-            const float v[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const unsigned k = fkey(v[c]);
-                if (i + c < L) {
-                    below += k < lo;
-                    if (k >= lo && k <= hi) stage[atomicAdd(&s_n, 1u)] = v[c];
-                }
-            }
+    auto take = [&](int n) {   // the queue's last n lines
+        nq -= n;
+        bool in = false;
+        float v = 0.f;
+        if (lane < n) {
+            const int64_t i = q[nq + lane];
+            float lnS, a;
+            v = line_terms(line_const(lines, i), r, sc[(size_t)s * n_sp + lines.species[i]], &lnS, &a);
+            const unsigned k = fkey(v);
+            below += k < lo;
+            in = k >= lo && k <= hi;
         }
-        __syncthreads();
-        if (s_n > kMedStage - 4 * kMedThreads) flush();
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        unsigned at = 0u;
+        if (lane == 0 && m) at = atomicAdd(&st[s].n, (unsigned)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (in) list[s * list_ld + at + __popc(m & lt)] = v;
+        __syncwarp();
+    };
+    const int64_t step = (int64_t)gridDim.x * kWarps * 128;
+    int64_t i0 = ((int64_t)blockIdx.x * kWarps + warp) * 128;
+    auto load = [&](int64_t j) {
+        return j + 4 * lane < L ? __ldg(reinterpret_cast<const float4*>(x + j) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    float4 next = load(i0);
+    for (; i0 < L; i0 += step) {
+        const float4 f = next;
+        next = load(i0 + step);
+        const float v[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int64_t i = i0 + 4 * lane + c;
+            const bool on = i < L, under = v[c] < flo;
+            below += on && under;
+            const bool open = on && !under && !(bound_low(v[c]) > fhi);
+            const unsigned m = __ballot_sync(0xffffffffu, open);
+            if (open) q[nq + __popc(m & lt)] = (int)i;
+            nq += __popc(m);
+        }
+        __syncwarp();
+        while (nq >= 32) take(32);
     }
+    if (nq > 0) take(nq);
     below = __reduce_add_sync(0xffffffffu, below);
-    if ((tid & 31) == 0 && below) atomicAdd(&s_below, below);
-    flush();
-    if (tid == 0 && s_below) atomicAdd(&st[s].below, s_below);
+    if (lane == 0 && below) atomicAdd(&st[s].below, below);
+}
+
+// whether the median lies in the row's bracket
+__device__ __forceinline__ bool med_found(const MedState& m, int64_t L) {
+    const unsigned rank = (unsigned)((L - 1) / 2);
+    return rank >= m.below && rank - m.below < m.n;
+}
+
+// ln kappa0 in place of its bound, for the rows whose bracket missed the median
+__global__ void __launch_bounds__(256) k_med_redo(int64_t L, size_t ld, LineList lines, int n_sp,
+                                                  const RowConst* __restrict__ rc, const SpConst* __restrict__ sc,
+                                                  const MedState* __restrict__ st, float* __restrict__ lnk0) {
+    const int s = blockIdx.y;
+    if (med_found(st[s], L)) return;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < L; i += (int64_t)gridDim.x * blockDim.x) {
+        float lnS, a;
+        lnk0[s * ld + i] = line_terms(line_const(lines, i), rc[s], sc[(size_t)s * n_sp + lines.species[i]], &lnS, &a);
+    }
 }
 
 // st: null, or the bracket whose lines are listed
@@ -402,7 +510,7 @@ __global__ void __launch_bounds__(kMedThreads) k_med_select(int64_t L, size_t ld
     int64_t n = L;
     unsigned rank = (unsigned)((L - 1) / 2), lo = 0u;
     int sh = 0;
-    if (st && rank >= st[s].below && rank - st[s].below < st[s].n) {
+    if (st && med_found(st[s], L)) {
         x = list + s * list_ld;
         n = st[s].n;
         rank -= st[s].below;
@@ -573,6 +681,9 @@ struct PrepOut {
 // logarithm, root or division: 3.4 -> 1.4 ms for 4e8 (row, line) pairs, which it reads at 16 B each.  The lines that
 // remain are appended, as one run per block in line order, to the row's list, and flagged for
 // k_place.  The block's class counts, which k_windows adds to, start at zero here.
+// BOUNDS: lnk0 holds upper bounds of ln kappa0 and lnS of ln(a S) (k_bounds; av is not read); lines that the
+// full terms drop may be listed, k_windows drops them.
+template <bool BOUNDS>
 __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, RowGrids grids,
                                                        const int* __restrict__ species,
                                                        const float* __restrict__ dist, unsigned char* __restrict__ flag,
@@ -592,7 +703,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, Row
     if (i0 < L) {   // rows are padded to a multiple of four lines
         const float4 k4 = __ldcs(reinterpret_cast<const float4*>(lnk0 + s * ld + i0));
         const float4 s4 = __ldg(reinterpret_cast<const float4*>(lnS + s * ld + i0));
-        const float4 a4 = __ldg(reinterpret_cast<const float4*>(av + s * ld + i0));
+        const float4 a4 = BOUNDS ? make_float4(1.f, 1.f, 1.f, 1.f) : __ldg(reinterpret_cast<const float4*>(av + s * ld + i0));
         const float4 d4 = __ldg(reinterpret_cast<const float4*>(dist + gL + i0));
         lk[0] = k4.x, lk[1] = k4.y, lk[2] = k4.z, lk[3] = k4.w;
         ls[0] = s4.x, ls[1] = s4.y, ls[2] = s4.z, ls[3] = s4.w;
@@ -606,13 +717,14 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, Row
     unsigned reach = 0u;   // bit k: line i0 + k is kept
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        if (i0 + k < L && lk[k] >= ltp) {
-            const float w2 = 8.f * kInvSqrtPi * 1.06f * la[k] * __expf(fminf(ls[k] - ltp, 88.f));
+        if (i0 + k < L && (BOUNDS ? !(lk[k] < ltp) : lk[k] >= ltp)) {
+            // (with bounds nothing is capped and a NaN keeps the line)
+            const float w2 = 8.f * kInvSqrtPi * 1.06f * la[k] * __expf(BOUNDS ? ls[k] - ltp : fminf(ls[k] - ltp, 88.f));
             float need = kv_min * di[k];
-            bool in = need <= 22.f || w2 >= need * need;
+            bool in = need <= 22.f || (BOUNDS ? !(w2 < need * need) : w2 >= need * need);
             if (in && need > 0.f) {   // off the grid, and not too far for the slowest species: its own kv
                 need = sc[(size_t)s * n_sp + species[i0 + k]].kv * di[k];
-                in = need <= 22.f || w2 >= need * need;
+                in = need <= 22.f || (BOUNDS ? !(w2 < need * need) : w2 >= need * need);
             }
             if (in) reach |= 1u << k;
         }
@@ -659,14 +771,18 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, Row
 // at their expected crossing (far wing, continued fraction, core): a warp whose lanes need
 // different tiers runs all of them at every evaluation.  The per-block class counts are integer
 // atomics, combined first across the lanes of a warp that hold lines of the same prep block.
-__global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids grids, const int* __restrict__ species,
+// BOUNDS: the list was made from bounds (k_prep): the lines take their full terms here, those whose
+// peak is below the cut are dropped, and ln S and a are stored.
+template <bool BOUNDS>
+__global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids grids, LineList lines,
                                                           const int* __restrict__ cpos, const float* __restrict__ fpos,
-                                                          int n_sp, const SpConst* __restrict__ sc,
-                                                          const float* __restrict__ lnS, const float* __restrict__ av,
+                                                          int n_sp, const RowConst* __restrict__ rc,
+                                                          const SpConst* __restrict__ sc, float* lnS, float* av,
                                                           const float* __restrict__ ln_tp, int nb, PrepOut o) {
     constexpr int kWarps = kPrepThreads / 32;
     __shared__ unsigned char perm[kPrepThreads];
     __shared__ int cnt[4][kWarps];
+    const int* __restrict__ species = lines.species;
     const int s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = o.nsurv[s];
     const GridDesc gd = grids.of(s);
@@ -678,10 +794,25 @@ __global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids
         {   // ---- sort by tier
             int cat = 3;
             if (base + tid < n) {
-                const size_t q = s * ld + o.surv[s * ld + base + tid];
-                const float rel = fminf(lnS[q] - ltp, 88.f), a = av[q];
+                const int64_t i = o.surv[s * ld + base + tid];
+                const size_t q = s * ld + i;
+                float ls, a;
+                bool kept = true;
+                if (BOUNDS) {
+                    kept = line_terms(line_const(lines, i), rc[s], sc[(size_t)s * n_sp + species[i]], &ls, &a) >= ltp;
+                    lnS[q] = ls;
+                    av[q] = a;
+                } else {
+                    ls = __ldg(lnS + q);
+                    a = __ldg(av + q);
+                }
+                const float rel = fminf(ls - ltp, 88.f);
                 const float z2 = fmaxf(a * kInvSqrtPi * __expf(rel), rel) + a * a;
                 cat = z2 >= 1600.f ? 0 : (z2 >= 36.f ? 1 : 2);
+                if (!kept) {   // sorted behind the others
+                    cat = 3;
+                    o.cls[s * ld + base + tid] = kDropped;
+                }
             }
             unsigned mine = 0u;
 #pragma unroll
@@ -701,15 +832,20 @@ __global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids
             __syncthreads();
         }
         const int t = base + perm[tid];
+        int live = 0;   // lines of the categories 0 to 2
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) live += cnt[q][w];
         int blk = 0, key2 = -1;
-        if (t < n) {
+        if (tid < live) {
             const int64_t i = o.surv[s * ld + t];
             const size_t q = s * ld + i;
             blk = (int)(i / kPrepLines);
-            const float rel = fminf(lnS[q] - ltp, 88.f);
+            const float rel = fminf((BOUNDS ? lnS[q] : __ldg(lnS + q)) - ltp, 88.f);
             const float r = expf(-rel);
             const int c = cpos[gL + i];
-            const float f = fpos[gL + i], a = av[q], kv = sc[(size_t)s * n_sp + species[i]].kv;
+            const float f = fpos[gL + i], a = BOUNDS ? av[q] : __ldg(av + q), kv = sc[(size_t)s * n_sp + species[i]].kv;
             unsigned char cl = kDropped;
             const float srel = expf(rel);
             float vo, vi;
@@ -1734,6 +1870,16 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     k_start<<<cb + (unsigned)((L + kStartThreads - 1) / kStartThreads), kStartThreads, 0, st>>>(
         cb, n_sel, d_sel, n_sp, ctx->d_sp_el, ctx->d_sp_stage, ctx->n_el, ctx->d_el, pop, ctx->vturb, pop32, b.rc, b.spc,
         b.po.nsurv, L, b.ld, b.n_grids, ctx->d_lam, grid, d_grids, b.dist, b.flag);
+    const LineList lines{ctx->d_species, ctx->d_loggf, ctx->d_E, ctx->d_lgR, ctx->d_lgS, ctx->d_lgW, ctx->d_lam};
+    int dev = 0, sms = 0;
+    MPSA_CUDA_TRY(cudaGetDevice(&dev));
+    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const bool small = L <= kMedSmall;
+    // Bounds first, where a grid covers less than a quarter of the list's range: a line that is kept
+    // takes its terms after its bounds; and where there are enough pairs to repay two more launches.  80 depths x 5e6 lines, 0.2 per cent of the range: 8.80 -> 7.09 ms for the call,
+    // 63 depths, 5 per cent: 20.4 -> 19.4 ms; two rows over the whole range 14.0 -> 14.1 ms (so not there);
+    // 8 rows x 5e5 lines a call, eight requests at once: 11.4 -> 10.9 ms, 8 x 66,753 lines 4.86 -> 5.04 ms.
+    const bool bounds = !small && (int64_t)n_sel * L >= 3000000 && (d_grids || 4.0 * grid.N * grid.lnq64 < ctx->log_span);
     {
         // ln S, a, ln kappa0 and the median; the record array, not in use yet, holds the listed lines
         // and the sample
@@ -1742,29 +1888,32 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
         const size_t ns_ld = ((size_t)ns + 3) & ~(size_t)3;
         float* const list = reinterpret_cast<float*>(b.rec);
         float* const sample = list + (size_t)n_sel * b.ld;
-        const bool small = L <= kMedSmall;
-        auto kappa0 = [&](auto kernel, int64_t lines, size_t ld, float* k0) {
-            kernel<<<dim3((unsigned)((lines + 255) / 256), rows), 256, 0, st>>>(
-                L, ld, n_sel, ctx->d_species, ctx->d_loggf, ctx->d_E, ctx->d_lgR, ctx->d_lgS, ctx->d_lgW, ctx->d_lam, n_sp,
-                b.rc, b.spc, b.lnS, b.av, k0);
-        };
+        const unsigned lb = (unsigned)((L + 255) / 256);
         if (!small) {
-            kappa0(k_kappa0<true>, ns, ns_ld, sample);
+            k_kappa0<true><<<dim3((unsigned)((ns + 255) / 256), rows), 256, 0, st>>>(L, ns_ld, n_sel, lines, n_sp, b.rc, b.spc,
+                                                                                     nullptr, nullptr, sample);
             k_med_bracket<<<n_sel, kMedThreads, 0, st>>>(ns, ns_ld, sample, b.med);
         }
-        kappa0(k_kappa0<false>, L, b.ld, b.lnk0);
+        if (bounds)
+            k_bounds<<<dim3(lb, rows), 256, 0, st>>>(L, b.ld, n_sel, lines, n_sp, b.rc, b.spc, b.lnS, b.lnk0);
+        else
+            k_kappa0<false><<<dim3(lb, rows), 256, 0, st>>>(L, b.ld, n_sel, lines, n_sp, b.rc, b.spc, b.lnS, b.av, b.lnk0);
         if (!small) {
-            const int per_row = (int)std::max<int64_t>(1, std::min<int64_t>(128, L / (8 * 4 * kMedThreads)));
-            k_med_collect<<<dim3(per_row, n_sel), kMedThreads, 0, st>>>(L, b.ld, b.lnk0, b.med, list, b.ld);
+            // eight groups of 128 lines per warp, and no more than four waves of CTAs in all
+            const int per_row = (int)std::max<int64_t>(1, std::min<int64_t>(L / 8192, 16ll * sms / n_sel));
+            k_med_collect<<<dim3(per_row, n_sel), kCollectThreads, 0, st>>>(L, b.ld, b.lnk0, lines, n_sp, b.rc, b.spc, b.med,
+                                                                            list, b.ld);
+            if (bounds) k_med_redo<<<dim3(64, n_sel), 256, 0, st>>>(L, b.ld, lines, n_sp, b.rc, b.spc, b.med, b.lnk0);
         }
         k_med_select<<<n_sel, kMedThreads, 0, st>>>(L, b.ld, b.lnk0, small ? nullptr : b.med, list, b.ld,
                                                     (float)log(kcf), (float)log(cut), b.ln_tp, out);
     }
-    k_prep<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS, b.av,
-                                                       b.lnk0, b.ln_tp, b.nb, b.po);
-    int dev = 0, sms = 0;
-    MPSA_CUDA_TRY(cudaGetDevice(&dev));
-    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    auto prep = [&](auto kernel) {
+        kernel<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS,
+                                                           b.av, b.lnk0, b.ln_tp, b.nb, b.po);
+    };
+    if (bounds) prep(k_prep<true>);
+    else prep(k_prep<false>);
     if ((int64_t)b.nb * b.n_grids >= 2 * sms)
         k_place<kPrepLines><<<dim3(b.nb, b.n_grids), kPrepThreads, 0, st>>>(L, b.ld, ctx->d_lam, grid, d_grids, b.flag, b.c,
                                                                             b.f);
@@ -1775,8 +1924,12 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
         // the listed lines' count is known on the device only: about eight CTAs per SM in all,
         // each running over its row's list
         const int gx = std::max(1, std::min(b.nb, (8 * sms + n_sel - 1) / n_sel));
-        k_windows<<<dim3(gx, n_sel), kPrepThreads, 0, st>>>(b.ld, grids, ctx->d_species, b.c, b.f, n_sp, b.spc, b.lnS, b.av,
-                                                            b.ln_tp, b.nb, b.po);
+        auto windows = [&](auto kernel) {
+            kernel<<<dim3(gx, n_sel), kPrepThreads, 0, st>>>(b.ld, grids, lines, b.c, b.f, n_sp, b.rc, b.spc, b.lnS, b.av,
+                                                             b.ln_tp, b.nb, b.po);
+        };
+        if (bounds) windows(k_windows<true>);
+        else windows(k_windows<false>);
     }
     k_scan_class<<<dim3(kNumClasses, n_sel), 1024, 0, st>>>(b.nb, b.po.blkcnt, b.classcnt, out);
     constexpr int kWarps = kPrepThreads / 32;
@@ -1997,7 +2150,7 @@ namespace {
 struct TuneCfg {
     int pts, threads, minb;
 };
-constexpr TuneCfg kCfgs[] = {{8, 256, 4}, {4, 256, 4}, {8, 128, 8}, {16, 128, 3}};
+constexpr TuneCfg kCfgs[] = {{8, 256, 4}, {4, 256, 4}, {8, 128, 8}, {16, 256, 3}};
 constexpr int kNumCfgs = sizeof(kCfgs) / sizeof(kCfgs[0]);
 
 template <int PREC, int PTS, int THREADS, int MINB>
@@ -2021,14 +2174,14 @@ int persistent_launch(int cfg, int prec, const RowDesc* rows, const int2* units,
             case 0: return persistent_launch_t<1, 8, 256, 4>(rows, units, n_units, counter, st);
             case 1: return persistent_launch_t<1, 4, 256, 4>(rows, units, n_units, counter, st);
             case 2: return persistent_launch_t<1, 8, 128, 8>(rows, units, n_units, counter, st);
-            default: return persistent_launch_t<1, 16, 128, 3>(rows, units, n_units, counter, st);
+            default: return persistent_launch_t<1, 16, 256, 3>(rows, units, n_units, counter, st);
         }
     }
     switch (cfg) {
         case 0: return persistent_launch_t<0, 8, 256, 4>(rows, units, n_units, counter, st);
         case 1: return persistent_launch_t<0, 4, 256, 4>(rows, units, n_units, counter, st);
         case 2: return persistent_launch_t<0, 8, 128, 8>(rows, units, n_units, counter, st);
-        default: return persistent_launch_t<0, 16, 128, 3>(rows, units, n_units, counter, st);
+        default: return persistent_launch_t<0, 16, 256, 3>(rows, units, n_units, counter, st);
     }
 }
 

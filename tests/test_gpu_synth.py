@@ -355,6 +355,39 @@ def test_shares_of_a_tile_and_wide_tiles(n_lines, N, R, rows):
         assert W <= evg[s] <= W + 8 * len(L) + 16
 
 
+@pytest.mark.parametrize("kind", ["random", "far infrared", "strong damping", "no damping", "no atoms", "sample off"])
+def test_bounds_keep_what_the_full_terms_keep(kind):
+    # calls of 3e6 (row, line) pairs or more on a narrow window sort lines out by bounds first; the same rows one by
+    # one form every line's full terms.  Continuum and evaluation counts follow from the lines kept and from
+    # their bits: equal.  Opacities: both within the opacity tolerance of the same sum, and a line at the cut
+    # (cut * kappa_c) may fall either way at one point
+    w = wl.config_tiny(n_lines=40, lam=(300.0, 300.3), R=5e5, seed=91)
+    w.T, w.P = np.array([2000.0, 3500.0, 5000.0, 6500.0, 8000.0, 10000.0, 13000.0, 20000.0]), 10.0 ** np.arange(8)
+    se, ss = wl.species_table(w.n_metals)
+    L = wl.linelist(400_000, len(se), 200.0, 500.0, 92)
+    ab = None
+    if kind == "far infrared":           # h nu / kT from 1e-4 up: 1 - e^-x by its first order
+        w.grid = wl.Grid(5e6, 5.005e6, 5e5)
+        L.lam_nm[:] *= 1.6e4
+    elif kind == "strong damping":       # a up to 1e4
+        L.log_gS[:] = np.linspace(-8.0, -2.0, len(L))
+    elif kind == "no damping":
+        L.log_gR[:] = L.log_gS[:] = L.log_gW[:] = -45.0
+    elif kind == "no atoms":
+        ab = np.ones((1, wl.elements(w.n_metals).n))
+        ab[0, 2:5] = 0.0
+    elif kind == "sample off":
+        L.log_gf[::128] = 9.0
+    ctx, _ = gpu_context(w, lines=L, abund=ab)
+    kap, kc, ev = gpu_synth(ctx, w, np.arange(8))
+    for s in range(8):
+        k1, kc1, ev1 = gpu_synth(ctx, w, [s])
+        assert kc[s] == kc1[0] and ev[s] == ev1[0], s
+        if kc[s] > 0:
+            bad, err, bound = opacity_violations(kap[s], k1[0].astype(np.float64), float(kc[s]), 2 * w.cut * float(kc[s]))
+            assert len(bad) == 0, (s, bad[:5], float((err / bound).max()))
+
+
 @pytest.mark.parametrize("n_lines,kind", [(1, "random"), (2, "random"), (6, "equal"), (65536, "random"), (65537, "random"),
                                           (70003, "equal"), (262147, "random"), (262146, "two values"),
                                           (131101, "sample off"), (131101, "no atoms")])
