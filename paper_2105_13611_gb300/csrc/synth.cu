@@ -678,7 +678,8 @@ struct PrepOut {
 // w^2 = 8 a s_rel/sqrt(pi), the second of which is below 19: a line whose nearest grid point
 // lies at |v| = kv dist is dropped if that is above 22 and 3 per cent above w (k_windows drops
 // exactly what is left).  The squares are compared, so the test costs one exponential and no
-// logarithm, root or division: 3.4 -> 1.4 ms for 4e8 (row, line) pairs, which it reads at 16 B each.  The lines that
+// logarithm, root or division: 3.4 -> 1.4 ms for 4e8 (row, line) pairs, and 0.94 ms for their bounds, of which
+// it reads 8 B each (4 more of the few lines that can reach).  The lines that
 // remain are appended, as one run per block in line order, to the row's list, and flagged for
 // k_place.  The block's class counts, which k_windows adds to, start at zero here.
 // BOUNDS: lnk0 holds upper bounds of ln kappa0 and lnS of ln(a S) (k_bounds; av is not read); lines that the
@@ -693,76 +694,110 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(int64_t L, size_t ld, Row
                                                        int nb, PrepOut o) {
     static_assert(kPrepLines == 4 * kPrepThreads, "four lines per thread");
     constexpr int kWarps = kPrepThreads / 32;
-    __shared__ int s_cnt[kWarps], s_base;
+    __shared__ int s_cnt[2][kWarps], s_base;
     const int s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t i0 = (int64_t)blockIdx.x * kPrepLines + 4 * tid;
-    if (tid < kNumClasses) o.blkcnt[((size_t)s * kNumClasses + tid) * nb + blockIdx.x] = 0;
     const size_t gL = grids.of(s).index * ld;
     const float ltp = ln_tp[s];
-    float lk[4], ls[4], la[4], di[4];
-    if (i0 < L) {   // rows are padded to a multiple of four lines
-        const float4 k4 = __ldcs(reinterpret_cast<const float4*>(lnk0 + s * ld + i0));
-        const float4 s4 = __ldg(reinterpret_cast<const float4*>(lnS + s * ld + i0));
-        const float4 a4 = BOUNDS ? make_float4(1.f, 1.f, 1.f, 1.f) : __ldg(reinterpret_cast<const float4*>(av + s * ld + i0));
-        const float4 d4 = __ldg(reinterpret_cast<const float4*>(dist + gL + i0));
-        lk[0] = k4.x, lk[1] = k4.y, lk[2] = k4.z, lk[3] = k4.w;
-        ls[0] = s4.x, ls[1] = s4.y, ls[2] = s4.z, ls[3] = s4.w;
-        la[0] = a4.x, la[1] = a4.y, la[2] = a4.z, la[3] = a4.w;
-        di[0] = d4.x, di[1] = d4.y, di[2] = d4.z, di[3] = d4.w;
-    }
+    // a block's four lines of the thread (rows are padded to a multiple of four); its bounds of ln kappa0
+    // are read for the lines that pass the other test only
+    struct Four {
+        float4 k, s, a, d;
+    };
+    auto load = [&](int blk) {
+        Four f{};
+        const int64_t i0 = (int64_t)blk * kPrepLines + 4 * tid;
+        if (blk < nb && i0 < L) {
+            if (!BOUNDS) {
+                f.k = __ldcs(reinterpret_cast<const float4*>(lnk0 + s * ld + i0));
+                f.a = __ldg(reinterpret_cast<const float4*>(av + s * ld + i0));
+            }
+            f.s = __ldg(reinterpret_cast<const float4*>(lnS + s * ld + i0));
+            f.d = __ldg(reinterpret_cast<const float4*>(dist + gL + i0));
+        }
+        return f;
+    };
+    Four next = load(blockIdx.x);
     float kv_min = INFINITY;   // of the row's species
     for (int p = lane; p < n_sp; p += 32) kv_min = fminf(kv_min, sc[(size_t)s * n_sp + p].kv);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) kv_min = fminf(kv_min, __shfl_xor_sync(0xffffffffu, kv_min, d));
-    unsigned reach = 0u;   // bit k: line i0 + k is kept
+    int par = 0;
+    for (int blk = blockIdx.x; blk < nb; blk += gridDim.x, par ^= 1) {
+        const Four f = next;
+        next = load(blk + gridDim.x);
+        const int64_t i0 = (int64_t)blk * kPrepLines + 4 * tid;
+        if (tid < kNumClasses) o.blkcnt[((size_t)s * kNumClasses + tid) * nb + blk] = 0;
+        const float lk[4] = {f.k.x, f.k.y, f.k.z, f.k.w}, ls[4] = {f.s.x, f.s.y, f.s.z, f.s.w};
+        const float la[4] = {f.a.x, f.a.y, f.a.z, f.a.w}, di[4] = {f.d.x, f.d.y, f.d.z, f.d.w};
+        // Peak and reach, the reach with the slowest species first; the few lines left take their own (off
+        // the grid only) and, with bounds, their peak.  Each gather is issued for the four lines at
+        // once: one after the other, inside the tests, they cost a block eight memory latencies.
+        // (With bounds nothing is capped and a NaN keeps the line.)
+        float w2[4], x[4];
+        int sp[4];
+        bool in[4];
+        auto reaches = [&](float w, float need) { return need <= 22.f || (BOUNDS ? !(w < need * need) : w >= need * need); };
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (i0 + k < L && (BOUNDS ? !(lk[k] < ltp) : lk[k] >= ltp)) {
-            // (with bounds nothing is capped and a NaN keeps the line)
-            const float w2 = 8.f * kInvSqrtPi * 1.06f * la[k] * __expf(BOUNDS ? ls[k] - ltp : fminf(ls[k] - ltp, 88.f));
-            float need = kv_min * di[k];
-            bool in = need <= 22.f || (BOUNDS ? !(w2 < need * need) : w2 >= need * need);
-            if (in && need > 0.f) {   // off the grid, and not too far for the slowest species: its own kv
-                need = sc[(size_t)s * n_sp + species[i0 + k]].kv * di[k];
-                in = need <= 22.f || (BOUNDS ? !(w2 < need * need) : w2 >= need * need);
+        for (int k = 0; k < 4; ++k) {
+            w2[k] = BOUNDS ? 8.f * kInvSqrtPi * 1.06f * __expf(ls[k] - ltp)
+                           : 8.f * kInvSqrtPi * 1.06f * la[k] * __expf(fminf(ls[k] - ltp, 88.f));
+            in[k] = i0 + k < L && (BOUNDS || lk[k] >= ltp) && reaches(w2[k], kv_min * di[k]);
+        }
+        unsigned reach = 0u;   // bit k: line i0 + k is kept
+        bool more = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            reach |= in[k] ? 1u << k : 0u;
+            more = more || (in[k] && (BOUNDS || di[k] > 0.f));
+        }
+        if (more) {
+            reach = 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                sp[k] = in[k] ? __ldg(species + i0 + k) : 0;
+                if (BOUNDS) x[k] = in[k] ? __ldg(lnk0 + s * ld + i0 + k) : 0.f;
             }
-            if (in) reach |= 1u << k;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float need = __ldg(&sc[(size_t)s * n_sp + sp[k]].kv) * di[k];
+                if (in[k] && (di[k] <= 0.f || reaches(w2[k], need)) && (!BOUNDS || !(x[k] < ltp))) reach |= 1u << k;
+            }
         }
-    }
-    // the lines' places in the run: within the warp, then over the warps
-    const int cnt = __popc(reach);
-    int incl = cnt;
+        // the lines' places in the run: within the warp, then over the warps
+        const int cnt = __popc(reach);
+        int incl = cnt;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += y;
-    }
-    if (lane == 31) s_cnt[warp] = incl;
-    __syncthreads();
-    int before = 0, n = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const int c = s_cnt[w];
-        if (w < warp) before += c;
-        n += c;
-    }
-    if (n == 0) {
-        if (tid == 0) o.run[(size_t)s * nb + blockIdx.x] = make_int2(0, 0);
-        return;
-    }
-    if (tid == 0) {
-        const int base = atomicAdd(&o.nsurv[s], n);
-        s_base = base;
-        o.run[(size_t)s * nb + blockIdx.x] = make_int2(base, n);
-    }
-    __syncthreads();
-    int pos = s_base + before + incl - cnt;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if ((reach >> k) & 1u) {
-            o.surv[s * ld + pos++] = (int)(i0 + k);
-            flag[gL + i0 + k] = 1;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += y;
         }
+        if (lane == 31) s_cnt[par][warp] = incl;
+        __syncthreads();
+        int before = 0, n = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const int c = s_cnt[par][w];
+            if (w < warp) before += c;
+            n += c;
+        }
+        if (n == 0) {
+            if (tid == 0) o.run[(size_t)s * nb + blk] = make_int2(0, 0);
+            continue;
+        }
+        if (tid == 0) {
+            const int base = atomicAdd(&o.nsurv[s], n);
+            s_base = base;
+            o.run[(size_t)s * nb + blk] = make_int2(base, n);
+        }
+        __syncthreads();
+        int pos = s_base + before + incl - cnt;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((reach >> k) & 1u) {
+                o.surv[s * ld + pos++] = (int)(i0 + k);
+                flag[gL + i0 + k] = 1;
+            }
+    }
 }
 
 // k_windows: the outer and inner cut windows of every listed line (crossing searches on the
@@ -1908,8 +1943,11 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
         k_med_select<<<n_sel, kMedThreads, 0, st>>>(L, b.ld, b.lnk0, small ? nullptr : b.med, list, b.ld,
                                                     (float)log(kcf), (float)log(cut), b.ln_tp, out);
     }
+    // up to four blocks of lines per CTA, while 16 CTAs per SM remain (80 rows x 5e6 lines: the call 7.26 ms
+    // with one block per CTA, 7.07 with two, 6.99 with four)
+    const int gx = (int)std::max<int64_t>((b.nb + 3) / 4, std::min<int64_t>(b.nb, (16 * sms + n_sel - 1) / n_sel));
     auto prep = [&](auto kernel) {
-        kernel<<<dim3(b.nb, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS,
+        kernel<<<dim3(gx, n_sel), kPrepThreads, 0, st>>>(L, b.ld, grids, ctx->d_species, b.dist, b.flag, n_sp, b.spc, b.lnS,
                                                            b.av, b.lnk0, b.ln_tp, b.nb, b.po);
     };
     if (bounds) prep(k_prep<true>);
