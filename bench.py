@@ -38,18 +38,18 @@ import workloads as wl  # noqa: E402
 
 METRIC = "Voigt line-evals/s (line-by-line opacity synthesis + ODF binning)"
 UNIT = "line-evals/s"
-# FP32 operations of one far-wing profile evaluation in the form that takes 97-99.6 % of the
-# evaluations of the table rows (plain rational form in units of sk, two points per
-# reciprocal, packed FP32): per pair of points {v0, v1} = fma(G, B', E'), {D0, D1} =
-# fma(v, v, c') and {s1, s0} += r {D0, D1} are three packed FFMAs (12 flop) and
-# r = rcp(D0 D1) one FMUL (1 flop): 13 flop per pair, 6.5 per evaluation, plus half a
-# reciprocal on the special-function unit (not counted).
-FLOP_PER_EVAL = 6.5
+# FP32 operations that the profile kernel executes per line-evaluation of the default rows, all forms and
+# overheads included (ncu's FP32 thread-instruction counters: FFMA2 4, FFMA, FADD2 and FMUL2 2, FADD and
+# FMUL 1; 1.609e12 operations for 1.0804e13 evaluations).  An evaluation is one line at one
+# grid point inside its cut window; most are not formed one by one but as the line's share of
+# an interpolated wing sum, so the figure is far below the 6.5 operations of the cheapest profile form.  It
+# varies with the row (0.075 to 4.2) and holds for the default rows only.
+FLOP_PER_EVAL = 0.1489
 FP32_LANES_PER_SM = 128
-# kernels of the library per timed step: synth_opacity (k_place, k_consts, k_kappa0, k_med_init,
-# three k_med_hist + k_med_pick levels, k_prep, k_windows, k_scan_class, k_scan_fin, k_scatter,
-# k_ranges, k_tiles) and build_odf (k_odf_gather, then k_odf for the intervals it leaves)
-LAUNCHES_PER_STEP = 19
+# kernels of the library per timed step: synth_opacity (k_start, k_kappa0 over the sample,
+# k_med_bracket, k_kappa0, k_med_collect, k_med_select, k_prep, k_place, k_windows, k_scan_class,
+# k_scatter, k_ranges, k_tiles) and build_odf (k_odf_gather, then k_odf for the intervals it leaves)
+LAUNCHES_PER_STEP = 15
 
 
 def parse():
@@ -116,13 +116,23 @@ class Clocks:
         self.gpu = gpu_index
         self.f = tempfile.NamedTemporaryFile("w+", suffix=".csv", delete=False)
         self.p = None
+        self.skip = 0
 
     def start(self):
+        """Returns when the first sample is there, so that nvidia-smi's start is not in the timed region."""
         try:
             self.p = subprocess.Popen(["nvidia-smi", "-i", str(self.gpu), f"--query-gpu={self.Q}", "--format=csv,noheader,nounits",
-                                       "-lms", "200"], stdout=self.f, stderr=subprocess.DEVNULL)
+                                       "-lms", "100"], stdout=self.f, stderr=subprocess.DEVNULL)
         except OSError:
             self.p = None
+            return
+        t0 = time.monotonic()
+        while time.monotonic() - t0 < 10 and self.p.poll() is None and os.path.getsize(self.f.name) == 0:
+            time.sleep(0.01)
+
+    def mark(self):
+        """The timed region begins: earlier samples do not count."""
+        self.skip = len(open(self.f.name).read().strip().splitlines())
 
     def stop(self):
         if self.p is None:
@@ -134,6 +144,7 @@ class Clocks:
             self.p.kill()
         self.f.flush()
         rows = [r.split(",") for r in open(self.f.name).read().strip().splitlines() if r.strip()]
+        rows = rows[self.skip:] or rows[-1:]   # (a region shorter than the interval: the sample before it)
         os.unlink(self.f.name)
         sm, mx, reasons = [], [], set()
         names = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"]
@@ -321,14 +332,17 @@ def native_arm(args):
         ctx.synth_opacity(w.grid, sel, kap, kc, ev, opts=opts, stream=stream)
         ctx.build_odf(kap, bounds, w.widths, odf, stream=stream)
 
+    clocks = Clocks(local)
+    clocks.start()
     for _ in range(args.warmup):
         step()
+        ev_tot.add_(ev)   # torch loads this kernel at its first use, 0.7 s on a host that does so for the first time
+    ev_tot.zero_()
     barrier()
     ctx.profile_enable(True)
     ctx.profile_read(binding.KERNEL_PROFILE)
     ctx.profile_read(binding.KERNEL_ODF)
-    clocks = Clocks(local)
-    clocks.start()
+    clocks.mark()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     barrier()
     e0.record(stream)
@@ -403,15 +417,15 @@ def native_arm(args):
     fp32_peak = sms * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12        # TFLOP/s at the maximum SM clock
     achieved = evals_per_launch * FLOP_PER_EVAL / (tiles_avg / 1e3) / 1e12
     traffic = measured_traffic("k_tiles", ["synth.cu", "voigt.cuh", "common.cuh"], sel)
-    counted = profile_value("k_tiles_fp32_ops_row1044.md", "flop_per_eval_counted", "k_tiles",
+    counted = profile_value("k_tiles_fp32_ops.md", "flop_per_eval_counted", "k_tiles",
                             ["synth.cu", "voigt.cuh", "common.cuh"])
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp32_peak, "traffic": traffic, "kernel": "k_tiles (profile synthesis)",
                 "fp32_counted": None if counted is None else {
                     "flop_per_eval": counted, "achieved": achieved * counted / FLOP_PER_EVAL,
                     "frac": achieved * counted / FLOP_PER_EVAL / fp32_peak,
-                    "source": "ncu FP32 thread-instruction counters (FFMA2 x4, FFMA x2, FMUL, FADD) on row 1044, "
-                              "profiles/k_tiles_fp32_ops_row1044.md"},
+                    "source": "ncu FP32 thread-instruction counters (FFMA2 x4; FFMA, FADD2, FMUL2 x2; FADD, FMUL) "
+                              "over the eight default rows, profiles/k_tiles_fp32_ops.md"},
                 "peak_kind": f"FP32 FMA peak {sms} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x {sm_max:.0f} MHz",
                 "sms": sms, "flop_per_eval": FLOP_PER_EVAL, "avg_launch_ms": tiles_avg, "launches": tiles_n}
     odf_avg = odf_ms / max(odf_n, 1)

@@ -504,13 +504,13 @@ int mpsa_profile_read(mpsa_ctx* ctx, int kernel, double* total_ms, int64_t* laun
 /*
  * mpsa_voigt -- the Voigt function H(v, a) = Re w(v + i a) of the line profile
  * (paper Sect. 2.1: argument v = (nu - nu0)/dnu_D, damping a = gamma/(4 pi dnu_D)),
- * evaluated on the device exactly as the synthesis kernels evaluate it, for
- * accuracy tests of the profile tiers.
+ * evaluated on the device as the profile kernel evaluates it at a grid point, for
+ * accuracy tests of its tiers.
  *   v, a (device, double[n]): arguments (a > 0; the sign of v is ignored).
  *   precision: MPSA_PREC_FP64 evaluates the FP64 tiers in double; any other value
  *     rounds v and a to FP32 and evaluates the FP32 tiers (far: rational or
- *     one-level continued fraction; mid: five-level continued fraction; core:
- *     shifted 12-point Gauss-Hermite).
+ *     one-level continued fraction; then the asymptotic series; core: a rational
+ *     form in v for a <= 0.03, else shifted 12-point Gauss-Hermite).
  *   out (device, double[n]): H, widened from FP32 for the FP32 tiers.
  * Stream-ordered.  Errors: MPSA_EINVAL, MPSA_ECUDA.
  */

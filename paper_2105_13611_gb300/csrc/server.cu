@@ -101,7 +101,7 @@ namespace mpsa {
 namespace {
 
 size_t synth_scratch_bytes(const mpsa_ctx* c, int rows, int N) {
-    // per (row, line) prep arrays, buckets and the crossing-search list (~61 B), per-line
+    // per (row, line) prep arrays, records and the crossing-search list (73 B, admitted at 64), per-line
     // placement (12 B), tile ranges, per (row, prep block) class counts
     const size_t nT = (size_t)(N + kTile - 1) / kTile, nb = (size_t)(c->L + kPrepLines - 1) / kPrepLines;
     return (size_t)rows * c->L * 64 + (size_t)c->L * 12 + (size_t)rows * kNumClasses * (nT + 3) * 4 +

@@ -7,18 +7,20 @@
 // opacity of the synthetic workload).
 //
 // Pipeline (all on the caller's stream):
-//   k_start        per line: how far off the grid its centre is, and per (row, species): ln(sqrt(pi) e^2/(m_e c) N/U / rho), u, c/u from the FP64 table
-//   k_kappa0       per (row, line): ln S, a, ln kappa0 in FP32 log space
+//   k_start        per line: how far off the grid its centre is; per (row, species):
+//                  ln(sqrt(pi) e^2/(m_e c) N/U / rho), u, c/u from the FP64 table
+//   k_kappa0       per (row, line): ln S, a, ln kappa0 in FP32 log space; on long lists and narrow
+//                  grids k_bounds instead: upper bounds of ln kappa0 and ln(a S)
 //   k_med_*        per row: lower median of ln kappa0 -> ln t_p, kappa_c
 //   k_prep         per (row, line): peak against the cut, reach of the wing; the lines left, listed
 //   k_place        the listed lines' centre index c and fraction f on the grid (FP64 log)
-//   k_windows      per listed line: cut windows (outer: no point beyond can pass the cut; inner:
-//                  every point inside passes), width class
+//   k_windows      per listed line: its terms where there are only bounds so far; cut windows (outer: no
+//                  point beyond can pass the cut; inner: every point inside passes), width class
 //   k_scan_class, k_scatter   stable counting sort of the kept lines by width class
 //   k_ranges       per (row, class, tile boundary): first line whose centre lies at or
 //                  beyond the boundary (binary search in the centre-sorted class)
-//   k_tiles        the profile kernel: one CTA per (row, 2048-point tile) (or several, on calls with
-//                  few tiles); wings summed at Chebyshev nodes, the rest point by point; FP32
+//   k_tiles        the profile kernel: one CTA per (row, tile of 2048 or 4096 points), or several on
+//                  calls with few tiles; wings summed at Chebyshev nodes, the rest point by point; FP32
 //                  partial sums folded into Kahan-compensated totals; no atomics; coalesced stores.
 #include <math.h>
 #include <stdio.h>
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(kStartThreads) k_start(int cb, int n_sel, cons
 // H(0, a) is bound by its arithmetic: at v = 0 the two poles of a pair of voigt_core give the same
 // term, so voigt_core0 forms it once (60 operations instead of 130), with every rounding that the general
 // form takes there (median, cut and windows follow from these bits).  4e8 (row, line) pairs: 3.60 ms
-// before, 2.58 ms now; their 12 bytes each would take 0.7 ms.
+// in the general form, 2.58 ms; their 12 bytes each would take 0.7 ms (k_bounds below avoids most of it).
 constexpr int kKappa0Rows = 16;
 
 __device__ __forceinline__ float voigt_core0(float a) {
@@ -346,8 +348,9 @@ __global__ void __launch_bounds__(256) k_bounds(int64_t L, size_t ld, int n_sel,
 // deviations of its rank on either side), one pass over the row counts the lines below the bracket
 // and lists the 3 per cent inside (k_med_collect), and the median is selected among those
 // (k_med_select again; from the whole row should the bracket have missed it).  5e6 lines x 80
-// rows: 1.10 ms for three passes, 0.62 ms now.  (Counting and listing in k_kappa0 itself took one
-// global atomic per warp and row: 2.6 -> 11.5 ms.)
+// rows: 1.10 ms for three passes, 0.62 ms over stored values, 0.80 ms over bounds of them (which save
+// 1.85 ms in k_kappa0).  (Counting and listing in k_kappa0 itself took one global atomic per warp
+// and row: 2.6 -> 11.5 ms.)
 constexpr int kMedBins = 2048, kMedThreads = 1024;
 constexpr int64_t kMedSmall = 65536;
 

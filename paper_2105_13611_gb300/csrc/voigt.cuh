@@ -22,6 +22,11 @@
 //        Re[R(z) - R(v)] comes from the sum, written with an explicit factor a
 //        ("region II").  The constants are computed on the host from the
 //        Hermite nodes and weights (mpsa::voigt_init).
+//
+// These tiers (voigt_H) decide the cut windows.  At its points the profile kernel takes cheaper
+// forms where their errors allow (voigt_point): for a <= 0.03 and |z|^2 < 64 a rational form of the
+// two leading terms in a (voigt_small2), from |z|^2 = 64 (a^2 <= 2; 100 above) the asymptotic series
+// of H to |z|^-10, else the core tier.
 #pragma once
 
 #include <cuda_runtime.h>
