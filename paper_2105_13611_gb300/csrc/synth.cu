@@ -332,7 +332,8 @@ __global__ void __launch_bounds__(256) k_bounds(int64_t L, size_t ld, int n_sel,
         const float x2 = r.hc_kT_cm * inv;   // x log2(e)
         const float w = x2 < 0.02f * kLog2E ? x2 * kLn2 : 1.f - ex2_fast(-x2);
         const float lnS = fmaf(kLn2, lg2_fast(w), fmaf(-l.E, r.inv_kT_eV, (q.lnC - q.lnu) + lgk));
-        const float k0 = fmaf(-kLn2, lg2_fast(a + sqrt_fast(fmaf(a, a, 1.2732395f))), lnS + 0.1207822f);   // ln(2/sqrt(pi))
+        float k0 = fmaf(-kLn2, lg2_fast(a + sqrt_fast(fmaf(a, a, 1.2732395f))), lnS + 0.1207822f);   // ln(2/sqrt(pi))
+        if (!(a < 1.0e18f)) k0 = __int_as_float(0x7fc00000);   // a^2 beyond FP32: no bound, the line takes its full terms
         const size_t o = s * ld + i;
         lnaS_up[o] = bound_up(fmaf(kLn2, lg2_fast(a), lnS));
         lnk0_up[o] = bound_up(k0);

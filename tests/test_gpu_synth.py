@@ -355,7 +355,8 @@ def test_shares_of_a_tile_and_wide_tiles(n_lines, N, R, rows):
         assert W <= evg[s] <= W + 8 * len(L) + 16
 
 
-@pytest.mark.parametrize("kind", ["random", "far infrared", "strong damping", "no damping", "no atoms", "sample off"])
+@pytest.mark.parametrize("kind", ["random", "far infrared", "strong damping", "no damping", "no atoms", "sample off",
+                                  "damping beyond FP32"])
 def test_bounds_keep_what_the_full_terms_keep(kind):
     # calls of 3e6 (row, line) pairs or more on a narrow window sort lines out by bounds first; the same rows one by
     # one form every line's full terms.  Continuum and evaluation counts follow from the lines kept and from
@@ -378,6 +379,9 @@ def test_bounds_keep_what_the_full_terms_keep(kind):
         ab[0, 2:5] = 0.0
     elif kind == "sample off":
         L.log_gf[::128] = 9.0
+    elif kind == "damping beyond FP32":
+        L.log_gR[::7] = 45.0
+        L.log_gS[3::11] = 30.0
     ctx, _ = gpu_context(w, lines=L, abund=ab)
     kap, kc, ev = gpu_synth(ctx, w, np.arange(8))
     for s in range(8):
