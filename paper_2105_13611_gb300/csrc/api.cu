@@ -60,28 +60,32 @@ int upload(T** dst, const T* src, size_t n) {
 // leave it), to a relative change of n_e below 1e-14.  The stage weights prod_{i<j} Phi_i / n_e
 // are formed in log space and scaled by their largest value, so no ratio overflows.
 //
-// One warp per row: lane l holds element l (and l + 32 with more than 32 elements, EPL = 2), and
-// every sum over the elements is a warp reduction whose result all lanes share, so the lanes
-// take the same Newton steps.  The FP64 exponentials bound the kernel, so what counts is how many
+// LANES lanes per row: lane l holds the elements l + LANES k, k < EPL, and
+// every sum over the elements is a reduction over the row's lanes whose result they share, so they
+// take the same Newton steps; a warp's rows iterate until the last is done.  The FP64 exponentials bound the kernel, so what counts is how many
 // iterations there are: 41 on average over the T-P table when the search started from the middle of
 // the bracket (n_e near 1e-143) and took a last step that rounds to y itself for one out of the
 // bracket, which restarted a bisection; 6 from the largest n_e that any one element gives by its
-// first ionisation alone, with that step accepted.  11,400 rows (8 compositions x 57 x 25): 7.45 ms
-// before, 0.78 ms now.  The stage loops run over all five stages (ln Phi = -inf where an element has
+// first ionisation alone, with that step accepted.  11,400 rows (8 compositions x 57 x 25) of 17
+// elements: 7.45 ms before, 0.78 ms with a warp per row, 0.43 ms with eight lanes per row.  The stage loops run over all five stages (ln Phi = -inf where an element has
 // no such stage), so that the stage arrays stay in registers.
 
-// sum over the warp, lane 0's result given to every lane (the same bits in all lanes)
-__device__ __forceinline__ double warp_sum(double v) {
-    for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
-    return __shfl_sync(0xffffffffu, v, 0);
+// sum over the row's lanes, the first's result given to all of them (the same bits in all lanes)
+template <int LANES>
+__device__ __forceinline__ double row_sum(double v) {
+#pragma unroll
+    for (int d = LANES / 2; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d, LANES);
+    return __shfl_sync(0xffffffffu, v, 0, LANES);
 }
 
-template <int EPL>
+template <int EPL, int LANES>
 __global__ void __launch_bounds__(128) k_populations(int rows, int n_points, int n_el, const double* __restrict__ el,
                                                      const double* __restrict__ abund, const double* __restrict__ T,
                                                      const double* __restrict__ P, double* __restrict__ pop) {
-    const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (r >= rows) return;   // the same for every lane of the warp
+    const int lane = threadIdx.x % LANES;
+    const int at = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES);
+    if (((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / LANES >= rows) return;   // the whole warp
+    const int r = min(at, rows - 1);   // lanes past the last row repeat it, and store nothing
     const int comp = r / n_points, pt = r % n_points;
     const double t = T[pt], p = P[pt];
     const double kT = kKB * t, eV_kT = kEV / kT;
@@ -92,18 +96,18 @@ __global__ void __launch_bounds__(128) k_populations(int rows, int n_points, int
     double eps_part = 0.0;
 #pragma unroll
     for (int k = 0; k < EPL; ++k) {
-        const int e = lane + 32 * k;
+        const int e = lane + LANES * k;
         eps[k] = e < n_el ? exp((el[e * kElStride + kElLogEps] - 12.0) * 2.302585092994045684) * abund[(size_t)comp * n_el + e] : 0.0;
         eps_part += eps[k];
     }
-    const double eps_sum = warp_sum(eps_part);
+    const double eps_sum = row_sum<LANES>(eps_part);
     const double n_tot = p / kT;
     double frac[EPL];
     double lphi[EPL][kMaxStages - 1];   // ln Phi_{e,j}; -inf beyond the element's stages
     double guess = 1e-300;
 #pragma unroll
     for (int k = 0; k < EPL; ++k) {
-        const int e = lane + 32 * k;
+        const int e = lane + LANES * k;
         frac[k] = 0.0;
 #pragma unroll
         for (int j = 0; j + 1 < kMaxStages; ++j) lphi[k][j] = -INFINITY;
@@ -126,7 +130,8 @@ __global__ void __launch_bounds__(128) k_populations(int rows, int n_points, int
         const double g = 2.0 * an / (1.0 + sqrt(1.0 + 4.0 * (an / ph)));   // ph = 0: an / inf = 0
         guess = fmax(guess, g);
     }
-    for (int d = 16; d > 0; d >>= 1) guess = fmax(guess, __shfl_xor_sync(0xffffffffu, guess, d));
+#pragma unroll
+    for (int d = LANES / 2; d > 0; d >>= 1) guess = fmax(guess, __shfl_xor_sync(0xffffffffu, guess, d));
     // stage weights of the lane's element k at y = ln n_e: w_j = exp(lp_j - max lp),
     // lp_j = sum_{i<j} (ln Phi_i - y)
     auto weights = [&](int k, double y, double* w) -> double {
@@ -153,7 +158,9 @@ __global__ void __launch_bounds__(128) k_populations(int rows, int n_points, int
     double w0[EPL][kMaxStages], y0 = y, ne0 = exp(y);
 #pragma unroll
     for (int k = 0; k < EPL; ++k) weights(k, y0, w0[k]);
+    bool done = false;
     for (int it = 0; it < 400; ++it) {
+        if (__all_sync(0xffffffffu, done)) break;
         if (fabs(y - y0) > 40.0) {
             y0 = y;
             ne0 = exp(y0);
@@ -177,27 +184,29 @@ __global__ void __launch_bounds__(128) k_populations(int rows, int n_points, int
             q += frac[k] * mean;
             v += frac[k] * fmax(s2 * r0 - mean * mean, 0.0);
         }
-        q = warp_sum(q);
-        v = warp_sum(v);
+        q = row_sum<LANES>(q);
+        v = row_sum<LANES>(v);
+        if (done) continue;
         const double g = ne - nn * q, dg = ne * (1.0 + q) + nn * v;   // g(y) and dg/dy
         if (g > 0.0) hi = y; else lo = y;
         double yn = (dg > 0.0) ? y - g / dg : 0.5 * (lo + hi);
         // at the root the step rounds to y itself, an end of the bracket: done, not outside
         if (dg > 0.0 && fabs(g) < 1e-14 * dg) {
             y = yn;
-            break;
+            done = true;
+            continue;
         }
         if (!(yn > lo && yn < hi)) yn = 0.5 * (lo + hi);
         const double dy = yn - y;
         y = yn;
-        if (fabs(dy) < 1e-14 || !(hi - lo > 0.0) || !(y > lo && y < hi && (0.5 * (lo + hi) != lo))) break;
+        done = fabs(dy) < 1e-14 || !(hi - lo > 0.0) || !(y > lo && y < hi && (0.5 * (lo + hi) != lo));
     }
     const double u = exp(y0 - y), ne = exp(y), nn = n_tot - ne;
     double mpart = 0.0, nHI = 0.0;
 #pragma unroll
     for (int k = 0; k < EPL; ++k) {
-        const int e = lane + 32 * k;
-        if (e >= n_el) continue;
+        const int e = lane + LANES * k;
+        if (e >= n_el || at >= rows) continue;
         const double* q = el + e * kElStride;
         const int ns = (int)q[kElStages];
         double w[kMaxStages], s0 = 0.0, up = 1.0;
@@ -221,8 +230,8 @@ __global__ void __launch_bounds__(128) k_populations(int rows, int n_points, int
         }
         mpart += frac[k] * q[kElMass] * kAMU;
     }
-    const double mmean = warp_sum(mpart);
-    if (lane == 0) {
+    const double mmean = row_sum<LANES>(mpart);
+    if (lane == 0 && at < rows) {
         row[kPopT] = t;
         row[kPopP] = p;
         row[kPopNe] = ne;
@@ -236,9 +245,27 @@ __global__ void __launch_bounds__(128) k_populations(int rows, int n_points, int
 int populations_device(int n_el, const double* d_el, const double* d_abund, int n_comp, int n_points,
                        const double* d_T, const double* d_P, double* d_pop, cudaStream_t s) {
     const int rows = n_comp * n_points;
-    const unsigned blocks = (unsigned)(((int64_t)rows * 32 + 127) / 128);
-    if (n_el <= 32) k_populations<1><<<blocks, 128, 0, s>>>(rows, n_points, n_el, d_el, d_abund, d_T, d_P, d_pop);
-    else k_populations<2><<<blocks, 128, 0, s>>>(rows, n_points, n_el, d_el, d_abund, d_T, d_P, d_pop);
+    int dev = 0, sms = 0;
+    MPSA_CUDA_TRY(cudaGetDevice(&dev));
+    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    auto go = [&](auto kernel, int lanes) {
+        const unsigned blocks = (unsigned)(((int64_t)rows * lanes + 127) / 128);
+        kernel<<<blocks, 128, 0, s>>>(rows, n_points, n_el, d_el, d_abund, d_T, d_P, d_pop);
+    };
+    // Eight lanes per row from eight rows per SM on: four rows share what a warp computes once per row, and
+    // 17 elements fill 17 of 24 slots instead of 17 of 32.  Fewer rows are bound by latency, and take a
+    // warp each.  The call with 17 elements, a warp per row and eight lanes: 400 rows 128 and 161 us, 1425 rows
+    // 208 and 168, 11,400 rows 1039 and 719; with 7 elements 133 and 131, 207 and 131, 1033 and 521.
+    if (n_el <= 32 && rows >= 8 * sms) {
+        if (n_el <= 8) go(k_populations<1, 8>, 8);
+        else if (n_el <= 16) go(k_populations<2, 8>, 8);
+        else if (n_el <= 24) go(k_populations<3, 8>, 8);
+        else go(k_populations<4, 8>, 8);
+    } else if (n_el <= 32) {
+        go(k_populations<1, 32>, 32);
+    } else {
+        go(k_populations<2, 32>, 32);
+    }
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
 }

@@ -100,3 +100,25 @@ def test_stage_beyond_the_table_is_rejected():
     with pytest.raises(binding.MpsaError) as e:
         ctx.synth_opacity(w.grid, [0], kap)
     assert e.value.code == binding.MPSA_EINVAL and "stage" in str(e.value)
+
+
+@pytest.mark.parametrize("n_el", [3, 8, 9, 16, 17, 24, 25, 32])
+def test_rows_that_share_a_warp(n_el):
+    # eight lanes per row from eight rows per SM on, with one to four elements a lane: the same points in
+    # calls of 200 rows, which take a warp each.  n_e is solved to 1e-14 in both; sums in another
+    # order and an exponential's argument of up to some hundreds leave 1e-11
+    from paper_2105_13611_gb300 import binding
+    base = wl.eos_table(15)
+    idx = [e if e < base.n else 2 + (e - base.n) % (base.n - 2) for e in range(n_el)]
+    eos = wl.EosTable([base.symbol[e] for e in idx], base.mass_amu[idx], base.log_eps[idx], base.n_stages[idx],
+                      base.chi_eV[idx], base.lnU[idx])
+    n = 3002
+    rng = np.random.default_rng(n_el)
+    T, P = np.exp(rng.uniform(np.log(1500.0), np.log(6e4), n)), 10.0 ** rng.uniform(-3.0, 8.0, n)
+    ctx = binding.Context(0)
+    ctx.set_atmosphere_grid_eos(eos, T, P)
+    many = ctx.get_populations(0, n)
+    for i in range(0, n, 200):
+        ctx.set_atmosphere_grid_eos(eos, T[i:i + 200], P[i:i + 200])
+        few = ctx.get_populations(0, len(T[i:i + 200]))
+        assert np.allclose(many[i:i + 200], few, rtol=1e-11, atol=1e-280)
