@@ -1100,7 +1100,12 @@ __global__ void k_ranges(int n_sel, size_t ld, RowDesc one, const RowDesc* __res
 // centre, a profile is smooth: s_rel H has its nearest singularity (the centre) at three
 // half-lengths from the stretch's middle, so its Chebyshev interpolant converges like
 // 5.8^-n.  With kNodes = 12 nodes the interpolant of 1/v^2 is within 2.3e-8 of it anywhere on
-// the stretch (10 nodes: 6.7e-7, 8: 1.8e-5), below the 1e-6 of the profile formulas.  The sum
+// the stretch (10 nodes: 6.7e-7, 8: 1.8e-5), below the 1e-6 of the profile formulas.  That is
+// so while v is linear in the grid index.  Blueward of a centre v grows like e^x, x = ln lambda, and a
+// stretch that is long in x takes more nodes: 2.1e-7 where it spans 1 in x, 7.9e-7 at 1.5, 3.3e-6 at 2,
+// 3.5e-4 at 3.5 (the interpolant restated in FP64, the centre one span beyond the end).  So a
+// stretch of more than kMaxStretch is not interpolated: tiles of 2048 points below R = 2048, of 4096
+// below 4096, warp parts below an eighth of that.  The sum
 // over such lines is therefore formed at the nodes only, and interpolated once per tile:
 // 12 evaluations per (line, stretch) instead of one per point.
 //
@@ -1108,6 +1113,7 @@ __global__ void k_ranges(int n_sel, size_t ld, RowDesc one, const RowDesc* __res
 // that neither level takes (centre too close, window edge inside, too small |z|) are
 // evaluated point by point.
 constexpr int kNodes = 12;
+constexpr float kMaxStretch = 1.f;   // in ln lambda
 // cos(i pi / 24): node k of a stretch is at (1 + x_k)/2 of its length, x_k = cos((2k + 1) pi / 24),
 // and T_m(x_k) = cos(m (2k + 1) pi / 24)
 __constant__ float c_cos24[48] = {
@@ -1439,6 +1445,8 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int J0, int size, in
     const bool active = Js <= Te;
     const float span0 = (float)(Te - J0), span1 = active ? (float)(Je - Js) : 0.f;
     const float gend0 = expm1f(-span0 * lnq), gend1 = expm1f(-span1 * lnq);
+    // a centre this far from the tile, or the part, is taken by interpolation
+    const float far0 = span0 * lnq <= kMaxStretch ? span0 : INFINITY, far1 = span1 * lnq <= kMaxStretch ? span1 : INFINITY;
     if (lane < kNodes) {
         const float x = 0.5f + 0.5f * c_cos24[2 * lane + 1];
         sG1[warp][lane] = expm1f(-span1 * x * lnq);
@@ -1505,7 +1513,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int J0, int size, in
                     sk = __int_as_float(r1.x) * a * kInvSqrtPi;
                     w = wing(Js, r0.x, f, kv, A, lnq, span1, gend1);
                     inside = inner_covers(r1.y, r1.z, (unsigned)r1.w, Js, Je);
-                    const bool smooth = inside && w.dist > span1;
+                    const bool smooth = inside && w.dist > far1;
                     const bool ra = rational_ok(w, A);
                     rat = smooth && ra;
                     ser = smooth && !ra && w.zmin2 >= (A <= kSeriesA ? kSeriesZ2Low : kSeriesZ2) && w.zmax2 <= 1.0e18f;
@@ -1526,7 +1534,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int J0, int size, in
                 np = 0;
             }
             if (direct) {
-                const bool away = w.dist > span1;
+                const bool away = w.dist > far1;
                 PointRec p;
                 p.ci = (float)(r0.x - Js);
                 p.f = f;
@@ -1593,7 +1601,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int J0, int size, in
                 if (r1.z >= J0 && r1.y <= Te) {
                     const float a = __int_as_float(r0.w), A = a * a;
                     const Wing w = wing(J0, r0.x, __int_as_float(r0.y), __int_as_float(r0.z), A, lnq, span0, gend0);
-                    if (inner_covers(r1.y, r1.z, (unsigned)r1.w, J0, Te) && w.dist > span0 && rational_ok(w, A))
+                    if (inner_covers(r1.y, r1.z, (unsigned)r1.w, J0, Te) && w.dist > far0 && rational_ok(w, A))
                         nodes_rational(w, A, __int_as_float(r1.x) * a * kInvSqrtPi, sG0, acc0);
                     else
                         queue = true;

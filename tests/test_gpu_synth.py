@@ -429,3 +429,31 @@ def test_median_continuum_of_lists_of_every_length(n_lines, kind):
             assert float(kc[s]) == 0.0
         else:
             assert abs(float(kc[s]) / pl.kappa_c - 1) < 1e-5, s
+
+
+@pytest.mark.parametrize("rows", [3, 160])
+@pytest.mark.parametrize("side", [-1, 1])
+@pytest.mark.parametrize("N,R", [(1750, 500.0), (2048, 1000.0), (2048, 2100.0), (1150, 300.0)])
+def test_lines_beyond_a_coarse_grid(N, R, side, rows):
+    # grids of some thousand points that span a factor of 2.7 to 46 in wavelength, and every line beyond
+    # the grid, further away than the grid is long: a profile then grows like e^2x over a tile, which twelve
+    # Chebyshev nodes follow only while the tile is short in ln lambda.  The cut lets every window cover the
+    # grid; opacities lie far below kappa_c, so the tolerance counts on the opacity itself.  Three rows share
+    # each tile out in parts of 256 points, 160 rows take it whole
+    lam0, lnq = 100.0, np.log1p(1 / R)
+    span = (N - 1) * lnq
+    w = wl.config_tiny(n_lines=20, lam=(lam0, lam0 * np.exp((N - 0.5) * lnq)), R=R, seed=71)
+    w.T, w.P, w.cut = np.array([6000.0, 9000.0, 15000.0]), np.array([1e4, 1e-2, 1e7]), 1e-22
+    se, ss = wl.species_table(w.n_metals)
+    edge = lam0 if side < 0 else w.grid.lam1_nm
+    lo, hi = sorted(edge * np.exp(side * (span + d)) for d in (0.05, 0.3))
+    L = wl.linelist(60, len(se), lo, hi, 72)
+    ctx, _ = gpu_context(w, lines=L)
+    kg, kcg, evg = gpu_synth(ctx, w, np.arange(rows) % 3)
+    assert kg.shape[1] == N
+    for s in range(3):
+        pl, k, slack, W = oracle_dense(w, L, w.T[s], w.P[s])
+        assert abs(kcg[s] / pl.kappa_c - 1) < 2e-5
+        bad, err, bound = opacity_violations(kg[s], k, 0.0, slack)
+        assert len(bad) == 0, (s, bad[:5], float((err / k).max()))
+        assert W <= evg[s] <= W + 8 * len(L) + 16
