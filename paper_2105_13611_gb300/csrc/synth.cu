@@ -1036,7 +1036,9 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
             r.srel = o.srel[sL + t];
             r.jlo = w.x;
             r.jhi = w.y;
-            r.in = pack_inner(w.x, w.y, w.z, w.w);
+            // s_rel a beyond FP32 (s_rel near e^88, a > 2): only the general form, which multiplies by H, may
+            // take the line, so no part of the grid counts as inside its window
+            r.in = r.srel * r.a < INFINITY ? pack_inner(w.x, w.y, w.z, w.w) : kNoInner;
             len_sum += (unsigned long long)(w.y - w.x + 1);
             rec[sL + placed[warp][b] + lrank] = r;
             line[sL + placed[warp][b] + lrank] = i;
@@ -1548,7 +1550,9 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int J0, int size, in
                 p.hi = r1.z - Js;
                 p.a = a;
                 int kind = kPtGen;
-                if (away && rational_ok(w, A)) {
+                if (!(sk < INFINITY)) {
+                    // s_rel H is in range where s_rel a is not
+                } else if (away && rational_ok(w, A)) {
                     kind = kPtRat;
                 } else if (A <= kSeriesA && away && w.zmin2 >= kSeriesZ2Low && w.zmax2 <= 1.0e18f) {
                     kind = kPtWing;

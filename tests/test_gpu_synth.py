@@ -457,3 +457,30 @@ def test_lines_beyond_a_coarse_grid(N, R, side, rows):
         bad, err, bound = opacity_violations(kg[s], k, 0.0, slack)
         assert len(bad) == 0, (s, bad[:5], float((err / k).max()))
         assert W <= evg[s] <= W + 8 * len(L) + 16
+
+
+@pytest.mark.parametrize("a0", [1.0, 30.0, 1000.0])
+@pytest.mark.parametrize("N", [60, 2048, 9000])
+def test_strong_damped_lines_at_the_end_of_fp32(N, a0):
+    # s_rel = S / t_p up to e^87 (FP32 ends at e^88.7) with a damping of a0 or so: s_rel a is beyond FP32, the
+    # profile s_rel H is not.  Centres on the grid and up to three tiles beside it, so that lines reach a tile from
+    # every distance; ln S of 100 in FP32 leaves 2e-5
+    R = 5e5
+    lnq = np.log1p(1 / R)
+    w = wl.config_tiny(n_lines=20, lam=(500.0, 500.0 * np.exp((N - 0.5) * lnq)), R=R, seed=73)
+    w.T, w.P = np.array([6000.0]), np.array([1e4])
+    se, ss = wl.species_table(w.n_metals)
+    pad = np.exp(6144 * lnq)
+    L = wl.linelist(40, len(se), 500.0 / pad, w.grid.lam1_nm * pad, 74)
+    el = wl.elements(w.n_metals)
+    L.species[:], L.E_eV[:], L.log_gS[:], L.log_gW[:], L.log_gf[:] = 2, 1.0, -8.0, -8.0, 4.0 + 0.2 * np.sin(np.arange(40))
+    u = np.sqrt(2 * 1.380649e-16 * 6000.0 / (el.mass_amu[se[2]] * 1.66053906660e-24))
+    L.log_gR[:] = np.log10(a0 * 4 * np.pi * u / 500e-7)
+    pl = sy.prepare(L, se, ss, el, w.T[0], w.P[0], w.grid, w.cut, w.kc_factor)
+    w.cut *= np.exp(np.log(pl.terms.S.max() / pl.t) - 87.0)
+    ctx, _ = gpu_context(w, lines=L)
+    kg, kcg, evg = gpu_synth(ctx, w, [0])
+    pl, k, slack, W = oracle_dense(w, L, w.T[0], w.P[0])
+    bad, err, bound = opacity_violations(kg[0], k, 0.0, slack)
+    assert len(bad) == 0 and np.isfinite(kg).all(), (bad[:5], float((err / k).max()))
+    assert W <= evg[0] <= W + 8 * len(L) + 16
