@@ -145,12 +145,11 @@ __global__ void __launch_bounds__(128) k_formal(int D, int N, const float* __res
 //    neighbouring bins and walks the depths from the bottom up, holding one intensity pair per
 //    direction.  The recurrence needs only the layer optical
 //    thicknesses dtau_d = (kappa_d + kappa_{d+1})(m_{d+1} - m_d)/2 and tau_0 = kappa_0 m_0, so
-//    no depth array is kept.  The cells and the Planck function of each bin and depth sit in
-//    shared memory; the per-bin Planck constants come from the host.
+//    no depth array is kept.  The cells and the Planck function of each bin at a window of depths
+//    sit in shared memory; the per-bin Planck constants come from the host.
 constexpr int kBinThreads = 192;            // at most
 constexpr int kBinCols = 2 * kBinThreads;   // sub-bins of a CTA, two per thread
 constexpr int kBinMaxKb = 64;
-
 
 struct DepthCell {
     int r00, dT, dP;        // table row of the lower corner, row offsets to the upper T and P corners
@@ -174,7 +173,8 @@ struct BinCellArgs {
 };
 
 struct BinArgs {
-    int K, ns, D, n_mu, kb;
+    int K, ns, D, n_mu;
+    int kb, Dw;            // bins of a CTA (even), depths in shared memory at a time
     const float2* tab;     // [nT*nP][ns][(K + 1) / 2] bin pairs, FP32
     const float3* pk;      // [K]: c1, ln c1, c2 of B_lambda at the bin centre
     const double* w;       // [ns]
@@ -200,25 +200,40 @@ __device__ __forceinline__ void axis_cell(const double* __restrict__ ax, int n, 
     *f = (x - ax[lo]) / (ax[lo + 1] - ax[lo]);
 }
 
-// a block turns one row's chunk of kTabBins bins in shared memory: coalesced reads and writes
-constexpr int kTabBins = 64;
-__global__ void __launch_bounds__(256) k_bin_table(const double* __restrict__ src, float* __restrict__ dst, int rows,
-                                                   int K, int ns) {
-    __shared__ float t[32][kTabBins + 1];
-    const int Kp = (K + 1) & ~1, chunks = (Kp + kTabBins - 1) / kTabBins;
-    for (long long it = blockIdx.x; it < (long long)rows * chunks; it += gridDim.x) {
-        const int row = (int)(it / chunks), k0 = (int)(it - (long long)row * chunks) * kTabBins;
-        const int nb = min(kTabBins, K - k0), nw = min(kTabBins, Kp - k0);
-        const double* in = src + ((size_t)row * K + k0) * ns;
-        __syncthreads();
-        if (nw > nb)
-            for (int s = threadIdx.x; s < ns; s += blockDim.x) t[s][nb] = 0.f;
-        for (int i = threadIdx.x; i < nb * ns; i += blockDim.x) t[i % ns][i / ns] = (float)in[i];
-        __syncthreads();
-        for (int i = threadIdx.x; i < ns * nw; i += blockDim.x) {
-            const int s = i / nw, k = i - s * nw;
-            dst[((size_t)row * ns + s) * Kp + k0 + k] = t[s][k];
-        }
+// A block turns kr rows' chunk of kc bins (even) in shared memory: coalesced reads and writes, at most
+// kTabTile values (ns <= 32), eight loads a thread in flight.  by_ns: 2^32 / ns rounded up, so that
+// i / ns = umulhi(i, by_ns) for the i < 2^16 here (ns > 1).  57 x 25 x 328 x 12 values: 14.3 us in their
+// order, 24.5 turned by blocks that looped over chunks of 64 bins, 16.5 now.
+constexpr int kTabTile = 2048;
+__global__ void __launch_bounds__(256) k_bin_table(const double* __restrict__ src, float* __restrict__ dst, int rows, int K,
+                                                   int ns, unsigned by_ns, int kc, int kr) {
+    __shared__ float t[kTabTile + 128];   // [kr][ns][kc + 1]
+    const int Kp = (K + 1) & ~1, chunks = (Kp + kc - 1) / kc;
+    const int rb = blockIdx.x / chunks, row0 = rb * kr, k0 = (blockIdx.x - rb * chunks) * kc;
+    const int nb = min(kc, K - k0), np = min(kc, Kp - k0) >> 1, nr = min(kr, rows - row0);
+    const int per = nb * ns, n = nr * per;   // values of a row, of the block (kr = 1 or the whole rows: contiguous)
+    const double* in = src + ((size_t)row0 * K + k0) * ns;
+    double v[kTabTile / 256];
+#pragma unroll
+    for (int u = 0; u < kTabTile / 256; ++u) {
+        const int i = u * 256 + threadIdx.x;
+        v[u] = i < n ? __ldg(in + i) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kTabTile / 256; ++u) {
+        const int i = u * 256 + threadIdx.x;
+        if (i >= n) break;
+        const int k = ns > 1 ? (int)__umulhi((unsigned)i, by_ns) : i, s = i - k * ns;   // bin over all rows, sub-bin
+        const int r = nr > 1 ? k / nb : 0;
+        t[(r * ns + s) * (kc + 1) + k - r * nb] = (float)v[u];
+    }
+    __syncthreads();
+    const bool odd = 2 * np > nb;   // the padded bin
+    float2* out = reinterpret_cast<float2*>(dst + (size_t)row0 * ns * Kp + k0);
+    for (int i = threadIdx.x; i < nr * ns * np; i += 256) {
+        const int q = i / np, p = i - q * np;   // q: row and sub-bin
+        const float* c = t + q * (kc + 1) + 2 * p;
+        out[(size_t)q * (Kp >> 1) + p] = make_float2(c[0], odd && p == np - 1 ? 0.f : c[1]);
     }
 }
 
@@ -259,76 +274,91 @@ __global__ void k_bin_cells(BinCellArgs a) {
 // warp's layers are mostly all thin or all thick and one of the two forms runs.
 // 1024 rays x 80 depths x 328 bins x 12 sub-bins x 5 directions: 1.53 ms one sub-bin per thread,
 // 1.37 ms in pairs within a bin, 1.35 ms in pairs across bins, 1.20 ms with the two short forms
-// below.  64 registers and 5 CTAs per SM: 6 CTAs (1.33 ms) reload the constants, and one choice
-// of form for all directions of a layer takes the same time with 93 registers.
+// below, 1.17 ms with CTAs of whole warps (bin_chunk).  64 registers and 10 CTAs of three warps per SM.  One
+// choice of form for all directions of a layer takes the same time with 93 registers.
+// A thread of two sub-bins and all directions is a long chain, and half as many threads share a CTA's
+// Planck function.  So a call of few rays spreads its bins and its directions over more CTAs (blockIdx.z
+// counts groups of NMU directions), adds threads for the Planck function, and a deep ray keeps a
+// window of its depths in shared memory.  Kernel times of one sub-bin per thread, of pairs without and with
+// this, in us: one ray of 80 depths, 328 x 12, 5 directions 49, 47, 27; 328 x 1 50, 86, 24; 8 rays of 256
+// depths, 16 directions 221, 268, 168; 1024 rays of 200 depths, 328 x 1, 1 direction 565, 1777, 431; 40 x 12,
+// 5 directions 213, 249, 167.
 template <int NMU>
 __global__ void __launch_bounds__(kBinThreads) k_bin_intensity(BinArgs a) {
     extern __shared__ __align__(16) unsigned char bsm[];
-    DepthCell* cell = reinterpret_cast<DepthCell*>(bsm);                      // [D]
-    float* Sb = reinterpret_cast<float*>(cell + a.D);                         // [D][kb]
-    float* part = Sb + (size_t)a.kb * a.D;                                    // [ns][kb][NMU]
-    const int ray = blockIdx.y, k0 = blockIdx.x * a.kb, tid = threadIdx.x;
-    const DepthCell* rc = a.cells + (size_t)ray * a.D;
-    for (int d = tid; d < a.D; d += blockDim.x) cell[d] = rc[d];
-    __syncthreads();
-    // Planck function at each bin centre and depth
-    for (int i = tid; i < a.kb * a.D; i += blockDim.x) {
-        const int d = i / a.kb, k = k0 + i - d * a.kb;
-        float S = 0.f;
-        if (k < a.K) {
-            const float3 p = a.pk[k];
-            S = planck_f32(p.x, p.y, p.z, cell[d].T);
+    DepthCell* cell = reinterpret_cast<DepthCell*>(bsm);                      // [Dw]
+    float* Sb = reinterpret_cast<float*>(cell + a.Dw);                        // [Dw][kb]
+    float* part = reinterpret_cast<float*>(bsm);                              // [ns][kb][NMU], after the last depth
+    const int ray = blockIdx.y, k0 = blockIdx.x * a.kb, tid = threadIdx.x, D = a.D;
+    const int q0 = blockIdx.z * NMU, n_mu = min(NMU, a.n_mu - q0);   // the CTA's directions
+    const DepthCell* rc = a.cells + (size_t)ray * D;
+    // the window of depths in shared memory: cells and Planck function of the depths w0..top
+    int w0;
+    auto fill = [&](int top) {
+        w0 = max(0, top - a.Dw + 1);
+        const int n = top - w0 + 1;
+        for (int d = tid; d < n; d += blockDim.x) cell[d] = rc[w0 + d];
+        __syncthreads();
+        for (int i = tid; i < a.kb * n; i += blockDim.x) {
+            const int d = i / a.kb, k = k0 + i - d * a.kb;
+            float S = 0.f;
+            if (k < a.K) {
+                const float3 p = a.pk[k];
+                S = planck_f32(p.x, p.y, p.z, cell[d].T);
+            }
+            Sb[i] = S;
         }
-        Sb[i] = S;
-    }
-    __syncthreads();
+        __syncthreads();
+    };
+    fill(D - 1);
 
     const int pairs = a.kb / 2, s = tid / pairs, pr = tid - s * pairs;
-    if (s < a.ns && k0 + 2 * pr < a.K) {
-    float2 I[NMU];
+    const bool act = s < a.ns && k0 + 2 * pr < a.K;
+    const int np = (a.K + 1) >> 1;
+    const float2* __restrict__ tab = a.tab + (size_t)s * np + (k0 >> 1) + pr;
+    const DepthCell* cw = cell - w0;                                            // depth d: cw[d]
+    const float2* Sw = reinterpret_cast<const float2*>(Sb) + pr - w0 * pairs;   // depth d: Sw[d * pairs]
+    // a depth's four table values (offsets below 2^31, checked on the host), and its opacity from them
+    auto load = [&](int d, float2 (&v)[4]) {
+        const int r = cw[d].r00, dT = cw[d].dT, dP = cw[d].dP;
+        v[0] = __ldg(tab + r);
+        v[1] = __ldg(tab + r + dP);
+        v[2] = __ldg(tab + r + dT);
+        v[3] = __ldg(tab + r + dT + dP);
+    };
+    auto kappa = [&](int d, const float2 (&v)[4]) -> float2 {
+        const DepthCell& c = cw[d];
+        float2 k = ffma2(dup2(c.w00), v[0], dup2(c.kc));
+        k = ffma2(dup2(c.w01), v[1], k);
+        k = ffma2(dup2(c.w10), v[2], k);
+        return ffma2(dup2(c.w11), v[3], k);
+    };
+    const float2 one = dup2(1.f), minus = dup2(-1.f);
+    const float2 nl2 = dup2(-1.4426950408889634f);   // e^{-x} = 2^{x * (-log2 e)}
+    float2 I[NMU], mu[NMU], rmu[NMU];                // per direction the intensity, mu and 1/mu
 #pragma unroll
-    for (int q = 0; q < NMU; ++q) I[q] = make_float2(0.f, 0.f);
-        float2 mu[NMU], rmu[NMU];   // per direction mu and 1/mu
-        const float2 nl2 = dup2(-1.4426950408889634f);   // e^{-x} = 2^{x * (-log2 e)}
-#pragma unroll
-        for (int q = 0; q < NMU; ++q) {
-            const float m = q < a.n_mu ? a.mu[q] : 1.f, r = 1.f / m;
-            mu[q] = dup2(m);
-            rmu[q] = dup2(r);
-        }
-        const int np = (a.K + 1) >> 1;
-        const float2* __restrict__ tab = a.tab + (size_t)s * np + (k0 >> 1) + pr;
-        const float2* __restrict__ Sp = reinterpret_cast<const float2*>(Sb) + pr;   // depth d: Sp[d * pairs]
-        // a depth's four table values (offsets below 2^31, checked on the host), and its opacity from them
-        auto load = [&](int d, float2 (&v)[4]) {
-            const int r = cell[d].r00, dT = cell[d].dT, dP = cell[d].dP;
-            v[0] = __ldg(tab + r);
-            v[1] = __ldg(tab + r + dP);
-            v[2] = __ldg(tab + r + dT);
-            v[3] = __ldg(tab + r + dT + dP);
-        };
-        auto kappa = [&](int d, const float2 (&v)[4]) -> float2 {
-            const DepthCell& c = cell[d];
-            float2 k = ffma2(dup2(c.w00), v[0], dup2(c.kc));
-            k = ffma2(dup2(c.w01), v[1], k);
-            k = ffma2(dup2(c.w10), v[2], k);
-            return ffma2(dup2(c.w11), v[3], k);
-        };
-        const float2 one = dup2(1.f), minus = dup2(-1.f);
-        const int D = a.D;
-        float2 v[4];
+    for (int q = 0; q < NMU; ++q) {
+        const float m = q < n_mu ? a.mu[q0 + q] : 1.f, r = 1.f / m;
+        mu[q] = dup2(m);
+        rmu[q] = dup2(r);
+        I[q] = make_float2(0.f, 0.f);
+    }
+    float2 v[4], k_hi, k_lo, dtau, S_hi, Sd;
+    if (act) {
         load(D - 1, v);
-        float2 k_hi = kappa(D - 1, v);
+        k_hi = kappa(D - 1, v);
         load(D - 2, v);
-        float2 k_lo = kappa(D - 2, v);
-        float2 dtau = fmul2(fadd2(k_lo, k_hi), dup2(0.5f * (cell[D - 1].m - cell[D - 2].m)));
-        float2 S_hi = Sp[(D - 1) * pairs], Sd = Sp[(D - 2) * pairs];
-        {
-            const float2 dS = make_float2((S_hi.x - Sd.x) / dtau.x, (S_hi.y - Sd.y) / dtau.y);
+        k_lo = kappa(D - 2, v);
+        dtau = fmul2(fadd2(k_lo, k_hi), dup2(0.5f * (cw[D - 1].m - cw[D - 2].m)));
+        S_hi = Sw[(D - 1) * pairs], Sd = Sw[(D - 2) * pairs];
+        const float2 dS = make_float2((S_hi.x - Sd.x) / dtau.x, (S_hi.y - Sd.y) / dtau.y);
 #pragma unroll
-            for (int q = 0; q < NMU; ++q) I[q] = ffma2(mu[q], dS, S_hi);
-        }
-        for (int d = D - 2;; --d) {
+        for (int q = 0; q < NMU; ++q) I[q] = ffma2(mu[q], dS, S_hi);
+    }
+    for (int top = D - 2;;) {
+        // the window's layers: d needs the depth below it in the window, but for the last
+        const int end = w0 > 0 ? w0 + 1 : 0;
+        for (int d = top; act && d >= end; --d) {
             if (d > 0) load(d - 1, v);   // in flight during the layer's directions
             // layer d .. d+1 of optical thickness dtau; per direction x = dtau / mu, e = e^{-x}:
             //   I <- I e + S_d (1 - e) + dS (1 - e(1 + x)) / x,  dS = S_{d+1} - S_d.
@@ -367,11 +397,20 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_intensity(BinArgs a) {
             if (d == 0) break;
             k_hi = k_lo;
             k_lo = kappa(d - 1, v);
-            dtau = fmul2(fadd2(k_lo, k_hi), dup2(0.5f * (cell[d].m - cell[d - 1].m)));
+            dtau = fmul2(fadd2(k_lo, k_hi), dup2(0.5f * (cw[d].m - cw[d - 1].m)));
             S_hi = Sd;
-            Sd = Sp[(d - 1) * pairs];
+            Sd = Sw[(d - 1) * pairs];
         }
-        const float2 tau0 = fmul2(k_lo, dup2(cell[0].m));
+        if (w0 == 0) break;
+        top = w0;
+        __syncthreads();
+        fill(top);
+        cw = cell - w0;
+        Sw = reinterpret_cast<const float2*>(Sb) + pr - w0 * pairs;
+    }
+    const float2 tau0 = fmul2(k_lo, dup2(cw[0].m));
+    __syncthreads();   // the window is free for the sub-bins' intensities
+    if (act) {
         const float2 ws = dup2((float)a.w[s]);
 #pragma unroll
         for (int q = 0; q < NMU; ++q) {
@@ -385,14 +424,14 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_intensity(BinArgs a) {
     __syncthreads();
     // sum over the sub-bins in order
     const bool bad = a.bad[ray] != 0;
-    for (int i = tid; i < a.kb * a.n_mu; i += blockDim.x) {
-        const int b = i / a.n_mu, q = i - b * a.n_mu, kk = k0 + b;
+    for (int i = tid; i < a.kb * n_mu; i += blockDim.x) {
+        const int b = i / n_mu, q = i - b * n_mu, kk = k0 + b;
         if (kk >= a.K) continue;
         float acc = 0.f;
         for (int t = 0; t < a.ns; ++t) acc += part[(t * a.kb + b) * NMU + q];
-        a.out[((size_t)ray * a.n_mu + q) * a.K + kk] = bad ? __int_as_float(0x7fc00000) : acc;
+        a.out[((size_t)ray * a.n_mu + q0 + q) * a.K + kk] = bad ? __int_as_float(0x7fc00000) : acc;
     }
-    if (tid == 0 && a.status && blockIdx.x == 0) a.status[ray] = bad ? 1 : 0;
+    if (tid == 0 && a.status && blockIdx.x == 0 && blockIdx.z == 0) a.status[ray] = bad ? 1 : 0;
 }
 
 unsigned g_spec_init = 0;
@@ -486,13 +525,35 @@ extern "C" int synth_spectrum(mpsa_ctx* ctx, const mpsa_atmos* atm, const mpsa_l
 namespace mpsa {
 namespace {
 
-constexpr size_t kBinSmemMax =
-    (size_t)kMaxDepth * sizeof(DepthCell) + (size_t)kBinMaxKb * kMaxDepth * sizeof(float) +
-    (size_t)kBinCols * kMaxMu * sizeof(float);
+constexpr size_t kBinSmemMax = 227 * 1024;
+constexpr int kBinWarps = 8;     // warps of an SM below which directions are shared out over CTAs
+constexpr int kPlanckWarps = 24; // warps of an SM below which CTAs take more threads for the Planck function
+
+// Bins of a CTA: an even number up to kBinCols sub-bins.  The warps that the busiest SM is given decide,
+// whatever they hold (a quarter of a warp stands for what a CTA costs beside its warps); up to
+// eight of them, two per scheduler, take as long as one, and then the spread over the SMs.
+int bin_chunk(int K, int ns, long long n_rays, int sms) {
+    int best = 2;
+    double least = 1e300;
+    for (int kb = 2; kb <= kBinMaxKb && kb * ns <= kBinCols; kb += 2) {
+        const long long ctas = (K + kb - 1) / kb * n_rays;
+        const double load = (double)((ctas + sms - 1) / sms) * ((ns * kb / 2 + 31) / 32 + 0.25);
+        const double cost = std::max(load, 8.0) + 0.01 * load;
+        if (cost < least) {
+            least = cost;
+            best = kb;
+        }
+    }
+    return best;
+}
 
 template <int NMU>
-int bin_launch(const BinArgs& a, int n_rays, cudaStream_t st) {
+int bin_launch(BinArgs a, int n_rays, int sms, cudaStream_t st) {
     static unsigned attr_set = 0;   // one bit per device
+    static const int regs = [] {
+        cudaFuncAttributes fa = {};
+        return cudaFuncGetAttributes(&fa, k_bin_intensity<NMU>) == cudaSuccess ? std::max(fa.numRegs, 1) : 128;
+    }();
     int dev = 0;
     MPSA_CUDA_TRY(cudaGetDevice(&dev));
     if (!(attr_set & (1u << (dev & 31)))) {
@@ -500,10 +561,17 @@ int bin_launch(const BinArgs& a, int n_rays, cudaStream_t st) {
                                            (int)kBinSmemMax));
         attr_set |= 1u << (dev & 31);
     }
-    const size_t smem = (size_t)a.D * sizeof(DepthCell) + (size_t)a.kb * a.D * sizeof(float) +
-                        (size_t)kBinCols * NMU * sizeof(float);
-    const dim3 grid((a.K + a.kb - 1) / a.kb, n_rays);
-    k_bin_intensity<NMU><<<grid, (a.ns * (a.kb / 2) + 31) / 32 * 32, smem, st>>>(a);
+    const dim3 grid((a.K + a.kb - 1) / a.kb, n_rays, (a.n_mu + NMU - 1) / NMU);
+    // the threads of the sub-bins, and more for the Planck function while the SMs have few warps
+    const long long ctas = (long long)grid.x * grid.y * grid.z;
+    int warps = (a.ns * (a.kb / 2) + 31) / 32;
+    warps = std::max(warps, (int)std::min<long long>(kBinThreads / 32, kPlanckWarps * sms / ctas));
+    // as many depths at a time as leave shared memory for the CTAs that the registers allow
+    const int fit = std::max(1, std::min(32, 65536 / (regs * 32 * warps)));
+    const size_t per_depth = sizeof(DepthCell) + a.kb * sizeof(float);
+    a.Dw = (int)std::min<size_t>(a.D, std::max<size_t>(16, (kBinSmemMax / fit - 1024) / per_depth));
+    const size_t smem = std::max(a.Dw * per_depth, (size_t)a.ns * a.kb * NMU * sizeof(float));
+    k_bin_intensity<NMU><<<grid, warps * 32, smem, st>>>(a);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
 }
@@ -577,9 +645,11 @@ extern "C" int odf_intensity(mpsa_ctx* ctx, const mpsa_odf_table* tab, int32_t n
     MPSA_CUDA_TRY(cudaMemcpyAsync(dw, tab->widths, ns * sizeof(double), cudaMemcpyHostToDevice, st));
     MPSA_CUDA_TRY(cudaMemcpyAsync(dmu, hmu.data(), n_mu * sizeof(float), cudaMemcpyHostToDevice, st));
     MPSA_CUDA_TRY(cudaMemsetAsync(dbad, 0, n_rays * sizeof(int), st));
-    const int rows = tab->nT * tab->nP;
-    const long long parts = (long long)rows * ((K + kTabBins) / kTabBins);
-    k_bin_table<<<(unsigned)std::min<long long>(parts, 4096), 256, 0, st>>>(tab->odf, dtab, rows, K, ns);
+    // whole rows, as many as fit a block, or equal chunks of a row
+    const int rows = tab->nT * tab->nP, Kp = (K + 1) & ~1, most = (kTabTile / ns) & ~1, chunks = (Kp + most - 1) / most;
+    const int kc = ((Kp + chunks - 1) / chunks + 1) & ~1, kr = chunks > 1 ? 1 : std::max(1, std::min(128 / ns, most / Kp));
+    const unsigned by_ns = (unsigned)(((1ull << 32) + ns - 1) / ns);
+    k_bin_table<<<(unsigned)((rows + kr - 1) / kr * ((Kp + kc - 1) / kc)), 256, 0, st>>>(tab->odf, dtab, rows, K, ns, by_ns, kc, kr);
     MPSA_CUDA_TRY(cudaGetLastError());
     BinCellArgs ca;
     ca.nT = tab->nT;
@@ -602,7 +672,6 @@ extern "C" int odf_intensity(mpsa_ctx* ctx, const mpsa_odf_table* tab, int32_t n
     a.ns = ns;
     a.D = n_depth;
     a.n_mu = n_mu;
-    a.kb = std::min(kBinCols / ns, kBinMaxKb) & ~1;   // even, at least 12 (ns <= 32)
     a.tab = reinterpret_cast<const float2*>(dtab);
     a.pk = dpk;
     a.w = dw;
@@ -612,16 +681,28 @@ extern "C" int odf_intensity(mpsa_ctx* ctx, const mpsa_odf_table* tab, int32_t n
     a.out = I_out;
     a.status = ray_status;
     prof_mark(ctx, MPSA_KERNEL_BINS, st);
-    switch (n_mu) {
-        case 1: r = bin_launch<1>(a, n_rays, st); break;
-        case 2: r = bin_launch<2>(a, n_rays, st); break;
-        case 3: r = bin_launch<3>(a, n_rays, st); break;
-        case 4: r = bin_launch<4>(a, n_rays, st); break;
-        case 5: r = bin_launch<5>(a, n_rays, st); break;
-        case 6: r = bin_launch<6>(a, n_rays, st); break;
-        case 7: r = bin_launch<7>(a, n_rays, st); break;
-        case 8: r = bin_launch<8>(a, n_rays, st); break;
-        default: r = bin_launch<16>(a, n_rays, st); break;
+    int dev = 0, sms = 0;
+    MPSA_CUDA_TRY(cudaGetDevice(&dev));
+    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // directions of a thread: all (in two groups above eight, which take 135 registers at once), or fewer
+    // while that leaves an SM no more than kBinWarps warps
+    int nq = 1;
+    for (; nq < n_mu; ++nq) {
+        const int z = (n_mu + nq - 1) / nq;
+        a.kb = bin_chunk(K, ns, (long long)n_rays * z, sms);
+        if ((long long)((K + a.kb - 1) / a.kb) * n_rays * z * ((ns * a.kb / 2 + 31) / 32) <= kBinWarps * sms) break;
+    }
+    if (nq > 8) nq = (n_mu + 1) / 2;
+    a.kb = bin_chunk(K, ns, (long long)n_rays * ((n_mu + nq - 1) / nq), sms);
+    switch (nq) {
+        case 1: r = bin_launch<1>(a, n_rays, sms, st); break;
+        case 2: r = bin_launch<2>(a, n_rays, sms, st); break;
+        case 3: r = bin_launch<3>(a, n_rays, sms, st); break;
+        case 4: r = bin_launch<4>(a, n_rays, sms, st); break;
+        case 5: r = bin_launch<5>(a, n_rays, sms, st); break;
+        case 6: r = bin_launch<6>(a, n_rays, sms, st); break;
+        case 7: r = bin_launch<7>(a, n_rays, sms, st); break;
+        default: r = bin_launch<8>(a, n_rays, sms, st); break;
     }
     prof_mark(ctx, MPSA_KERNEL_BINS, st);
     // pageable host-to-device copies are staged before cudaMemcpyAsync returns,

@@ -84,6 +84,24 @@ def test_parity_bin_counts(K, ns):
         assert ok, (r, rel)
 
 
+@pytest.mark.parametrize("rays,D,K,ns,n_mu", [(1, 256, 64, 1, 16), (2, 200, 131, 3, 9), (1, 2, 328, 12, 5), (40, 33, 64, 12, 7),
+                                             (4000, 97, 64, 1, 2), (1500, 21, 64, 1, 5), (900, 256, 65, 4, 1),
+                                             (300, 256, 40, 12, 10)])
+def test_parity_spread_of_the_work(rays, D, K, ns, n_mu):
+    """Few rays share their bins and directions out over more CTAs; many deep rays of small bins keep a window of
+    16 and more depths in shared memory at a time (up to nine windows here)."""
+    lt, lp, odf, kc, lam = wl.odf_table_synthetic(3, 4, K, ns, seed=60 + K + ns)
+    w = np.full(ns, 1.0 / ns)
+    mus = np.linspace(1.0, 0.1, n_mu)
+    m, T, P = wl.ray_atmospheres(rays, D, seed=61)
+    g, st = run_gpu(lt, lp, odf, kc, lam, w, m, T, P, mus, status=True)
+    assert (st == 0).all() and np.isfinite(g).all()
+    for r in {0, rays // 2, rays - 1}:
+        o = oracle(lt, lp, odf, kc, lam, w, m[r], T[r], P[r], mus)
+        ok, rel = close(g[r], o)
+        assert ok, (r, rel)
+
+
 def test_isothermal_is_planck():
     lt, lp, odf, kc, lam = wl.odf_table_synthetic(5, 4, 33, 12, seed=35)
     D = 50
