@@ -1550,9 +1550,7 @@ __device__ __forceinline__ void tile_body(const RowDesc& g, int J0, int size, in
                 p.hi = r1.z - Js;
                 p.a = a;
                 int kind = kPtGen;
-                if (!(sk < INFINITY)) {
-                    // s_rel H is in range where s_rel a is not
-                } else if (away && rational_ok(w, A)) {
+                if (away && sk < INFINITY && rational_ok(w, A)) {   // (sk beyond FP32: a > 2, so the next two don't take it)
                     kind = kPtRat;
                 } else if (A <= kSeriesA && away && w.zmin2 >= kSeriesZ2Low && w.zmax2 <= 1.0e18f) {
                     kind = kPtWing;
