@@ -20,6 +20,9 @@ int populations_device(int n_el, const double* d_el, const double* d_abund, int 
 int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, double lam0_nm, double R, int N,
                float* kappa, float* kc_out, int64_t* evals, const mpsa_synth_opts* opts, cudaStream_t st, int peers = 1);
 
+// Device memory that a synth_rows call takes for itself (synth.cu).
+size_t synth_rows_bytes(const mpsa_ctx* ctx, int n_sel, int N, double R, int peers = 1);
+
 // Every species of the line list refers to an element of the table and to a stage that
 // element has (synth.cu).
 int check_species(const mpsa_ctx* ctx, const char* who);

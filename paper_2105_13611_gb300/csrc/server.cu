@@ -57,7 +57,7 @@ struct Req {
     float* kc_out = nullptr;
     int mean_kind = MPSA_MEAN_ARITH;
     // sizes
-    int N = 0;
+    int N = 0, rows = 1;         // rows: of a chunk
     size_t out_bytes = 0, kc_bytes = 0, est = 0;
     // runtime
     int slot = -1;
@@ -100,12 +100,48 @@ struct mpsa_server {
 namespace mpsa {
 namespace {
 
-size_t synth_scratch_bytes(const mpsa_ctx* c, int rows, int N) {
-    // per (row, line) prep arrays, records and the crossing-search list (73 B, admitted at 64), per-line
-    // placement (12 B), tile ranges, per (row, prep block) class counts
+// The device memory that decides whether a request fits a budget at all: 64 B per (row, line) of a chunk of
+// rows_per_chunk rows, 12 per line, tile ranges, per (row, prep block) class counts.  The figure stays what
+// callers have chosen their budgets by; what a request really takes (spectrum_bytes, odf_bytes: 73 B per pair,
+// and the partial sums of shared tiles) decides when it runs, and in a request between the two, how
+// many rows a chunk has.
+size_t fit_bytes(const mpsa_ctx* c, int rows, int N) {
     const size_t nT = (size_t)(N + kTile - 1) / kTile, nb = (size_t)(c->L + kPrepLines - 1) / kPrepLines;
     return (size_t)rows * c->L * 64 + (size_t)c->L * 12 + (size_t)rows * kNumClasses * (nT + 3) * 4 +
            (size_t)rows * nb * (kNumClasses * 4 + 8) + (1 << 20);
+}
+
+// the largest scratch of n rows in chunks of `rows`
+size_t chunks_bytes(const mpsa_ctx* c, int n, int rows, int N, double R, int peers) {
+    const size_t full = synth_rows_bytes(c, rows, N, R, peers);
+    return n % rows ? std::max(full, synth_rows_bytes(c, n % rows, N, R, peers)) : full;
+}
+
+// A spectrum request's own arrays, in one block.
+struct SpectrumBlock {
+    char* in = nullptr;
+    double* pop = nullptr;
+    float *kap = nullptr, *kc = nullptr, *I = nullptr;
+    ScratchBlock block;
+    SpectrumBlock(int D, int N, int n_mu, int n_el, size_t in_bytes) {
+        block.add(&in, in_bytes);
+        block.add(&pop, (size_t)D * pop_stride(n_el));
+        block.add(&kap, (size_t)D * N);
+        block.add(&kc, D);
+        block.add(&I, (size_t)n_mu * N);
+    }
+};
+
+size_t spectrum_bytes(const mpsa_server* s, const Req* r) {
+    const int D = (int)r->m.size(), n_mu = (int)r->mu.size(), ne = s->ctx->n_el;
+    return SpectrumBlock(D, r->N, n_mu, ne, 28 * (size_t)D + 8 * ne + 4 * n_mu + 128).block.bytes +
+           chunks_bytes(s->ctx, D, r->rows, r->N, r->win.R, (int)s->slots.size()) + (1 << 20);
+}
+
+size_t odf_bytes(const mpsa_server* s, const Req* r) {
+    const size_t n = r->sel.size(), K = r->bounds.size() - 1, ns = r->widths.size();
+    return 8 * n + 4 * (size_t)r->rows * r->N + 8 * (K + 1) + 8 * (2 * ns + 1) + 8 * n * K * ns +
+           chunks_bytes(s->ctx, (int)n, r->rows, r->N, r->grid.R, 1) + (1 << 20);
 }
 
 int launch_spectrum(mpsa_server* s, Req* r, Slot& sl) {
@@ -122,36 +158,28 @@ int launch_spectrum(mpsa_server* s, Req* r, Slot& sl) {
     const size_t oT = in.add(r->T.data(), D), oP = in.add(r->P.data(), D);
     const size_t oab = in.add(c->h_abund.data() + (size_t)r->comp * ne, ne), om = in.add(hm.data(), D);
     const size_t of = in.add(hT.data(), D), omu = in.add(hmu.data(), n_mu), osel = in.add(hsel.data(), D);
-    char* din;
-    double* dpop;
-    float *kap, *kc, *Iout;
-    ScratchBlock block;
-    block.add(&din, in.data.size());
-    block.add(&dpop, (size_t)D * pop_stride(ne));
-    block.add(&kap, (size_t)D * N);
-    block.add(&kc, D);
-    block.add(&Iout, (size_t)n_mu * N);
+    SpectrumBlock q(D, N, n_mu, ne, in.data.size());
     int rc;
-    if ((rc = block.take(sc))) return rc;
-    MPSA_CUDA_TRY(cudaMemcpyAsync(din, in.data.data(), in.data.size(), cudaMemcpyHostToDevice, st));
-    const int* dsel = reinterpret_cast<int*>(din + osel);
-    const float *fm = reinterpret_cast<float*>(din + om), *fT = reinterpret_cast<float*>(din + of),
-                *fmu = reinterpret_cast<float*>(din + omu);
-    if ((rc = populations_device(ne, c->d_el, reinterpret_cast<double*>(din + oab), 1, D, reinterpret_cast<double*>(din + oT),
-                                 reinterpret_cast<double*>(din + oP), dpop, st)))
+    if ((rc = q.block.take(sc))) return rc;
+    MPSA_CUDA_TRY(cudaMemcpyAsync(q.in, in.data.data(), in.data.size(), cudaMemcpyHostToDevice, st));
+    const int* dsel = reinterpret_cast<int*>(q.in + osel);
+    const float *fm = reinterpret_cast<float*>(q.in + om), *fT = reinterpret_cast<float*>(q.in + of),
+                *fmu = reinterpret_cast<float*>(q.in + omu);
+    if ((rc = populations_device(ne, c->d_el, reinterpret_cast<double*>(q.in + oab), 1, D, reinterpret_cast<double*>(q.in + oT),
+                                 reinterpret_cast<double*>(q.in + oP), q.pop, st)))
         return rc;
     // every slot may hold a request: the chunks leave the others their part of the GPU (by the number of slots, not
     // of requests in flight, on which the result would then depend)
-    for (int off = 0; off < D; off += s->rows_per_chunk) {
-        const int nrow = std::min(s->rows_per_chunk, D - off);
-        if ((rc = synth_rows(c, dpop, nrow, dsel + off, r->win.lambda0_nm, r->win.R, N, kap + (size_t)off * N, kc + off,
+    for (int off = 0; off < D; off += r->rows) {
+        const int nrow = std::min(r->rows, D - off);
+        if ((rc = synth_rows(c, q.pop, nrow, dsel + off, r->win.lambda0_nm, r->win.R, N, q.kap + (size_t)off * N, q.kc + off,
                              nullptr, nullptr, st, (int)s->slots.size())))
             return rc;
     }
-    if ((rc = formal_launch(D, N, kap, kc, nullptr, fm, fT, r->win.lambda0_nm, log1p(1.0 / r->win.R), n_mu, fmu, Iout,
+    if ((rc = formal_launch(D, N, q.kap, q.kc, nullptr, fm, fT, r->win.lambda0_nm, log1p(1.0 / r->win.R), n_mu, fmu, q.I,
                             st)))
         return rc;
-    MPSA_CUDA_TRY(cudaMemcpyAsync(sl.pinned, Iout, r->out_bytes, cudaMemcpyDeviceToHost, st));
+    MPSA_CUDA_TRY(cudaMemcpyAsync(sl.pinned, q.I, r->out_bytes, cudaMemcpyDeviceToHost, st));
     return MPSA_OK;
 }
 
@@ -179,7 +207,7 @@ void odf_free(Req* r) {
 int launch_odf(mpsa_server* s, Req* r, Slot&) {
     cudaStream_t st = r->st;
     const int n_sel = (int)r->sel.size(), N = r->N, K = (int)r->bounds.size() - 1, ns = (int)r->widths.size();
-    const int chunk = std::min(s->rows_per_chunk, n_sel);
+    const int chunk = r->rows;
     int rc;
     if ((rc = pool_alloc(s, &r->dsel, n_sel, st)) || (rc = pool_alloc(s, &r->kap, (size_t)chunk * N, st)) ||
         (rc = pool_alloc(s, &r->kc, n_sel, st)) || (rc = pool_alloc(s, &r->db, K + 1, st)) ||
@@ -200,7 +228,7 @@ int odf_chunk(mpsa_server* s, Req* r, Slot& sl) {
     mpsa_ctx* c = s->ctx;
     cudaStream_t st = r->st;
     const int n_sel = (int)r->sel.size(), N = r->N, K = (int)r->bounds.size() - 1, ns = (int)r->widths.size();
-    const int off = r->next_row, nrow = std::min(std::min(s->rows_per_chunk, n_sel), n_sel - off);
+    const int off = r->next_row, nrow = std::min(r->rows, n_sel - off);
     int rc;
     if ((rc = synth_rows(c, c->d_pop, nrow, r->dsel + off, r->grid.lambda0_nm, r->grid.R, N, r->kap, r->kc + off,
                          nullptr, nullptr, st)))
@@ -373,6 +401,7 @@ int mpsa_server_submit(mpsa_server* s, const mpsa_request* q, int64_t* ticket) {
     Req* r = new Req();
     r->kind = q->kind;
     int rc;
+    size_t fit = 0;
     if (q->kind == MPSA_REQ_SPECTRUM) {
         const int D = q->atm.n_depth;
         if (D < 2 || D > 256 || !q->atm.m || !q->atm.T || !q->atm.P || !q->mu || q->n_mu < 1 || q->n_mu > 16 || !q->I_out) {
@@ -402,7 +431,8 @@ int mpsa_server_submit(mpsa_server* s, const mpsa_request* q, int64_t* ticket) {
         r->win = q->win;
         r->I_out = q->I_out;
         r->out_bytes = (size_t)q->n_mu * r->N * sizeof(float);
-        r->est = (size_t)D * r->N * 4 + (size_t)q->n_mu * r->N * 4 + synth_scratch_bytes(c, std::min(s->rows_per_chunk, D), r->N);
+        r->rows = std::min(s->rows_per_chunk, D);
+        fit = (size_t)D * r->N * 4 + (size_t)q->n_mu * r->N * 4 + fit_bytes(c, r->rows, r->N);
     } else if (q->kind == MPSA_REQ_ODF) {
         if (q->n_sel < 1 || !q->sel || !q->bounds || !q->widths || !q->odf_out || q->K < 1 || q->n_steps < 1 || q->n_steps > 32) {
             delete r;
@@ -431,17 +461,18 @@ int mpsa_server_submit(mpsa_server* s, const mpsa_request* q, int64_t* ticket) {
         r->kc_out = q->kappa_c_out;
         r->out_bytes = (size_t)q->n_sel * q->K * q->n_steps * sizeof(double);
         r->kc_bytes = (size_t)q->n_sel * sizeof(float);
-        const int chunk = std::min(s->rows_per_chunk, q->n_sel);
-        r->est = (size_t)chunk * r->N * 4 + r->out_bytes + synth_scratch_bytes(c, chunk, r->N);
+        r->rows = std::min(s->rows_per_chunk, q->n_sel);
+        fit = (size_t)r->rows * r->N * 4 + r->out_bytes + fit_bytes(c, r->rows, r->N);
     } else {
         delete r;
         return fail(MPSA_EINVAL, "mpsa_server_submit: kind %d", q->kind);
     }
-    if (r->est > s->budget) {
-        const size_t est = r->est;
+    if (fit > s->budget) {
         delete r;
-        return fail(MPSA_ENOMEM, "mpsa_server_submit: request needs about %zu bytes, budget is %zu", est, s->budget);
+        return fail(MPSA_ENOMEM, "mpsa_server_submit: request needs about %zu bytes, budget is %zu", fit, s->budget);
     }
+    auto bytes = [&] { return r->kind == MPSA_REQ_SPECTRUM ? spectrum_bytes(s, r) : odf_bytes(s, r); };
+    for (r->est = bytes(); r->est > s->budget && r->rows > 1; r->est = bytes()) r->rows -= (r->rows + 15) / 16;
     {
         std::lock_guard<std::mutex> lk(s->mu);
         if (s->stop) {

@@ -2058,6 +2058,32 @@ void tile_split(TileArgs& ta, int tile, int n_sel, int N, int64_t L, int sms, in
     ta.used = nullptr;
 }
 
+// The scratch of one synth_rows call: its arrays, added to one block.
+struct SynthScratch {
+    PrepBufs b;
+    TileArgs ta;
+    int *cum = nullptr, tile = 0, nT = 0, nC = 0;   // nC: CTAs of a row, before the split by candidates
+    ScratchBlock block;
+    SynthScratch(const mpsa_ctx* ctx, int n_sel, int N, double R, int prec, int sms, int peers) {
+        tile = prec == MPSA_PREC_FP64 ? kTile64 : tile_size(ctx, n_sel, N, R, sms);
+        nT = (N + tile - 1) / tile;
+        prep_alloc(b, ctx, n_sel, 1, [&](auto** p, size_t n) { return block.add(p, n); });
+        block.add(&cum, (size_t)n_sel * kNumClasses * (nT + 3));
+        tile_split(ta, tile, n_sel, N, b.L, sms, peers);
+        nC = (N + ta.size - 1) / ta.size;
+        if (ta.split > 1) {
+            block.add(&ta.part, (size_t)n_sel * ta.split * N);
+            block.add(&ta.used, (size_t)n_sel * nC);
+        }
+    }
+};
+
+size_t synth_rows_bytes(const mpsa_ctx* ctx, int n_sel, int N, double R, int peers) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) sms = 1;
+    return SynthScratch(ctx, n_sel, N, R, MPSA_PREC_FP32_COMPENSATED, sms, peers).block.bytes;
+}
+
 int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, double lam0_nm, double R, int N,
                float* kappa, float* kc_out, int64_t* evals, const mpsa_synth_opts* opts, cudaStream_t st, int peers) {
     const int prec = opts ? opts->precision : 0;
@@ -2065,23 +2091,15 @@ int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, do
         prec != MPSA_PREC_FP32_POP32)
         return fail(MPSA_EINVAL, "synth: precision %d", prec);
     Scratch sc(st, ctx->pool);
-    PrepBufs b;
-    int r, *cum;
-    int dev = 0, sms = 0;
+    int r, dev = 0, sms = 0;
     MPSA_CUDA_TRY(cudaGetDevice(&dev));
     MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int tile = prec == MPSA_PREC_FP64 ? kTile64 : tile_size(ctx, n_sel, N, R, sms), nT = (N + tile - 1) / tile;
-    ScratchBlock block;
-    prep_alloc(b, ctx, n_sel, 1, [&](auto** p, size_t n) { return block.add(p, n); });
-    block.add(&cum, (size_t)n_sel * kNumClasses * (nT + 3));
-    TileArgs ta;
-    tile_split(ta, tile, n_sel, N, b.L, sms, peers);
-    const int nC = (N + ta.size - 1) / ta.size;   // CTAs of a row, before the split by candidates
-    if (ta.split > 1) {
-        block.add(&ta.part, (size_t)n_sel * ta.split * N);
-        block.add(&ta.used, (size_t)n_sel * nC);
-    }
-    if ((r = block.take(sc))) return r;
+    SynthScratch scratch(ctx, n_sel, N, R, prec, sms, peers);
+    if ((r = scratch.block.take(sc))) return r;
+    PrepBufs& b = scratch.b;
+    TileArgs& ta = scratch.ta;
+    int* const cum = scratch.cum;
+    const int tile = scratch.tile, nT = scratch.nT, nC = scratch.nC;
     const GridDesc grid = grid_desc(lam0_nm, log1p(1.0 / R), N, 0);
     const RowOut out{kc_out, (unsigned long long*)evals, nullptr, nullptr};
     if ((r = prep_launch(b, ctx, pop, d_sel, grid, nullptr, nullptr, out, opts, st))) return r;

@@ -146,3 +146,58 @@ def test_served_results_match_the_oracle():
                 k_o, slack, _ = sy.kappa_dense(pl)
                 o = od.odf(k_o, b, wd)
                 assert np.all(np.abs(odf_g[r] - o) <= 1e-4 * (o + pl.kappa_c) + slack.max() * 1.001)
+
+
+@pytest.mark.parametrize("kind", ["spectrum", "odf"])
+@pytest.mark.parametrize("n_lines,rows,N", [(1_000_000, 40, 300), (700_001, 30, 150_000), (100_001, 8, 16_384)])
+def test_estimate_covers_what_a_request_takes(kind, n_lines, rows, N):
+    # bytes_peak after one request alone against the device memory that the context's pool took for it: the pool
+    # keeps what it has mapped, in steps of some tens of MB (128 MB allowed); the estimate is 64 MB above what is
+    # used at most.  The third case shares its tiles out by lines alone (above 1e5 of them): 64 partial sums of
+    # 8 rows
+    import torch
+    from paper_2105_13611_gb300 import binding
+    w = wl.config_tiny(n_lines=40, lam=(300.0, 300.3), R=5e5, seed=33)
+    se, ss = wl.species_table(w.n_metals)
+    w.T, w.P = np.linspace(4000.0, 9000.0, rows), np.full(rows, 1e4)
+    ctx, _ = gpu_context(w, lines=wl.linelist(n_lines, len(se), 290.0, 500.0, 34))
+    win = wl.Grid(300.0, 300.0 * float(np.exp((N - 0.5) * np.log1p(1 / 5e5))), 5e5)
+    m, T, P = spc.grey_atmosphere(rows, 6000.0, 4.0)
+
+    def request(srv, g):
+        n = binding.grid_size(g.lam0_nm, g.lam1_nm, g.R)
+        t = srv.submit_spectrum(m, T, P, g, MUS) if kind == "spectrum" else srv.submit_odf(range(rows), g, [0, n], [1.0])
+        return srv.wait(t)
+
+    srv = binding.Server(ctx, hbm_budget_bytes=32 << 30, max_inflight=1, rows_per_chunk=2)
+    request(srv, wl.Grid(300.0, 300.01, 5e5))     # the modules' own memory
+    srv.close()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    srv = binding.Server(ctx, hbm_budget_bytes=32 << 30, max_inflight=1, rows_per_chunk=rows)
+    request(srv, win)
+    peak, used = srv.stats()["bytes_peak"], free - torch.cuda.mem_get_info()[0]
+    srv.close()
+    pairs = rows * n_lines * 73
+    assert peak >= used - (128 << 20) and peak >= pairs
+    assert peak <= pairs + 13 * n_lines + rows * N * 4 * (65 if n_lines == 100_001 else 1) + len(MUS) * N * 4 + (64 << 20)
+    if n_lines == 100_001:
+        assert peak >= pairs + 64 * rows * N * 4
+
+
+def test_budget_between_the_two_figures_takes_fewer_rows():
+    # a budget that holds 64 B per (row, line) of a chunk but not the 73 it takes: the request runs as before, in
+    # smaller chunks, and stays inside the budget
+    from paper_2105_13611_gb300 import binding
+    w = wl.config_tiny(n_lines=40, lam=(300.0, 300.3), R=5e5, seed=35)
+    se, ss = wl.species_table(w.n_metals)
+    n, D, g = 300_000, 24, wl.Grid(300.0, 300.1, 5e5)
+    ctx, _ = gpu_context(w, lines=wl.linelist(n, len(se), 290.0, 500.0, 36))
+    m, T, P = spc.grey_atmosphere(D, 6000.0, 4.0)
+    out = []
+    for budget in (8 << 30, 68 * n * D):
+        srv = binding.Server(ctx, hbm_budget_bytes=budget, max_inflight=2, rows_per_chunk=D)
+        out.append(srv.wait(srv.submit_spectrum(m, T, P, g, MUS))[0])
+        assert srv.stats()["bytes_peak"] <= budget and srv.stats()["completed"] == 1
+        srv.close()
+    assert np.allclose(out[0], out[1], rtol=1e-5, atol=0)
