@@ -75,7 +75,6 @@ struct Target {
     unsigned long long iv_lt;    // exact sum (group units) of the group's values below the prefix range
     long long cnt_in;            // values inside the current prefix range
     unsigned prefix;             // bits resolved so far
-    int slot;                    // distinct-prefix slot at the current level
     int total;                   // 1 when k >= n (S is the total)
 };
 
@@ -383,7 +382,8 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
     __shared__ unsigned tbits[kL1Bins / 32];                 // bitmap of the targets' level-1 bins
     __shared__ unsigned long long gsum[256];
     __shared__ double gpre[257];
-    __shared__ Target tg[kMaxTargets];
+    __shared__ Target tg[kMaxTargets];          // CLUSTER: written by CTA 0 between two merges only, the others copy it
+    __shared__ int tslot[kMaxTargets];          // distinct-prefix slot of each target at the current level
     __shared__ unsigned dpre[kMaxTargets];
     __shared__ int n_distinct, n_cand;
     __shared__ unsigned s_zero;
@@ -498,7 +498,6 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         // the floor of the correctly rounded product whatever the compiler contracts
         t.k = (long long)floor(__dmul_rn(cw[lane + 1], (double)n));
         t.total = t.k >= n;
-        t.slot = -1;
         t.prefix = 0;
         t.cnt_lt = 0;
         t.cnt_in = 0;
@@ -554,7 +553,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
             const bool leader = act && first == lane;
             const unsigned lm = __ballot_sync(kFull, leader);
             const int slot = __popc(lm & ((1u << first) - 1u));
-            if (act) tg[lane].slot = slot;
+            if (act) tslot[lane] = slot;
             long long in = 0;
             if (leader) {
                 dpre[slot] = p;
@@ -639,7 +638,8 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         for (int t = warp; t < nt && rank == 0; t += kOdfWarps) {
             if (tg[t].total) continue;
             Target tt = tg[t];
-            const Hist hs{h2.c + tt.slot * kL2Bins, h2.hi + tt.slot * kL2Bins, h2.lo + tt.slot * kL2Bins};
+            const int at = tslot[t] * kL2Bins;
+            const Hist hs{h2.c + at, h2.hi + at, h2.lo + at};
             resolve_warp(tt, hs, wb, sh, lane);
             if (lane == 0) tg[t] = tt;
         }
