@@ -504,16 +504,25 @@ int mpsa_profile_read(mpsa_ctx* ctx, int kernel, double* total_ms, int64_t* laun
 /*
  * mpsa_voigt -- the Voigt function H(v, a) = Re w(v + i a) of the line profile
  * (paper Sect. 2.1: argument v = (nu - nu0)/dnu_D, damping a = gamma/(4 pi dnu_D)),
- * evaluated on the device as the profile kernel evaluates it at a grid point, for
- * accuracy tests of its tiers.
+ * evaluated on the device by the functions of the kernels, for accuracy tests.
  *   v, a (device, double[n]): arguments (a > 0; the sign of v is ignored).
- *   precision: MPSA_PREC_FP64 evaluates the FP64 tiers in double; any other value
- *     rounds v and a to FP32 and evaluates the FP32 tiers (far: rational or
- *     one-level continued fraction; then the asymptotic series; core: a rational
- *     form in v for a <= 0.03, else shifted 12-point Gauss-Hermite).
+ *   precision: MPSA_PREC_FP64 evaluates the FP64 tiers in double.  Everything else
+ *     rounds v and a to FP32: MPSA_VOIGT_POINT as the profile kernel takes a grid
+ *     point on its own (the asymptotic series from |z| = 10, inside it a rational form
+ *     in v for a <= 0.03, else the tiers); MPSA_VOIGT_PAIR and MPSA_VOIGT_NODE its
+ *     packed forms for points beside a core (the series, a^2 <= 2, from |z| = 8) and
+ *     for the nodes of a wing (far rational form, series), and the form of a point
+ *     where these are not taken; MPSA_VOIGT_CENTRE H(0, a) as the line terms take it (v
+ *     is ignored); any other value the tiers that decide the cut windows (far, from
+ *     |z| = 40: rational or one-level continued fraction; mid, from 6: five-level
+ *     continued fraction; core: shifted 12-point Gauss-Hermite).
  *   out (device, double[n]): H, widened from FP32 for the FP32 tiers.
  * Stream-ordered.  Errors: MPSA_EINVAL, MPSA_ECUDA.
  */
+#define MPSA_VOIGT_POINT  16
+#define MPSA_VOIGT_PAIR   17
+#define MPSA_VOIGT_NODE   18
+#define MPSA_VOIGT_CENTRE 19
 int mpsa_voigt(mpsa_ctx* ctx, const double* v, const double* a, int64_t n, int32_t precision, double* out,
                void* stream);
 

@@ -16,6 +16,7 @@ LIB_PATH = os.environ.get("MPSA_LIBRARY") or os.path.join(HERE, "_lib", "libmpsa
 
 MPSA_OK, MPSA_EINVAL, MPSA_ENOMEM, MPSA_ECUDA, MPSA_ESTATE, MPSA_ETIMEOUT = 0, -1, -2, -3, -4, -5
 PREC_FP32_COMPENSATED, PREC_FP32_NAIVE, PREC_FP64, PREC_FP32_POP32 = 0, 1, 2, 3
+VOIGT_POINT, VOIGT_PAIR, VOIGT_NODE, VOIGT_CENTRE = 16, 17, 18, 19
 MEAN_ARITH, MEAN_GEOM = 0, 1
 
 EXPORTED = ["mpsa_create", "mpsa_destroy", "mpsa_last_error", "mpsa_version", "mpsa_grid_size",
@@ -344,7 +345,8 @@ class Context:
                                         _dev(kappa_out), _stream(stream)))
 
     def voigt(self, v, a, out, precision=0, stream=None):
-        """H(v, a) on the device as the kernels evaluate it; v, a, out: device float64 tensors."""
+        """H(v, a) on the device as the kernels evaluate it (precision: PREC_FP64, VOIGT_*, else the FP32 tiers of
+        the cut windows); v, a, out: device float64 tensors."""
         _check(self.lib.mpsa_voigt(self.h, _dev(v), _dev(a), int(v.numel()), int(precision), _dev(out),
                                    _stream(stream)))
 

@@ -1841,11 +1841,32 @@ __global__ void __launch_bounds__(256) k_tiles64(Tile64Args g) {
 
 int g_init_mask = 0;
 
-__global__ void k_voigt_eval(int64_t n, const double* __restrict__ v, const double* __restrict__ a, bool fp64,
+// H in the FP32 form of `which` (mpsa_voigt)
+__device__ float voigt_form(float v, float a, int which) {
+    const float A = a * a, Z = fmaf(v, v, A);
+    if (which == MPSA_VOIGT_CENTRE) return A >= 36.f ? voigt_H(0.f, a) : voigt_core0(a);
+    if (which == MPSA_VOIGT_PAIR && A <= kSeriesA && Z >= kSeriesZ2Low && Z <= 1.0e18f)
+        return pair_series(make_float2(v, v), A, a * kInvSqrtPi, series_k2(A), series_k3(A), series_k4(A)).x;
+    if (which == MPSA_VOIGT_NODE) {
+        // every node of the stretch at v; a line that is interpolated passes the cut there, so s_rel (here a
+        // power of two) is what makes s_rel H one or more
+        const Wing w{v, 0.f, 0.f, Z, Z};
+        const float G[kNodes] = {}, ka = a * kInvSqrtPi, srel = exp2f(ceilf(log2f(Z / ka)));
+        float2 acc[kNodes / 2] = {};
+        if (rational_ok(w, A)) nodes_rational(w, A, srel * ka, G, acc);
+        else if (A <= kSeriesA && Z >= kSeriesZ2Low) nodes_series<true>(w, A, srel * ka, G, acc);
+        else if (A > kSeriesA && Z >= kSeriesZ2 && Z <= 1.0e18f) nodes_series<false>(w, A, srel * ka, G, acc);
+        else return voigt_point(v, a);
+        return acc[0].x / srel;
+    }
+    return which >= MPSA_VOIGT_POINT && which <= MPSA_VOIGT_NODE ? voigt_point(v, a) : voigt_H(v, a);
+}
+
+__global__ void k_voigt_eval(int64_t n, const double* __restrict__ v, const double* __restrict__ a, int which,
                              double* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    out[i] = fp64 ? voigt_H64(v[i], a[i]) : (double)voigt_point((float)v[i], (float)a[i]);
+    out[i] = which == MPSA_PREC_FP64 ? voigt_H64(v[i], a[i]) : (double)voigt_form((float)v[i], (float)a[i], which);
 }
 
 }  // namespace
@@ -2613,7 +2634,7 @@ int mpsa_voigt(mpsa_ctx* ctx, const double* v, const double* a, int64_t n, int32
     const int threads = 256;
     const int64_t blocks = (n + threads - 1) / threads;
     if (blocks > 0x7fffffff) return fail(MPSA_EINVAL, "mpsa_voigt: n = %lld too large", (long long)n);
-    k_voigt_eval<<<(unsigned)blocks, threads, 0, (cudaStream_t)stream>>>(n, v, a, precision == MPSA_PREC_FP64, out);
+    k_voigt_eval<<<(unsigned)blocks, threads, 0, (cudaStream_t)stream>>>(n, v, a, precision, out);
     MPSA_CUDA_TRY(cudaGetLastError());
     return MPSA_OK;
 }

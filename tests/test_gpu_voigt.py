@@ -81,3 +81,50 @@ def test_weakly_damped_and_series_forms_against_oracle():
     rel = np.abs(device_H(ctx, vf, af, binding.PREC_FP32_COMPENSATED) / H(vf, af) - 1)
     assert rel.max() <= FP32_RTOL, (rel.max(), vf[np.argmax(rel)], af[np.argmax(rel)])
     ctx.close()
+
+
+@pytest.mark.parametrize("form", ["POINT", "PAIR", "NODE"])
+def test_profile_forms_against_oracle(form):
+    # the forms of the profile kernel beside those of the cut windows (the two tests above): points on their own,
+    # packed pairs, wing nodes, over every damping and hugging |z|^2 = 64 and 100 (the series' edges, a^2 <= 2 and
+    # above), a = 3e-4, 0.03 and sqrt 2, and the rational form's switch
+    from paper_2105_13611_gb300 import binding
+    ctx = binding.Context(0)
+    e = 1e-6
+    a = np.r_[np.geomspace(1e-16, 1e3, 115), [x * (1 + s * e) for x in (3e-4, 0.03, np.sqrt(2.0)) for s in (-1, 1)]]
+    v = np.r_[0.0, np.linspace(1e-3, 10.2, 1200), np.geomspace(10.0, 1e7, 300)]
+    V, A = (x.ravel() for x in np.meshgrid(v, a, indexing="ij"))
+    edge = [(np.sqrt(z * f - x * x), x) for x in a for z in (64.0, 100.0, 1e3 * np.sqrt(2 + 2 * x * x))
+            for f in (1 - e, 1 + e) if z * f > x * x]
+    V, A = np.r_[V, [x for x, _ in edge]], np.r_[A, [y for _, y in edge]]
+    vf, af = V.astype(np.float32).astype(np.float64), A.astype(np.float32).astype(np.float64)
+    rel = np.abs(device_H(ctx, vf, af, getattr(binding, "VOIGT_" + form)) / H(vf, af) - 1)
+    assert rel.max() <= FP32_RTOL, (rel.max(), vf[np.argmax(rel)], af[np.argmax(rel)])
+    ctx.close()
+
+
+def test_line_centre_against_oracle_and_tiers():
+    # H(0, a) of the line terms: within the tiers' error of the oracle, and within rounding of the core tier, which
+    # forms the two poles of a pair apart (terms of one sign, some 30 roundings: 2e-6)
+    from paper_2105_13611_gb300 import binding
+    ctx = binding.Context(0)
+    a = np.r_[np.geomspace(1e-16, 1e4, 4000), [x * (1 + s * 1e-6) for x in (2.0, 6.0) for s in (-1, 1)]]
+    a = a.astype(np.float32).astype(np.float64)
+    g, t = (device_H(ctx, v, a, p) for v, p in ((np.full_like(a, 7.0), binding.VOIGT_CENTRE), (np.zeros_like(a), 0)))
+    assert np.abs(g / H(np.zeros_like(a), a) - 1).max() <= FP32_RTOL
+    assert np.abs(g / t - 1).max() <= 2e-6
+    ctx.close()
+
+
+def test_cut_window_tiers_of_weak_damping():
+    # the tiers that decide the cut windows, down to the damping of low-pressure lines (test_fp32_tiers above starts
+    # at a = 1e-5): where e^{-v^2} makes up H its argument's rounding costs v^2 2^-24, 2e-6 at v^2 = 36
+    from paper_2105_13611_gb300 import binding
+    ctx = binding.Context(0)
+    a = np.geomspace(1e-16, 1e-5, 40)
+    v = np.r_[0.0, np.linspace(1e-3, 10.2, 2500), np.geomspace(10.0, 1e4, 200)]
+    V, A = (x.ravel() for x in np.meshgrid(v, a, indexing="ij"))
+    vf, af = V.astype(np.float32).astype(np.float64), A.astype(np.float32).astype(np.float64)
+    rel = np.abs(device_H(ctx, vf, af, binding.PREC_FP32_COMPENSATED) / H(vf, af) - 1)
+    assert rel.max() <= FP32_RTOL, (rel.max(), vf[np.argmax(rel)], af[np.argmax(rel)])
+    ctx.close()
