@@ -203,7 +203,8 @@ __device__ __forceinline__ float voigt_series(float t, float A) {
 // rational function of V of degree 8/9, fitted by iteratively weighted least squares to D1 in 40
 // digits on 0 <= V <= 100, with the errors measured against the H of a = 0.03 (7.2e-8); q3 and q5
 // share its denominator (their terms' errors 1.1e-7 and 3e-8).  In FP32 the error is that of
-// the quotient and e^{-V}, 6e-7.  Below a = 3e-4 the a^2 terms are under 1e-7.  The 12-point sum of
+// the quotient and e^{-V}, 6e-7.  Up to a = 3e-4 of the terms in a^2 and above only e^{-V} (1 - 2 a^2 V) counts
+// (1.3e-6 of H at v = 2.95; the others 1e-7), and it rides in the exponent's correction.  The 12-point sum of
 // voigt_core takes about 150 FP32 operations a point, this 33 (a <= 3e-4) or 50, half of them
 // instructions.
 constexpr float kSmallA = 0.03f, kTinyA = 3e-4f;
@@ -236,7 +237,8 @@ __device__ __forceinline__ float2 voigt_small2(float2 v, float A, float a) {
     den = ffma2(V, den, dup2(7.589423457e-01f));
     den = ffma2(V, den, dup2(1.f));
     const float2 hi = fmul2(V, dup2(1.44269504f));
-    const float2 lo = ffma2(V, dup2(-1.44269504f), hi);              // hi - V log2e (its rounding)
+    const float l2e = TINY ? fmaf(2.f * A, 1.44269504f, 1.44269504f) : 1.44269504f;
+    const float2 lo = ffma2(V, dup2(-l2e), hi);                      // hi - V log2e (its rounding, TINY: 2 a^2 V too)
     const float cx = fmaf(lo.x, 0.69314718f, fmaf(-v.x, v.x, V.x));   // ... and that of V
     const float cy = fmaf(lo.y, 0.69314718f, fmaf(-v.y, v.y, V.y));
     const float ex = ex2_approx(-hi.x), ey = ex2_approx(-hi.y);

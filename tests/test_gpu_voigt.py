@@ -128,3 +128,16 @@ def test_cut_window_tiers_of_weak_damping():
     rel = np.abs(device_H(ctx, vf, af, binding.PREC_FP32_COMPENSATED) / H(vf, af) - 1)
     assert rel.max() <= FP32_RTOL, (rel.max(), vf[np.argmax(rel)], af[np.argmax(rel)])
     ctx.close()
+
+
+def test_weak_damping_has_no_step():
+    # a <= 3e-4 inside |z| = 10 (the terms in a^3 and a^4 left out, 8e-8 in all) and just above it: the error of
+    # ex2.approx (2^-22), of the reciprocal and of some FP32 roundings of the quotient leave less than 1e-6
+    from paper_2105_13611_gb300 import binding
+    ctx = binding.Context(0)
+    a = np.r_[np.geomspace(1e-8, 3e-4, 40), 3.001e-4, 4e-4]
+    V, A = (x.ravel() for x in np.meshgrid(np.linspace(0.0, 9.99, 5000), a, indexing="ij"))
+    vf, af = V.astype(np.float32).astype(np.float64), A.astype(np.float32).astype(np.float64)
+    rel = np.abs(device_H(ctx, vf, af, binding.VOIGT_POINT) / H(vf, af) - 1)
+    assert rel.max() <= 1e-6, (rel.max(), vf[np.argmax(rel)], af[np.argmax(rel)])
+    ctx.close()
