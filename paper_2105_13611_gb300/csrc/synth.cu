@@ -1946,9 +1946,11 @@ int prep_launch(const PrepBufs& b, const mpsa_ctx* ctx, const double* pop, const
     MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const bool small = L <= kMedSmall;
     // Bounds first, where a grid covers less than a quarter of the list's range: a line that is kept
-    // takes its terms after its bounds; and where there are enough pairs to repay two more launches.  80 depths x 5e6 lines, 0.2 per cent of the range: 8.80 -> 7.09 ms for the call,
-    // 63 depths, 5 per cent: 20.4 -> 19.4 ms; two rows over the whole range 14.0 -> 14.1 ms (so not there);
-    // 8 rows x 5e5 lines a call, eight requests at once: 11.4 -> 10.9 ms, 8 x 66,753 lines 4.86 -> 5.04 ms.
+    // takes its terms after its bounds; and where there are enough pairs to repay two more launches.  80 depths x 5e6
+    // lines, 0.2 per cent of the range: 8.80 -> 7.09 ms for the call, 63 depths, 5 per cent: 20.4 -> 19.4 ms; two rows
+    // over the whole range 14.0 -> 14.1 ms (so not there); 8 rows x 5e5 lines a call, eight requests at once: 11.4 ->
+    // 10.9 ms, 8 x 66,753 lines 4.86 -> 5.04 ms.  Batches always: 8 rows x 1e6 lines on grids over the whole range
+    // take 3.95 ms with bounds and 3.93 without, over 41 per cent of it 1.92 and 1.94 ms.
     const bool bounds = !small && (int64_t)n_sel * L >= 3000000 && (d_grids || 4.0 * grid.N * grid.lnq64 < ctx->log_span);
     {
         // ln S, a, ln kappa0 and the median; the record array, not in use yet, holds the listed lines
