@@ -71,7 +71,7 @@ __device__ __forceinline__ void layer_weights(float x, float e, float rx, float*
 // the layers' optical thicknesses, so nothing is kept per depth: with tau and S of every
 // depth in local memory, and three exponentials per layer and direction, 80 depths x 7300 points x 5
 // directions took 134 us, now 54 us.  All directions of a point share its Planck function
-// (NMU = 5); a window too narrow to fill the GPU spreads them over threads (NMU = 1).
+// (NMU = 5); a window too narrow to fill the GPU spreads them over threads (NMU = 1; formal_launch).
 template <int NMU>
 __global__ void __launch_bounds__(128) k_formal(int D, int N, const float* __restrict__ kappa,
                                                 const float* __restrict__ kc, const float* __restrict__ kcont,
@@ -441,7 +441,13 @@ unsigned g_spec_init = 0;
 int formal_launch(int D, int N, const float* kappa, const float* kc, const float* kcont, const float* m, const float* T,
                   double lam0_nm, double lnq, int n_mu, const float* mu, float* I_out, cudaStream_t st) {
     const int blocks = (N + 127) / 128;
-    if (n_mu > 1 && blocks >= 152)   // a CTA of 128 points per SM at least
+    int dev = 0, sms = 0;
+    MPSA_CUDA_TRY(cudaGetDevice(&dev));
+    MPSA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // One direction per thread while that gives an SM fewer than seven CTAs.  The 80-depth call with one and with
+    // five directions per thread: 25,000 points, 5 directions 512 and 517 us, 7 directions 528 and 518; 40,000 points, 2
+    // directions 605 and 617, 3 directions 614 and 615, 5 directions 641 and 620; 80,000 points, 2 directions 727 and 731.
+    if ((long long)blocks * n_mu >= 7ll * sms)
         k_formal<5><<<dim3(blocks, (n_mu + 4) / 5), 128, 0, st>>>(D, N, kappa, kc, kcont, m, T, lam0_nm, lnq, n_mu, mu, I_out);
     else
         k_formal<1><<<dim3(blocks, n_mu), 128, 0, st>>>(D, N, kappa, kc, kcont, m, T, lam0_nm, lnq, n_mu, mu, I_out);

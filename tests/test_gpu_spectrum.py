@@ -76,3 +76,28 @@ def test_spectrum_parity_realistic(Teff, logg, D, win, lines_lam, n_lines):
     o, dI = spc.spectrum_at(L, se, ss, el, m, T, P, g, MUS, js)
     err = np.abs(I[:, js].astype(np.float64) - o)
     assert np.all(err <= 1e-4 * o + dI * 1.001), (err / o).max()
+
+
+@pytest.mark.parametrize("n_mu", [1, 2, 4, 6, 7, 16])
+@pytest.mark.parametrize("N", [8_400, 20_000, 70_000])
+def test_spectrum_parity_direction_counts(N, n_mu):
+    # from seven CTAs of 128 points and one direction per SM on, a thread takes five directions, and the last group may
+    # be short: from 8,500 points with 16 directions, 68,100 with two
+    import torch
+    from paper_2105_13611_gb300 import binding
+    lam1 = 300.0 * np.exp((N - 0.5) * np.log1p(1 / 5e5))
+    w = wl.config_tiny(n_lines=400, lam=(299.0, lam1 + 1.0), R=5e5, seed=25)
+    ctx, L = gpu_context(w)
+    m, T, P = spc.grey_atmosphere(20, 5772.0, 4.44)
+    win, mus = wl.Grid(300.0, lam1, 5e5), np.linspace(1.0, 0.1, n_mu)
+    assert binding.grid_size(win.lam0_nm, win.lam1_nm, win.R) == N
+    out = torch.full((n_mu, N), -1.0, device="cuda")
+    ctx.synth_spectrum(m, T, P, win, mus, out)
+    torch.cuda.synchronize()
+    I = out.cpu().numpy().astype(np.float64)
+    assert (I > 0).all()
+    js = np.unique(np.r_[0, N - 1, np.random.default_rng(n_mu).integers(0, N, 20)])
+    el = wl.elements(w.n_metals)
+    se, ss = wl.species_table(w.n_metals)
+    o, dI = spc.spectrum_at(L, se, ss, el, m, T, P, win, mus, js)
+    assert np.all(np.abs(I[:, js] - o) <= 1e-4 * o + dI * 1.001)
