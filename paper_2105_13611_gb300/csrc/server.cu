@@ -169,7 +169,9 @@ int launch_spectrum(mpsa_server* s, Req* r, Slot& sl) {
                                  reinterpret_cast<double*>(q.in + oP), q.pop, st)))
         return rc;
     // every slot may hold a request: the chunks leave the others their part of the GPU (by the number of slots, not
-    // of requests in flight, on which the result would then depend)
+    // of requests in flight, on which the result would then depend).  It costs a request that is alone on a server of
+    // eight slots, 40 depths, against one slot: 20,000 lines 1 nm 0.95 -> 1.21 ms, 5 nm 1.22 -> 1.99, 30 nm 2.02 -> 2.79;
+    // 2000 lines up to 5 nm and 5e5 lines up to 30 nm nothing.
     for (int off = 0; off < D; off += r->rows) {
         const int nrow = std::min(r->rows, D - off);
         if ((rc = synth_rows(c, q.pop, nrow, dsel + off, r->win.lambda0_nm, r->win.R, N, q.kap + (size_t)off * N, q.kc + off,

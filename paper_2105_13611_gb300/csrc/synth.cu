@@ -2062,11 +2062,15 @@ int tile_size(const mpsa_ctx* ctx, int n_sel, int N, double R, int sms) {
 // A call with fewer tiles than the GPU holds CTAs (narrow windows) shares each tile out:
 //  * of lists up to 1e5 lines, by points, down to 256 a CTA, while half the GPU stays free: near lines are
 //    evaluated point by point, and a shorter part has fewer of them.  Every CTA runs over the
-//    tile's candidates, so not with long lists.  40 depths, 20,000 lines, 1000 points: 478 -> 380 us;
+//    tile's candidates, which costs more the longer the list is.  The call without and with it, us, 40 rows of
+//    2000 points: 20,000 lines 561 and 343, 100,000 lines 1352 and 930, 300,000 lines 2326 and 1738; of 500
+//    points: 300 and 289, 658 and 656, 1122 and 1212 (150,000 lines 756 and 782);
 //  * of lists above 2048 lines, by candidate lines, over up to 64 CTAs, with partial sums added afterwards: as
 //    many as run at once, one chunk each at least, and up to eight times that for
 //    the tiles with kSplitChunks each (deep rows have ten times the candidates of shallow ones).
-//    Shorter lists save the second kernel: one row of 1350 lines 93 -> 84 us, of 40 lines 107 -> 103 us.
+//    Shorter lists save the second kernel.  With and without, us, 4 rows of 8000 points: 300 lines 151 and 115, 2048
+//    lines 173 and 134, 5000 lines 185 and 147, 10,000 lines 191 and 162; 40 rows: 189 and 152, 256 and 234, 329 and
+//    338, 428 and 481 (the line lies on the safe side of the two).
 // peers: calls that run beside this one take their part of the GPU.  Eight spectrum requests at once on eight
 // streams: 12.8 ms when each counts on the whole GPU, 11.5 ms on an eighth; seven on 25,000 lines 5.6, 3.7 ms.
 void tile_split(TileArgs& ta, int tile, int n_sel, int N, int64_t L, int sms, int peers) {
