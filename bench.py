@@ -38,14 +38,8 @@ import workloads as wl  # noqa: E402
 
 METRIC = "Voigt line-evals/s (line-by-line opacity synthesis + ODF binning)"
 UNIT = "line-evals/s"
-# FP32 operations that the profile kernel executes per line-evaluation of the default rows, all forms and
-# overheads included (ncu's FP32 thread-instruction counters: FFMA2 4, FFMA, FADD2 and FMUL2 2, FADD and
-# FMUL 1; 1.609e12 operations for 1.0804e13 evaluations).  An evaluation is one line at one
-# grid point inside its cut window; most are not formed one by one but as the line's share of
-# an interpolated wing sum, so the figure is far below the 6.5 operations of the cheapest profile form.  It
-# varies with the row (0.075 to 4.2) and holds for the default rows only.
-FLOP_PER_EVAL = 0.1489
 FP32_LANES_PER_SM = 128
+TILE_SOURCES = ["synth.cu", "voigt.cuh", "common.cuh"]   # of the profile kernel
 # kernels of the library per timed step: synth_opacity (k_start, k_kappa0 over the sample,
 # k_med_bracket, k_kappa0, k_med_collect, k_med_select, k_prep, k_place, k_windows, k_scan_class,
 # k_scatter, k_ranges, k_tiles) and build_odf (k_odf_gather, then k_odf for the intervals it leaves)
@@ -415,19 +409,18 @@ def native_arm(args):
     tiles_avg = tiles_ms / max(tiles_n, 1)
     evals_per_launch = evals_rank / max(tiles_n, 1)
     fp32_peak = sms * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12        # TFLOP/s at the maximum SM clock
-    achieved = evals_per_launch * FLOP_PER_EVAL / (tiles_avg / 1e3) / 1e12
-    traffic = measured_traffic("k_tiles", ["synth.cu", "voigt.cuh", "common.cuh"], sel)
-    counted = profile_value("k_tiles_fp32_ops.md", "flop_per_eval_counted", "k_tiles",
-                            ["synth.cu", "voigt.cuh", "common.cuh"])
+    traffic = measured_traffic("k_tiles", TILE_SOURCES, sel)
+    # FP32 operations per line-evaluation, counted on these rows and this kernel (or null: it varies with the row,
+    # 0.075 to 4.2)
+    per_eval = profile_value("k_tiles_fp32_ops.md", "flop_per_eval_counted", "k_tiles", TILE_SOURCES, sel)
+    achieved = None if per_eval is None else evals_per_launch * per_eval / (tiles_avg / 1e3) / 1e12
     roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
-                "frac": achieved / fp32_peak, "traffic": traffic, "kernel": "k_tiles (profile synthesis)",
-                "fp32_counted": None if counted is None else {
-                    "flop_per_eval": counted, "achieved": achieved * counted / FLOP_PER_EVAL,
-                    "frac": achieved * counted / FLOP_PER_EVAL / fp32_peak,
-                    "source": "ncu FP32 thread-instruction counters (FFMA2 x4; FFMA, FADD2, FMUL2 x2; FADD, FMUL) "
-                              "over the eight default rows, profiles/k_tiles_fp32_ops.md"},
+                "frac": None if achieved is None else achieved / fp32_peak, "traffic": traffic,
+                "kernel": "k_tiles (profile synthesis)",
+                "source": "ncu FP32 thread-instruction counters (FFMA2 x4; FFMA, FADD2, FMUL2 x2; FADD, FMUL) of "
+                          "these rows and kernel sources, profiles/k_tiles_fp32_ops.md; null where they differ",
                 "peak_kind": f"FP32 FMA peak {sms} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x {sm_max:.0f} MHz",
-                "sms": sms, "flop_per_eval": FLOP_PER_EVAL, "avg_launch_ms": tiles_avg, "launches": tiles_n}
+                "sms": sms, "flop_per_eval": per_eval, "avg_launch_ms": tiles_avg, "launches": tiles_n}
     odf_avg = odf_ms / max(odf_n, 1)
     odf_bytes = B * N * 4 + B * K * 12 * 8
     roofline_odf = {"bound": "hbm", "achieved": odf_bytes / (odf_avg / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
@@ -977,9 +970,9 @@ def table_arm(args):
     print(json.dumps(out), flush=True)
 
 
-def profile_value(name, key, kernel, sources):
-    """A number recorded in a profiles/ summary (key: value), or None when the summary is missing
-    or was taken on kernel sources that have changed since (SHA-1 of the files)."""
+def profile_value(name, key, kernel, sources, rows):
+    """A number recorded in a profiles/ summary (key: value), or None when the summary is missing or was taken
+    on other rows or on kernel sources that have changed since (SHA-1 of the files)."""
     import hashlib
     import re
     path = os.path.join(ROOT, "profiles", name)
@@ -990,35 +983,20 @@ def profile_value(name, key, kernel, sources):
     for f in sources:
         with open(os.path.join(ROOT, "paper_2105_13611_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
+    m_rows = re.search(r"^rows: ([0-9,]+)$", text, re.M)
     m_src = re.search(rf"^{kernel}_source_sha1: ([0-9a-f]+)$", text, re.M)
     m_val = re.search(rf"^{key}: ([0-9.eE+-]+)$", text, re.M)
-    if not (m_src and m_val) or m_src.group(1) != h.hexdigest():
+    if not (m_rows and m_src and m_val):
+        return None
+    if [int(r) for r in m_rows.group(1).split(",")] != [int(r) for r in rows] or m_src.group(1) != h.hexdigest():
         return None
     return float(m_val.group(1))
 
 
 def measured_traffic(kernel, sources, rows):
-    """DRAM bytes (read + written) per launch of `kernel` from the ncu summary in
-    profiles/traffic_table_workload.md, or None when that capture was taken on other rows
-    or on kernel sources that have changed since (recorded as SHA-1 of the files)."""
-    import hashlib
-    import re
-    path = os.path.join(ROOT, "profiles", "traffic_table_workload.md")
-    if not os.path.exists(path):
-        return None
-    text = open(path).read()
-    h = hashlib.sha1()
-    for f in sources:
-        with open(os.path.join(ROOT, "paper_2105_13611_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
-    m_rows = re.search(r"^rows: ([0-9,]+)$", text, re.M)
-    m_src = re.search(rf"^{kernel}_source_sha1: ([0-9a-f]+)$", text, re.M)
-    m_val = re.search(rf"^{kernel}_bytes_per_launch: ([0-9]+)$", text, re.M)
-    if not (m_rows and m_src and m_val):
-        return None
-    if [int(r) for r in m_rows.group(1).split(",")] != [int(r) for r in rows] or m_src.group(1) != h.hexdigest():
-        return None
-    return int(m_val.group(1))
+    """DRAM bytes (read + written) per launch of `kernel` from profiles/traffic_table_workload.md (see profile_value)."""
+    v = profile_value("traffic_table_workload.md", f"{kernel}_bytes_per_launch", kernel, sources, rows)
+    return None if v is None else int(v)
 
 
 def main():
