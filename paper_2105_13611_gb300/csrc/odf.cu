@@ -400,7 +400,8 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
     const int64_t b0 = bounds[k], b1 = bounds[k + 1];
     const long long n = b1 - b0;
     // this CTA's slice [x, x + nx) of the interval's n values
-    const long long per = (((n + C - 1) / C) + 3) & ~3ll, s0 = min(n, rank * per), nx = min(per, n - s0);
+    const long long per = CLUSTER ? (((n + C - 1) / C) + 3) & ~3ll : n, s0 = CLUSTER ? min(n, rank * per) : 0ll;
+    const long long nx = CLUSTER ? min(per, n - s0) : n;
     const float* x = kappa + (size_t)row * N + b0 + s0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // the targets as CTA 0 has them
