@@ -75,6 +75,7 @@ struct Target {
     unsigned long long iv_lt;    // exact sum (group units) of the group's values below the prefix range
     long long cnt_in;            // values inside the current prefix range
     unsigned prefix;             // bits resolved so far
+    int slot;                    // distinct-prefix slot at the current level (k_odf<false>)
     int total;                   // 1 when k >= n (S is the total)
 };
 
@@ -383,7 +384,9 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
     __shared__ unsigned long long gsum[256];
     __shared__ double gpre[257];
     __shared__ Target tg[kMaxTargets];          // CLUSTER: written by CTA 0 between two merges only, the others copy it
-    __shared__ int tslot[kMaxTargets];          // distinct-prefix slot of each target at the current level
+    // each target's slot at the current level; not in tg where other CTAs copy that (1 % slower with one CTA)
+    __shared__ int tslot[CLUSTER ? kMaxTargets : 1];
+    auto slot_at = [&](int t) -> int& { return CLUSTER ? tslot[CLUSTER ? t : 0] : tg[t].slot; };
     __shared__ unsigned dpre[kMaxTargets];
     __shared__ int n_distinct, n_cand;
     __shared__ unsigned s_zero;
@@ -554,7 +557,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
             const bool leader = act && first == lane;
             const unsigned lm = __ballot_sync(kFull, leader);
             const int slot = __popc(lm & ((1u << first) - 1u));
-            if (act) tslot[lane] = slot;
+            if (act) slot_at(lane) = slot;
             long long in = 0;
             if (leader) {
                 dpre[slot] = p;
@@ -639,7 +642,7 @@ __global__ void __launch_bounds__(kOdfThreads, ODF_MINB) k_odf(const float* __re
         for (int t = warp; t < nt && rank == 0; t += kOdfWarps) {
             if (tg[t].total) continue;
             Target tt = tg[t];
-            const int at = tslot[t] * kL2Bins;
+            const int at = (CLUSTER ? tslot[CLUSTER ? t : 0] : tt.slot) * kL2Bins;
             const Hist hs{h2.c + at, h2.hi + at, h2.lo + at};
             resolve_warp(tt, hs, wb, sh, lane);
             if (lane == 0) tg[t] = tt;
