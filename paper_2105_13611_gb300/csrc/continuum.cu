@@ -46,7 +46,7 @@ __global__ void k_cont_rows(int n_sel, const int* __restrict__ sel, int n_el, co
                             ContRow* __restrict__ out) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n_sel) return;
-    const double* row = pop + (size_t)sel[s] * pop_stride(n_el);
+    const double* row = pop + (size_t)(sel ? sel[s] : s) * pop_stride(n_el);
     const double T = row[kPopT], ne = row[kPopNe], nHI = row[kPopNHI], rho = row[kPopRho];
     const double kT = kKB * T, x = log(T / 5040.0);
     // partition functions of H I and H II at T (element 0 is hydrogen)

@@ -14,7 +14,7 @@ constexpr int kPrepLines = 1024;
 int populations_device(int n_el, const double* d_el, const double* d_abund, int n_comp, int n_points,
                        const double* d_T, const double* d_P, double* d_pop, cudaStream_t s);
 
-// Line-by-line opacity for rows d_sel of a population table onto the grid
+// Line-by-line opacity for rows d_sel of a population table (null: its first n_sel) onto the grid
 // (lam0_nm, R, N): kappa [n_sel][N], optional kappa_c [n_sel] and evaluation counts; peers: calls that
 // share the GPU with this one on other streams (synth.cu).
 int synth_rows(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, double lam0_nm, double R, int N,
@@ -47,7 +47,7 @@ int odf_setup();
 int odf_check(const char* who, int n_rows, int64_t N, int K, const int64_t* bounds, int n_steps,
               const double* widths, int mean_kind, double* cw);
 
-// Continuous opacity of rows d_sel of `pop` on the grid (lam0, R, N) from the MPSA_CONT_* sources
+// Continuous opacity of rows d_sel of `pop` (null: the first n_sel) on the grid (lam0, R, N) from the MPSA_CONT_* sources
 // into out [n_sel][N] (continuum.cu).
 int continuum_launch(mpsa_ctx* ctx, const double* pop, int n_sel, const int* d_sel, double lam0_nm, double R, int N,
                      int sources, float* out, cudaStream_t st);

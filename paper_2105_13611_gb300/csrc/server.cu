@@ -134,7 +134,7 @@ struct SpectrumBlock {
 
 size_t spectrum_bytes(const mpsa_server* s, const Req* r) {
     const int D = (int)r->m.size(), n_mu = (int)r->mu.size(), ne = s->ctx->n_el;
-    return SpectrumBlock(D, r->N, n_mu, ne, 28 * (size_t)D + 8 * ne + 4 * n_mu + 128).block.bytes +
+    return SpectrumBlock(D, r->N, n_mu, ne, 24 * (size_t)D + 8 * ne + 4 * n_mu + 128).block.bytes +
            chunks_bytes(s->ctx, D, r->rows, r->N, r->win.R, (int)s->slots.size()) + (1 << 20);
 }
 
@@ -151,18 +151,16 @@ int launch_spectrum(mpsa_server* s, Req* r, Slot& sl) {
     Scratch sc(st, s->ctx->pool);
     // the request's small inputs, in one copy
     std::vector<float> hm(D), hT(D), hmu(n_mu);
-    std::vector<int> hsel(D);
-    for (int d = 0; d < D; ++d) hm[d] = (float)r->m[d], hT[d] = (float)r->T[d], hsel[d] = d;
+    for (int d = 0; d < D; ++d) hm[d] = (float)r->m[d], hT[d] = (float)r->T[d];
     for (int q = 0; q < n_mu; ++q) hmu[q] = (float)r->mu[q];
     HostPack in;
     const size_t oT = in.add(r->T.data(), D), oP = in.add(r->P.data(), D);
     const size_t oab = in.add(c->h_abund.data() + (size_t)r->comp * ne, ne), om = in.add(hm.data(), D);
-    const size_t of = in.add(hT.data(), D), omu = in.add(hmu.data(), n_mu), osel = in.add(hsel.data(), D);
+    const size_t of = in.add(hT.data(), D), omu = in.add(hmu.data(), n_mu);
     SpectrumBlock q(D, N, n_mu, ne, in.data.size());
     int rc;
     if ((rc = q.block.take(sc))) return rc;
     MPSA_CUDA_TRY(cudaMemcpyAsync(q.in, in.data.data(), in.data.size(), cudaMemcpyHostToDevice, st));
-    const int* dsel = reinterpret_cast<int*>(q.in + osel);
     const float *fm = reinterpret_cast<float*>(q.in + om), *fT = reinterpret_cast<float*>(q.in + of),
                 *fmu = reinterpret_cast<float*>(q.in + omu);
     if ((rc = populations_device(ne, c->d_el, reinterpret_cast<double*>(q.in + oab), 1, D, reinterpret_cast<double*>(q.in + oT),
@@ -174,7 +172,7 @@ int launch_spectrum(mpsa_server* s, Req* r, Slot& sl) {
     // 2000 lines up to 5 nm and 5e5 lines up to 30 nm nothing.
     for (int off = 0; off < D; off += r->rows) {
         const int nrow = std::min(r->rows, D - off);
-        if ((rc = synth_rows(c, q.pop, nrow, dsel + off, r->win.lambda0_nm, r->win.R, N, q.kap + (size_t)off * N, q.kc + off,
+        if ((rc = synth_rows(c, q.pop + (size_t)off * pop_stride(ne), nrow, nullptr, r->win.lambda0_nm, r->win.R, N, q.kap + (size_t)off * N, q.kc + off,
                              nullptr, nullptr, st, (int)s->slots.size())))
             return rc;
     }

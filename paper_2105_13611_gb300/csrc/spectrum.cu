@@ -493,12 +493,11 @@ extern "C" int synth_spectrum(mpsa_ctx* ctx, const mpsa_atmos* atm, const mpsa_l
     const int ne = ctx->n_el;
     // the call's small inputs, in one copy
     std::vector<float> hm(D), hT(D), hmu(n_mu);
-    std::vector<int> hsel(D);
-    for (int d = 0; d < D; ++d) hm[d] = (float)atm->m[d], hT[d] = (float)atm->T[d], hsel[d] = d;
+    for (int d = 0; d < D; ++d) hm[d] = (float)atm->m[d], hT[d] = (float)atm->T[d];
     for (int q = 0; q < n_mu; ++q) hmu[q] = (float)mu[q];
     HostPack in;
     const size_t oT = in.add(atm->T, D), oP = in.add(atm->P, D), oab = in.add(ctx->h_abund.data() + (size_t)atm->comp * ne, ne);
-    const size_t om = in.add(hm.data(), D), of = in.add(hT.data(), D), omu = in.add(hmu.data(), n_mu), osel = in.add(hsel.data(), D);
+    const size_t om = in.add(hm.data(), D), of = in.add(hT.data(), D), omu = in.add(hmu.data(), n_mu);
     char* din;
     double* dpop;
     float *kap, *kc, *kcont = nullptr;
@@ -510,16 +509,15 @@ extern "C" int synth_spectrum(mpsa_ctx* ctx, const mpsa_atmos* atm, const mpsa_l
     if (cont) block.add(&kcont, (size_t)D * N);
     if ((r = block.take(sc))) return r;
     MPSA_CUDA_TRY(cudaMemcpyAsync(din, in.data.data(), in.data.size(), cudaMemcpyHostToDevice, st));
-    const int* dsel = reinterpret_cast<int*>(din + osel);
     const float *fm = reinterpret_cast<float*>(din + om), *fT = reinterpret_cast<float*>(din + of),
                 *fmu = reinterpret_cast<float*>(din + omu);
     if ((r = populations_device(ne, ctx->d_el, reinterpret_cast<double*>(din + oab), 1, D, reinterpret_cast<double*>(din + oT),
                                 reinterpret_cast<double*>(din + oP), dpop, st)))
         return r;
-    if ((r = synth_rows(ctx, dpop, D, dsel, win->lambda0_nm, win->R, N, kap, kc, nullptr, opts, st))) return r;
+    if ((r = synth_rows(ctx, dpop, D, nullptr, win->lambda0_nm, win->R, N, kap, kc, nullptr, opts, st))) return r;
     if (cont) {
         if (cont & ~MPSA_CONT_ALL) return fail(MPSA_EINVAL, "synth_spectrum: continuum = %d", cont);
-        if ((r = continuum_launch(ctx, dpop, D, dsel, win->lambda0_nm, win->R, N, cont, kcont, st))) return r;
+        if ((r = continuum_launch(ctx, dpop, D, nullptr, win->lambda0_nm, win->R, N, cont, kcont, st))) return r;
     }
     if ((r = formal_launch(D, N, kap, kc, kcont, fm, fT, win->lambda0_nm, log1p(1.0 / win->R), n_mu, fmu, I_out, st)))
         return r;

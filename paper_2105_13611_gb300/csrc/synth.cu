@@ -119,7 +119,7 @@ __device__ __forceinline__ void sp_consts(int t, const int* __restrict__ sel, in
                                           const double* __restrict__ pop, double vturb, int pop32,
                                           RowConst* __restrict__ rc, SpConst* __restrict__ sc) {
     const int s = t / n_sp, sp = t % n_sp;
-    const double* row = pop + (size_t)sel[s] * pop_stride(n_el);
+    const double* row = pop + (size_t)(sel ? sel[s] : s) * pop_stride(n_el);
     const double T = row[kPopT];
     const int e = sp_el[sp], st = sp_stage[sp];
     const double m = el[e * kElStride + kElMass] * kAMU;
@@ -1774,7 +1774,7 @@ __global__ void __launch_bounds__(256) k_tiles64(Tile64Args g) {
     const int s = blockIdx.y, tile = blockIdx.x, tid = threadIdx.x;
     const RowDesc r = row_desc(g.t, s);
     const int J0 = tile * TILE;
-    const double* row = g.pop + (size_t)g.sel[s] * g.pop_stride_;
+    const double* row = g.pop + (size_t)(g.sel ? g.sel[s] : s) * g.pop_stride_;
     const double T = row[kPopT], ne = row[kPopNe], nHI = row[kPopNHI], rho = row[kPopRho];
     const double tp = exp((double)*r.ln_tp);
     double nu[PTS], acc[PTS];

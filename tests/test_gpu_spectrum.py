@@ -101,3 +101,25 @@ def test_spectrum_parity_direction_counts(N, n_mu):
     se, ss = wl.species_table(w.n_metals)
     o, dI = spc.spectrum_at(L, se, ss, el, m, T, P, win, mus, js)
     assert np.all(np.abs(I[:, js] - o) <= 1e-4 * o + dI * 1.001)
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2, 3])
+@pytest.mark.parametrize("continuum", [0, 15])
+def test_depths_are_rows_of_the_call_itself(precision, continuum):
+    # the depths' rows are the call's own populations in order, in every precision and with the closed-form
+    # continuum (no list of rows goes to the device: a captured call would read it from host memory that is gone)
+    import torch
+    from paper_2105_13611_gb300 import binding
+    w = wl.config_tiny(n_lines=60, lam=(300.0, 300.5), R=5e5, seed=26)
+    ctx, L = gpu_context(w)
+    m, T, P = spc.grey_atmosphere(11, 5772.0, 4.44)
+    win = wl.Grid(300.1, 300.3, 5e5)
+    N = binding.grid_size(win.lam0_nm, win.lam1_nm, win.R)
+    I = torch.empty((len(MUS), N), device="cuda")
+    ctx.synth_spectrum(m, T, P, win, MUS, I, opts=binding.make_opts(1e-3, 1e-2, precision, continuum=continuum))
+    torch.cuda.synchronize()
+    el = wl.elements(w.n_metals)
+    se, ss = wl.species_table(w.n_metals)
+    src = ("elec", "bf", "ff", "ray") if continuum else None
+    o = spc.spectrum(L, se, ss, el, m, T, P, win, MUS, continuum=src)
+    assert np.abs(I.cpu().numpy() / o - 1).max() < 1e-4
