@@ -897,7 +897,9 @@ __global__ void __launch_bounds__(kPrepThreads, 3) k_windows(size_t ld, RowGrids
             if (lo <= hi) {
                 const int jlo = (int)lo, jhi = (int)hi;
                 int ilo = 1, ihi = 0;
-                if (vi >= 0.f) {
+                // (s_rel a beyond FP32, s_rel near e^88 and a > 2: no inner window, so that no level interpolates the
+                // line; its points multiply s_rel by H)
+                if (vi >= 0.f && srel * a < INFINITY) {
                     const float vi2 = vi * (1.f - 1e-5f);
                     long long ih = (long long)c + (long long)floorf(fminf(f + d_red(vi2, kv, lnq), 1.0e9f)) - 2;
                     long long il = (long long)c + (long long)ceilf(fmaxf(f - d_blue(vi2, kv, lnq), -1.0e9f)) + 2;
@@ -1036,9 +1038,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_scatter(size_t ld, RowGrids gr
             r.srel = o.srel[sL + t];
             r.jlo = w.x;
             r.jhi = w.y;
-            // s_rel a beyond FP32 (s_rel near e^88, a > 2): only the general form, which multiplies by H, may
-            // take the line, so no part of the grid counts as inside its window
-            r.in = r.srel * r.a < INFINITY ? pack_inner(w.x, w.y, w.z, w.w) : kNoInner;
+            r.in = pack_inner(w.x, w.y, w.z, w.w);
             len_sum += (unsigned long long)(w.y - w.x + 1);
             rec[sL + placed[warp][b] + lrank] = r;
             line[sL + placed[warp][b] + lrank] = i;
